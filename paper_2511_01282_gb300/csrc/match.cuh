@@ -1,0 +1,418 @@
+// match.cuh -- the part that rs_match_scan and rs_match_scan_indexed share:
+// one cluster of 8 CTAs (512 threads each) per request tests its candidate
+// positions against the key, counts and lists the matches in ascending order,
+// ranks those that clear theta_score and gathers the selected continuations.
+//
+// The candidates come from a source (every position of the buffer, or the
+// index's lists) in rows of 128: element e = 0..3 of lane l.  A warp tests
+// kRows rows at a time with all their loads in flight; the outcome is four
+// ballots per row, kept in shared memory (16 bytes per 128 candidates), so
+// that the ascending ranks come from one block scan of popcounts and no
+// candidate is tested twice.  A request with few rows is handled by CTA 0
+// alone (the other seven leave at once and no cluster barrier is used);
+// otherwise the rows are split in eighths, every CTA pushes its count to all
+// peers and its best top_c to CTA 0 through distributed shared memory, and
+// after the cluster barrier nobody touches another CTA's shared memory.
+//
+// What bounds it: a chain of dependent reads (offsets, key, candidates,
+// scores, spans) of about 0.5 us each, then for long buffers the reads of one
+// request's eight SMs (~100 GB/s per SM).
+#pragma once
+
+#include <cooperative_groups.h>
+#include <math.h>
+
+#include "common.cuh"
+
+namespace rs {
+
+constexpr int kMatCluster = 8;
+constexpr int kMatThreads = 512;
+constexpr int kMatWarps = kMatThreads / 32;
+constexpr int kMatCand = 512;       // matches ranked from the shared buffer
+constexpr int kMatBitRows = 4096;   // rows whose ballots a CTA keeps (524288 candidates)
+constexpr size_t kMatSmem = (size_t)kMatBitRows * 4 * sizeof(uint32_t);
+
+// (s, p) before (s2, p2): higher score first, then the more recent position
+__device__ __forceinline__ bool sp_before(float s, int p, float s2, int p2) {
+    return s > s2 || (s == s2 && p > p2);
+}
+
+// Rank of (s, p) among n distinct (score, position) pairs in shared memory:
+// the number of pairs before it in (score desc, position desc) order.
+__device__ __forceinline__ int sp_rank(float s, int p, const float *cs, const int *cp, int n) {
+    int r = 0;
+    for (int q = 0; q < n; ++q) r += sp_before(cs[q], cp[q], s, p);
+    return r;
+}
+
+struct MatShared {
+    float cs[kMatCand];  // matches with S >= theta_score (first kMatCand)
+    int cp[kMatCand];
+    int ccnt;
+    int warp_sums[kMatWarps];
+    float wv[kMatWarps];
+    int wp[kMatWarps];
+    long long peer_cnt[kMatCluster];           // match count of each CTA (pushed by its owner)
+    float peer_s[kMatCluster][RS_MAX_TOPC];    // CTA 0: each CTA's best top_c
+    int peer_p[kMatCluster][RS_MAX_TOPC];
+    int peer_n[kMatCluster];
+    float top_s[RS_MAX_TOPC];                  // this CTA's best top_c
+    int top_p[RS_MAX_TOPC];
+    int ntop;
+    int sel[RS_MAX_TOPC];
+};
+
+struct MatOut {
+    int32_t *count, *pos, *sel_pos, *sel_len, *spans, *n_sel, *status;
+    float theta_score;
+    int top_c, span_len, pos_cap;
+};
+
+// The request's token buffer and key, as both kernels read them first.
+struct MatReq {
+    const int32_t *X;
+    const float *S;
+    long long t;
+    int k, st;  // key length; status bits
+    bool run;
+    int key[RS_MAX_L];  // key[i] = X[t - k + i]
+    int k1, k2;         // its last token, and the one before (-1: none)
+};
+
+// ok: the caller's own condition for reading the request (its index is valid).
+__device__ __forceinline__ void mat_request(MatReq &q, const int32_t *__restrict__ tokens,
+                                            const int64_t *__restrict__ tok_off, const int32_t *__restrict__ k_star,
+                                            const uint8_t *__restrict__ gate_ok, const float *__restrict__ scores, int b,
+                                            int B, bool ok) {
+    const long long t0 = tok_off[b], t1 = tok_off[b + 1], tend = tok_off[B];
+    q.k = k_star[b];
+    const bool gate = gate_ok == nullptr || gate_ok[b] != 0;
+    q.t = t1 - t0;
+    // the buffers hold tok_off[B] tokens: a range outside them is not read
+    const bool off_ok = ok && t0 >= 0 && q.t >= 0 && t0 + q.t <= tend;
+    q.X = tokens + (off_ok ? t0 : 0);
+    q.S = scores + (off_ok ? t0 : 0);
+    q.st = off_ok ? 0 : RS_ST_BAD_OFFSET;
+    q.run = off_ok && q.k > 0 && gate;
+    if (q.run && q.k > RS_MAX_L) {
+        q.st = RS_ST_TOO_LARGE;
+        q.run = false;
+    }
+    if (q.run && (long long)q.k > q.t) q.run = false;
+#pragma unroll
+    for (int i = 0; i < RS_MAX_L; ++i) q.key[i] = (q.run && i < q.k) ? q.X[q.t - q.k + i] : -1;
+    q.k1 = q.run ? q.X[q.t - 1] : -1;
+    q.k2 = q.run && q.k > 1 ? q.X[q.t - 2] : -1;
+}
+
+// Whether the k - 1 tokens before position p (p >= k - 1) are the key's; every
+// load is issued before the first comparison.
+__device__ __forceinline__ bool mat_prefix(const MatReq &q, long long p) {
+    int v[RS_MAX_L];
+#pragma unroll
+    for (int j = 0; j < RS_MAX_L; ++j) v[j] = j < q.k - 1 ? q.X[p - (q.k - 1) + j] : -1;
+    bool m = true;
+#pragma unroll
+    for (int j = 0; j < RS_MAX_L; ++j) m &= j >= q.k - 1 || v[j] == q.key[j];
+    return m;
+}
+
+// Exclusive scan of one int per thread over the block; *total gets the sum.
+__device__ __forceinline__ int mat_excl_scan(int v, MatShared &sh, int *total) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) sh.warp_sums[warp] = x;
+    __syncthreads();
+    int before = 0, sum = 0;
+#pragma unroll
+    for (int w = 0; w < kMatWarps; ++w) {
+        const int y = sh.warp_sums[w];
+        before += w < warp ? y : 0;
+        sum += y;
+    }
+    __syncthreads();  // warp_sums reusable
+    *total = sum;
+    return before + x - v;
+}
+
+// Best head of the block's register lists; every thread gets it.
+__device__ __forceinline__ void mat_block_best(float hv, int hp, MatShared &sh, float *bv, int *bp) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const float ov = __shfl_xor_sync(0xffffffffu, hv, o);
+            const int op = __shfl_xor_sync(0xffffffffu, hp, o);
+            if (sp_before(ov, op, hv, hp)) {
+                hv = ov;
+                hp = op;
+            }
+        }
+        if (r == 0) {
+            if (lane == 0) {
+                sh.wv[warp] = hv;
+                sh.wp[warp] = hp;
+            }
+            __syncthreads();
+            hv = lane < kMatWarps ? sh.wv[lane] : -INFINITY;
+            hp = lane < kMatWarps ? sh.wp[lane] : -1;
+        }
+    }
+    __syncthreads();  // wv / wp reusable
+    *bv = hv;
+    *bp = hp;
+}
+
+// The tests of a source's rows [r0, r0 + kRows) by one warp: this lane's hits,
+// bit 4 u + e for element e of row r0 + u; rows at or past `end` give none.
+// The warp's ballots go to bits[4 (r0 - base) ..] (rows below cap only).
+template <class Src>
+__device__ __forceinline__ uint32_t mat_rows(const Src &src, const MatReq &q, long long r0, long long end,
+                                             uint32_t *bits, long long base) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t hits = src.test(q, r0, end, lane);
+    uint32_t mine = 0;
+#pragma unroll
+    for (int j = 0; j < 4 * Src::kRows; ++j) {
+        const uint32_t bal = __ballot_sync(0xffffffffu, (hits >> j) & 1u);
+        mine = lane == j ? bal : mine;
+    }
+    if (lane < 4 * Src::kRows && r0 - base + (lane >> 2) < kMatBitRows) bits[4 * (r0 - base) + lane] = mine;
+    return hits;
+}
+
+// The whole of a request once its source is known (see the file comment).
+// rows: candidate rows; solo: CTA 0 alone handles them.
+template <class Src>
+__device__ __forceinline__ void mat_body(const Src &src, const MatReq &q, long long rows, bool solo, int b, int crank,
+                                         MatShared &sh, uint32_t *bits, const MatOut &o) {
+    namespace cg = cooperative_groups;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int top_c = o.top_c, pos_cap = o.pos_cap;
+    if (!solo) cluster_arrive_relaxed();  // this CTA runs; the wait sits before the first push
+    const long long per = solo ? rows : (rows + kMatCluster - 1) / kMatCluster;
+    const long long lo = solo ? 0 : (per * crank < rows ? per * crank : rows);
+    const long long hi = lo + per < rows ? lo + per : rows;
+    if (tid == 0) sh.ccnt = 0;
+    __syncthreads();
+
+    // ---- every candidate once: ballots, count, the matches that clear theta ----
+    float ls[RS_MAX_TOPC];  // this thread's best (used when more match than the buffer holds)
+    int lp[RS_MAX_TOPC];
+#pragma unroll
+    for (int i = 0; i < RS_MAX_TOPC; ++i) {
+        ls[i] = -INFINITY;
+        lp[i] = -1;
+    }
+    int cnt = 0;
+    for (long long r0 = lo + warp * Src::kRows; r0 < hi; r0 += kMatWarps * Src::kRows) {
+        uint32_t rem = mat_rows(src, q, r0, hi, bits, lo);
+        cnt += __popc(rem);
+        while (rem) {
+            const int j = __ffs(rem) - 1;
+            rem &= rem - 1;
+            const int p = src.pos(r0 + (j >> 2), lane, j & 3);
+            const float s = q.S[p];
+            if (!(s >= o.theta_score)) continue;
+            const int slot = atomicAdd(&sh.ccnt, 1);
+            if (slot < kMatCand) {
+                sh.cs[slot] = s;
+                sh.cp[slot] = p;
+            }
+            if (sp_before(s, p, ls[RS_MAX_TOPC - 1], lp[RS_MAX_TOPC - 1])) {
+                float cs = s;
+                int cp = p;
+#pragma unroll
+                for (int i = 0; i < RS_MAX_TOPC; ++i) {
+                    if (sp_before(cs, cp, ls[i], lp[i])) {
+                        const float ts = ls[i];
+                        const int tp = lp[i];
+                        ls[i] = cs;
+                        lp[i] = cp;
+                        cs = ts;
+                        cp = tp;
+                    }
+                }
+            }
+        }
+    }
+    int cta_total = 0;
+    (void)mat_excl_scan(cnt, sh, &cta_total);
+    // the CTA's best top_c: rank every buffered match by counting
+    const int ncand = sh.ccnt;
+    if (ncand <= kMatCand) {
+        for (int e = tid; e < ncand; e += kMatThreads) {
+            const float sv = sh.cs[e];
+            const int pv = sh.cp[e];
+            const int r = sp_rank(sv, pv, sh.cs, sh.cp, ncand);
+            if (r < top_c) {
+                sh.top_s[r] = sv;
+                sh.top_p[r] = pv;
+            }
+        }
+        if (tid == 0) sh.ntop = ncand < top_c ? ncand : top_c;
+    } else {
+        int ntop = 0;
+        for (int c = 0; c < top_c; ++c) {
+            float bv;
+            int bp;
+            mat_block_best(ls[0], lp[0], sh, &bv, &bp);
+            if (bp < 0) break;
+            if (tid == 0) {
+                sh.top_s[c] = bv;
+                sh.top_p[c] = bp;
+            }
+            ntop = c + 1;
+            if (lp[0] == bp) {  // the owner pops its head
+#pragma unroll
+                for (int i = 0; i < RS_MAX_TOPC - 1; ++i) {
+                    ls[i] = ls[i + 1];
+                    lp[i] = lp[i + 1];
+                }
+                ls[RS_MAX_TOPC - 1] = -INFINITY;
+                lp[RS_MAX_TOPC - 1] = -1;
+            }
+        }
+        if (tid == 0) sh.ntop = ntop;
+    }
+
+    // ---- the slice's global rank (pushed counts) ----
+    long long offset = 0, total = cta_total;
+    __syncthreads();  // this CTA's top list is complete
+    if (!solo) {
+        cg::cluster_group cluster = cg::this_cluster();
+        cluster_wait();  // every CTA of the cluster is running
+        if (tid < kMatCluster) *cluster.map_shared_rank(&sh.peer_cnt[crank], tid) = cta_total;
+        if (tid < RS_MAX_TOPC && tid < sh.ntop) {
+            *cluster.map_shared_rank(&sh.peer_s[crank][tid], 0) = sh.top_s[tid];
+            *cluster.map_shared_rank(&sh.peer_p[crank][tid], 0) = sh.top_p[tid];
+        }
+        if (tid == 0) *cluster.map_shared_rank(&sh.peer_n[crank], 0) = sh.ntop;
+        cluster_arrive_release();  // every push is visible after the wait
+        cluster_wait();
+        total = 0;
+        for (int r = 0; r < kMatCluster; ++r) {
+            const long long c = sh.peer_cnt[r];
+            if (r < crank) offset += c;
+            total += c;
+        }
+    }
+
+    // ---- positions in ascending order: the kept ballots, then (slices of more
+    // rows than are kept) further rows tested again ----
+    long long base = offset;
+    int32_t *pos = o.pos + (long long)b * pos_cap;
+    for (long long w0 = lo; w0 < hi && base < pos_cap; w0 += kMatBitRows) {
+        const int nr = (int)(hi - w0 < kMatBitRows ? hi - w0 : kMatBitRows);
+        if (w0 != lo) {
+            __syncthreads();  // the previous rows are consumed
+            for (long long r0 = w0 + warp * Src::kRows; r0 < w0 + nr; r0 += kMatWarps * Src::kRows)
+                (void)mat_rows(src, q, r0, w0 + nr, bits, w0);
+            __syncthreads();
+        }
+        const int mr = (nr + kMatThreads - 1) / kMatThreads;  // consecutive rows per thread
+        const int a = tid * mr < nr ? tid * mr : nr, z = a + mr < nr ? a + mr : nr;
+        int n = 0;
+        for (int r = a; r < z; ++r) {
+            const uint4 w = *reinterpret_cast<const uint4 *>(bits + 4 * r);
+            n += __popc(w.x) + __popc(w.y) + __popc(w.z) + __popc(w.w);
+        }
+        int wtotal = 0;
+        long long idx = base + mat_excl_scan(n, sh, &wtotal);
+        if (n) {
+            for (int r = a; r < z && idx < pos_cap; ++r) {
+                const uint4 w = *reinterpret_cast<const uint4 *>(bits + 4 * r);
+                if (Src::kLaneMajor) {
+                    uint32_t any = w.x | w.y | w.z | w.w;
+                    while (any) {
+                        const int l = __ffs(any) - 1;
+                        any &= any - 1;
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const uint32_t we = e == 0 ? w.x : e == 1 ? w.y : e == 2 ? w.z : w.w;
+                            if ((we >> l) & 1u) {
+                                if (idx < pos_cap) pos[idx] = src.pos(w0 + r, l, e);
+                                ++idx;
+                            }
+                        }
+                    }
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        uint32_t we = e == 0 ? w.x : e == 1 ? w.y : e == 2 ? w.z : w.w;
+                        while (we) {
+                            const int l = __ffs(we) - 1;
+                            we &= we - 1;
+                            if (idx < pos_cap) pos[idx] = src.pos(w0 + r, l, e);
+                            ++idx;
+                        }
+                    }
+                }
+            }
+        }
+        base += wtotal;
+    }
+    if (crank != 0) return;
+
+    // ---- CTA 0: merge the per-CTA lists, selection outputs ----
+    const long long stored = total < pos_cap ? total : pos_cap;
+    for (long long i = stored + tid; i < pos_cap; i += kMatThreads) pos[i] = -1;
+    int nsel;
+    if (solo) {
+        nsel = sh.ntop;
+        if (tid < nsel) sh.sel[tid] = sh.top_p[tid];  // already ranked
+    } else {
+        // the cluster's candidates (at most kMatCluster * RS_MAX_TOPC), ranked by counting
+        float *ms = sh.cs;  // reused: the CTA's own buffer is no longer needed
+        int *mp = sh.cp;
+        int nm = 0;
+        for (int r = 0; r < kMatCluster; ++r) {
+            const int n = sh.peer_n[r];
+            if (tid < n) {
+                ms[nm + tid] = sh.peer_s[r][tid];
+                mp[nm + tid] = sh.peer_p[r][tid];
+            }
+            nm += n;
+        }
+        __syncthreads();
+        if (tid < nm) {
+            const int r = sp_rank(ms[tid], mp[tid], ms, mp, nm);
+            if (r < top_c) sh.sel[r] = mp[tid];
+        }
+        nsel = nm < top_c ? nm : top_c;
+    }
+    __syncthreads();
+    for (int i = tid; i < top_c * o.span_len; i += kMatThreads) {
+        const int c = i / o.span_len, j = i - c * o.span_len;
+        int v = -1;
+        if (c < nsel) {
+            const long long p = sh.sel[c];
+            if (j < q.t - 1 - p) v = q.X[p + 1 + j];
+        }
+        o.spans[(long long)b * top_c * o.span_len + i] = v;
+    }
+    if (tid < top_c) {
+        int sp = -1, sl = 0;
+        if (tid < nsel) {
+            sp = sh.sel[tid];
+            const long long len = q.t - 1 - sp;
+            sl = (int)(len > o.span_len ? o.span_len : len);
+        }
+        o.sel_pos[(long long)b * top_c + tid] = sp;
+        o.sel_len[(long long)b * top_c + tid] = sl;
+    }
+    if (tid == 0) {
+        o.count[b] = (int32_t)total;
+        o.n_sel[b] = nsel;
+        o.status[b] = q.st | (total > pos_cap ? RS_ST_TRUNCATED : 0);
+    }
+}
+
+}  // namespace rs

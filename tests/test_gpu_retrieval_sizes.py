@@ -1,0 +1,72 @@
+"""The retrieval kernels at the edges of their splits, bit for bit against the
+oracle: buffers that start at every offset from a 16-byte boundary, one
+round of a single CTA and one position more, more candidates than a CTA keeps
+ballots for and more matches than the ranking buffer holds."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from gpu_helpers import f32
+from paper_2511_01282_gb300 import respec as rs
+from test_gpu_index import _cuda
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import __graft_entry__
+    __graft_entry__.build()
+    assert torch.cuda.is_available()
+
+
+def _buffers(rng, lens, V, k):
+    tok_off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    tokens = rng.integers(0, V, int(tok_off[-1])).astype(np.int32)
+    for b, t in enumerate(lens):
+        a = int(tok_off[b])
+        if t > 4 * k + 8:  # the key at both ends of the buffer and in between
+            for q in [k - 1, t - 2 - k] + rng.integers(k, t - k, 3).tolist():
+                tokens[a + q - k + 1:a + q + 1] = tokens[a + t - k:a + t]
+    return tokens, tok_off
+
+
+def _scan(tokens, tok_off, ks, scores, theta, top_c, span_len, pos_cap):
+    B = len(tok_off) - 1
+    z = lambda *shape: torch.full(shape, -7, dtype=torch.int32, device="cuda")  # noqa: E731
+    out = dict(count=z(B), pos=z(B, pos_cap), sel_pos=z(B, top_c), sel_len=z(B, top_c), spans=z(B, top_c, span_len),
+               n_sel=z(B), status=z(B))
+    p = rs.params(theta_score=theta, top_c=top_c, span_len=span_len)
+    rs.rs_match_scan(_cuda(tokens), _cuda(tok_off), B, _cuda(ks), None, _cuda(scores), p, pos_cap, out["count"], out["pos"],
+                     out["sel_pos"], out["sel_len"], out["spans"], out["n_sel"], out["status"])
+    torch.cuda.synchronize()
+    ref = oracle.match_scan(tokens, tok_off, ks, scores, f32(theta), top_c, span_len, pos_cap, gate_ok=None)
+    for key, got in out.items():
+        assert (got.cpu().numpy() == ref[key]).all(), key
+    return ref
+
+
+@pytest.mark.parametrize("k", [1, 2, 3, 8])
+@pytest.mark.parametrize("V", [3, 400])
+def test_scan_alignments_and_round_edges(k, V):
+    # request lengths of 1 mod 4 walk through every alignment; 16384 candidate
+    # positions are one round of one CTA
+    rng = np.random.default_rng(100 * k + V)
+    lens = [1, 5, 129, 2049, 16381, 16385, 16389, 33, 8193, 17, 20001]
+    tokens, tok_off = _buffers(rng, lens, V, k)
+    scores = rng.random(len(tokens)).astype(np.float32)
+    scores[rng.random(len(tokens)) < 0.2] = 0.5
+    for pos_cap in (0, 1, 700):
+        _scan(tokens, tok_off, np.full(len(lens), k, np.int32), scores, 0.3, 3, 8, pos_cap)
+
+
+def test_scan_beyond_the_kept_ballots():
+    # 8 x 4096 rows x 128 positions = 4194304: the last rows are tested again
+    # for their positions, which the capacity reaches only with few matches
+    rng = np.random.default_rng(7)
+    tokens, tok_off = _buffers(rng, [3, 4194304 + 70001], 50000, 2)
+    scores = rng.random(len(tokens)).astype(np.float32)
+    ref = _scan(tokens, tok_off, np.array([1, 1], np.int32), scores, 0.3, 8, 4, 300)
+    assert 20 < ref["count"][1] < 300
+    _scan(tokens, tok_off, np.array([0, 2], np.int32), scores, 0.3, 8, 4, 300)
