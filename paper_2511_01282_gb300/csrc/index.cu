@@ -10,12 +10,15 @@
 // instead of O(t); an append touches O(appended tokens).
 //
 // Layout of the index (per request b, sizes from rs_match_index_bytes):
-//   start[b][0 .. V+1]  bucket offsets: the positions holding token v are
-//                       bucket[start[v] .. start[v] + len[v]) in ascending
-//                       order; ids outside [0, V) share bucket V
-//                       (verification compares the real tokens).  Bucket v
-//                       has room for count_v + count_v / 4 + 2 entries
-//                       (count_v: occurrences at build time);
+//   first[b][0 .. V+1]  number of build-time tokens with an id below v (ids
+//                       outside [0, V) count as id V, the last bucket;
+//                       verification compares the real tokens), first[V + 1] =
+//                       t_b.  Bucket v holds the ascending positions of id v:
+//                       list slots start(v) .. start(v) + len[v) with
+//                       start(v) = first[v] + first[v] / 4 + 2 v, so bucket v
+//                       has room for at least count_v + count_v / 4 + 2
+//                       entries (count_v: occurrences at build time) and no
+//                       prefix over the rooms is needed;
 //   len[b][0 .. V]      entries in each bucket;
 //   list (per request, at base[b]): kOvf overflow slots, then the buckets.
 //                       A position whose bucket is full goes to the overflow
@@ -26,64 +29,73 @@
 //                       left out when the overflow list was full) are tested
 //                       one by one (a linear tail).
 // base[b] = tok_off[b] + tok_off[b] / 4 + b (2 (V + 1) + kOvf) at build time:
-// request b's share is at least t_b + t_b / 4 + 2 (V + 1) + kOvf slots, which
-// holds every bucket's room (sum of count_v / 4 <= t_b / 4).
+// a bound that telescopes over the requests (start(V + 1) <= t_b + t_b / 4 +
+// 2 (V + 1)).
 //
-// Build: every token's key (request, bucket) is sorted with a stable LSD
-// radix sort (8-bit digits; per 4096-key tile a histogram, a two-level scan
-// of the digit x tile counts, then a stable scatter that ranks each key within
-// its tile by warp match and per-warp digit counters), so every bucket's
-// positions come out ascending; a last pass places each sorted position at
-// its bucket's start plus its rank.  All of it is parallel over the tokens
-// of all requests.
+// Build: the (request, bucket) keys of all tokens are sorted, with their
+// positions, by a stable LSD radix sort over all requests at once (digits of
+// at most 9 bits, so 18-bit keys -- 128K ids, one request -- take two
+// passes).  A pass is three kernels: the digit counts of every tile of keys,
+// their offsets, and the stable scatter, which ranks a tile's keys by warp
+// match and per-warp counters, orders the tile in shared memory and writes
+// whole runs of equal digits.  first[] is then a binary search per bucket in
+// the sorted keys (no atomics: counting buckets with them made a text's most
+// common tokens the bottleneck, 270 of 700 us for 4 x 1M tokens), and the
+// last kernel moves each sorted position to its bucket's slots.  A pass over
+// 4M tokens reads 32 MB and writes 32 MB in L2 and takes ~46 us cold (counts
+// 10, offsets 7.5, scatter 27-31, bound by the ballots and the 64-byte runs).
+// Build, four appends and four queries on 4 x 1M tokens: 1018 -> 150 us in a
+// graph; build, eight appends and eight queries on 4 x 32K: 242 -> 97 us.
 // Append: one CTA per request takes the new positions in rounds of 256; each
 // position's rank among the round's positions of its bucket gives its slot
 // after the bucket's entries; full buckets spill to the overflow list in
 // position order; if that is full too, indexing stops at the first such
 // position (it and every later one stay in the linear tail, and the status
 // word says so).
-// Query: one CTA per request walks the candidates in rounds of 1024 (bucket,
-// overflow list, then tail), verifies them, writes matches at their ascending
-// rank (block scan of the round's hits) and ranks the matches that clear
-// theta_score by counting, as the scan does.
-#include <math.h>
+// Query: the candidates (the key's last token's bucket, the overflow list,
+// then the tail) are tested by one cluster per request as match.cuh
+// describes (70K candidates for a text's most common token: 79-120 us with one
+// CTA, 10.8 so; a handful: 10.4 -> 8.8, the chain of reads).
+#include "match.cuh"
 
 #include <algorithm>
-
-#include "common.cuh"
 
 namespace rs {
 namespace {
 
-constexpr int kIdxThreads = 1024;
-constexpr int kQryThreads = 256;
-constexpr int kQryRound = 1024;          // candidates per query round (4 per thread)
-constexpr int kQryCand = 256;            // matches ranked from the shared buffer
 constexpr int kOvf = 4096;               // overflow slots per request
-constexpr int kRadixBins = 256;          // 8-bit digits
-constexpr int kTile = 4096;              // keys per radix tile
-constexpr int kRadixThreads = 256;       // 8 warps x 512 keys per tile
+constexpr int kMaxDigitBits = 9;
+constexpr int kMaxBins = 1 << kMaxDigitBits;
+constexpr int kRadixThreads = 256;
+constexpr int kRadixWarps = kRadixThreads / 32;
 constexpr int kAppThreads = 256;         // positions per append round
+
+// Keys per tile: 4096, or 1024 for builds of at most kSmallBuild tokens, whose
+// 4096-key tiles would leave most SMs idle (4 x 32K tokens: 32 tiles).
+constexpr int kTileRounds = 16, kTileRoundsSmall = 4;
+constexpr long long kSmallBuild = 1 << 19;
+inline int tile_rounds(long long t_total) { return t_total <= kSmallBuild ? kTileRoundsSmall : kTileRounds; }
+inline long long n_tiles(long long t_total) {
+    const long long tile = (long long)tile_rounds(t_total) * kRadixThreads;
+    return (t_total + tile - 1) / tile;
+}
 
 struct IndexView {
     int32_t *valid;         // 1 when the build's offsets were consistent (else the index holds nothing)
     int64_t *built, *base;  // per request: positions indexed, first list slot
     int32_t *ovf_n;         // per request: overflow entries
-    int32_t *start;         // [B][V + 2]
+    int32_t *first;         // [B][V + 2]
     int32_t *len;           // [B][V + 1]
     int32_t *list;
     // build scratch
-    int32_t *sstart;        // [B][V + 1]: exclusive prefix of the bucket counts
-    uint32_t *key[2];
-    int32_t *val[2];
-    int32_t *hist;          // [kRadixBins][ntiles]
-    int32_t *dtot;          // [kRadixBins]
+    uint2 *pair[2];         // (key, position) of every token
+    int32_t *hist;          // [ntiles][bins]
+    int32_t *dtot;          // [kMaxBins]
 };
 
 inline long long list_slots(int B, int V, long long t_total) {
     return t_total + t_total / 4 + (long long)B * (2ll * (V + 1) + kOvf);
 }
-inline long long n_tiles(long long t_total) { return (t_total + kTile - 1) / kTile; }
 
 // Carves the index (and its build scratch) out of `base`; returns the bytes used.
 inline size_t carve_index(void *base, int B, int V, long long t_total, IndexView *v) {
@@ -92,16 +104,13 @@ inline size_t carve_index(void *base, int B, int V, long long t_total, IndexView
     v->built = cv.take<int64_t>((size_t)B);
     v->base = cv.take<int64_t>((size_t)B);
     v->ovf_n = cv.take<int32_t>((size_t)B);
-    v->start = cv.take<int32_t>((size_t)B * (V + 2));
+    v->first = cv.take<int32_t>((size_t)B * (V + 2));
     v->len = cv.take<int32_t>((size_t)B * (V + 1));
     v->list = cv.take<int32_t>((size_t)list_slots(B, V, t_total));
-    v->sstart = cv.take<int32_t>((size_t)B * (V + 1));
-    v->key[0] = cv.take<uint32_t>((size_t)t_total);
-    v->key[1] = cv.take<uint32_t>((size_t)t_total);
-    v->val[0] = cv.take<int32_t>((size_t)t_total);
-    v->val[1] = cv.take<int32_t>((size_t)t_total);
-    v->hist = cv.take<int32_t>((size_t)kRadixBins * n_tiles(t_total));
-    v->dtot = cv.take<int32_t>((size_t)kRadixBins);
+    v->pair[0] = cv.take<uint2>((size_t)t_total);
+    v->pair[1] = cv.take<uint2>((size_t)t_total);
+    v->hist = cv.take<int32_t>((size_t)kMaxBins * n_tiles(t_total));
+    v->dtot = cv.take<int32_t>((size_t)kMaxBins);
     return cv.used();
 }
 inline size_t index_bytes(int B, int V, long long t_total) {
@@ -116,272 +125,320 @@ inline int bits_for(long long n) {  // smallest b with n < 2^b
 }
 
 __device__ __forceinline__ int bucket_of(int tok, int V) { return (tok >= 0 && tok < V) ? tok : V; }
-__device__ __forceinline__ int room_of(int count) { return count + count / 4 + 2; }
+__device__ __forceinline__ long long start_of(int first, int v) { return (long long)first + first / 4 + 2ll * v; }
 
 // (0) the build's offsets: tok_off[0] = 0, ascending, tok_off[B] = t_total;
 // every later build kernel does nothing unless they are
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(1024)
 index_check(const int64_t *__restrict__ tok_off, int B, long long t_total, IndexView ix) {
     pdl_enter();
-    __shared__ int s_bad;
-    if (threadIdx.x == 0) s_bad = tok_off[0] != 0 || tok_off[B] != t_total;
-    __syncthreads();
-    for (int b = threadIdx.x; b < B; b += blockDim.x)
-        if (tok_off[b + 1] < tok_off[b]) s_bad = 1;
-    __syncthreads();
-    if (threadIdx.x == 0) *ix.valid = s_bad ? 0 : 1;
+    int bad = threadIdx.x == 0 && (tok_off[0] != 0 || tok_off[B] != t_total);
+    for (int b = threadIdx.x; b < B; b += blockDim.x) bad |= tok_off[b + 1] < tok_off[b];
+    bad = __syncthreads_or(bad);
+    if (threadIdx.x == 0) *ix.valid = bad ? 0 : 1;
 }
 
-// (1) per request: zero the bucket counts, record the request's extent
-__global__ void __launch_bounds__(256)
-index_init(const int64_t *__restrict__ tok_off, int V, IndexView ix) {
+// The keys of a pass: pass 0 makes them from the tokens (the request of token
+// i is the last b with tok_off[b] <= i), later passes read the pairs.
+struct TokenKeys {
+    const int32_t *tokens;
+    const int64_t *tok_off;
+    int B, V, vbits;
+    int b0;        // the request of the tile's first token
+    long long b1;  // where that request ends
+    __device__ __forceinline__ int request(long long i) const {
+        int lo = 0, hi = B - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (tok_off[mid] <= i) lo = mid;
+            else hi = mid - 1;
+        }
+        return lo;
+    }
+    __device__ __forceinline__ void tile(long long i0) {
+        b0 = request(i0);
+        b1 = tok_off[b0 + 1];
+    }
+    // the load, apart from what is made of it, so that a thread's loads are all
+    // in flight before any is used
+    __device__ __forceinline__ int load(long long i) const { return tokens[i]; }
+    __device__ __forceinline__ uint2 pair(int tok, long long i) const {
+        const int b = i < b1 ? b0 : request(i);
+        const uint32_t k = (uint32_t)bucket_of(tok, V) | (vbits >= 32 ? 0u : ((uint32_t)b << vbits));
+        return make_uint2(k, (uint32_t)i);
+    }
+};
+struct PairKeys {
+    const uint2 *in;
+    __device__ __forceinline__ void tile(long long) {}
+    __device__ __forceinline__ uint2 load(long long i) const { return in[i]; }
+    __device__ __forceinline__ uint2 pair(uint2 x, long long) const { return x; }
+};
+
+// Each radix kernel handles one tile of kR * 256 keys; a thread's keys are all
+// loaded before any is used.
+template <class Keys, int kR>
+__global__ void __launch_bounds__(kRadixThreads)
+radix_hist(Keys src, long long N, int shift, int bins, int32_t *__restrict__ hist, const int32_t *__restrict__ valid) {
+    pdl_enter();
+    if (!*valid) return;
+    __shared__ int cnt[kMaxBins];
+    const long long tile = blockIdx.x, i0 = tile * (kR * kRadixThreads);
+    for (int d = threadIdx.x; d < bins; d += kRadixThreads) cnt[d] = 0;
+    decltype(src.load(0)) x[kR];
+#pragma unroll
+    for (int q = 0; q < kR; ++q) {
+        const long long i = i0 + q * kRadixThreads + threadIdx.x;
+        x[q] = src.load(i < N ? i : i0);
+    }
+    src.tile(i0);
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < kR; ++q) {
+        const long long i = i0 + q * kRadixThreads + threadIdx.x;
+        if (i < N) atomicAdd(&cnt[(src.pair(x[q], i).x >> shift) & (bins - 1)], 1);
+    }
+    __syncthreads();
+    for (int d = threadIdx.x; d < bins; d += kRadixThreads) hist[tile * bins + d] = cnt[d];
+}
+
+// The exclusive sum over the block of one value per thread.
+__device__ __forceinline__ int radix_excl_scan(int v, int *s_w, int *total) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) s_w[warp] = x;
+    __syncthreads();
+    int before = 0, sum = 0;
+#pragma unroll
+    for (int w = 0; w < kRadixWarps; ++w) {
+        const int y = s_w[w];
+        before += w < warp ? y : 0;
+        sum += y;
+    }
+    __syncthreads();
+    *total = sum;
+    return before + x - v;
+}
+
+// (tile, digit) offsets: each digit's exclusive prefix over the tiles, and
+// its total.  A block takes eight digits (one 32-byte sector of a tile's
+// counts); thread (group g, digit d) takes eight consecutive tiles a round.
+constexpr int kOffDigits = 8, kOffTiles = 8;
+__global__ void __launch_bounds__(kRadixThreads)
+radix_offsets(int32_t *__restrict__ hist, long long ntiles, int bins, int32_t *__restrict__ dtot,
+              const int32_t *__restrict__ valid) {
+    pdl_enter();
+    if (!*valid) return;
+    constexpr int kGroups = kRadixThreads / kOffDigits;
+    __shared__ int s_sum[kGroups][kOffDigits + 1];
+    const int d = threadIdx.x % kOffDigits, g = threadIdx.x / kOffDigits;
+    int32_t *col = hist + blockIdx.x * kOffDigits + d;
+    const bool live = (int)blockIdx.x * kOffDigits + d < bins;
+    int carry = 0;
+    for (long long base = 0; base < ntiles; base += kGroups * kOffTiles) {
+        const long long t = base + g * kOffTiles;
+        int c[kOffTiles], sum = 0;
+#pragma unroll
+        for (int q = 0; q < kOffTiles; ++q) c[q] = live && t + q < ntiles ? col[(t + q) * bins] : 0;
+#pragma unroll
+        for (int q = 0; q < kOffTiles; ++q) sum += c[q];
+        s_sum[g][d] = sum;
+        __syncthreads();
+        int x = carry;
+#pragma unroll
+        for (int h = 0; h < kGroups; ++h) {
+            const int y = s_sum[h][d];
+            x += h < g ? y : 0;
+            carry += y;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < kOffTiles; ++q) {
+            if (live && t + q < ntiles) col[(t + q) * bins] = x;
+            x += c[q];
+        }
+    }
+    if (live && g == 0) dtot[blockIdx.x * kOffDigits + d] = carry;
+}
+
+// The stable scatter.  Warp w takes keys w 32 kR .. of the tile, 32 at a time;
+// a key's rank is the count of equal digits before it in the tile (earlier
+// warps, earlier rounds of its warp, lower lanes of its round).  The tile is
+// put in digit order in shared memory and leaves from there, so that equal
+// digits -- consecutive addresses -- are written by neighbouring threads.
+template <class Keys, int kR>
+__global__ void __launch_bounds__(kRadixThreads, 3)
+radix_scatter(Keys src, uint2 *__restrict__ out, long long N, int shift, int bins,
+              const int32_t *__restrict__ hist, const int32_t *__restrict__ dtot, const int32_t *__restrict__ valid) {
+    pdl_enter();
+    if (!*valid) return;
+    constexpr int kTile = kR * kRadixThreads;
+    __shared__ uint2 s_pair[kTile];
+    __shared__ uint16_t s_cnt[kRadixWarps][kMaxBins];
+    __shared__ int s_dst[kMaxBins];  // global index of the digit's first key, less its place in the tile
+    __shared__ int s_w[kRadixWarps];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const long long tile = blockIdx.x, i0 = tile * kTile;
+    const int n = (int)(N - i0 < kTile ? N - i0 : kTile);
+    decltype(src.load(0)) x[kR];
+#pragma unroll
+    for (int q = 0; q < kR; ++q) {
+        const int e = warp * (32 * kR) + q * 32 + lane;
+        x[q] = src.load(i0 + (e < n ? e : 0));
+    }
+    src.tile(i0);
+    // this thread's digits 2 tid and 2 tid + 1 (bins is even): where the tile's
+    // keys of each begin, within the digit and over all digits
+    int2 g = make_int2(0, 0), tot = make_int2(0, 0);
+    if (2 * tid < bins) {
+        g = *reinterpret_cast<const int2 *>(hist + tile * bins + 2 * tid);
+        tot = *reinterpret_cast<const int2 *>(dtot + 2 * tid);
+    }
+    for (int x = tid; x < kRadixWarps * kMaxBins / 2; x += kRadixThreads) reinterpret_cast<uint32_t *>(&s_cnt[0][0])[x] = 0;
+    uint2 k[kR];
+#pragma unroll
+    for (int q = 0; q < kR; ++q) {
+        const int e = warp * (32 * kR) + q * 32 + lane;
+        k[q] = e < n ? src.pair(x[q], i0 + e) : make_uint2(0u, 0u);
+    }
+    int all;
+    const int below = radix_excl_scan(tot.x + tot.y, s_w, &all);  // ends with a barrier
+    g.x += below;
+    g.y += below + tot.x;
+    const unsigned lt = (1u << lane) - 1u;
+    int rk[kR];
+#pragma unroll
+    for (int q = 0; q < kR; ++q) {
+        const bool ok = warp * (32 * kR) + q * 32 + lane < n;
+        const int dg = (int)((k[q].x >> shift) & (bins - 1));
+        // the lanes of this round with the same digit, one ballot per bit
+        // (match.any is slow where a round holds many distinct digits: first
+        // pass over 4 x 1M tokens 47.2 us with it, 31.2 so; second pass, few
+        // distinct digits, 25.7 against 27.4)
+        unsigned peers = __ballot_sync(0xffffffffu, ok);
+#pragma unroll
+        for (int bit = 0; bit < kMaxDigitBits; ++bit) {
+            const bool one = (dg >> bit) & 1;
+            const unsigned bal = __ballot_sync(0xffffffffu, one);
+            peers &= one ? bal : ~bal;
+        }
+        const int before = ok ? s_cnt[warp][dg] : 0;
+        __syncwarp();
+        if (ok && (peers & lt) == 0) s_cnt[warp][dg] = (uint16_t)(before + __popc(peers));
+        __syncwarp();
+        rk[q] = before + __popc(peers & lt);
+    }
+    __syncthreads();
+    {  // each digit's counts over the warps, then over the digits
+        int run[2] = {0, 0};
+#pragma unroll
+        for (int w = 0; w < kRadixWarps; ++w) {
+            uint32_t *p = reinterpret_cast<uint32_t *>(&s_cnt[w][2 * tid]);
+            const uint32_t c = *p;
+            *p = (uint32_t)run[0] | ((uint32_t)run[1] << 16);
+            run[0] += (int)(c & 0xffffu);
+            run[1] += (int)(c >> 16);
+        }
+        int total;
+        const int x = radix_excl_scan(run[0] + run[1], s_w, &total);
+        s_dst[2 * tid] = g.x - x;
+        s_dst[2 * tid + 1] = g.y - (x + run[0]);
+        // the counters become places in the ordered tile
+#pragma unroll
+        for (int w = 0; w < kRadixWarps; ++w) {
+            uint32_t *p = reinterpret_cast<uint32_t *>(&s_cnt[w][2 * tid]);
+            const uint32_t c = *p;
+            *p = ((c & 0xffffu) + (uint32_t)x) | (((c >> 16) + (uint32_t)(x + run[0])) << 16);
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < kR; ++q) {
+        if (warp * (32 * kR) + q * 32 + lane < n) {
+            const int dg = (int)((k[q].x >> shift) & (bins - 1));
+            s_pair[s_cnt[warp][dg] + rk[q]] = k[q];
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < kR; ++q) {
+        const int e = q * kRadixThreads + tid;
+        if (e < n) {
+            const uint2 v = s_pair[e];
+            out[(long long)s_dst[(v.x >> shift) & (bins - 1)] + e] = v;
+        }
+    }
+}
+static_assert(kMaxBins == 2 * kRadixThreads, "two digits per thread");
+static_assert(kTileRounds * kRadixThreads <= 65535, "16-bit tile counters");
+
+// first[b][v]: where the keys of (b, v) begin in the sorted order, by binary
+// search; the lengths are the differences.  Blocks of 256 threads cover 255
+// buckets (the last thread only serves its neighbour).
+constexpr int kFirstPer = 255;
+__global__ void __launch_bounds__(kFirstPer + 1)
+index_first(const uint2 *__restrict__ sorted, const int64_t *__restrict__ tok_off, int V, int vbits, IndexView ix) {
     pdl_enter();
     if (!*ix.valid) return;
-    const int b = blockIdx.y;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < V + 1; i += stride)
-        ix.len[(long long)b * (V + 1) + i] = 0;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        const long long o = tok_off[b];
-        ix.built[b] = tok_off[b + 1] - o;
-        ix.base[b] = o + o / 4 + (long long)b * (2ll * (V + 1) + kOvf);
+    __shared__ int s_first[kFirstPer + 1];
+    const int b = blockIdx.y, tid = threadIdx.x;
+    const long long v = (long long)blockIdx.x * kFirstPer + tid;
+    const long long t0 = tok_off[b], t1 = tok_off[b + 1];
+    int f = (int)(t1 - t0);
+    if (v <= V) {
+        const uint32_t key = (uint32_t)v | (vbits >= 32 ? 0u : ((uint32_t)b << vbits));
+        long long lo = t0, hi = t1;  // first key >= (b, v)
+        while (lo < hi) {
+            const long long mid = (lo + hi) >> 1;
+            if (sorted[mid].x < key) lo = mid + 1;
+            else hi = mid;
+        }
+        f = (int)(lo - t0);
+    }
+    s_first[tid] = f;
+    __syncthreads();
+    if (tid < kFirstPer && v <= V + 1) {
+        ix.first[(long long)b * (V + 2) + v] = f;
+        if (v <= V) ix.len[(long long)b * (V + 1) + v] = s_first[tid + 1] - f;
+    }
+    if (blockIdx.x == 0 && tid == 0) {
+        ix.built[b] = t1 - t0;
+        ix.base[b] = t0 + t0 / 4 + (long long)b * (2ll * (V + 1) + kOvf);
         ix.ovf_n[b] = 0;
     }
 }
 
-// (2) count every bucket and write each token's sort key (request, bucket)
-// and its global position
+// Each sorted position into its bucket: its rank among the request's
+// positions of that bucket is its sorted index minus the bucket's first.
+constexpr int kPlacePer = 4;
 __global__ void __launch_bounds__(256)
-index_count(const int32_t *__restrict__ tokens, const int64_t *__restrict__ tok_off, int V, int vbits,
+index_place(const uint2 *__restrict__ sorted, long long N, const int64_t *__restrict__ tok_off, int V, int vbits,
             IndexView ix) {
     pdl_enter();
     if (!*ix.valid) return;
-    const int b = blockIdx.y;
-    int32_t *cnt = ix.len + (long long)b * (V + 1);
-    const long long t0 = tok_off[b], t = tok_off[b + 1] - t0;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < t; i += stride) {
-        const int bk = bucket_of(tokens[t0 + i], V);
-        atomicAdd(&cnt[bk], 1);
-        ix.key[0][t0 + i] = ((uint32_t)b << vbits) | (uint32_t)bk;
-        ix.val[0][t0 + i] = (int32_t)(t0 + i);
-    }
-}
-
-// (3) per request: bucket starts (prefix of the rooms) and the sorted starts
-// (prefix of the counts); len keeps the counts.  Each thread takes kOffPer
-// consecutive buckets, so one round of the block covers 8192 of them.
-constexpr int kOffPer = 8;
-__global__ void __launch_bounds__(kIdxThreads)
-index_offsets(int V, IndexView ix) {
-    pdl_enter();
-    if (!*ix.valid) return;
-    __shared__ int s_w[2][kIdxThreads / 32];
-    __shared__ int s_carry[2];
-    const int b = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int32_t *cnt = ix.len + (long long)b * (V + 1);
-    int32_t *start = ix.start + (long long)b * (V + 2);
-    int32_t *sstart = ix.sstart + (long long)b * (V + 1);
-    if (threadIdx.x < 2) s_carry[threadIdx.x] = 0;
-    __syncthreads();
-    for (int base = 0; base < V + 1; base += kIdxThreads * kOffPer) {
-        const int i0 = base + threadIdx.x * kOffPer;
-        int c[kOffPer];
-        int r0 = 0, r1 = 0;  // this thread's rooms and counts
-#pragma unroll
-        for (int q = 0; q < kOffPer; ++q) {
-            c[q] = i0 + q < V + 1 ? cnt[i0 + q] : 0;
-            r0 += i0 + q < V + 1 ? room_of(c[q]) : 0;
-            r1 += c[q];
-        }
-        int x0 = r0, x1 = r1;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y0 = __shfl_up_sync(0xffffffffu, x0, o), y1 = __shfl_up_sync(0xffffffffu, x1, o);
-            if (lane >= o) {
-                x0 += y0;
-                x1 += y1;
-            }
-        }
-        if (lane == 31) {
-            s_w[0][warp] = x0;
-            s_w[1][warp] = x1;
-        }
-        __syncthreads();
-        int b0 = 0, b1 = 0, t0s = 0, t1s = 0;
-        for (int w = 0; w < kIdxThreads / 32; ++w) {
-            b0 += w < warp ? s_w[0][w] : 0;
-            b1 += w < warp ? s_w[1][w] : 0;
-            t0s += s_w[0][w];
-            t1s += s_w[1][w];
-        }
-        int e0 = s_carry[0] + b0 + x0 - r0, e1 = s_carry[1] + b1 + x1 - r1;
-#pragma unroll
-        for (int q = 0; q < kOffPer; ++q) {
-            if (i0 + q < V + 1) {
-                start[i0 + q] = e0;
-                sstart[i0 + q] = e1;
-                e0 += room_of(c[q]);
-                e1 += c[q];
-            }
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            s_carry[0] += t0s;
-            s_carry[1] += t1s;
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) start[V + 1] = s_carry[0];
-}
-
-// (4) radix sort passes: tile histograms ...
-__global__ void __launch_bounds__(kRadixThreads)
-radix_hist(const uint32_t *__restrict__ key, long long N, int shift, long long ntiles, int32_t *__restrict__ hist,
-           const int32_t *__restrict__ valid) {
-    pdl_enter();
-    if (!*valid) return;
-    __shared__ int cnt[kRadixBins];
-    const long long tile = blockIdx.x;
-    cnt[threadIdx.x] = 0;
-    __syncthreads();
-    for (int e = threadIdx.x; e < kTile; e += kRadixThreads) {
-        const long long i = tile * kTile + e;
-        if (i < N) atomicAdd(&cnt[(key[i] >> shift) & (kRadixBins - 1)], 1);
-    }
-    __syncthreads();
-    hist[(long long)threadIdx.x * ntiles + tile] = cnt[threadIdx.x];
-}
-
-// ... each digit's total over the tiles ...
-__global__ void __launch_bounds__(kRadixThreads)
-radix_total(const int32_t *__restrict__ hist, long long ntiles, int32_t *__restrict__ dtot,
-            const int32_t *__restrict__ valid) {
-    pdl_enter();
-    if (!*valid) return;
-    __shared__ int s_w[kRadixThreads / 32];
-    const int d = blockIdx.x;
-    int sum = 0;
-    for (long long t = threadIdx.x; t < ntiles; t += kRadixThreads) sum += hist[(long long)d * ntiles + t];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5] = sum;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int tot = 0;
-        for (int w = 0; w < kRadixThreads / 32; ++w) tot += s_w[w];
-        dtot[d] = tot;
-    }
-}
-
-// ... (digit, tile) offsets: the digits below d, then the tiles before t ...
-__global__ void __launch_bounds__(kRadixThreads)
-radix_offsets(int32_t *__restrict__ hist, long long ntiles, const int32_t *__restrict__ dtot,
-              const int32_t *__restrict__ valid) {
-    pdl_enter();
-    if (!*valid) return;
-    __shared__ int s_w[kRadixThreads / 32];
-    __shared__ int s_carry;
-    const int d = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (threadIdx.x == 0) {
-        int c = 0;
-        for (int e = 0; e < d; ++e) c += dtot[e];
-        s_carry = c;
-    }
-    __syncthreads();
-    for (long long base = 0; base < ntiles; base += kRadixThreads) {
-        const long long t = base + threadIdx.x;
-        const int v = t < ntiles ? hist[(long long)d * ntiles + t] : 0;
-        int x = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31) s_w[warp] = x;
-        __syncthreads();
-        int before = 0, sum = 0;
-        for (int w = 0; w < kRadixThreads / 32; ++w) {
-            before += w < warp ? s_w[w] : 0;
-            sum += s_w[w];
-        }
-        if (t < ntiles) hist[(long long)d * ntiles + t] = s_carry + before + x - v;
-        __syncthreads();
-        if (threadIdx.x == 0) s_carry += sum;
-        __syncthreads();
-    }
-}
-
-// ... and the stable scatter: warp w takes keys w*512 .. w*512 + 511 of the
-// tile, 32 at a time; a key's rank is the count of equal digits before it in
-// the tile (earlier warps, earlier rounds of its warp, lower lanes of its round)
-__global__ void __launch_bounds__(kRadixThreads)
-radix_scatter(const uint32_t *__restrict__ kin, const int32_t *__restrict__ vin, uint32_t *__restrict__ kout,
-              int32_t *__restrict__ vout, long long N, int shift, long long ntiles, const int32_t *__restrict__ hist,
-              const int32_t *__restrict__ valid) {
-    pdl_enter();
-    if (!*valid) return;
-    constexpr int kWarps = kRadixThreads / 32;
-    constexpr int kRounds = kTile / kRadixThreads;
-    __shared__ int wcnt[kWarps][kRadixBins];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const long long tile = blockIdx.x;
-    for (int i = threadIdx.x; i < kWarps * kRadixBins; i += kRadixThreads) (&wcnt[0][0])[i] = 0;
-    __syncthreads();
-    uint32_t k[kRounds];
-    int v[kRounds], rk[kRounds], dg[kRounds];
-    const unsigned lt = (1u << lane) - 1u;
-#pragma unroll
-    for (int q = 0; q < kRounds; ++q) {
-        const long long i = tile * kTile + warp * (kTile / kWarps) + q * 32 + lane;
-        const bool ok = i < N;
-        k[q] = ok ? kin[i] : 0u;
-        v[q] = ok ? vin[i] : 0;
-        dg[q] = ok ? (int)((k[q] >> shift) & (kRadixBins - 1)) : kRadixBins + lane;  // padding: a digit of its own
-        const unsigned peers = __match_any_sync(0xffffffffu, dg[q]);
-        const int base = ok ? wcnt[warp][dg[q]] : 0;
-        __syncwarp();
-        if (ok && (peers & lt) == 0) wcnt[warp][dg[q]] = base + __popc(peers);
-        __syncwarp();
-        rk[q] = ok ? base + __popc(peers & lt) : -1;
-    }
-    __syncthreads();
-    {  // exclusive prefix of each digit's counts over the warps
-        const int d = threadIdx.x;
-        int run = 0;
-#pragma unroll
-        for (int w = 0; w < kWarps; ++w) {
-            const int c = wcnt[w][d];
-            wcnt[w][d] = run;
-            run += c;
-        }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < kRounds; ++q) {
-        if (rk[q] < 0) continue;
-        const long long dst = (long long)hist[(long long)dg[q] * ntiles + tile] + wcnt[warp][dg[q]] + rk[q];
-        kout[dst] = k[q];
-        vout[dst] = v[q];
-    }
-}
-
-// (5) each sorted position into its bucket: its rank among the request's
-// positions of that bucket is its sorted index minus the bucket's sorted start
-__global__ void __launch_bounds__(256)
-index_place(const uint32_t *__restrict__ key, const int32_t *__restrict__ val, long long N,
-            const int64_t *__restrict__ tok_off, int V, int vbits, IndexView ix) {
-    pdl_enter();
-    if (!*ix.valid) return;
-    const long long stride = (long long)gridDim.x * blockDim.x;
     const uint32_t vmask = (vbits >= 32) ? 0xffffffffu : ((1u << vbits) - 1u);
-    for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < N; j += stride) {
-        const uint32_t kk = key[j];
-        const int b = (int)(vbits >= 32 ? 0 : (kk >> vbits));
-        const int bk = (int)(kk & vmask);
+    const long long j0 = (long long)blockIdx.x * (256 * kPlacePer) + threadIdx.x;
+    uint2 p[kPlacePer];
+    int f[kPlacePer];
+#pragma unroll
+    for (int q = 0; q < kPlacePer; ++q) p[q] = j0 + 256 * q < N ? sorted[j0 + 256 * q] : make_uint2(0u, 0u);
+#pragma unroll
+    for (int q = 0; q < kPlacePer; ++q) {
+        const int b = (int)(vbits >= 32 ? 0 : (p[q].x >> vbits));
+        f[q] = ix.first[(long long)b * (V + 2) + (p[q].x & vmask)];
+    }
+#pragma unroll
+    for (int q = 0; q < kPlacePer; ++q) {
+        const long long j = j0 + 256 * q;
+        if (j >= N) break;
+        const int b = (int)(vbits >= 32 ? 0 : (p[q].x >> vbits));
         const long long t0 = tok_off[b];
-        const long long rank = j - t0 - ix.sstart[(long long)b * (V + 1) + bk];
-        ix.list[ix.base[b] + kOvf + ix.start[(long long)b * (V + 2) + bk] + rank] = (int32_t)(val[j] - t0);
+        ix.list[ix.base[b] + kOvf + start_of(f[q], (int)(p[q].x & vmask)) + (j - t0 - f[q])] = (int32_t)((long long)p[q].y - t0);
     }
 }
 
@@ -406,7 +463,7 @@ index_append(const int32_t *__restrict__ tokens, const int64_t *__restrict__ tok
         return;
     }
     const int32_t *X = tokens + t0;
-    int32_t *start = ix.start + (long long)b * (V + 2);
+    const int32_t *first = ix.first + (long long)b * (V + 2);
     int32_t *len = ix.len + (long long)b * (V + 1);
     int32_t *ovf = ix.list + ix.base[b];
     int32_t *buckets = ovf + kOvf;
@@ -420,10 +477,13 @@ index_append(const int32_t *__restrict__ tokens, const int64_t *__restrict__ tok
         s_bk[tid] = bk;
         if (tid == 0) s_cut = t;
         __syncthreads();
-        int rank = 0;
-        for (int j = 0; j < tid; ++j) rank += s_bk[j] == bk;
         const int lo = valid ? len[bk] : 0;
-        const int room = valid ? start[bk + 1] - start[bk] : 0;
+        const int f0 = valid ? first[bk] : 0, f1 = valid ? first[bk + 1] : 0;
+        const long long start = start_of(f0, valid ? bk : 0);
+        const int room = valid ? (f1 - f0) + (f1 - f0) / 4 + 2 : 0;
+        const int nr = (int)(t - r0 < kAppThreads ? t - r0 : kAppThreads);  // positions of this round
+        int rank = 0;
+        for (int j = 0; j < tid && j < nr; ++j) rank += s_bk[j] == bk;
         const int slot = lo + rank;
         const bool inb = valid && slot < room;
         const bool ov = valid && !inb;
@@ -447,14 +507,14 @@ index_append(const int32_t *__restrict__ tokens, const int64_t *__restrict__ tok
         const long long cut = s_cut;
         const bool in = valid && p < cut;
         s_ok[tid] = (unsigned char)(in && inb);
-        if (in && inb) buckets[start[bk] + slot] = (int32_t)p;
+        if (in && inb) buckets[start + slot] = (int32_t)p;
         if (in && ov) ovf[oslot] = (int32_t)p;
         if (tid == 0) s_novf = 0;
         __syncthreads();
         // the last indexed position of a bucket in this round sets its length
         if (in && inb) {
             bool last = true;
-            for (int j = tid + 1; j < kAppThreads; ++j)
+            for (int j = tid + 1; j < nr; ++j)
                 if (s_bk[j] == bk && s_ok[j]) last = false;
             if (last) len[bk] = slot + 1;
         }
@@ -476,228 +536,81 @@ index_append(const int32_t *__restrict__ tokens, const int64_t *__restrict__ tok
     }
 }
 
-// (s, p) before (s2, p2): higher score first, then the more recent position
-__device__ __forceinline__ bool sp_before(float s, int p, float s2, int p2) {
-    return s > s2 || (s == s2 && p > p2);
-}
+// Query candidates, ascending: the bucket of the key's last token, the
+// overflow list (every token's overflow entries are newer than its bucket's),
+// then the positions not indexed (built .. t - 2); row r's element e of lane l
+// is candidate 128 r + 32 e + l.
+struct ListSource {
+    static constexpr int kRows = 2;
+    static constexpr bool kLaneMajor = false;
+    const int32_t *blist, *olist;
+    long long nb, no, ncand, tail0;
+    __device__ __forceinline__ int cand(long long c) const {
+        if (c < nb) return blist[c];
+        if (c < nb + no) return olist[c - nb];
+        return (int)(tail0 + (c - nb - no));
+    }
+    __device__ __forceinline__ int pos(long long row, int lane, int e) const { return cand(128 * row + 32 * e + lane); }
+    __device__ __forceinline__ uint32_t test(const MatReq &q, long long r0, long long end, int lane) const {
+        int p[4 * kRows], x0[4 * kRows], x1[4 * kRows];
+#pragma unroll
+        for (int j = 0; j < 4 * kRows; ++j) {
+            const long long c = 128 * (r0 + (j >> 2)) + 32 * (j & 3) + lane;
+            p[j] = r0 + (j >> 2) < end && c < ncand ? cand(c) : -1;
+        }
+#pragma unroll
+        for (int j = 0; j < 4 * kRows; ++j) {
+            const bool in = p[j] >= q.k - 1 && (long long)p[j] <= q.t - 2;
+            if (!in) p[j] = -1;
+            x0[j] = in ? q.X[p[j]] : 0;
+            x1[j] = in && q.k > 1 ? q.X[p[j] - 1] : 0;
+        }
+        const int kl = q.k1, k2 = q.k2;
+        uint32_t hits = 0;
+#pragma unroll
+        for (int j = 0; j < 4 * kRows; ++j)
+            if (p[j] >= 0 && x0[j] == kl && (q.k < 2 || x1[j] == k2)) hits |= 1u << j;
+        if (q.k > 2) {
+#pragma unroll
+            for (int j = 0; j < 4 * kRows; ++j)
+                if (((hits >> j) & 1u) && !mat_prefix(q, p[j])) hits &= ~(1u << j);
+        }
+        return hits;
+    }
+};
 
-__global__ void __launch_bounds__(kQryThreads)
+// One round of CTA 0's warps; longer candidate lists are split over the cluster.
+constexpr long long kQrySoloRows = kMatWarps * ListSource::kRows;
+
+__global__ void __cluster_dims__(kMatCluster, 1, 1) __launch_bounds__(kMatThreads)
 index_query(const int32_t *__restrict__ tokens, const int64_t *__restrict__ tok_off, int V,
             const int32_t *__restrict__ k_star, const uint8_t *__restrict__ gate_ok,
-            const float *__restrict__ scores, float theta_score, int top_c, int span_len, int pos_cap,
-            IndexView ix, int32_t *__restrict__ count, int32_t *__restrict__ pos, int32_t *__restrict__ sel_pos,
-            int32_t *__restrict__ sel_len, int32_t *__restrict__ spans, int32_t *__restrict__ n_sel,
-            int32_t *__restrict__ status) {
+            const float *__restrict__ scores, IndexView ix, MatOut o) {
     pdl_enter();
-    constexpr int kPer = kQryRound / kQryThreads;
-    __shared__ int s_key[RS_MAX_L];
-    __shared__ int s_w[kQryThreads / 32];
-    __shared__ float s_cs[kQryCand];
-    __shared__ int s_cp[kQryCand];
-    __shared__ int s_ccnt;
-    __shared__ float s_bv[kQryThreads / 32];
-    __shared__ int s_bp[kQryThreads / 32];
-    __shared__ int s_sel[RS_MAX_TOPC];
-    __shared__ int s_nsel;
-    const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const long long t0 = tok_off[b];
-    const long long t = tok_off[b + 1] - t0;
-    // an index whose build saw inconsistent offsets holds nothing, and the
-    // buffers hold tok_off[B] tokens: otherwise the request is not read
-    const bool off_ok = *ix.valid && t0 >= 0 && t >= 0 && t0 + t <= tok_off[gridDim.x];
-    const int32_t *X = tokens + (off_ok ? t0 : 0);
-    const float *S = scores + (off_ok ? t0 : 0);
-    const int k = k_star[b];
-    int st = off_ok ? 0 : RS_ST_BAD_OFFSET;
-    bool run = off_ok && k > 0 && (gate_ok == nullptr || gate_ok[b] != 0);
-    if (run && k > RS_MAX_L) {
-        st = RS_ST_TOO_LARGE;
-        run = false;
+    __shared__ MatShared sh;
+    extern __shared__ __align__(16) uint32_t qry_bits[];
+    const int crank = (int)cooperative_groups::this_cluster().block_rank();
+    const int b = blockIdx.y;
+    // an index whose build saw inconsistent offsets holds nothing: the request is not read
+    const long long built = ix.built[b], base = ix.base[b];  // read beside the request's own records
+    const int novf = ix.ovf_n[b];
+    MatReq q;
+    mat_request(q, tokens, tok_off, k_star, gate_ok, scores, b, gridDim.y, *ix.valid != 0);
+    ListSource src{nullptr, nullptr, 0, 0, 0, q.t};
+    if (q.run) {
+        const int bk = bucket_of(q.k1, V);
+        src.olist = ix.list + base;
+        src.blist = src.olist + kOvf + start_of(ix.first[(long long)b * (V + 2) + bk], bk);
+        src.nb = ix.len[(long long)b * (V + 1) + bk];
+        src.no = novf;
+        src.tail0 = built < q.t ? built : q.t;
+        const long long nt = q.t - 1 - src.tail0;  // tail: positions tail0 .. t - 2
+        src.ncand = src.nb + src.no + (nt > 0 ? nt : 0);
     }
-    if (run && (long long)k > t) run = false;
-    if (run && tid < k) s_key[tid] = X[t - k + tid];
-    if (tid == 0) s_ccnt = 0;
-    __syncthreads();
-    int key[RS_MAX_L];
-#pragma unroll
-    for (int i = 0; i < RS_MAX_L; ++i) key[i] = (run && i < k) ? s_key[i] : 0;
-    // candidates, ascending: the bucket of the key's last token, the overflow
-    // list (every token's overflow entries are newer than its bucket's), then
-    // the positions not indexed (built .. t - 2)
-    long long nb = 0, no = 0, tail0 = t;
-    const int32_t *blist = nullptr, *olist = nullptr;
-    if (run) {
-        const int bk = bucket_of(key[k - 1], V);
-        olist = ix.list + ix.base[b];
-        blist = olist + kOvf + ix.start[(long long)b * (V + 2) + bk];
-        nb = ix.len[(long long)b * (V + 1) + bk];
-        no = ix.ovf_n[b];
-        const long long built = ix.built[b];
-        tail0 = built < t ? built : t;
-    }
-    const long long nt = run ? (t - 1) - tail0 : 0;  // tail: positions tail0 .. t-2
-    const long long ncand = nb + no + (nt > 0 ? nt : 0);
-
-    float ls[RS_MAX_TOPC];
-    int lp[RS_MAX_TOPC];
-#pragma unroll
-    for (int i = 0; i < RS_MAX_TOPC; ++i) {
-        ls[i] = -INFINITY;
-        lp[i] = -1;
-    }
-    long long total = 0;  // matches so far (the next match's rank)
-    for (long long c0 = 0; c0 < ncand; c0 += kQryRound) {
-        int cp[kPer];
-        bool hit[kPer];
-        int nh = 0;
-#pragma unroll
-        for (int q = 0; q < kPer; ++q) {  // candidate c0 + kPer * tid + q, in order
-            const long long c = c0 + (long long)kPer * tid + q;
-            cp[q] = -1;
-            if (c < nb) cp[q] = blist[c];
-            else if (c < nb + no) cp[q] = olist[c - nb];
-            else if (c < ncand) cp[q] = (int)(tail0 + (c - nb - no));
-        }
-#pragma unroll
-        for (int q = 0; q < kPer; ++q) {
-            const int p = cp[q];
-            bool m = p >= k - 1 && (long long)p <= t - 2;
-            if (m) {
-                for (int i = 0; i < k; ++i) m = m && (X[p - i] == key[k - 1 - i]);
-            }
-            hit[q] = m;
-            nh += m;
-        }
-        // ascending rank of this thread's hits in the round
-        int x = nh;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31) s_w[warp] = x;
-        __syncthreads();
-        int before = 0, sum = 0;
-#pragma unroll
-        for (int w = 0; w < kQryThreads / 32; ++w) {
-            const int y = s_w[w];
-            before += w < warp ? y : 0;
-            sum += y;
-        }
-        __syncthreads();
-        long long r = total + before + x - nh;
-#pragma unroll
-        for (int q = 0; q < kPer; ++q) {
-            if (!hit[q]) continue;
-            const int p = cp[q];
-            if (r < pos_cap) pos[(long long)b * pos_cap + r] = p;
-            ++r;
-            const float s = S[p];
-            if (!(s >= theta_score)) continue;
-            const int slot = atomicAdd(&s_ccnt, 1);
-            if (slot < kQryCand) {
-                s_cs[slot] = s;
-                s_cp[slot] = p;
-            }
-            if (sp_before(s, p, ls[RS_MAX_TOPC - 1], lp[RS_MAX_TOPC - 1])) {
-                float cs = s;
-                int cq = p;
-#pragma unroll
-                for (int i = 0; i < RS_MAX_TOPC; ++i)
-                    if (sp_before(cs, cq, ls[i], lp[i])) {
-                        const float ts = ls[i];
-                        const int tq = lp[i];
-                        ls[i] = cs;
-                        lp[i] = cq;
-                        cs = ts;
-                        cq = tq;
-                    }
-            }
-        }
-        total += sum;
-    }
-    __syncthreads();
-    // the best top_c: rank the buffered matches by counting, else merge the per-thread lists
-    const int nc = s_ccnt;
-    if (nc <= kQryCand) {
-        for (int e = tid; e < nc; e += kQryThreads) {
-            int rk = 0;
-            for (int q = 0; q < nc; ++q) rk += sp_before(s_cs[q], s_cp[q], s_cs[e], s_cp[e]);
-            if (rk < top_c) s_sel[rk] = s_cp[e];
-        }
-        if (tid == 0) s_nsel = nc < top_c ? nc : top_c;
-    } else {
-        int nsel = 0;
-        for (int c = 0; c < top_c; ++c) {
-            float hv = ls[0];
-            int hp = lp[0];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const float ov = __shfl_xor_sync(0xffffffffu, hv, o);
-                const int op = __shfl_xor_sync(0xffffffffu, hp, o);
-                if (sp_before(ov, op, hv, hp)) {
-                    hv = ov;
-                    hp = op;
-                }
-            }
-            if (lane == 0) {
-                s_bv[warp] = hv;
-                s_bp[warp] = hp;
-            }
-            __syncthreads();
-            hv = s_bv[0];
-            hp = s_bp[0];
-            for (int w = 1; w < kQryThreads / 32; ++w)
-                if (sp_before(s_bv[w], s_bp[w], hv, hp)) {
-                    hv = s_bv[w];
-                    hp = s_bp[w];
-                }
-            __syncthreads();
-            if (hp < 0) break;
-            if (tid == 0) s_sel[c] = hp;
-            nsel = c + 1;
-            if (lp[0] == hp) {  // the owner pops its head
-#pragma unroll
-                for (int i = 0; i < RS_MAX_TOPC - 1; ++i) {
-                    ls[i] = ls[i + 1];
-                    lp[i] = lp[i + 1];
-                }
-                ls[RS_MAX_TOPC - 1] = -INFINITY;
-                lp[RS_MAX_TOPC - 1] = -1;
-            }
-        }
-        if (tid == 0) s_nsel = nsel;
-    }
-    const long long stored = total < pos_cap ? total : pos_cap;
-    for (long long i = stored + tid; i < pos_cap; i += kQryThreads) pos[(long long)b * pos_cap + i] = -1;
-    __syncthreads();
-    const int nsel = s_nsel;
-    for (int i = tid; i < top_c * span_len; i += kQryThreads) {
-        const int c = i / span_len, j = i - c * span_len;
-        int v = -1;
-        if (c < nsel) {
-            const long long p = s_sel[c];
-            long long len = t - 1 - p;
-            if (len > span_len) len = span_len;
-            if (j < len) v = X[p + 1 + j];
-        }
-        spans[(long long)b * top_c * span_len + i] = v;
-    }
-    if (tid < top_c) {
-        int sp = -1, sl = 0;
-        if (tid < nsel) {
-            sp = s_sel[tid];
-            const long long len = t - 1 - sp;
-            sl = (int)(len > span_len ? span_len : len);
-        }
-        sel_pos[(long long)b * top_c + tid] = sp;
-        sel_len[(long long)b * top_c + tid] = sl;
-    }
-    if (tid == 0) {
-        count[b] = (int32_t)total;
-        n_sel[b] = nsel;
-        status[b] = st | (total > pos_cap ? RS_ST_TRUNCATED : 0);
-    }
+    const long long rows = (src.ncand + 127) / 128;
+    const bool solo = rows <= kQrySoloRows;
+    if (solo && crank != 0) return;
+    mat_body(src, q, rows, solo, b, crank, sh, qry_bits, o);
 }
 
 }  // namespace
@@ -727,6 +640,31 @@ static rs_status check_index(const char *who, int B, int V, int64_t t_total, con
     return RS_OK;
 }
 
+// One pass of the sort: digit `pass` of the keys, from the tokens or from the
+// pairs the last pass left.
+template <int kR>
+static rs_status radix_pass(const int32_t *tokens, const int64_t *tok_off, int B, int V, int vbits, int keybits,
+                            int passes, int pass, long long N, const IndexView &ix, cudaStream_t st) {
+    const int bits = (keybits + passes - 1) / passes, shift = pass * bits, bins = 1 << bits;
+    const long long nt = n_tiles(N);
+    const TokenKeys tk{tokens, tok_off, B, V, vbits, 0, 0};
+    const PairKeys pk{ix.pair[(pass & 1) ^ 1]};
+    const dim3 grid((unsigned)nt), block(kRadixThreads);
+    if (pass == 0) launch_pdl(radix_hist<TokenKeys, kR>, grid, block, 0, st, tk, N, shift, bins, ix.hist, ix.valid);
+    else launch_pdl(radix_hist<PairKeys, kR>, grid, block, 0, st, pk, N, shift, bins, ix.hist, ix.valid);
+    RS_CHECK_LAUNCH("rs_match_index_build/radix_hist");
+    launch_pdl(radix_offsets, dim3((unsigned)(bins + kOffDigits - 1) / kOffDigits), block, 0, st, ix.hist, nt, bins, ix.dtot,
+               ix.valid);
+    RS_CHECK_LAUNCH("rs_match_index_build/radix_offsets");
+    if (pass == 0)
+        launch_pdl(radix_scatter<TokenKeys, kR>, grid, block, 0, st, tk, ix.pair[0], N, shift, bins, ix.hist, ix.dtot, ix.valid);
+    else
+        launch_pdl(radix_scatter<PairKeys, kR>, grid, block, 0, st, pk, ix.pair[pass & 1], N, shift, bins, ix.hist, ix.dtot,
+                   ix.valid);
+    RS_CHECK_LAUNCH("rs_match_index_build/radix_scatter");
+    return RS_OK;
+}
+
 extern "C" rs_status rs_match_index_build(const int32_t *tokens, const int64_t *tok_off, int B, int V,
                                           int64_t t_total, void *index, size_t index_bytes_avail, void *stream) {
     clear_error();
@@ -739,34 +677,22 @@ extern "C" rs_status rs_match_index_build(const int32_t *tokens, const int64_t *
     carve_index(index, B, V, t_total, &ix);
     const int vbits = bits_for(V);
     const int keybits = vbits + bits_for(B - 1);
-    launch_pdl(index_check, dim3(1), dim3(256), 0, st, tok_off, B, (long long)t_total, ix);
+    launch_pdl(index_check, dim3(1), dim3(1024), 0, st, tok_off, B, (long long)t_total, ix);
     RS_CHECK_LAUNCH("rs_match_index_build/check");
-    const unsigned zx = (unsigned)std::min<long long>((V + 1 + 255) / 256, 64);
-    launch_pdl(index_init, dim3(zx, B), dim3(256), 0, st, tok_off, V, ix);
-    RS_CHECK_LAUNCH("rs_match_index_build/init");
-    const unsigned cx = (unsigned)std::max<long long>(1, std::min<long long>((t_total / B + 1023) / 1024, 256));
-    launch_pdl(index_count, dim3(cx, B), dim3(256), 0, st, tokens, tok_off, V, vbits, ix);
-    RS_CHECK_LAUNCH("rs_match_index_build/count");
-    launch_pdl(index_offsets, dim3(B), dim3(kIdxThreads), 0, st, V, ix);
-    RS_CHECK_LAUNCH("rs_match_index_build/offsets");
-    if (t_total == 0) return RS_OK;
-    // stable LSD radix sort of the (request, bucket) keys, 8 bits per pass
-    const long long N = t_total, nt = n_tiles(t_total);
-    int cur = 0;
-    for (int shift = 0; shift < keybits; shift += 8, cur ^= 1) {
-        launch_pdl(radix_hist, dim3((unsigned)nt), dim3(kRadixThreads), 0, st, ix.key[cur], N, shift, nt, ix.hist,
-                   ix.valid);
-        RS_CHECK_LAUNCH("rs_match_index_build/radix_hist");
-        launch_pdl(radix_total, dim3(kRadixBins), dim3(kRadixThreads), 0, st, ix.hist, nt, ix.dtot, ix.valid);
-        RS_CHECK_LAUNCH("rs_match_index_build/radix_total");
-        launch_pdl(radix_offsets, dim3(kRadixBins), dim3(kRadixThreads), 0, st, ix.hist, nt, ix.dtot, ix.valid);
-        RS_CHECK_LAUNCH("rs_match_index_build/radix_offsets");
-        launch_pdl(radix_scatter, dim3((unsigned)nt), dim3(kRadixThreads), 0, st, ix.key[cur], ix.val[cur],
-                   ix.key[cur ^ 1], ix.val[cur ^ 1], N, shift, nt, ix.hist, ix.valid);
-        RS_CHECK_LAUNCH("rs_match_index_build/radix_scatter");
+    const int passes = t_total > 0 ? (keybits + kMaxDigitBits - 1) / kMaxDigitBits : 0;
+    const bool small = tile_rounds(t_total) == kTileRoundsSmall;
+    for (int pass = 0; pass < passes; ++pass) {
+        const rs_status s = small ? radix_pass<kTileRoundsSmall>(tokens, tok_off, B, V, vbits, keybits, passes, pass, t_total, ix, st)
+                                  : radix_pass<kTileRounds>(tokens, tok_off, B, V, vbits, keybits, passes, pass, t_total, ix, st);
+        if (s != RS_OK) return s;
     }
-    const unsigned px = (unsigned)std::min<long long>((N + 255) / 256, 148ll * 16);
-    launch_pdl(index_place, dim3(px), dim3(256), 0, st, ix.key[cur], ix.val[cur], N, tok_off, V, vbits, ix);
+    const uint2 *sorted = ix.pair[(passes - 1) & 1];
+    launch_pdl(index_first, dim3((unsigned)((V + 2ll + kFirstPer - 1) / kFirstPer), B), dim3(kFirstPer + 1), 0, st, sorted,
+        tok_off, V, vbits, ix);
+    RS_CHECK_LAUNCH("rs_match_index_build/first");
+    if (t_total == 0) return RS_OK;
+    launch_pdl(index_place, dim3((unsigned)((t_total + 256 * kPlacePer - 1) / (256 * kPlacePer))), dim3(256), 0, st, sorted,
+        (long long)t_total, tok_off, V, vbits, ix);
     RS_CHECK_LAUNCH("rs_match_index_build/place");
     return RS_OK;
 }
@@ -806,9 +732,20 @@ extern "C" rs_status rs_match_scan_indexed(const int32_t *tokens, const int64_t 
     if (B == 0) return RS_OK;
     IndexView ix;
     carve_index(const_cast<void *>(index), B, V, t_total, &ix);
-    launch_pdl(index_query, dim3(B), dim3(kQryThreads), 0, (cudaStream_t)stream, tokens, tok_off, V, k_star,
-        gate_ok, scores, p.theta_score, p.top_c, p.span_len, pos_cap, ix, count, pos, sel_pos, sel_len, spans, n_sel,
-        status);
+    static int attr_done[64] = {0};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev >= 0 && dev < 64 && !attr_done[dev]) {
+        const cudaError_t ce = cudaFuncSetAttribute(index_query, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMatSmem);
+        if (ce != cudaSuccess) {
+            set_error("rs_match_scan_indexed: cudaFuncSetAttribute: %s", cudaGetErrorString(ce));
+            return RS_ERR_CUDA;
+        }
+        attr_done[dev] = 1;
+    }
+    const MatOut o{count, pos, sel_pos, sel_len, spans, n_sel, status, p.theta_score, p.top_c, p.span_len, pos_cap};
+    launch_pdl(index_query, dim3(kMatCluster, B), dim3(kMatThreads), kMatSmem, (cudaStream_t)stream, tokens, tok_off, V,
+        k_star, gate_ok, scores, ix, o);
     RS_CHECK_LAUNCH("rs_match_scan_indexed");
     return RS_OK;
 }

@@ -1,7 +1,8 @@
 """The retrieval kernels at the edges of their splits, bit for bit against the
 oracle: buffers that start at every offset from a 16-byte boundary, one
 round of a single CTA and one position more, more candidates than a CTA keeps
-ballots for and more matches than the ranking buffer holds."""
+ballots for, more matches than the ranking buffer holds, and (the index)
+tiles, digits and passes of the sort at their edges."""
 import numpy as np
 import pytest
 import torch
@@ -9,7 +10,7 @@ import torch
 import oracle
 from gpu_helpers import f32
 from paper_2511_01282_gb300 import respec as rs
-from test_gpu_index import _cuda
+from test_gpu_index import _cuda, compare
 
 pytestmark = pytest.mark.gpu
 
@@ -70,3 +71,30 @@ def test_scan_beyond_the_kept_ballots():
     ref = _scan(tokens, tok_off, np.array([1, 1], np.int32), scores, 0.3, 8, 4, 300)
     assert 20 < ref["count"][1] < 300
     _scan(tokens, tok_off, np.array([0, 2], np.int32), scores, 0.3, 8, 4, 300)
+
+
+@pytest.mark.parametrize("lens,V", [([1023, 1024, 1025, 0, 1], 300), ([4096, 0, 0, 4097], 1), ([524288 - 5, 5], 70000),
+                                    ([524289], 511), ([70001] * 3, 512), ([3] * 700, 1 << 18)])
+def test_index_sort_edges(lens, V):
+    # tiles of 1024 and 4096 keys (524288 tokens is the last total with small
+    # tiles), one to four passes, empty requests, ids that nothing holds
+    rng = np.random.default_rng(len(lens) + V)
+    tokens, tok_off = _buffers(rng, lens, max(V, 2), 1)  # V = 1: ids 0 and (foreign) 1
+    scores = rng.random(len(tokens)).astype(np.float32)
+    ks = rng.integers(1, 3, len(lens)).astype(np.int32)
+    compare(tokens, tok_off, ks, None, scores, 0.3, 4, 8, 50, V)
+
+
+@pytest.mark.parametrize("common", [4095, 4096, 4097, 40000, 4300000])
+def test_index_query_of_a_common_token(common):
+    # the key's last token fills one round of one CTA, one more, several rounds
+    # of the cluster, and more than the ballots it keeps
+    rng = np.random.default_rng(common)
+    t = common + common // 3 + 100
+    tokens = rng.integers(1, 1000, t).astype(np.int32)
+    tokens[rng.permutation(t - 1)[:common]] = 0
+    tokens[-1] = 0
+    tok_off = np.array([0, t], np.int64)
+    scores = rng.random(t).astype(np.float32)
+    for k in (1, 3):
+        compare(tokens, tok_off, np.array([k], np.int32), None, scores, 0.3, 8, 4, 5000, 1000)
