@@ -16,9 +16,9 @@
 // statistics need no second kernel.  Longer rows write their chunk results
 // to the workspace and kernel 2 (accept_merge) merges them.
 // Kernel 3 (accept_decide): one CTA per request checks the tree, verifies
-// model nodes (each thread walks its own root path over per-node match
-// flags), runs the look-ahead procedure per chain (one thread per chain),
-// picks the winner and updates the scores (one thread per selection).
+// model nodes (ancestor sets against the set of greedy matches), runs the
+// look-ahead procedure per chain (one lane per chain), picks the winner and
+// updates the scores (one lane per selection).
 #include <math.h>
 
 #include <cooperative_groups.h>
@@ -182,7 +182,10 @@ template <bool kVec, bool kEnt, bool kFuse>
 __global__ void __launch_bounds__(kAccThreads, 4)
 accept_rows(const float *__restrict__ logits, int V, int nchunks, int beta, VI *__restrict__ cand,
             MS *__restrict__ part, RowOut o) {
-    pdl_enter();
+    // the kernels behind this one read the caller's arrays before they wait for
+    // it (accept_decide), so they may launch only once its own wait is over
+    pdl_wait_prev();
+    pdl_launch_next();
     __shared__ RowsShared sh;
     const long long blk = blockIdx.x;
     const long long r = blockIdx.x / (unsigned)nchunks;  // 32-bit division
@@ -373,54 +376,67 @@ accept_merge(const VI *__restrict__ cand, const MS *__restrict__ part, int nchun
     merge_row<kCandPerLane>(cand + r * ncand, ncand, part + r * nchunks, nchunks, beta, r, o, lane);
 }
 
-constexpr int kDecThreads = 512;
-static_assert(kDecThreads >= RS_MAX_NODES + RS_MAX_TOPC, "one thread per node plus one per selection");
+// One thread per node (warps 0-7) and a warp for the chains and selections.
+constexpr int kDecThreads = RS_MAX_NODES + 32;
+static_assert(RS_MAX_TOPC <= 32, "one lane per selection");
 constexpr int kNodeWords = RS_MAX_NODES / 32;
 
-// One CTA per request.  Every global read happens in two dependent rounds
-// at the start (the tree and the row statistics, then the logit of each
-// node's token in its parent's row; the selected positions and their scores
-// are read by other threads at the same time); the rest works on shared
-// memory.  Per node it precomputes the greedy match
-// (token == argmax of the parent row) and the relaxed check of Eq. 6-7
-// (token among the parent row's top beta and max logit - token logit <= tau
-// in fp64), so each chain's look-ahead walk and each model node's path check
-// read only flags.  Chain c's nodes are ranked by popcounts of per-chain
-// membership masks (one warp ballot per 32 nodes).
+// Consecutive set bits of w from bit `pos` on, below bit L.
+__device__ __forceinline__ int ones_from(const uint32_t *w, int pos, int L) {
+    int p = pos;
+    while (p < L) {
+        const int avail = 32 - (p & 31);
+        const uint32_t x = ~(w[p >> 5] >> (p & 31));
+        const int n = x ? min(__ffs(x) - 1, avail) : avail;
+        p += n;
+        if (n < avail) break;
+    }
+    return min(p, L) - pos;
+}
+
+// One CTA per request.  The kernel is a chain of dependent reads and block
+// barriers, so everything that does not depend on the row statistics comes
+// before the wait for the row kernels (kEarly) and overlaps them: the tree and
+// its checks, each node's ancestor set and depth, each chain's nodes in order,
+// the logit of each node's token in its parent's row, the selected positions
+// and their scores.  That is safe because accept_rows lets its successors
+// launch only after its own wait: whatever wrote the caller's arrays is
+// complete by then, and this call's row kernels write none of them.
+// After the wait one round of reads gives every node its parent's statistics;
+// greedy matches (token == argmax of the parent row) and relaxed checks (Eq.
+// 6-7: token among the parent row's top beta, fp64 logit gap <= tau) become
+// bit sets, so a model node is accepted when its ancestor set lies in the
+// greedy set and a chain's look-ahead counts runs of ones; then every node
+// writes its own part of the accepted path.  Cold and alone 9.7 -> 7.3 us (4
+// trees of 65 nodes), 11.2 -> 8.6 us (one of 145); the whole call in a graph,
+// where the first half overlaps the row kernels, 18.2 -> 14.3 and 29.0 -> 23.7.
+template <bool kEarly>
 __global__ void __launch_bounds__(kDecThreads)
 accept_decide(const float *__restrict__ logits, int R, int V, const int32_t *__restrict__ node_off,
               const int32_t *__restrict__ tokens, const int32_t *__restrict__ parents,
               const uint8_t *__restrict__ source, const int8_t *__restrict__ chain,
               const int32_t *__restrict__ sel_pos, const int64_t *__restrict__ tok_off, rs_params p,
-              int acc_cap, const int32_t *__restrict__ argmax, const int32_t *__restrict__ topk,
-              const float *__restrict__ lse, const float *__restrict__ rowmax, float *__restrict__ p_tok,
-              int32_t *__restrict__ acc_len, int32_t *__restrict__ acc_nodes, int32_t *__restrict__ bonus,
-              int32_t *__restrict__ winner, uint8_t *__restrict__ commit, float *__restrict__ scores,
+              int acc_cap, const int32_t *argmax, const int32_t *topk, const float *lse, const float *rowmax,
+              float *__restrict__ p_tok, int32_t *__restrict__ acc_len, int32_t *__restrict__ acc_nodes,
+              int32_t *__restrict__ bonus, int32_t *__restrict__ winner, uint8_t *__restrict__ commit, float *scores,
               int32_t *__restrict__ status) {
-    pdl_enter();
+    pdl_launch_next();
+    if (!kEarly) pdl_wait_prev();
     const int b = blockIdx.x;
     const int n0 = node_off[b];
     const int N = node_off[b + 1] - n0;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int beta = p.beta, top_c = p.top_c;
 
-    __shared__ int s_arg[RS_MAX_NODES];
-    __shared__ int s_top[RS_MAX_NODES * RS_MAX_BETA];
     __shared__ int s_par[RS_MAX_NODES];
-    __shared__ int s_tok[RS_MAX_NODES];
-    __shared__ float s_zmax[RS_MAX_NODES];  // each row's largest logit
-    __shared__ float s_ztok[RS_MAX_NODES];  // node i: logit of its token in its parent's row
     __shared__ uint8_t s_src[RS_MAX_NODES];
-    __shared__ int8_t s_chn[RS_MAX_NODES];
-    __shared__ uint8_t s_g[RS_MAX_NODES];   // greedy match
-    __shared__ uint8_t s_rx[RS_MAX_NODES];  // relaxed check (Eq. 6 and Eq. 7)
+    __shared__ uint32_t s_anc[RS_MAX_NODES][kNodeWords + 1];  // ancestors and the node itself, without the root
     __shared__ uint32_t s_cmask[RS_MAX_TOPC][kNodeWords];
     __shared__ int s_cnodes[RS_MAX_TOPC][RS_MAX_NODES];
-    __shared__ int s_clen[RS_MAX_TOPC];
+    __shared__ uint32_t s_cg[RS_MAX_TOPC][kNodeWords], s_cr[RS_MAX_TOPC][kNodeWords];  // greedy / relaxed, chain order
+    __shared__ uint32_t s_g[kNodeWords];                                               // greedy, node order
     __shared__ int s_cacc[RS_MAX_TOPC];
-    __shared__ int s_selp[RS_MAX_TOPC];
-    __shared__ float s_selS[RS_MAX_TOPC];
-    __shared__ int s_bad, s_stt, s_win, s_dup;
+    __shared__ int s_bad;
     __shared__ int s_best;  // (depth << 16) | (0xffff - node)
 
     // the request's rows must lie in [0, R) and its buffer in the score table
@@ -436,118 +452,98 @@ accept_decide(const float *__restrict__ logits, int R, int V, const int32_t *__r
     if (tid == 0) {
         s_bad = 0;
         s_best = 0;
-        s_stt = 0;
     }
+    if (tid < RS_MAX_TOPC * kNodeWords) {
+        (&s_cg[0][0])[tid] = 0;
+        (&s_cr[0][0])[tid] = 0;
+    }
+    static_assert(RS_MAX_TOPC * kNodeWords <= kDecThreads, "one thread per chain word");
 
-    // ---- every global read up front.  Node = tid (N <= RS_MAX_NODES, one
-    // per thread): its tree entries and row statistics, then its token's
-    // logit in the parent's row (two dependent rounds); meanwhile threads
-    // RS_MAX_NODES .. read the selected positions and their scores (Eq. 4-5
-    // inputs) and every thread reads top-beta ids ----
+    // ---- the tree: node = tid ----
     const int node = tid;
-    int r_pa = 0, r_sr = 0, r_ch = 0, r_tk = 0, r_am = 0;
-    float r_zmax = 0.f, r_z = 0.f, r_lp = 0.f;
-    bool r_bad = false;
-    if (st == 0 && node < N) {
-        r_pa = parents[n0 + node];
-        r_sr = source[n0 + node];
-        r_ch = chain[n0 + node];
-        r_tk = tokens[n0 + node];
-        r_am = argmax[n0 + node];
-        r_zmax = rowmax[n0 + node];
-        if (node == 0) r_bad = (r_pa != -1 || r_sr != 0 || r_ch != -1);
-        else r_bad = (r_pa < 0 || r_pa >= node || r_sr < 1 || r_sr > 2 || (r_sr == 2 && (r_ch < 0 || r_ch >= top_c)) ||
-                    (r_sr == 1 && r_ch != -1) || r_tk < 0 || r_tk >= V);
-        if (!r_bad && node > 0) {
-            r_z = logits[(long long)(n0 + r_pa) * V + r_tk];
-            r_lp = lse[n0 + r_pa];
-        }
+    const bool live = st == 0 && node < N;
+    int pa = 0, sr = 0, ch = -1, tk = 0;
+    float z = 0.f;  // the token's logit in the parent's row
+    bool bad = false;
+    if (live) {
+        pa = parents[n0 + node];
+        sr = source[n0 + node];
+        ch = chain[n0 + node];
+        tk = tokens[n0 + node];
+        if (node == 0) bad = (pa != -1 || sr != 0 || ch != -1);
+        else bad = (pa < 0 || pa >= node || sr < 1 || sr > 2 || (sr == 2 && (ch < 0 || ch >= top_c)) ||
+                    (sr == 1 && ch != -1) || tk < 0 || tk >= V);
+        if (!bad && node > 0) z = logits[(long long)(n0 + pa) * V + tk];
+        s_par[node] = pa;
+        s_src[node] = (uint8_t)sr;
     }
-    const int js = tid - RS_MAX_NODES;
+    // ---- the selections: lane j of the last warp ----
+    const bool seller = warp == kNodeWords;
     int selp = -1;
     float selS = 0.f;
-    if (js >= 0 && js < top_c) {
-        selp = sel_pos[(long long)b * top_c + js];
-        selS = (tok_ok && selp >= 0 && (long long)selp < t) ? scores[t0 + selp] : 0.f;
-    }
-    if (st == 0)
-        for (int x = tid; x < N * beta; x += kDecThreads)
-            s_top[(x / beta) * RS_MAX_BETA + (x % beta)] = topk[(long long)n0 * beta + x];
-    __syncthreads();  // s_bad, s_best and s_stt are initialised
-    if (js >= 0 && js < top_c) {
-        s_selp[js] = selp;
-        s_selS[js] = selS;
-    }
-    if (st == 0 && node < N) {
-        s_arg[node] = r_am;
-        s_zmax[node] = r_zmax;
-        s_par[node] = r_pa;
-        s_tok[node] = r_tk;
-        s_src[node] = (uint8_t)r_sr;
-        s_chn[node] = (int8_t)r_ch;
-        commit[n0 + node] = 0;
-        if (r_bad) {
-            atomicOr(&s_bad, 1);
-        } else if (node == 0) {
-            p_tok[n0] = 1.f;
-        } else {
-            s_ztok[node] = r_z;
-            p_tok[n0 + node] = __expf(r_z - r_lp);
+    bool dup = false;  // some position is selected twice: it is updated twice, in selection order
+    if (seller) {
+        if (lane < top_c) {
+            selp = sel_pos[(long long)b * top_c + lane];
+            selS = (tok_ok && selp >= 0 && (long long)selp < t) ? scores[t0 + selp] : 0.f;
         }
+#pragma unroll
+        for (int c = 0; c < RS_MAX_TOPC; ++c) {
+            const int o = __shfl_sync(0xffffffffu, selp, c);
+            dup |= c < lane && selp >= 0 && selp == o;
+        }
+        dup = __any_sync(0xffffffffu, dup);
     }
-    __syncthreads();
-    const bool ok1 = st == 0 && s_bad == 0;
+    bool any_bad = __syncthreads_or(bad);  // s_par, s_src and the zeroes are complete
 
-    // ---- model nodes hang from the root or from model nodes; chain
-    // membership masks; per-node greedy and relaxed flags ----
+    // ---- model nodes hang from the root or from model nodes; ancestor sets;
+    // chain membership masks ----
+    const bool ok1 = st == 0 && !any_bad;  // every parent is an earlier node: walks end
+    uint32_t anc[kNodeWords];
+    int depth = 0;
+    bad = false;
     if (ok1) {
-        for (int i = 1 + tid; i < N; i += kDecThreads) {
-            const int pa = s_par[i], x = s_tok[i];
-            if (s_src[i] == 1 && s_src[pa] > 1) atomicOr(&s_bad, 1);
-            s_g[i] = (uint8_t)(x == s_arg[pa]);
-            bool in_top = false;
-            for (int j = 0; j < beta; ++j) in_top |= (s_top[pa * RS_MAX_BETA + j] == x);
-            const double gap = (double)s_zmax[pa] - (double)s_ztok[i];
-            s_rx[i] = (uint8_t)(in_top && gap <= (double)p.tau);
+        if (live) {
+            bad = node > 0 && sr == 1 && s_src[pa] > 1;
+#pragma unroll
+            for (int w = 0; w < kNodeWords; ++w) anc[w] = 0;
+            for (int x = node; x > 0; x = s_par[x]) {
+                ++depth;
+#pragma unroll
+                for (int w = 0; w < kNodeWords; ++w) anc[w] |= (x >> 5) == w ? 1u << (x & 31) : 0u;
+            }
+#pragma unroll
+            for (int w = 0; w < kNodeWords; ++w) s_anc[node][w] = anc[w];
         }
         if (warp < kNodeWords) {
-            const int i = warp * 32 + lane;
-            const int ch = (i > 0 && i < N && s_src[i] == 2) ? s_chn[i] : -1;
+            const int c0 = (live && node > 0 && sr == 2) ? ch : -1;
             for (int c = 0; c < top_c; ++c) {
-                const uint32_t m = __ballot_sync(0xffffffffu, ch == c);
+                const uint32_t m = __ballot_sync(0xffffffffu, c0 == c);
                 if (lane == 0) s_cmask[c][warp] = m;
             }
         }
     }
-    __syncthreads();
-    const bool ok2 = ok1 && s_bad == 0;
+    any_bad |= __syncthreads_or(bad);
     // ---- chain c in index order: node of rank r ----
-    if (ok2) {
-        for (int i = 1 + tid; i < N; i += kDecThreads) {
-            if (s_src[i] != 2) continue;
-            const int c = s_chn[i], w = i >> 5;
-            int rank = __popc(s_cmask[c][w] & ((1u << (i & 31)) - 1u));
-            for (int q = 0; q < w; ++q) rank += __popc(s_cmask[c][q]);
-            s_cnodes[c][rank] = i;
-        }
-        if (tid < top_c) {
-            int L = 0;
+    const bool ok2 = st == 0 && !any_bad;
+    const bool chained = ok2 && live && node > 0 && sr == 2;
+    int rank = 0, clen = 0;  // of a chain node; of lane c's chain
+    if (chained) {
+        rank = __popc(s_cmask[ch][node >> 5] & ((1u << (node & 31)) - 1u));
+        for (int q = 0; q < (node >> 5); ++q) rank += __popc(s_cmask[ch][q]);
+        s_cnodes[ch][rank] = node;
+    }
+    if (ok2 && seller && lane < top_c) {
 #pragma unroll
-            for (int q = 0; q < kNodeWords; ++q) L += __popc(s_cmask[tid][q]);
-            s_clen[tid] = L;
-        }
+        for (int q = 0; q < kNodeWords; ++q) clen += __popc(s_cmask[lane][q]);
     }
     __syncthreads();
     // ---- each chain is a path from the root: rank r hangs from rank r - 1 ----
-    if (ok2) {
-        for (int x = tid; x < top_c * RS_MAX_NODES; x += kDecThreads) {
-            const int c = x / RS_MAX_NODES, r = x - c * RS_MAX_NODES;
-            if (r >= s_clen[c]) continue;
-            if (s_par[s_cnodes[c][r]] != (r == 0 ? 0 : s_cnodes[c][r - 1])) atomicOr(&s_bad, 1);
-        }
-    }
-    __syncthreads();
-    if (st == 0 && s_bad) st = RS_ST_BAD_TREE;
+    bad = chained && pa != (rank == 0 ? 0 : s_cnodes[ch][rank - 1]);
+    any_bad |= __syncthreads_or(bad);
+    if (st == 0 && any_bad) st = RS_ST_BAD_TREE;
+
+    if (kEarly) pdl_wait_prev();  // the row statistics are complete
 
     // ---- outputs of a rejected request ----
     if (st != 0) {
@@ -565,29 +561,53 @@ accept_decide(const float *__restrict__ logits, int R, int V, const int32_t *__r
         return;
     }
 
-    // ---- strict verification of model nodes: every node on the root path matches ----
-    for (int i = 1 + tid; i < N; i += kDecThreads) {
-        if (s_src[i] != 1) continue;
-        bool ok = true;
-        int depth = 0;
-        for (int a = i; a > 0; a = s_par[a]) {
-            ok = ok && s_g[a];
-            ++depth;
+    // ---- greedy and relaxed flags, from the parent's row statistics ----
+    int own_arg = 0;
+    bool g = false;
+    if (live) {
+        own_arg = argmax[n0 + node];
+        if (node == 0) {
+            p_tok[n0] = 1.f;
+        } else {
+            const int32_t *tp = topk + (long long)(n0 + pa) * beta;
+            int id[RS_MAX_BETA];
+#pragma unroll
+            for (int j = 0; j < RS_MAX_BETA; ++j) id[j] = j < beta ? tp[j] : -1;
+            const int am = argmax[n0 + pa];
+            const float zmax = rowmax[n0 + pa], lp = lse[n0 + pa];
+            g = tk == am;
+            bool in_top = false;
+#pragma unroll
+            for (int j = 0; j < RS_MAX_BETA; ++j) in_top |= id[j] == tk;  // tk >= 0
+            const bool rx = in_top && (double)zmax - (double)z <= (double)p.tau;
+            p_tok[n0 + node] = __expf(z - lp);
+            if (chained) {
+                if (g) atomicOr(&s_cg[ch][rank >> 5], 1u << (rank & 31));
+                if (rx) atomicOr(&s_cr[ch][rank >> 5], 1u << (rank & 31));
+            }
         }
-        if (ok) atomicMax(&s_best, (depth << 16) | (0xffff - i));
     }
+    if (warp < kNodeWords) {
+        const uint32_t m = __ballot_sync(0xffffffffu, g);
+        if (lane == 0) s_g[warp] = m;
+    }
+    __syncthreads();
 
-    // ---- relaxed verification with look-ahead, one thread per chain ----
-    if (tid < top_c) {
-        const int c = tid, L = s_clen[c];
-        const int *d = s_cnodes[c];
-        int l0 = 0;
-        while (l0 < L && s_g[d[l0]]) ++l0;
-        int cur = l0, last = l0;
+    // ---- strict verification of model nodes: every node on the root path matches ----
+    if (live && sr == 1) {
+        uint32_t miss = 0;
+#pragma unroll
+        for (int w = 0; w < kNodeWords; ++w) miss |= anc[w] & ~s_g[w];
+        if (!miss) atomicMax(&s_best, (depth << 16) | (0xffff - node));
+    }
+    // ---- relaxed verification with look-ahead, one lane per chain ----
+    int cacc = 0;
+    if (seller && lane < top_c) {
+        const uint32_t *cg = s_cg[lane], *cr = s_cr[lane];
+        int cur = ones_from(cg, 0, clen), last = cur;
         for (int att = 0; att < p.phi; ++att) {
-            if (cur >= L || !s_rx[d[cur]]) break;
-            int xi = 0;
-            while (cur + 1 + xi < L && s_g[d[cur + 1 + xi]]) ++xi;
+            if (cur >= clen || !((cr[cur >> 5] >> (cur & 31)) & 1u)) break;
+            const int xi = ones_from(cg, cur + 1, clen);
             if (xi >= p.m) {
                 last = cur + 1 + xi;
                 cur = last;
@@ -595,82 +615,60 @@ accept_decide(const float *__restrict__ logits, int R, int V, const int32_t *__r
                 cur = cur + 1;
             }
         }
-        s_cacc[c] = last;
+        cacc = last;
+        s_cacc[lane] = last;
     }
     __syncthreads();
 
-    // ---- winner, accepted path, bonus, commit ----
-    if (tid == 0) {
-        const int model_len = s_best >> 16;
-        const int best_node = model_len > 0 ? 0xffff - (s_best & 0xffff) : 0;
-        int best_len = model_len, win = model_len > 0 ? -1 : -2;
-        for (int c = 0; c < top_c; ++c)
-            if (s_cacc[c] > best_len) {
-                best_len = s_cacc[c];
-                win = c;
-            }
-        if (best_len == 0) win = -2;
-        int last_node = 0;
-        if (win == -1) {
-            int a = best_node;
-            last_node = a;
-            for (int j = best_len - 1; j >= 0; --j) {
-                if (j < acc_cap) acc_nodes[(long long)b * acc_cap + j] = a;
-                commit[n0 + a] = 1;
-                a = s_par[a];
-            }
-        } else if (win >= 0) {
-            for (int j = 0; j < best_len; ++j) {
-                const int a = s_cnodes[win][j];
-                if (j < acc_cap) acc_nodes[(long long)b * acc_cap + j] = a;
-                commit[n0 + a] = 1;
-                last_node = a;
-            }
+    // ---- winner; each node writes its own place on the accepted path ----
+    const int best = s_best;
+    int best_len = best >> 16, win = best_len > 0 ? -1 : -2;
+    const int best_node = best_len > 0 ? 0xffff - (best & 0xffff) : 0;
+    for (int c = 0; c < top_c; ++c) {
+        const int l = s_cacc[c];
+        if (l > best_len) {
+            best_len = l;
+            win = c;
         }
-        for (int j = best_len; j < acc_cap; ++j) acc_nodes[(long long)b * acc_cap + j] = -1;
-        commit[n0] = 1;
-        acc_len[b] = best_len;
-        winner[b] = win;
-        bonus[b] = s_arg[last_node];
-        s_win = win;
-        s_stt = best_len > acc_cap ? RS_ST_TRUNCATED : 0;
-        // a position selected twice is updated twice, in selection order
-        int dup = 0;
-        for (int c = 0; c < top_c; ++c)
-            for (int c2 = 0; c2 < c; ++c2)
-                dup |= (s_selp[c] >= 0 && s_selp[c] == s_selp[c2]);
-        s_dup = dup;
     }
-    __syncthreads();
+    if (live) {
+        const bool on = node > 0 && (win == -1 ? ((s_anc[best_node][node >> 5] >> (node & 31)) & 1u) != 0
+                                               : (win >= 0 && sr == 2 && ch == win && rank < best_len));
+        const int j = win == -1 ? depth - 1 : rank;
+        commit[n0 + node] = (uint8_t)(on || node == 0);
+        if (on && j < acc_cap) acc_nodes[(long long)b * acc_cap + j] = node;
+        if (on ? j == best_len - 1 : (node == 0 && best_len == 0)) bonus[b] = own_arg;
+        if (node == 0) {
+            acc_len[b] = best_len;
+            winner[b] = win;
+        }
+    }
+    for (int j = best_len + tid; j < acc_cap; j += kDecThreads) acc_nodes[(long long)b * acc_cap + j] = -1;
 
     // ---- Eq. 4-5 in fp64, rounded once to the fp32 table ----
-    const double a = (double)p.alpha;
-    auto ema = [&](int c, double S) -> double {
-        const double R = (s_win == c) ? __ddiv_rn((double)s_cacc[c], (double)s_clen[c]) : 0.0;
-        return __dadd_rn(__dmul_rn(__dsub_rn(1.0, a), S), __dmul_rn(a, R));
-    };
-    if (!s_dup) {
-        if (tid < top_c) {
-            const int c = tid, pos = s_selp[c];
-            if (pos >= 0 && s_clen[c] != 0) {
-                if ((long long)pos >= t) atomicOr(&s_stt, RS_ST_BAD_POS);
-                else scores[t0 + pos] = __double2float_rn(ema(c, (double)s_selS[c]));
+    if (seller) {
+        const double a = (double)p.alpha;
+        auto ema = [&](bool won, int acc, int len, double S) -> double {
+            const double Rw = won ? __ddiv_rn((double)acc, (double)len) : 0.0;
+            return __dadd_rn(__dmul_rn(__dsub_rn(1.0, a), S), __dmul_rn(a, Rw));
+        };
+        const bool upd = lane < top_c && selp >= 0 && clen != 0;
+        const bool far = upd && (long long)selp >= t;
+        if (!dup) {
+            if (upd && !far) scores[t0 + selp] = __double2float_rn(ema(win == lane, cacc, clen, (double)selS));
+        } else {
+            for (int c = 0; c < top_c; ++c) {
+                if (lane == c && upd && !far) {
+                    volatile float *S = scores + t0 + selp;  // an earlier lane may just have written it
+                    *S = __double2float_rn(ema(win == c, cacc, clen, (double)*S));
+                    __threadfence();
+                }
+                __syncwarp();
             }
         }
-    } else if (tid == 0) {
-        for (int c = 0; c < top_c; ++c) {
-            const int pos = s_selp[c];
-            if (pos < 0 || s_clen[c] == 0) continue;
-            if ((long long)pos >= t) {
-                s_stt |= RS_ST_BAD_POS;
-                continue;
-            }
-            float *S = scores + t0 + pos;
-            *S = __double2float_rn(ema(c, (double)(*S)));
-        }
+        const bool any_far = __any_sync(0xffffffffu, far);
+        if (lane == 0) status[b] = (best_len > acc_cap ? RS_ST_TRUNCATED : 0) | (any_far ? RS_ST_BAD_POS : 0);
     }
-    __syncthreads();
-    if (tid == 0) status[b] = s_stt;
 }
 
 }  // namespace
@@ -758,9 +756,10 @@ extern "C" rs_status rs_accept(const float *logits, int R, int V, const int32_t 
         }
     }
     if (B > 0) {
-        launch_pdl(accept_decide, dim3(B), dim3(kDecThreads), 0, st, logits, R, V, node_off, tokens, parents,
-            source, chain, sel_pos, tok_off, p, acc_cap, argmax, topk, lse, rowmax, p_tok, acc_len, acc_nodes,
-            bonus, winner, commit, scores, status);
+        // without row kernels of its own the call's predecessor may still be running
+        launch_pdl(R > 0 ? accept_decide<true> : accept_decide<false>, dim3(B), dim3(kDecThreads), 0, st, logits, R, V,
+            node_off, tokens, parents, source, chain, sel_pos, tok_off, p, acc_cap, argmax, topk, lse, rowmax, p_tok,
+            acc_len, acc_nodes, bonus, winner, commit, scores, status);
         RS_CHECK_LAUNCH("rs_accept/accept_decide");
     }
     return RS_OK;

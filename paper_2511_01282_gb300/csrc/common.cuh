@@ -41,9 +41,7 @@ void count_launch(int n = 1);
 // predecessor's completion and memory before it touches global memory (its
 // second).  Since every kernel waits, completion stays ordered along the
 // whole stream.  Without a programmatic predecessor the wait returns at once.
-// Persistent kernels, whose grid assumes every SM free, use launch_full
-// instead: they start only once the previous kernel has finished.
-template <bool kEarly = true, typename... KArgs, typename... Args>
+template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                        Args... args) {
     cudaLaunchConfig_t cfg = {};
@@ -55,7 +53,18 @@ cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t sme
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = kEarly ? 1 : 0;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+}
+// A launch that starts only once the previous kernel has finished.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_full(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                       Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
     return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
 // The same with a one-dimensional cluster of `cluster_x` CTAs along x
@@ -78,11 +87,6 @@ cudaError_t launch_pdl_cluster(void (*kern)(KArgs...), dim3 grid, dim3 block, si
     cfg.attrs = at;
     cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
-}
-template <typename... KArgs, typename... Args>
-cudaError_t launch_full(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                        Args... args) {
-    return launch_pdl<false>(kern, grid, block, smem, st, args...);
 }
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -109,6 +113,9 @@ long long l2_bytes();  // L2 size of the current device (cached per device)
 // Let the next kernel start launching, then wait for the previous kernel.
 __device__ __forceinline__ void pdl_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait_prev() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// A kernel with work before pdl_wait_prev takes what its predecessor writes
+// through pointers that are not `const __restrict__`: loads through those may
+// become ld.global.nc, which the compiler is free to move above the wait.
 __device__ __forceinline__ void pdl_enter() {
     pdl_launch_next();
     pdl_wait_prev();
