@@ -8,7 +8,7 @@
 // chunk's.  Row entropy is then H = ln s - w / s for the merged triple (the
 // log-sum-exp form of -sum p ln p).
 // Kernel 2 (entropy_merge): one warp per row merges its chunk triples into
-// the row entropy.  Kernel 3 (gate_push): one CTA per request pushes the
+// the row entropy (rows of one chunk need no merge: kernel 1 writes theirs).  Kernel 3 (gate_push): one CTA per request pushes the
 // committed rows' entropies into the history and evaluates H_k, C_k, k* and
 // the trigger in fp64.  rs_entropy_gate_rows runs kernel 3 alone on row
 // entropies that rs_accept already produced from the same logits.
@@ -49,6 +49,9 @@ __device__ __forceinline__ Ent3 ent_shfl(Ent3 a, int o) {
     return b;
 }
 
+// Row entropy in nats of the whole row's triple.
+__device__ __forceinline__ float ent_of(Ent3 t) { return t.s > 0.f ? (__logf(t.s) - t.w / t.s) : 0.f; }
+
 __device__ __forceinline__ float ex2f_approx(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -59,8 +62,12 @@ __device__ __forceinline__ float ex2f_approx(float x) {
 // 0 and 16-byte alignment; else 1).
 template <int kW>
 __global__ void __launch_bounds__(kGateThreads)
-entropy_partial(const float *__restrict__ logits, int V, int nchunks, Ent3 *__restrict__ part) {
-    pdl_enter();
+entropy_partial(const float *__restrict__ logits, int V, int nchunks, Ent3 *__restrict__ part,
+                float *__restrict__ entropy) {
+    // gate_push reads the caller's arrays before it waits for this call's row
+    // kernels, so it may launch only once this kernel's own wait is over
+    pdl_wait_prev();
+    pdl_launch_next();
     const long long blk = blockIdx.x;
     const long long r = blockIdx.x / (unsigned)nchunks;  // 32-bit division
     const int chunk = (int)(blk - r * nchunks);
@@ -142,7 +149,8 @@ entropy_partial(const float *__restrict__ logits, int V, int nchunks, Ent3 *__re
         Ent3 a = sw[0];
 #pragma unroll
         for (int w = 1; w < kGateThreads / 32; ++w) a = ent_merge(a, sw[w]);
-        part[blk] = a;
+        if (nchunks == 1) entropy[r] = ent_of(a);  // the chunk is the row: nothing to merge
+        else part[blk] = a;
     }
 }
 
@@ -158,7 +166,7 @@ entropy_merge(const Ent3 *__restrict__ part, int nchunks, int R, float *__restri
     for (int c = lane; c < nchunks; c += 32) t = ent_merge(t, part[r * nchunks + c]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) t = ent_merge(t, ent_shfl(t, o));
-    if (lane == 0) entropy[r] = t.s > 0.f ? (__logf(t.s) - t.w / t.s) : 0.f;
+    if (lane == 0) entropy[r] = ent_of(t);
 }
 
 // Per request: the committed rows' entropies, in row order, extend the
@@ -193,43 +201,71 @@ __device__ __forceinline__ int push_scan(int v, int *s_w, int *total) {
     return before + x - v;
 }
 
+// kEarly: behind this call's own row kernels, whose first lets its successors
+// launch only after its own wait; everything but the row entropies is then
+// read before the wait.  Otherwise two rounds of reads follow the wait: the
+// offsets with the old history, then the flags with the rows' entropies (all of
+// them, so that the entropies do not wait for the flags).  lambda / k, the
+// longest operation, comes before the wait either way.  Cold and alone 6.7 ->
+// 5.3 us (kEarly) and 6.5 -> 6.1 us.
+template <bool kEarly>
 __global__ void __launch_bounds__(kPushThreads)
-gate_push(const float *__restrict__ entropy, const int32_t *__restrict__ row_off,
-          const uint8_t *__restrict__ row_commit, int R, rs_params p, float *__restrict__ hist,
-          int32_t *__restrict__ hist_n, int32_t *__restrict__ k_star, float *__restrict__ h_best,
+gate_push(const float *entropy, const int32_t *__restrict__ row_off, const uint8_t *__restrict__ row_commit, int R,
+          rs_params p, float *hist, int32_t *hist_n, int32_t *__restrict__ k_star, float *__restrict__ h_best,
           uint8_t *__restrict__ entropy_ok) {
-    pdl_enter();
+    pdl_launch_next();
     const int b = blockIdx.x, tid = threadIdx.x;
+    const int l = p.l;
+    const double pen = tid < RS_MAX_L ? __ddiv_rn((double)p.lambda_e, (double)(tid + 1)) : 0.0;
+    if (!kEarly) pdl_wait_prev();
     // rows [r0, r1) must lie in [0, R) (R < 0: the row offsets' last entry);
     // a range outside them pushes nothing
     const int rend = R >= 0 ? R : row_off[gridDim.x];
     int r0 = row_off[b], r1 = row_off[b + 1];
+    int n = hist_n[b];
+    const float old = tid < l ? hist[(long long)b * l + tid] : 0.f;
     if (r0 < 0 || r1 < r0 || r1 > rend) r0 = r1 = 0;
-    const int l = p.l;
     __shared__ float s_h[RS_MAX_L];
     __shared__ int s_w[kPushWarps];
-    int n = hist_n[b];
     n = n < 0 ? 0 : (n > l ? l : n);
+    const bool one_round = r1 - r0 <= kPushThreads;  // a row per thread (at most RS_MAX_NODES rows per tree)
+    const bool f0 = tid < r1 - r0 && row_commit[r0 + tid] != 0;
 
     // committed rows c; the newest m = min(c, l) of them and the newest
     // keep = min(n, l - m) old entries form the new history
-    int cnt = 0;
-    for (int r = r0 + tid; r < r1; r += kPushThreads) cnt += row_commit[r] != 0;
-    int c = 0;
-    (void)push_scan(cnt, s_w, &c);
+    int c = 0, q0 = 0;
+    float e0 = 0.f;
+    if (one_round) {
+        if (kEarly) {
+            q0 = push_scan(f0 ? 1 : 0, s_w, &c);
+            pdl_wait_prev();
+            if (f0) e0 = entropy[r0 + tid];
+        } else {
+            if (tid < r1 - r0) e0 = entropy[r0 + tid];
+            q0 = push_scan(f0 ? 1 : 0, s_w, &c);
+        }
+    } else {
+        int cnt = 0;
+        for (int r = r0 + tid; r < r1; r += kPushThreads) cnt += row_commit[r] != 0;
+        (void)push_scan(cnt, s_w, &c);
+        if (kEarly) pdl_wait_prev();
+    }
     const int m = c < l ? c : l;
     const int keep = n < l - m ? n : l - m;
     const int nn = keep + m;
-    const float old = tid < keep ? hist[(long long)b * l + n - keep + tid] : 0.f;
-    if (tid < keep) s_h[tid] = old;
-    int carry = 0;
-    for (int base = r0; base < r1; base += kPushThreads) {
-        const int r = base + tid;
-        const bool f = r < r1 && row_commit[r] != 0;
-        int tot = 0;
-        const int q = carry + push_scan(f ? 1 : 0, s_w, &tot);
-        if (f && q >= c - m) s_h[keep + q - (c - m)] = entropy[r];
-        carry += tot;
+    if (tid < n && tid >= n - keep) s_h[tid - (n - keep)] = old;
+    if (one_round) {
+        if (f0 && q0 >= c - m) s_h[keep + q0 - (c - m)] = e0;
+    } else {
+        int carry = 0;
+        for (int base = r0; base < r1; base += kPushThreads) {
+            const int r = base + tid;
+            const bool f = r < r1 && row_commit[r] != 0;
+            int tot = 0;
+            const int q = carry + push_scan(f ? 1 : 0, s_w, &tot);
+            if (f && q >= c - m) s_h[keep + q - (c - m)] = entropy[r];
+            carry += tot;
+        }
     }
     __syncthreads();
     if (tid < nn) hist[(long long)b * l + tid] = s_h[tid];
@@ -241,12 +277,13 @@ gate_push(const float *__restrict__ entropy, const int32_t *__restrict__ row_off
         double sum = 0.0;
         for (int i = nn - k; i < nn; ++i) sum = __dadd_rn(sum, (double)s_h[i]);
         hk = __ddiv_rn(sum, (double)k);
-        ck = __dadd_rn(hk, __ddiv_rn((double)p.lambda_e, (double)k));
+        ck = __dadd_rn(hk, pen);
         if (ck != ck) ck = INFINITY;  // a NaN never wins the strict comparison
     }
     int bk = k;
+    static_assert(RS_MAX_L == 8, "the keys live in lanes 0 .. 7");
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
+    for (int o = RS_MAX_L / 2; o > 0; o >>= 1) {
         const double oc = __shfl_xor_sync(0xffffffffu, ck, o);
         const double oh = __shfl_xor_sync(0xffffffffu, hk, o);
         const int ok = __shfl_xor_sync(0xffffffffu, bk, o);
@@ -267,7 +304,7 @@ gate_push(const float *__restrict__ entropy, const int32_t *__restrict__ row_off
     }
 }
 
-// The three launches of a gate call over the chunk triples in `part`.
+// The launches of a gate call over the chunk triples in `part`.
 rs_status launch_gate(const char *who, const float *logits, int R, int V, int nchunks, Ent3 *part,
                       const int32_t *row_off, const uint8_t *row_commit, int B, rs_params p, float *hist,
                       int32_t *hist_n, float *entropy, int32_t *k_star, float *h_best, uint8_t *entropy_ok,
@@ -282,20 +319,22 @@ rs_status launch_gate(const char *who, const float *logits, int R, int V, int nc
                       : (V % 4 == 0 && ((uintptr_t)logits & 15) == 0) ? 4 : 1;
         if (w == 8)
             launch_pdl(entropy_partial<8>, dim3((unsigned)blocks), dim3(kGateThreads), 0, st, logits, V, nchunks,
-                part);
+                part, entropy);
         else if (w == 4)
             launch_pdl(entropy_partial<4>, dim3((unsigned)blocks), dim3(kGateThreads), 0, st, logits, V, nchunks,
-                part);
+                part, entropy);
         else
             launch_pdl(entropy_partial<1>, dim3((unsigned)blocks), dim3(kGateThreads), 0, st, logits, V, nchunks,
-                part);
+                part, entropy);
         RS_CHECK_LAUNCH(who);
-        launch_pdl(entropy_merge, dim3((R + kMergeThreads / 32 - 1) / (kMergeThreads / 32)), dim3(kMergeThreads),
-            0, st, part, nchunks, R, entropy);
-        RS_CHECK_LAUNCH(who);
+        if (nchunks > 1) {
+            launch_pdl(entropy_merge, dim3((R + kMergeThreads / 32 - 1) / (kMergeThreads / 32)), dim3(kMergeThreads),
+                0, st, part, nchunks, R, entropy);
+            RS_CHECK_LAUNCH(who);
+        }
     }
     if (B > 0) {
-        launch_pdl(gate_push, dim3(B), dim3(kPushThreads), 0, st, entropy, row_off, row_commit, R, p, hist, hist_n,
+        launch_pdl(R > 0 ? gate_push<true> : gate_push<false>, dim3(B), dim3(kPushThreads), 0, st, entropy, row_off, row_commit, R, p, hist, hist_n,
             k_star, h_best, entropy_ok);
         RS_CHECK_LAUNCH(who);
     }
@@ -445,7 +484,7 @@ extern "C" rs_status rs_entropy_gate_rows(const float *entropy, const int32_t *r
     RS_CHECK_ARG(B == 0 || (entropy && row_off && row_commit && hist && hist_n && k_star && h_best && entropy_ok),
                  "rs_entropy_gate_rows: null pointer");
     if (B == 0) return RS_OK;
-    launch_pdl(gate_push, dim3(B), dim3(kPushThreads), 0, (cudaStream_t)stream, entropy, row_off, row_commit, -1,
+    launch_pdl(gate_push<false>, dim3(B), dim3(kPushThreads), 0, (cudaStream_t)stream, entropy, row_off, row_commit, -1,
         p, hist, hist_n, k_star, h_best, entropy_ok);
     RS_CHECK_LAUNCH("rs_entropy_gate_rows");
     return RS_OK;

@@ -1,6 +1,7 @@
-"""rs_accept's decisions at the edges of their words, bit for bit against the
-oracle: trees of up to 256 nodes, chains and model paths that cross 32-node
-words, positions selected twice, more accepted nodes than the list holds."""
+"""rs_accept's decisions and the trigger's push at the edges of their words and
+rounds, bit for bit against the oracle: trees of up to 256 nodes, chains and
+model paths that cross 32-node words, positions selected twice, more accepted
+nodes than the list holds, and requests of one round of rows and more."""
 import numpy as np
 import pytest
 import torch
@@ -78,3 +79,38 @@ def test_decisions_over_long_trees(seed, accept, phi, m, acc_cap):
     for k in ("argmax", "topk", "acc_len", "acc_nodes", "bonus", "winner", "commit", "scores", "status"):
         assert (o[k].cpu().numpy() == ref[k]).all(), k
     assert (ref["status"] & rs.RS_ST_BAD_POS).any()
+
+
+@pytest.mark.parametrize("V", [500, 8193])
+def test_trigger_over_row_ranges(V):
+    # a row per thread up to 256 rows of a request, more in rounds; rows of one
+    # chunk (V <= 8192) need no merge
+    rng = np.random.default_rng(V)
+    l, n = 5, np.array([1, 255, 256, 257, 0, 600])
+    B, R = len(n), int(n.sum())
+    row_off = np.concatenate([[0], np.cumsum(n)]).astype(np.int32)
+    z = (rng.standard_normal((R, V)) * rng.uniform(0.5, 6, (R, 1))).astype(np.float32)
+    for share in (0.0, 0.01, 0.5, 1.0):
+        commit = (rng.random(R) < share).astype(np.uint8)
+        hist, hist_n = rng.uniform(0.1, 3, (B, l)).astype(np.float32), rng.integers(0, l + 1, B).astype(np.int32)
+        p = rs.params(l=l)
+        h, hn = _cuda(hist), _cuda(hist_n)
+        ent, hb = torch.zeros(R, device="cuda"), torch.zeros(B, device="cuda")
+        ks, ok = torch.zeros(B, dtype=torch.int32, device="cuda"), torch.zeros(B, dtype=torch.uint8, device="cuda")
+        ws = torch.empty(max(256, rs.rs_entropy_gate_workspace_size(R, V)), dtype=torch.uint8, device="cuda")
+        for rows in (False, True):  # the whole call, then the push alone on its entropies
+            h.copy_(_cuda(hist))
+            hn.copy_(_cuda(hist_n))
+            if rows:
+                rs.rs_entropy_gate_rows(ent, _cuda(row_off), _cuda(commit), B, p, h, hn, ks, hb, ok)
+            else:
+                rs.rs_entropy_gate(_cuda(z), R, V, _cuda(row_off), _cuda(commit), B, p, h, hn, ent, ks, hb, ok, ws)
+            torch.cuda.synchronize()
+            got = ent.cpu().numpy().astype(np.float64)
+            assert np.abs(got - oracle.entropy_rows(z)).max() < 1e-3
+            g = oracle.gate(got, row_off, commit, hist, hist_n, l, f32(p.lambda_e), f32(p.theta_entropy))
+            assert (ks.cpu().numpy() == g["k_star"]).all() and (ok.cpu().numpy() == g["ok"]).all()
+            assert (hb.cpu().numpy() == g["h_best"].astype(np.float32)).all() and (hn.cpu().numpy() == g["hist_n"]).all()
+            for b in range(B):
+                k = int(g["hist_n"][b])
+                assert (h.cpu().numpy()[b, :k] == g["hist"].astype(np.float32)[b, :k]).all()
