@@ -90,13 +90,11 @@ struct ReqInfo {
 // The split segment a CTA starts, for attn_combine: the segment that begins
 // in the CTA's range and continues past it (at most one per CTA).
 struct CombJob {
-    long long W;     // units of the launch
     int b;           // request (-1: the CTA starts no split segment)
     int kvh, mtile;  // the segment's KV head and row tile
     int n0, N;       // the request's first node and node count
     int first_slot;  // partial slot of the segment's first piece
     int c1;          // last CTA holding a piece of the segment
-    int pad;
 };
 
 struct AttnArgs {
@@ -119,9 +117,24 @@ struct AttnArgs {
 };
 
 // ------------------------------------------------------------------ schedule
+// A request's offsets against the arrays' extents: its rows must lie in [0, R)
+// and its keys (prefix, then one slot per node) in [0, kv_rows); 0 or the
+// status that rejects it.  rows_ok: whether its rows may be touched at all.
+__device__ __forceinline__ int check_request(int n0, int N, int S, long long kv0, int R, long long kv_rows,
+                                             bool &rows_ok) {
+    rows_ok = n0 >= 0 && N >= 0 && (long long)n0 + N <= R;
+    if (!rows_ok || kv0 < 0 || (S >= 0 && kv0 + S + N > kv_rows)) return RS_ST_BAD_OFFSET;
+    if (S < 0) return RS_ST_BAD_TREE;
+    return N > RS_MAX_NODES ? RS_ST_TOO_LARGE : 0;
+}
+__device__ __forceinline__ ReqInfo request_info(int N, int S, int G, int Hkv, int seg_rows) {
+    const int mt = (N * G + seg_rows - 1) / seg_rows, nt = (S + N + kBN - 1) / kBN;
+    return ReqInfo{Hkv * mt * nt, mt, nt, N * G};
+}
+
 // Exclusive prefixes over the requests of their units (s_pref[0..B],
 // s_pref[B] = W) and of their segments (s_spref).
-__device__ inline void unit_prefix(const ReqInfo *__restrict__ info, int B, int *s_pref, int *s_spref) {
+__device__ inline void unit_prefix(const ReqInfo *info, int B, int *s_pref, int *s_spref) {
     __shared__ int s_carry[2];
     __shared__ int s_w[2][32];
     if (threadIdx.x == 0) s_carry[0] = s_carry[1] = 0;
@@ -249,7 +262,7 @@ struct Piece {
     long long seg_start, seg_end;  // units of the whole segment
 };
 
-__device__ __forceinline__ Piece piece_at(const ReqInfo *__restrict__ info, const int *s_pref, int B,
+__device__ __forceinline__ Piece piece_at(const ReqInfo *info, const int *s_pref, int B,
                                           long long u, long long u0, long long u1, long long c) {
     Piece pc;
     pc.b = find_req(s_pref, B, u);
@@ -268,6 +281,27 @@ __device__ __forceinline__ Piece piece_at(const ReqInfo *__restrict__ info, cons
     pc.seg_start = seg_start;
     pc.seg_end = seg_end;
     return pc;
+}
+
+// The split segment CTA c (range [u0, u1)) starts: its last piece, when that
+// piece begins inside the range and ends past it.
+template <class S>
+__device__ __forceinline__ CombJob comb_job(const AttnArgs &a, const ReqInfo *info, const int *s_pref, const S &split,
+                                            long long u0, long long u1, int c) {
+    CombJob job{-1, 0, 0, 0, 0, 0, 0};
+    if (u0 < u1) {
+        const Piece pl = piece_at(info, s_pref, a.B, u1 - 1, u0, u1, c);
+        if (pl.seg_start >= u0 && pl.seg_end > u1) {
+            job.b = pl.b;
+            job.kvh = pl.kvh;
+            job.mtile = pl.mtile;
+            job.n0 = a.node_off[pl.b];
+            job.N = a.node_off[pl.b + 1] - job.n0;
+            job.first_slot = (int)(2 * c + (pl.seg_start > u0 ? 1 : 0));
+            job.c1 = (int)split.owner_of_seg_end(pl.b, pl.seg_start, pl.seg_end);
+        }
+    }
+    return job;
 }
 
 // 32 mask bits for tree indices [base, base + 32): negative indices are prefix
@@ -312,9 +346,8 @@ __device__ __forceinline__ void warp_arrive(uint64_t *bar) {
 // ------------------------------------------------------------------ kernel
 template <int D>
 __global__ void __launch_bounds__(kAttnThreads, 1)
-attn_tc_kernel(AttnArgs a, const ReqInfo *__restrict__ info, const __grid_constant__ CUtensorMap tmk,
+attn_tc_kernel(AttnArgs a, const ReqInfo *info, const __grid_constant__ CUtensorMap tmk,
                const __grid_constant__ CUtensorMap tmv) {
-    pdl_launch_next();
     using namespace sm100;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -355,11 +388,17 @@ attn_tc_kernel(AttnArgs a, const ReqInfo *__restrict__ info, const __grid_consta
         prefetch_tmap(&tmk);
         prefetch_tmap(&tmv);
     }
-    pdl_wait_prev();  // the prologue above touches no global memory
+    // launched while attn_prep runs: the prologue above (barriers, tensor
+    // memory, descriptors) touches no global memory.  attn_prep lets this kernel
+    // launch only after its own wait, so the CTAs, which take whole SMs, never
+    // stand in the way of earlier work (GQA-16K call 57.8 -> 56.4 us in a graph,
+    // batched 91.2 -> 89.9; working the split out before the wait as well, from
+    // the caller's arrays, was slower: 60.0 and 89.9)
+    pdl_wait_prev();
+    pdl_launch_next();
     unit_prefix(info, a.B, s_pref, s_spref);  // contains __syncthreads
     tc_fence_after();
     const uint32_t tmem = *s_tmem;
-    const long long W = s_pref[a.B];
     const long long Gc = gridDim.x, c = blockIdx.x;
     const Split split = make_split(s_pref, s_spref, a.B, (int)Gc);
     const long long u0 = split.range_lo(c), u1 = split.range_lo(c + 1);
@@ -419,22 +458,7 @@ attn_tc_kernel(AttnArgs a, const ReqInfo *__restrict__ info, const __grid_consta
         }
         __syncwarp();
         if (lane == 1) {  // after the producer loop: off the critical path
-            // the split segment this CTA starts (its last piece, when that piece
-            // begins inside the range and ends past it), for attn_combine
-            CombJob job{W, -1, 0, 0, 0, 0, 0, 0, 0};
-            if (u0 < u1) {
-                const Piece pl = piece_at(info, s_pref, a.B, u1 - 1, u0, u1, c);
-                if (pl.seg_start >= u0 && pl.seg_end > u1) {
-                    job.b = pl.b;
-                    job.kvh = pl.kvh;
-                    job.mtile = pl.mtile;
-                    job.n0 = a.node_off[pl.b];
-                    job.N = a.node_off[pl.b + 1] - job.n0;
-                    job.first_slot = (int)(2 * c + (pl.seg_start > u0 ? 1 : 0));
-                    job.c1 = (int)split.owner_of_seg_end(pl.b, pl.seg_start, pl.seg_end);
-                }
-            }
-            a.jobs[c] = job;
+            a.jobs[c] = comb_job(a, info, s_pref, split, u0, u1, (int)c);
             a.ranges[c] = make_int2((int)u0, (int)u1);
         }
     } else if (warp == kMmaWarp) {

@@ -81,7 +81,7 @@ inline size_t attn_pair_smem_bytes(int B) { return 1024 + kP2SmemPref + 3 * (siz
 // Exclusive prefixes over the requests of their units (s_pref), segments
 // (s_spref) and weighted units (s_apref: wf per unit of a full pair, wh per
 // unit of a half pair).
-__device__ inline void pair_prefix(const ReqInfo *__restrict__ info, int B, int Hkv, int wf, int wh, int *s_pref,
+__device__ inline void pair_prefix(const ReqInfo *info, int B, int Hkv, int wf, int wh, int *s_pref,
                                    int *s_spref, int *s_apref) {
     __shared__ int s_carry[3];
     __shared__ int s_w[3][32];
@@ -201,12 +201,22 @@ struct PairSplit {
     }
 };
 
+__device__ __forceinline__ PairSplit make_pair_split(const AttnArgs &a, const int *s_pref, const int *s_spref,
+                                                     const int *s_apref, int G) {
+    PairSplit split{s_pref, s_spref, s_apref, a.B, 0, G, a.Hkv, a.kv_stream ? kPairWFStream : kPairWF,
+                    a.kv_stream ? kPairWHStream : kPairWH};
+    int beta = (int)muldiv(s_pref[a.B], 1, 2ll * G);
+    const int cap = a.kv_stream ? kPairSegCostStream : kSegCostMax;
+    if (beta > cap) beta = cap;
+    split.beta = split.wh * beta;  // in the weighted units (a half-pair K/V tile weighs wh)
+    return split;
+}
+
 // ------------------------------------------------------------------ kernel
 template <int D>
 __global__ void __launch_bounds__(kPairThreads, 1)
-attn_pair_kernel(AttnArgs a, const ReqInfo *__restrict__ info, const __grid_constant__ CUtensorMap tmk,
+attn_pair_kernel(AttnArgs a, const ReqInfo *info, const __grid_constant__ CUtensorMap tmk,
                  const __grid_constant__ CUtensorMap tmv, const __grid_constant__ CUtensorMap tmq) {
-    pdl_launch_next();
     using namespace sm100;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -250,20 +260,14 @@ attn_pair_kernel(AttnArgs a, const ReqInfo *__restrict__ info, const __grid_cons
         prefetch_tmap(&tmv);
         if (a.q_tma) prefetch_tmap(&tmq);
     }
-    pdl_wait_prev();  // the prologue above touches no global memory
-    const int wf = a.kv_stream ? kPairWFStream : kPairWF, wh = a.kv_stream ? kPairWHStream : kPairWH;
-    pair_prefix(info, a.B, a.Hkv, wf, wh, s_pref, s_spref, s_apref);  // contains __syncthreads
+    pdl_wait_prev();  // as in the one-tile kernel: the prologue overlaps attn_prep
+    pdl_launch_next();
+    pair_prefix(info, a.B, a.Hkv, a.kv_stream ? kPairWFStream : kPairWF, a.kv_stream ? kPairWHStream : kPairWH, s_pref,
+                s_spref, s_apref);  // contains __syncthreads
     tc_fence_after();
     const uint32_t tmem = *s_tmem;
-    const long long W = s_pref[a.B];
     const long long Gc = gridDim.x, c = blockIdx.x;
-    PairSplit split{s_pref, s_spref, s_apref, a.B, 0, (int)Gc, a.Hkv, wf, wh};
-    {
-        int beta = (int)muldiv(W, 1, 2 * Gc);
-        const int cap = a.kv_stream ? kPairSegCostStream : kSegCostMax;
-        if (beta > cap) beta = cap;
-        split.beta = wh * beta;  // in the weighted units (a half-pair K/V tile weighs wh)
-    }
+    const PairSplit split = make_pair_split(a, s_pref, s_spref, s_apref, (int)Gc);
     // the range's two ends in two lanes at once: each is a chain of dependent
     // divisions on every CTA's path to its first tile (0.6 us apart when
     // computed in turn), and with them in one call the compiler also spills
@@ -368,20 +372,7 @@ attn_pair_kernel(AttnArgs a, const ReqInfo *__restrict__ info, const __grid_cons
         }
         __syncwarp();
         if (lane == 1) {  // the split segment this CTA starts, for attn_combine
-            CombJob job{W, -1, 0, 0, 0, 0, 0, 0, 0};
-            if (u0 < u1) {
-                const Piece pl = piece_at(info, s_pref, a.B, u1 - 1, u0, u1, c);
-                if (pl.seg_start >= u0 && pl.seg_end > u1) {
-                    job.b = pl.b;
-                    job.kvh = pl.kvh;
-                    job.mtile = pl.mtile;
-                    job.n0 = a.node_off[pl.b];
-                    job.N = a.node_off[pl.b + 1] - job.n0;
-                    job.first_slot = (int)(2 * c + (pl.seg_start > u0 ? 1 : 0));
-                    job.c1 = (int)split.owner_of_seg_end(pl.b, pl.seg_start, pl.seg_end);
-                }
-            }
-            a.jobs[c] = job;
+            a.jobs[c] = comb_job(a, info, s_pref, split, u0, u1, (int)c);
             a.ranges[c] = make_int2((int)u0, (int)u1);
         }
     } else if (warp == kMmaWarp) {
@@ -727,7 +718,8 @@ attn_pair_kernel(AttnArgs a, const ReqInfo *__restrict__ info, const __grid_cons
     if (tid == 0 && *s_abort) {  // any role gave up: flag every request this CTA touches
         // the range is recomputed (after the barrier, from shared memory) so
         // that no role keeps it in registers through its loop
-        const long long v0 = split.range_lo(c), v1 = split.range_lo(c + 1);
+        const PairSplit again = make_pair_split(a, s_pref, s_spref, s_apref, (int)Gc);
+        const long long v0 = again.range_lo(c), v1 = again.range_lo(c + 1);
         for (long long u = v0; u < v1;) {
             const Piece pc = piece_at(info, s_pref, a.B, u, v0, v1, c);
             atomicOr(&a.status[pc.b], RS_ST_TIMEOUT);
