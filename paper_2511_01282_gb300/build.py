@@ -1,14 +1,18 @@
-"""Build ``librespec.so`` (sm_103a) in-tree with nvcc.
+"""Build ``librespec.so`` (sm_103a) and its Python binding in-tree.
 
-Each translation unit under ``csrc/`` is compiled in parallel, then linked
-into one shared library next to this file.  The CUDA runtime is linked
-statically, so the library needs only the driver at run time.
+Each CUDA translation unit under ``csrc/`` is compiled in parallel with nvcc,
+then linked into one shared library next to this file.  The CUDA runtime is
+linked statically, so the library needs only the driver at run time.
+``csrc/bind.cpp`` (the marshalling of ``respec.py``) is compiled beside them
+with g++ against the installed torch and linked to the library.
 """
 import concurrent.futures as cf
+import importlib.util
 import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
@@ -16,6 +20,8 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "librespec.so")
+BIND_SRC = os.path.join(CSRC, "bind.cpp")
+BIND = os.path.join(HERE, "_respec_bind.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -24,6 +30,13 @@ def _nvcc():
         if c and os.path.exists(c):
             return c
     raise RuntimeError("nvcc not found")
+
+
+def _torch_dir():
+    spec = importlib.util.find_spec("torch")
+    if spec is None:
+        raise RuntimeError("torch not found")
+    return list(spec.submodule_search_locations)[0]
 
 
 def sources():
@@ -56,12 +69,22 @@ def build(force=False, verbose=False, extra_flags=()):
         if force or _stale(obj, [src] + hdrs):
             jobs.append([nvcc] + flags + ["-c", src, "-o", obj])
 
+    torch_dir = _torch_dir()
+    torch_lib = os.path.join(torch_dir, "lib")
+    cuda_include = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc))), "include")
+    bind_obj = os.path.join(BUILD, "bind.o")
+    if force or _stale(bind_obj, [BIND_SRC, os.path.join(torch_dir, "version.py")] + hdrs):
+        jobs.append(["g++", "-O2", "-std=c++17", "-fPIC", "-I", INCLUDE, "-I", sysconfig.get_paths()["include"],
+                     "-I", os.path.join(torch_dir, "include"),
+                     "-I", os.path.join(torch_dir, "include", "torch", "csrc", "api", "include"),
+                     "-I", cuda_include, "-c", BIND_SRC, "-o", bind_obj])
+
     def run(cmd):
         r = subprocess.run(cmd, capture_output=True, text=True)
         if verbose or r.returncode != 0:
             sys.stderr.write(r.stdout + r.stderr)
         if r.returncode != 0:
-            raise RuntimeError("nvcc failed: " + " ".join(cmd))
+            raise RuntimeError("compile failed: " + " ".join(cmd))
         return r
 
     if jobs:
@@ -71,6 +94,12 @@ def build(force=False, verbose=False, extra_flags=()):
         tmp = LIB + ".tmp.%d" % os.getpid()
         run([nvcc] + ARCH + ["-shared", "-o", tmp] + objs)
         os.replace(tmp, LIB)
+    if force or _stale(BIND, [bind_obj]):
+        tmp = BIND + ".tmp.%d" % os.getpid()
+        run(["g++", "-shared", "-o", tmp, bind_obj, "-L", HERE, "-l:" + os.path.basename(LIB), "-L", torch_lib,
+             "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda", "-Wl,-rpath,$ORIGIN",
+             "-Wl,-rpath," + torch_lib])
+        os.replace(tmp, BIND)
     return LIB
 
 

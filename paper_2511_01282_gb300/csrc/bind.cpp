@@ -1,0 +1,402 @@
+// bind.cpp -- the marshalling of respec.py's entry points, in C++.
+//
+// Every function takes the arguments of the Python function of its name, in
+// order (tensors, None or integer addresses for the pointers; the workspace
+// tensor for (pointer, bytes); a stream, None or an integer handle), calls the
+// C entry point of librespec.so without the interpreter lock and returns its
+// status.  A call of 25 arguments cost ~10 us through ctypes on the host of a
+// GB300 (0.23 us a tensor for three attribute calls, 2.9 us to build a stream
+// object, 1.8 us of conversions), more than some of the kernels behind it.
+//
+// Integers and floats are converted as ctypes converts them (an int wraps to
+// the C type; anything else is refused).
+#define PY_SSIZE_T_CLEAN
+#include <Python.h>
+#include <c10/cuda/CUDAStream.h>
+#include <string.h>
+#include <torch/csrc/autograd/python_variable.h>
+#include <torch/version.h>
+
+#include <stdexcept>
+
+#include "respec.h"
+
+namespace {
+
+PyObject *g_params_type = nullptr, *g_argument_error = nullptr;
+
+struct PyFail {};  // a Python exception is set
+
+// The arguments of one call, taken in order.
+struct Args {
+    PyObject *const *v;
+    Py_ssize_t n, i = 0;
+    PyObject *next() {
+        if (i >= n) {
+            PyErr_SetString(PyExc_TypeError, "too few arguments");
+            throw PyFail{};
+        }
+        return v[i++];
+    }
+    [[noreturn]] void refuse(const char *what, PyObject *o) {
+        PyErr_Format(g_argument_error, "argument %zd: TypeError: %s instead of %s instance", i, what, Py_TYPE(o)->tp_name);
+        throw PyFail{};
+    }
+    // The address of a tensor, or of an object with a tensor's attributes; its
+    // bytes too where asked for.
+    void *address(PyObject *o, size_t *bytes) {
+        if (THPVariable_Check(o)) {
+            const at::Tensor &t = THPVariable_Unpack(o);
+            check(t.is_cuda(), t.is_contiguous(), o);
+            if (bytes) *bytes = (size_t)t.numel() * (size_t)t.element_size();
+            return t.data_ptr();
+        }
+        const bool cuda = number(PyObject_GetAttrString(o, "is_cuda")) != 0;
+        check(cuda, cuda && number(PyObject_CallMethod(o, "is_contiguous", nullptr)) != 0, o);
+        if (bytes)
+            *bytes = (size_t)(number(PyObject_CallMethod(o, "numel", nullptr)) *
+                              number(PyObject_CallMethod(o, "element_size", nullptr)));
+        return reinterpret_cast<void *>(number(PyObject_CallMethod(o, "data_ptr", nullptr)));
+    }
+    void check(bool cuda, bool contiguous, PyObject *o) {
+        if (!cuda) {
+            PyObject *d = PyObject_GetAttrString(o, "device");
+            if (d) PyErr_Format(PyExc_ValueError, "expected a CUDA tensor, got one on %S", d);
+            Py_XDECREF(d);
+            throw PyFail{};
+        }
+        if (!contiguous) {
+            PyErr_SetString(PyExc_ValueError, "expected a contiguous tensor");
+            throw PyFail{};
+        }
+    }
+    unsigned long long number(PyObject *x) {  // takes the reference
+        if (!x) throw PyFail{};
+        const unsigned long long r = PyLong_Check(x) ? PyLong_AsUnsignedLongLongMask(x) : (unsigned long long)PyObject_IsTrue(x);
+        Py_DECREF(x);
+        return r;
+    }
+    template <class T>
+    T *ptr() {
+        PyObject *o = next();
+        if (o == Py_None) return nullptr;
+        if (PyLong_Check(o)) return reinterpret_cast<T *>(masked(o));
+        return static_cast<T *>(address(o, nullptr));
+    }
+    unsigned long long masked(PyObject *o) {
+        const unsigned long long x = PyLong_AsUnsignedLongLongMask(o);
+        if (x == (unsigned long long)-1 && PyErr_Occurred()) throw PyFail{};
+        return x;
+    }
+    long long i64() {
+        PyObject *o = next();
+        if (!PyLong_Check(o)) refuse("int expected", o);
+        return (long long)masked(o);
+    }
+    int i32() { return (int)i64(); }
+    float f32() {
+        PyObject *o = next();
+        const double x = PyFloat_AsDouble(o);
+        if (x == -1.0 && PyErr_Occurred()) {
+            PyErr_Clear();
+            refuse("float expected", o);
+        }
+        return (float)x;
+    }
+    rs_params params() {
+        PyObject *o = next();
+        const int is = PyObject_IsInstance(o, g_params_type);
+        if (is < 0) throw PyFail{};
+        if (!is) refuse("expected rs_params", o);
+        Py_buffer b;
+        if (PyObject_GetBuffer(o, &b, PyBUF_SIMPLE) != 0) throw PyFail{};
+        rs_params p;
+        const bool fits = b.len == (Py_ssize_t)sizeof p;
+        if (fits) memcpy(&p, b.buf, sizeof p);
+        PyBuffer_Release(&b);
+        if (!fits) {
+            PyErr_SetString(PyExc_TypeError, "rs_params has another size");
+            throw PyFail{};
+        }
+        return p;
+    }
+    // a tensor as (pointer, bytes); None as (null, 0)
+    void *sized(size_t *bytes, bool optional) {
+        PyObject *o = next();
+        *bytes = 0;
+        if (o == Py_None && optional) return nullptr;
+        return address(o, bytes);
+    }
+    void *stream() {
+        PyObject *o = next();
+        if (o == Py_None) return c10::cuda::getCurrentCUDAStream().stream();
+        if (PyLong_Check(o)) return reinterpret_cast<void *>(masked(o));
+        PyObject *h = PyObject_GetAttrString(o, "cuda_stream");
+        if (!h) throw PyFail{};
+        unsigned long long x = 0;
+        const bool ok = PyLong_Check(h);
+        if (ok) x = PyLong_AsUnsignedLongLongMask(h);
+        Py_DECREF(h);
+        if (!ok) refuse("stream handle expected", o);
+        return reinterpret_cast<void *>(x);
+    }
+};
+
+// body(args) converts and returns a callable that makes the C call.
+template <class F>
+PyObject *guarded(PyObject *const *v, Py_ssize_t n, F body) {
+    try {
+        Args a{v, n};
+        auto call = body(a);
+        if (a.i != n) {
+            PyErr_SetString(PyExc_TypeError, "too many arguments");
+            return nullptr;
+        }
+        rs_status st;
+        Py_BEGIN_ALLOW_THREADS
+        st = call();
+        Py_END_ALLOW_THREADS
+        return PyLong_FromLong((long)st);
+    } catch (const PyFail &) {
+        return nullptr;
+    } catch (const std::exception &e) {
+        PyErr_SetString(PyExc_RuntimeError, e.what());
+        return nullptr;
+    }
+}
+
+#define RS_BIND(name) PyObject *name(PyObject *, PyObject *const *v, Py_ssize_t n)
+
+RS_BIND(entropy_gate) {
+    return guarded(v, n, [](Args &a) {
+        auto *logits = a.ptr<const float>();
+        const int R = a.i32(), V = a.i32();
+        auto *row_off = a.ptr<const int32_t>();
+        auto *row_commit = a.ptr<const uint8_t>();
+        const int B = a.i32();
+        const rs_params p = a.params();
+        auto *hist = a.ptr<float>();
+        auto *hist_n = a.ptr<int32_t>();
+        auto *entropy = a.ptr<float>();
+        auto *k_star = a.ptr<int32_t>();
+        auto *h_best = a.ptr<float>();
+        auto *ok = a.ptr<uint8_t>();
+        size_t wb;
+        void *ws = a.sized(&wb, true), *st = a.stream();
+        return [=] {
+            return rs_entropy_gate(logits, R, V, row_off, row_commit, B, p, hist, hist_n, entropy, k_star, h_best, ok, ws, wb, st);
+        };
+    });
+}
+
+RS_BIND(entropy_gate_noalloc) {
+    return guarded(v, n, [](Args &a) {
+        auto *logits = a.ptr<const float>();
+        const int R = a.i32(), V = a.i32();
+        auto *row_off = a.ptr<const int32_t>();
+        auto *row_commit = a.ptr<const uint8_t>();
+        const int B = a.i32();
+        const rs_params p = a.params();
+        auto *hist = a.ptr<float>();
+        auto *hist_n = a.ptr<int32_t>();
+        auto *entropy = a.ptr<float>();
+        auto *k_star = a.ptr<int32_t>();
+        auto *h_best = a.ptr<float>();
+        auto *ok = a.ptr<uint8_t>();
+        void *st = a.stream();
+        return [=] {
+            return rs_entropy_gate_noalloc(logits, R, V, row_off, row_commit, B, p, hist, hist_n, entropy, k_star, h_best, ok, st);
+        };
+    });
+}
+
+RS_BIND(entropy_gate_rows) {
+    return guarded(v, n, [](Args &a) {
+        auto *entropy = a.ptr<const float>();
+        auto *row_off = a.ptr<const int32_t>();
+        auto *row_commit = a.ptr<const uint8_t>();
+        const int B = a.i32();
+        const rs_params p = a.params();
+        auto *hist = a.ptr<float>();
+        auto *hist_n = a.ptr<int32_t>();
+        auto *k_star = a.ptr<int32_t>();
+        auto *h_best = a.ptr<float>();
+        auto *ok = a.ptr<uint8_t>();
+        void *st = a.stream();
+        return [=] { return rs_entropy_gate_rows(entropy, row_off, row_commit, B, p, hist, hist_n, k_star, h_best, ok, st); };
+    });
+}
+
+RS_BIND(match_scan) {
+    return guarded(v, n, [](Args &a) {
+        auto *tokens = a.ptr<const int32_t>();
+        auto *tok_off = a.ptr<const int64_t>();
+        const int B = a.i32();
+        auto *k_star = a.ptr<const int32_t>();
+        auto *gate_ok = a.ptr<const uint8_t>();
+        auto *scores = a.ptr<const float>();
+        const rs_params p = a.params();
+        const int cap = a.i32();
+        auto *count = a.ptr<int32_t>(), *pos = a.ptr<int32_t>(), *sel_pos = a.ptr<int32_t>(), *sel_len = a.ptr<int32_t>();
+        auto *spans = a.ptr<int32_t>(), *n_sel = a.ptr<int32_t>(), *status = a.ptr<int32_t>();
+        size_t wb;
+        void *ws = a.sized(&wb, true), *st = a.stream();
+        return [=] {
+            return rs_match_scan(tokens, tok_off, B, k_star, gate_ok, scores, p, cap, count, pos, sel_pos, sel_len, spans, n_sel,
+                                 status, ws, wb, st);
+        };
+    });
+}
+
+RS_BIND(tree_verify_attn) {
+    return guarded(v, n, [](Args &a) {
+        auto *q = a.ptr<const uint16_t>(), *k = a.ptr<const uint16_t>(), *vv = a.ptr<const uint16_t>();
+        const int64_t kv_rows = a.i64();
+        auto *kv_off = a.ptr<const int64_t>();
+        auto *ctx_len = a.ptr<const int32_t>(), *node_off = a.ptr<const int32_t>(), *parents = a.ptr<const int32_t>();
+        const int B = a.i32(), R = a.i32(), Hq = a.i32(), Hkv = a.i32(), D = a.i32();
+        const float scale = a.f32();
+        auto *out = a.ptr<float>(), *lse = a.ptr<float>();
+        auto *status = a.ptr<int32_t>();
+        size_t wb;
+        void *ws = a.sized(&wb, true), *st = a.stream();
+        return [=] {
+            return rs_tree_verify_attn(q, k, vv, kv_rows, kv_off, ctx_len, node_off, parents, B, R, Hq, Hkv, D, scale, out, lse,
+                                       status, ws, wb, st);
+        };
+    });
+}
+
+RS_BIND(accept) {
+    return guarded(v, n, [](Args &a) {
+        auto *logits = a.ptr<const float>();
+        const int R = a.i32(), V = a.i32();
+        auto *node_off = a.ptr<const int32_t>();
+        const int B = a.i32();
+        auto *tokens = a.ptr<const int32_t>(), *parents = a.ptr<const int32_t>();
+        auto *source = a.ptr<const uint8_t>();
+        auto *chain = a.ptr<const int8_t>();
+        auto *sel_pos = a.ptr<const int32_t>();
+        auto *tok_off = a.ptr<const int64_t>();
+        const rs_params p = a.params();
+        const int cap = a.i32();
+        auto *argmax = a.ptr<int32_t>(), *topk = a.ptr<int32_t>();
+        auto *lse = a.ptr<float>(), *p_tok = a.ptr<float>(), *entropy = a.ptr<float>();
+        auto *acc_len = a.ptr<int32_t>(), *acc_nodes = a.ptr<int32_t>(), *bonus = a.ptr<int32_t>(), *winner = a.ptr<int32_t>();
+        auto *commit = a.ptr<uint8_t>();
+        auto *scores = a.ptr<float>();
+        auto *status = a.ptr<int32_t>();
+        size_t wb;
+        void *ws = a.sized(&wb, true), *st = a.stream();
+        return [=] {
+            return rs_accept(logits, R, V, node_off, B, tokens, parents, source, chain, sel_pos, tok_off, p, cap, argmax, topk, lse,
+                             p_tok, entropy, acc_len, acc_nodes, bonus, winner, commit, scores, status, ws, wb, st);
+        };
+    });
+}
+
+RS_BIND(match_index_build) {
+    return guarded(v, n, [](Args &a) {
+        auto *tokens = a.ptr<const int32_t>();
+        auto *tok_off = a.ptr<const int64_t>();
+        const int B = a.i32(), V = a.i32();
+        const int64_t total = a.i64();
+        size_t ib;
+        void *index = a.sized(&ib, false), *st = a.stream();
+        return [=] { return rs_match_index_build(tokens, tok_off, B, V, total, index, ib, st); };
+    });
+}
+
+RS_BIND(match_index_append) {
+    return guarded(v, n, [](Args &a) {
+        auto *tokens = a.ptr<const int32_t>();
+        auto *tok_off = a.ptr<const int64_t>();
+        const int B = a.i32(), V = a.i32();
+        const int64_t total = a.i64();
+        size_t ib;
+        void *index = a.sized(&ib, false);
+        auto *status = a.ptr<int32_t>();
+        void *st = a.stream();
+        return [=] { return rs_match_index_append(tokens, tok_off, B, V, total, index, ib, status, st); };
+    });
+}
+
+RS_BIND(match_scan_indexed) {
+    return guarded(v, n, [](Args &a) {
+        auto *tokens = a.ptr<const int32_t>();
+        auto *tok_off = a.ptr<const int64_t>();
+        const int B = a.i32();
+        auto *k_star = a.ptr<const int32_t>();
+        auto *gate_ok = a.ptr<const uint8_t>();
+        auto *scores = a.ptr<const float>();
+        const rs_params p = a.params();
+        const int cap = a.i32();
+        auto *count = a.ptr<int32_t>(), *pos = a.ptr<int32_t>(), *sel_pos = a.ptr<int32_t>(), *sel_len = a.ptr<int32_t>();
+        auto *spans = a.ptr<int32_t>(), *n_sel = a.ptr<int32_t>(), *status = a.ptr<int32_t>();
+        const int V = a.i32();
+        const int64_t total = a.i64();
+        size_t ib;
+        void *index = a.sized(&ib, false), *st = a.stream();
+        return [=] {
+            return rs_match_scan_indexed(tokens, tok_off, B, k_star, gate_ok, scores, p, cap, count, pos, sel_pos, sel_len, spans,
+                                         n_sel, status, V, total, index, ib, st);
+        };
+    });
+}
+
+RS_BIND(tree_sample) {
+    return guarded(v, n, [](Args &a) {
+        auto *logits = a.ptr<const float>();
+        const int R = a.i32(), V = a.i32();
+        auto *node_off = a.ptr<const int32_t>();
+        const int B = a.i32();
+        auto *tokens = a.ptr<const int32_t>(), *parents = a.ptr<const int32_t>();
+        auto *source = a.ptr<const uint8_t>();
+        const float T = a.f32();
+        auto *uniforms = a.ptr<const float>();
+        const int cap = a.i32();
+        auto *draw = a.ptr<int32_t>(), *acc_len = a.ptr<int32_t>(), *acc_nodes = a.ptr<int32_t>(), *bonus = a.ptr<int32_t>();
+        auto *status = a.ptr<int32_t>();
+        size_t wb;
+        void *ws = a.sized(&wb, true), *st = a.stream();
+        return [=] {
+            return rs_tree_sample(logits, R, V, node_off, B, tokens, parents, source, T, uniforms, cap, draw, acc_len, acc_nodes,
+                                  bonus, status, ws, wb, st);
+        };
+    });
+}
+
+// setup(rs_params type): the type the params argument must have.
+PyObject *setup(PyObject *, PyObject *type) {
+    Py_INCREF(type);
+    Py_XSETREF(g_params_type, type);
+    Py_RETURN_NONE;
+}
+
+#define RS_METHOD(name) {"rs_" #name, reinterpret_cast<PyCFunction>(reinterpret_cast<void *>(name)), METH_FASTCALL, nullptr}
+PyMethodDef kMethods[] = {RS_METHOD(entropy_gate),
+                          RS_METHOD(entropy_gate_noalloc),
+                          RS_METHOD(entropy_gate_rows),
+                          RS_METHOD(match_scan),
+                          RS_METHOD(tree_verify_attn),
+                          RS_METHOD(accept),
+                          RS_METHOD(match_index_build),
+                          RS_METHOD(match_index_append),
+                          RS_METHOD(match_scan_indexed),
+                          RS_METHOD(tree_sample),
+                          {"setup", setup, METH_O, nullptr},
+                          {nullptr, nullptr, 0, nullptr}};
+PyModuleDef kModule = {PyModuleDef_HEAD_INIT, "_respec_bind", nullptr, -1, kMethods, nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit__respec_bind() {
+    PyObject *ctypes = PyImport_ImportModule("ctypes");
+    if (!ctypes) return nullptr;
+    g_argument_error = PyObject_GetAttrString(ctypes, "ArgumentError");
+    Py_DECREF(ctypes);
+    if (!g_argument_error) return nullptr;
+    PyObject *m = PyModule_Create(&kModule);
+    if (m && PyModule_AddStringConstant(m, "torch_version", TORCH_VERSION) != 0) Py_CLEAR(m);
+    return m;
+}

@@ -3,17 +3,21 @@
 Argument marshalling only: every function here has the name and argument
 order of its C entry point, turns torch tensors into device pointers, calls
 the library and raises ``RespecError`` with the library's message when the
-call returns a non-zero status.  All computation happens in the CUDA
+call returns a non-zero status.  The calls that launch kernels are marshalled
+in C++ (``csrc/bind.cpp``): a decoding step is many small calls, and through
+ctypes each cost ~10 us of host time.  All computation happens in the CUDA
 kernels; there is no fallback of any kind -- without the compiled library
 (or without a GPU) every call fails.
 """
 import ctypes as C
+import importlib.util
 import os
 
 import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "librespec.so")
+BIND_PATH = os.path.join(_HERE, "_respec_bind.so")
 
 RS_OK, RS_ERR_INVALID_ARG, RS_ERR_UNSUPPORTED, RS_ERR_CAPACITY, RS_ERR_CUDA = range(5)
 RS_ST_BAD_TREE, RS_ST_TRUNCATED, RS_ST_BAD_POS, RS_ST_TOO_LARGE, RS_ST_TIMEOUT = 1, 2, 4, 8, 16
@@ -98,24 +102,26 @@ def exported_symbols():
     return list(_SIGS)
 
 
-def _ptr(t):
-    if t is None:
-        return None
-    if isinstance(t, int):
-        return t
-    if not t.is_cuda:
-        raise ValueError("expected a CUDA tensor, got one on %s" % t.device)
-    if not t.is_contiguous():
-        raise ValueError("expected a contiguous tensor")
-    return t.data_ptr()
+_bind = None
 
 
-def _stream(stream):
-    if stream is None:
-        return torch.cuda.current_stream().cuda_stream
-    if isinstance(stream, int):
-        return stream
-    return stream.cuda_stream
+def _native():
+    """The C++ marshalling module, built in-tree beside the library."""
+    global _bind
+    if _bind is None:
+        lib()
+        if not os.path.exists(BIND_PATH):
+            raise RuntimeError("_respec_bind.so is not built: run paper_2511_01282_gb300.build.build() "
+                               "(or __graft_entry__.build())")
+        spec = importlib.util.spec_from_file_location("_respec_bind", BIND_PATH)
+        m = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(m)
+        if not torch.__version__.startswith(m.torch_version):
+            raise RuntimeError("_respec_bind.so was built for torch %s, this is %s: rebuild it"
+                               % (m.torch_version, torch.__version__))
+        m.setup(rs_params)
+        _bind = m
+    return _bind
 
 
 def _check(status):
@@ -135,12 +141,6 @@ def rs_launch_count():
     return int(lib().rs_launch_count())
 
 
-def _ws(ws):
-    if ws is None:
-        return None, 0
-    return _ptr(ws), ws.numel() * ws.element_size()
-
-
 # ------------------------------------------------------------ entry points
 def rs_entropy_gate_workspace_size(R, V):
     return int(lib().rs_entropy_gate_workspace_size(R, V))
@@ -148,10 +148,8 @@ def rs_entropy_gate_workspace_size(R, V):
 
 def rs_entropy_gate(logits, R, V, row_off, row_commit, B, p, hist, hist_n, entropy, k_star,
                     h_best, entropy_ok, workspace, stream=None):
-    wp, wb = _ws(workspace)
-    _check(lib().rs_entropy_gate(_ptr(logits), R, V, _ptr(row_off), _ptr(row_commit), B, p,
-                                 _ptr(hist), _ptr(hist_n), _ptr(entropy), _ptr(k_star),
-                                 _ptr(h_best), _ptr(entropy_ok), wp, wb, _stream(stream)))
+    _check((_bind or _native()).rs_entropy_gate(logits, R, V, row_off, row_commit, B, p, hist, hist_n, entropy,
+                                                k_star, h_best, entropy_ok, workspace, stream))
 
 
 RS_GATE_NOALLOC_MAX_PARTIALS = 65536
@@ -161,9 +159,8 @@ def rs_entropy_gate_noalloc(logits, R, V, row_off, row_commit, B, p, hist, hist_
                             h_best, entropy_ok, stream=None):
     """rs_entropy_gate with the library's fixed scratch array instead of a
     caller workspace (for callers that cannot allocate device memory)."""
-    _check(lib().rs_entropy_gate_noalloc(_ptr(logits), R, V, _ptr(row_off), _ptr(row_commit), B, p,
-                                         _ptr(hist), _ptr(hist_n), _ptr(entropy), _ptr(k_star),
-                                         _ptr(h_best), _ptr(entropy_ok), _stream(stream)))
+    _check((_bind or _native()).rs_entropy_gate_noalloc(logits, R, V, row_off, row_commit, B, p, hist, hist_n,
+                                                        entropy, k_star, h_best, entropy_ok, stream))
 
 
 def rs_match_scan_workspace_size(B):
@@ -172,11 +169,8 @@ def rs_match_scan_workspace_size(B):
 
 def rs_match_scan(tokens, tok_off, B, k_star, gate_ok, scores, p, pos_cap, count, pos, sel_pos,
                   sel_len, spans, n_sel, status, workspace=None, stream=None):
-    wp, wb = _ws(workspace)
-    _check(lib().rs_match_scan(_ptr(tokens), _ptr(tok_off), B, _ptr(k_star), _ptr(gate_ok),
-                               _ptr(scores), p, pos_cap, _ptr(count), _ptr(pos), _ptr(sel_pos),
-                               _ptr(sel_len), _ptr(spans), _ptr(n_sel), _ptr(status), wp, wb,
-                               _stream(stream)))
+    _check((_bind or _native()).rs_match_scan(tokens, tok_off, B, k_star, gate_ok, scores, p, pos_cap, count,
+                                              pos, sel_pos, sel_len, spans, n_sel, status, workspace, stream))
 
 
 def rs_tree_verify_attn_workspace_size(B, R, Hq, Hkv, D):
@@ -185,11 +179,8 @@ def rs_tree_verify_attn_workspace_size(B, R, Hq, Hkv, D):
 
 def rs_tree_verify_attn(q, k, v, kv_rows, kv_off, ctx_len, node_off, parents, B, R, Hq, Hkv, D,
                         scale, out, lse, status, workspace, stream=None):
-    wp, wb = _ws(workspace)
-    _check(lib().rs_tree_verify_attn(_ptr(q), _ptr(k), _ptr(v), kv_rows, _ptr(kv_off),
-                                     _ptr(ctx_len), _ptr(node_off), _ptr(parents), B, R, Hq, Hkv,
-                                     D, scale, _ptr(out), _ptr(lse), _ptr(status), wp, wb,
-                                     _stream(stream)))
+    _check((_bind or _native()).rs_tree_verify_attn(q, k, v, kv_rows, kv_off, ctx_len, node_off, parents, B, R,
+                                                    Hq, Hkv, D, scale, out, lse, status, workspace, stream))
 
 
 def rs_accept_workspace_size(R, V, beta):
@@ -201,22 +192,18 @@ def rs_match_index_bytes(B, V, t_total):
 
 
 def rs_match_index_build(tokens, tok_off, B, V, t_total, index, stream=None):
-    _check(lib().rs_match_index_build(_ptr(tokens), _ptr(tok_off), B, V, t_total, _ptr(index),
-                                      index.numel() * index.element_size(), _stream(stream)))
+    _check((_bind or _native()).rs_match_index_build(tokens, tok_off, B, V, t_total, index, stream))
 
 
 def rs_match_index_append(tokens, tok_off, B, V, t_total, index, status=None, stream=None):
-    _check(lib().rs_match_index_append(_ptr(tokens), _ptr(tok_off), B, V, t_total, _ptr(index),
-                                       index.numel() * index.element_size(), _ptr(status), _stream(stream)))
+    _check((_bind or _native()).rs_match_index_append(tokens, tok_off, B, V, t_total, index, status, stream))
 
 
 def rs_match_scan_indexed(tokens, tok_off, B, k_star, gate_ok, scores, p, pos_cap, count, pos, sel_pos,
                           sel_len, spans, n_sel, status, V, t_total, index, stream=None):
-    _check(lib().rs_match_scan_indexed(_ptr(tokens), _ptr(tok_off), B, _ptr(k_star), _ptr(gate_ok),
-                                       _ptr(scores), p, pos_cap, _ptr(count), _ptr(pos), _ptr(sel_pos),
-                                       _ptr(sel_len), _ptr(spans), _ptr(n_sel), _ptr(status), V, t_total,
-                                       _ptr(index), index.numel() * index.element_size(),
-                                       _stream(stream)))
+    _check((_bind or _native()).rs_match_scan_indexed(tokens, tok_off, B, k_star, gate_ok, scores, p, pos_cap,
+                                                      count, pos, sel_pos, sel_len, spans, n_sel, status, V,
+                                                      t_total, index, stream))
 
 
 def rs_tree_sample_workspace_size(R, V):
@@ -225,26 +212,20 @@ def rs_tree_sample_workspace_size(R, V):
 
 def rs_tree_sample(logits, R, V, node_off, B, tokens, parents, source, temperature, uniforms,
                    acc_cap, draw, acc_len, acc_nodes, bonus, status, workspace, stream=None):
-    wp, wb = _ws(workspace)
-    _check(lib().rs_tree_sample(_ptr(logits), R, V, _ptr(node_off), B, _ptr(tokens),
-                                _ptr(parents), _ptr(source), float(temperature), _ptr(uniforms),
-                                acc_cap, _ptr(draw), _ptr(acc_len), _ptr(acc_nodes), _ptr(bonus),
-                                _ptr(status), wp, wb, _stream(stream)))
+    _check((_bind or _native()).rs_tree_sample(logits, R, V, node_off, B, tokens, parents, source,
+                                               float(temperature), uniforms, acc_cap, draw, acc_len, acc_nodes,
+                                               bonus, status, workspace, stream))
 
 
 def rs_accept(logits, R, V, node_off, B, tokens, parents, source, chain, sel_pos, tok_off, p,
               acc_cap, argmax, topk, lse, p_tok, entropy, acc_len, acc_nodes, bonus, winner, commit,
               scores, status, workspace, stream=None):
-    wp, wb = _ws(workspace)
-    _check(lib().rs_accept(_ptr(logits), R, V, _ptr(node_off), B, _ptr(tokens), _ptr(parents),
-                           _ptr(source), _ptr(chain), _ptr(sel_pos), _ptr(tok_off), p, acc_cap,
-                           _ptr(argmax), _ptr(topk), _ptr(lse), _ptr(p_tok), _ptr(entropy),
-                           _ptr(acc_len), _ptr(acc_nodes), _ptr(bonus), _ptr(winner),
-                           _ptr(commit), _ptr(scores), _ptr(status), wp, wb, _stream(stream)))
+    _check((_bind or _native()).rs_accept(logits, R, V, node_off, B, tokens, parents, source, chain, sel_pos,
+                                          tok_off, p, acc_cap, argmax, topk, lse, p_tok, entropy, acc_len,
+                                          acc_nodes, bonus, winner, commit, scores, status, workspace, stream))
 
 
 def rs_entropy_gate_rows(entropy, row_off, row_commit, B, p, hist, hist_n, k_star, h_best,
                          entropy_ok, stream=None):
-    _check(lib().rs_entropy_gate_rows(_ptr(entropy), _ptr(row_off), _ptr(row_commit), B, p,
-                                      _ptr(hist), _ptr(hist_n), _ptr(k_star), _ptr(h_best),
-                                      _ptr(entropy_ok), _stream(stream)))
+    _check((_bind or _native()).rs_entropy_gate_rows(entropy, row_off, row_commit, B, p, hist, hist_n, k_star,
+                                                     h_best, entropy_ok, stream))
