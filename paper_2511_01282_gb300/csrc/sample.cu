@@ -429,7 +429,11 @@ template <int kW>
 __global__ void __launch_bounds__(kSmpThreads)
 sample_partial(const float *__restrict__ logits, int V, int nchunks, float scale, ChunkMass *__restrict__ part,
                int *__restrict__ n_flag) {
-    pdl_enter();
+    // the later kernels read the caller's arrays before they wait for this
+    // call's (uniforms, the chosen logits' tree), so they may launch only once
+    // this kernel's own wait is over
+    pdl_wait_prev();
+    pdl_launch_next();
     if (blockIdx.x == 0 && threadIdx.x == 0) *n_flag = 0;  // the flagged list of this call (filled by kernel 2)
     __shared__ float s_w[kSmpWarps];
     __shared__ float2 s_w2[kSmpWarps];
@@ -467,10 +471,10 @@ sample_partial(const float *__restrict__ logits, int V, int nchunks, float scale
 template <int kW>
 __global__ void __launch_bounds__(kSmpThreads)
 sample_pick(const float *__restrict__ logits, int V, int nchunks, float scale, float lam_h, float lam_l,
-            const Exp2Tab tab, const ChunkMass *__restrict__ part, const float *__restrict__ uniforms, int force,
+            const Exp2Tab tab, const ChunkMass *part, const float *__restrict__ uniforms, int force,
             int *__restrict__ n_flag, FlagRow *__restrict__ flags, int *__restrict__ done,
             int32_t *__restrict__ draw) {
-    pdl_enter();
+    pdl_launch_next();
     __shared__ float2 s_tab[64];
     __shared__ RowDecision s_dec;
     __shared__ float s_wt[kSmpWarps];
@@ -481,9 +485,11 @@ sample_pick(const float *__restrict__ logits, int V, int nchunks, float scale, f
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const float *row = logits + (long long)r * V;
     if (tid < 64) s_tab[tid] = tab.t[tid];
+    const float ur = uniforms[r];
     __syncthreads();
+    pdl_wait_prev();  // the chunk masses are complete
     if (warp == 0) {
-        const RowDecision d = decide_row(part + (long long)r * nchunks, nchunks, uniforms[r], lam_h, lam_l, s_tab);
+        const RowDecision d = decide_row(part + (long long)r * nchunks, nchunks, ur, lam_h, lam_l, s_tab);
         if (lane == 0) s_dec = d;
     }
     __syncthreads();
@@ -665,10 +671,10 @@ __device__ int last_with_mass(const float *row, long long end, float M, double i
 // paths (u Z below 2^-40 Z, the last id with mass).
 __global__ void __launch_bounds__(kSmpThreads)
 sample_exact(const float *__restrict__ logits, int V, int nslices, float lam_h, float lam_l, double inv_t, double T,
-             const Exp2Tab tab, const float *__restrict__ uniforms, const int *__restrict__ n_flag,
-             const FlagRow *__restrict__ flags, int *__restrict__ done, float2 *__restrict__ slice_sum,
+             const Exp2Tab tab, const float *__restrict__ uniforms, const int *n_flag,
+             const FlagRow *flags, int *__restrict__ done, float2 *__restrict__ slice_sum,
              int32_t *__restrict__ draw) {
-    pdl_enter();
+    pdl_launch_next();
     __shared__ float2 s_tab[64];
     __shared__ DF s_w[kSmpWarps + 1];
     __shared__ double s_wd[kSmpWarps];
@@ -676,13 +682,14 @@ sample_exact(const float *__restrict__ logits, int V, int nslices, float lam_h, 
     __shared__ int s_i, s_fin;
     __shared__ DF s_pk;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid < 64) s_tab[tid] = tab.t[tid];
+    pdl_wait_prev();  // the flagged list is complete
     const int n = *n_flag;
     const long long want = (long long)n * nslices;
     const int G = (int)max(1ll, (want + gridDim.x - 1) / gridDim.x);  // slices per item
     const int ng = (nslices + G - 1) / G;                              // items per row
     const long long items = (long long)n * ng;
     if (blockIdx.x >= items) return;  // uniform over the CTA
-    if (tid < 64) s_tab[tid] = tab.t[tid];
     __syncthreads();
     {
         for (long long it = blockIdx.x; it < items; it += gridDim.x) {
@@ -812,18 +819,21 @@ sample_exact(const float *__restrict__ logits, int V, int nslices, float lam_h, 
 }
 
 // One warp per request: the tree check and the walk along model children.
+// kEarly: behind this call's own row kernels, the tree is read and checked
+// before the wait for them; only the draws are read after it.
+template <bool kEarly>
 __global__ void __launch_bounds__(32)
 sample_walk(const int32_t *__restrict__ node_off, int R, const int32_t *__restrict__ tokens,
             const int32_t *__restrict__ parents, const uint8_t *__restrict__ source,
-            const int32_t *__restrict__ draw, int acc_cap, int32_t *__restrict__ acc_len,
+            const int32_t *draw, int acc_cap, int32_t *__restrict__ acc_len,
             int32_t *__restrict__ acc_nodes, int32_t *__restrict__ bonus, int32_t *__restrict__ status) {
-    pdl_enter();
+    pdl_launch_next();
+    if (!kEarly) pdl_wait_prev();
     constexpr int kPer = RS_MAX_NODES / 32;
     const int b = blockIdx.x, lane = threadIdx.x;
     const int n0 = node_off[b];
     const int N = node_off[b + 1] - n0;
     int32_t *an = acc_nodes + (long long)b * acc_cap;
-    for (int j = lane; j < acc_cap; j += 32) an[j] = -1;
     int st = 0;
     if (n0 < 0 || N < 0 || (long long)n0 + N > R) st = RS_ST_BAD_OFFSET;  // rows outside [0, R): not read
     else if (N > RS_MAX_NODES) st = RS_ST_TOO_LARGE;
@@ -843,13 +853,20 @@ sample_walk(const int32_t *__restrict__ node_off, int R, const int32_t *__restri
             const int pa = parents[n0 + i], sr = source[n0 + i];
             par[q] = pa;
             tok[q] = tokens[n0 + i];
-            drw[q] = draw[n0 + i];
             model[q] = sr == 1;
             if (i == 0) bad |= pa != -1 || sr != 0;
             else bad |= pa < 0 || pa >= i || sr < 1 || sr > 2;
         }
     }
     if (st == 0 && __any_sync(0xffffffffu, bad)) st = RS_ST_BAD_TREE;
+    if (kEarly) pdl_wait_prev();  // the draws are complete
+    if (st == 0) {
+#pragma unroll
+        for (int q = 0; q < kPer; ++q)
+            if (lane + 32 * q < N) drw[q] = draw[n0 + lane + 32 * q];
+    }
+    for (int j = lane; j < acc_cap; j += 32) an[j] = -1;
+    __syncwarp();  // before lane 0 writes the accepted nodes over them
     if (st != 0) {
         if (lane == 0) {
             acc_len[b] = 0;
@@ -993,14 +1010,18 @@ extern "C" rs_status rs_tree_sample(const float *logits, int R, int V, const int
             launch_pdl(sample_pick<1>, dim3(R), blk, 0, st, logits, V, nchunks, scale, lam_h, lam_l, tab, part,
                        uniforms, force, n_flag, flags, done, draw);
         RS_CHECK_LAUNCH("rs_tree_sample/pick");
+        // eight blocks an SM: the slices of a few flagged rows (one or two in a
+        // hundred) are an item each, with none to do in turn (145 rows, V = 128256,
+        // the call: 33.7 us with two blocks an SM, 33.0 with four, 32.4 with eight);
+        // blocks without items leave at once
         const long long items = (long long)R * nslices;
-        const unsigned egrid = (unsigned)std::min<long long>(items, 2ll * num_sms());
+        const unsigned egrid = (unsigned)std::min<long long>(items, 8ll * num_sms());
         launch_pdl(sample_exact, dim3(egrid), blk, 0, st, logits, V, nslices, lam_h, lam_l, inv_t, T, tab, uniforms,
                    n_flag, flags, done, sums, draw);
         RS_CHECK_LAUNCH("rs_tree_sample/exact");
     }
     if (B > 0) {
-        launch_pdl(sample_walk, dim3(B), dim3(32), 0, st, node_off, R, tokens, parents, source, draw, acc_cap, acc_len,
+        launch_pdl(R > 0 ? sample_walk<true> : sample_walk<false>, dim3(B), dim3(32), 0, st, node_off, R, tokens, parents, source, draw, acc_cap, acc_len,
             acc_nodes, bonus, status);
         RS_CHECK_LAUNCH("rs_tree_sample/walk");
     }
