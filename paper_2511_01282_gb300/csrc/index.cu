@@ -455,6 +455,8 @@ index_append(const int32_t *__restrict__ tokens, const int64_t *__restrict__ tok
     __shared__ long long s_cut;
     __shared__ int s_novf;
     const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    long long built = ix.built[b];  // read beside the offsets; unused in an index that holds nothing
+    int novf = ix.ovf_n[b];
     const long long t0 = tok_off[b], t = tok_off[b + 1] - t0;
     // an index whose build saw inconsistent offsets holds nothing, and the
     // buffers hold tok_off[B] tokens: otherwise nothing is read or written
@@ -467,8 +469,6 @@ index_append(const int32_t *__restrict__ tokens, const int64_t *__restrict__ tok
     int32_t *len = ix.len + (long long)b * (V + 1);
     int32_t *ovf = ix.list + ix.base[b];
     int32_t *buckets = ovf + kOvf;
-    long long built = ix.built[b];
-    int novf = ix.ovf_n[b];
     bool full = false;
     for (long long r0 = built; r0 < t && !full; r0 += kAppThreads) {
         const long long p = r0 + tid;
@@ -544,23 +544,23 @@ struct ListSource {
     static constexpr int kRows = 2;
     static constexpr bool kLaneMajor = false;
     const int32_t *blist, *olist;
-    long long nb, no, ncand, tail0;
-    __device__ __forceinline__ int cand(long long c) const {
+    int nb, no, ncand, tail0;
+    __device__ __forceinline__ int cand(int c) const {
         if (c < nb) return blist[c];
         if (c < nb + no) return olist[c - nb];
-        return (int)(tail0 + (c - nb - no));
+        return tail0 + (c - nb - no);
     }
-    __device__ __forceinline__ int pos(long long row, int lane, int e) const { return cand(128 * row + 32 * e + lane); }
-    __device__ __forceinline__ uint32_t test(const MatReq &q, long long r0, long long end, int lane) const {
+    __device__ __forceinline__ int pos(int row, int lane, int e) const { return cand(128 * row + 32 * e + lane); }
+    __device__ __forceinline__ uint32_t test(const MatReq &q, int r0, int end, int lane) const {
         int p[4 * kRows], x0[4 * kRows], x1[4 * kRows];
 #pragma unroll
         for (int j = 0; j < 4 * kRows; ++j) {
-            const long long c = 128 * (r0 + (j >> 2)) + 32 * (j & 3) + lane;
+            const int c = 128 * (r0 + (j >> 2)) + 32 * (j & 3) + lane;
             p[j] = r0 + (j >> 2) < end && c < ncand ? cand(c) : -1;
         }
 #pragma unroll
         for (int j = 0; j < 4 * kRows; ++j) {
-            const bool in = p[j] >= q.k - 1 && (long long)p[j] <= q.t - 2;
+            const bool in = p[j] >= q.k - 1 && p[j] <= q.t - 2;
             if (!in) p[j] = -1;
             x0[j] = in ? q.X[p[j]] : 0;
             x1[j] = in && q.k > 1 ? q.X[p[j] - 1] : 0;
@@ -579,10 +579,7 @@ struct ListSource {
     }
 };
 
-// One round of CTA 0's warps; longer candidate lists are split over the cluster.
-constexpr long long kQrySoloRows = kMatWarps * ListSource::kRows;
-
-__global__ void __cluster_dims__(kMatCluster, 1, 1) __launch_bounds__(kMatThreads)
+__global__ void __launch_bounds__(kMatThreads)
 index_query(const int32_t *__restrict__ tokens, const int64_t *__restrict__ tok_off, int V,
             const int32_t *__restrict__ k_star, const uint8_t *__restrict__ gate_ok,
             const float *__restrict__ scores, IndexView ix, MatOut o) {
@@ -603,14 +600,14 @@ index_query(const int32_t *__restrict__ tokens, const int64_t *__restrict__ tok_
         src.blist = src.olist + kOvf + start_of(ix.first[(long long)b * (V + 2) + bk], bk);
         src.nb = ix.len[(long long)b * (V + 1) + bk];
         src.no = novf;
-        src.tail0 = built < q.t ? built : q.t;
-        const long long nt = q.t - 1 - src.tail0;  // tail: positions tail0 .. t - 2
+        src.tail0 = (int)(built < q.t ? built : q.t);
+        const int nt = q.t - 1 - src.tail0;  // tail: positions tail0 .. t - 2
         src.ncand = src.nb + src.no + (nt > 0 ? nt : 0);
     }
-    const long long rows = (src.ncand + 127) / 128;
-    const bool solo = rows <= kQrySoloRows;
-    if (solo && crank != 0) return;
-    mat_body(src, q, rows, solo, b, crank, sh, qry_bits, o);
+    const int rows = (src.ncand + 127) / 128;
+    const int nc = mat_ctas<ListSource>(rows);
+    if (crank >= nc) return;
+    mat_body(src, q, rows, nc, b, crank, sh, qry_bits, o);
 }
 
 }  // namespace
@@ -732,20 +729,8 @@ extern "C" rs_status rs_match_scan_indexed(const int32_t *tokens, const int64_t 
     if (B == 0) return RS_OK;
     IndexView ix;
     carve_index(const_cast<void *>(index), B, V, t_total, &ix);
-    static int attr_done[64] = {0};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev >= 0 && dev < 64 && !attr_done[dev]) {
-        const cudaError_t ce = cudaFuncSetAttribute(index_query, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMatSmem);
-        if (ce != cudaSuccess) {
-            set_error("rs_match_scan_indexed: cudaFuncSetAttribute: %s", cudaGetErrorString(ce));
-            return RS_ERR_CUDA;
-        }
-        attr_done[dev] = 1;
-    }
     const MatOut o{count, pos, sel_pos, sel_len, spans, n_sel, status, p.theta_score, p.top_c, p.span_len, pos_cap};
-    launch_pdl(index_query, dim3(kMatCluster, B), dim3(kMatThreads), kMatSmem, (cudaStream_t)stream, tokens, tok_off, V,
-        k_star, gate_ok, scores, ix, o);
-    RS_CHECK_LAUNCH("rs_match_scan_indexed");
-    return RS_OK;
+    static int attr_done[64] = {0};
+    return mat_launch("rs_match_scan_indexed", attr_done, index_query, B, (cudaStream_t)stream, tokens, tok_off, V, k_star,
+                      gate_ok, scores, ix, o);
 }

@@ -1,7 +1,7 @@
 // match.cuh -- the part that rs_match_scan and rs_match_scan_indexed share:
-// one cluster of 8 CTAs (512 threads each) per request tests its candidate
-// positions against the key, counts and lists the matches in ascending order,
-// ranks those that clear theta_score and gathers the selected continuations.
+// one cluster of CTAs per request tests its candidate positions against the
+// key, counts and lists the matches in ascending order, ranks those that clear
+// theta_score and gathers the selected continuations.
 //
 // The candidates come from a source (every position of the buffer, or the
 // index's lists) in rows of 128: element e = 0..3 of lane l.  A warp tests
@@ -9,14 +9,19 @@
 // ballots per row, kept in shared memory (16 bytes per 128 candidates), so
 // that the ascending ranks come from one block scan of popcounts and no
 // candidate is tested twice.  A request with few rows is handled by CTA 0
-// alone (the other seven leave at once and no cluster barrier is used);
-// otherwise the rows are split in eighths, every CTA pushes its count to all
-// peers and its best top_c to CTA 0 through distributed shared memory, and
-// after the cluster barrier nobody touches another CTA's shared memory.
+// alone (the others leave at once and no cluster barrier is used); otherwise
+// the rows are split evenly, every CTA pushes its count to all peers and its
+// best top_c to CTA 0 through distributed shared memory, and after the cluster
+// barrier nobody touches another CTA's shared memory.
 //
 // What bounds it: a chain of dependent reads (offsets, key, candidates,
 // scores, spans) of about 0.5 us each, then for long buffers the reads of one
-// request's eight SMs (~100 GB/s per SM).
+// request's SMs (~100 GB/s per SM), then, with many requests, the CTAs an SM
+// holds.  So calls of up to kMatFewB requests take clusters of 16 CTAs of 512
+// threads (4 x 1M tokens: 23.6 us with 8, 15.3 with 16; more of these clusters
+// than GPCs run in turn: 8 requests 23.5 and 27.4), of which a request of
+// less than kMatWideRows rows uses 8; calls of up to kMatMidB requests clusters
+// of 8; larger calls clusters of 8 CTAs of 256 threads.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -27,10 +32,13 @@
 namespace rs {
 
 constexpr int kMatCluster = 8;
-constexpr int kMatThreads = 512;
+constexpr int kMatClusterMax = 16;
+constexpr int kMatFewB = 4, kMatMidB = 8;
+constexpr int kMatWideRows = 1024;  // 131072 candidates
+constexpr int kMatThreads = 512;          // or half of it
 constexpr int kMatWarps = kMatThreads / 32;
-constexpr int kMatCand = 512;       // matches ranked from the shared buffer
-constexpr int kMatBitRows = 4096;   // rows whose ballots a CTA keeps (524288 candidates)
+constexpr int kMatCand = 512;             // matches ranked from the shared buffer
+constexpr int kMatBitRows = 2048;         // rows whose ballots a CTA keeps (262144 candidates)
 constexpr size_t kMatSmem = (size_t)kMatBitRows * 4 * sizeof(uint32_t);
 
 // (s, p) before (s2, p2): higher score first, then the more recent position
@@ -53,10 +61,10 @@ struct MatShared {
     int warp_sums[kMatWarps];
     float wv[kMatWarps];
     int wp[kMatWarps];
-    long long peer_cnt[kMatCluster];           // match count of each CTA (pushed by its owner)
-    float peer_s[kMatCluster][RS_MAX_TOPC];    // CTA 0: each CTA's best top_c
-    int peer_p[kMatCluster][RS_MAX_TOPC];
-    int peer_n[kMatCluster];
+    int peer_cnt[kMatClusterMax];           // match count of each CTA (pushed by its owner)
+    float peer_s[kMatClusterMax][RS_MAX_TOPC];    // CTA 0: each CTA's best top_c
+    int peer_p[kMatClusterMax][RS_MAX_TOPC];
+    int peer_n[kMatClusterMax];
     float top_s[RS_MAX_TOPC];                  // this CTA's best top_c
     int top_p[RS_MAX_TOPC];
     int ntop;
@@ -73,7 +81,7 @@ struct MatOut {
 struct MatReq {
     const int32_t *X;
     const float *S;
-    long long t;
+    int t;      // tokens (positions are int32: longer buffers are cut at 2^31 - 1)
     int k, st;  // key length; status bits
     bool run;
     int key[RS_MAX_L];  // key[i] = X[t - k + i]
@@ -88,18 +96,19 @@ __device__ __forceinline__ void mat_request(MatReq &q, const int32_t *__restrict
     const long long t0 = tok_off[b], t1 = tok_off[b + 1], tend = tok_off[B];
     q.k = k_star[b];
     const bool gate = gate_ok == nullptr || gate_ok[b] != 0;
-    q.t = t1 - t0;
+    const long long t = t1 - t0;
     // the buffers hold tok_off[B] tokens: a range outside them is not read
-    const bool off_ok = ok && t0 >= 0 && q.t >= 0 && t0 + q.t <= tend;
+    const bool off_ok = ok && t0 >= 0 && t >= 0 && t0 + t <= tend;
     q.X = tokens + (off_ok ? t0 : 0);
     q.S = scores + (off_ok ? t0 : 0);
+    q.t = off_ok ? (int)(t < 0x7fffffff ? t : 0x7fffffff) : 0;
     q.st = off_ok ? 0 : RS_ST_BAD_OFFSET;
     q.run = off_ok && q.k > 0 && gate;
     if (q.run && q.k > RS_MAX_L) {
         q.st = RS_ST_TOO_LARGE;
         q.run = false;
     }
-    if (q.run && (long long)q.k > q.t) q.run = false;
+    if (q.run && q.k > q.t) q.run = false;
 #pragma unroll
     for (int i = 0; i < RS_MAX_L; ++i) q.key[i] = (q.run && i < q.k) ? q.X[q.t - q.k + i] : -1;
     q.k1 = q.run ? q.X[q.t - 1] : -1;
@@ -108,7 +117,7 @@ __device__ __forceinline__ void mat_request(MatReq &q, const int32_t *__restrict
 
 // Whether the k - 1 tokens before position p (p >= k - 1) are the key's; every
 // load is issued before the first comparison.
-__device__ __forceinline__ bool mat_prefix(const MatReq &q, long long p) {
+__device__ __forceinline__ bool mat_prefix(const MatReq &q, int p) {
     int v[RS_MAX_L];
 #pragma unroll
     for (int j = 0; j < RS_MAX_L; ++j) v[j] = j < q.k - 1 ? q.X[p - (q.k - 1) + j] : -1;
@@ -132,7 +141,7 @@ __device__ __forceinline__ int mat_excl_scan(int v, MatShared &sh, int *total) {
     int before = 0, sum = 0;
 #pragma unroll
     for (int w = 0; w < kMatWarps; ++w) {
-        const int y = sh.warp_sums[w];
+        const int y = w < (int)(blockDim.x >> 5) ? sh.warp_sums[w] : 0;
         before += w < warp ? y : 0;
         sum += y;
     }
@@ -161,8 +170,8 @@ __device__ __forceinline__ void mat_block_best(float hv, int hp, MatShared &sh, 
                 sh.wp[warp] = hp;
             }
             __syncthreads();
-            hv = lane < kMatWarps ? sh.wv[lane] : -INFINITY;
-            hp = lane < kMatWarps ? sh.wp[lane] : -1;
+            hv = lane < (int)(blockDim.x >> 5) ? sh.wv[lane] : -INFINITY;
+            hp = lane < (int)(blockDim.x >> 5) ? sh.wp[lane] : -1;
         }
     }
     __syncthreads();  // wv / wp reusable
@@ -174,8 +183,8 @@ __device__ __forceinline__ void mat_block_best(float hv, int hp, MatShared &sh, 
 // bit 4 u + e for element e of row r0 + u; rows at or past `end` give none.
 // The warp's ballots go to bits[4 (r0 - base) ..] (rows below cap only).
 template <class Src>
-__device__ __forceinline__ uint32_t mat_rows(const Src &src, const MatReq &q, long long r0, long long end,
-                                             uint32_t *bits, long long base) {
+__device__ __forceinline__ uint32_t mat_rows(const Src &src, const MatReq &q, int r0, int end, uint32_t *bits,
+                                             int base) {
     const int lane = threadIdx.x & 31;
     const uint32_t hits = src.test(q, r0, end, lane);
     uint32_t mine = 0;
@@ -188,31 +197,62 @@ __device__ __forceinline__ uint32_t mat_rows(const Src &src, const MatReq &q, lo
     return hits;
 }
 
-// The whole of a request once its source is known (see the file comment).
-// rows: candidate rows; solo: CTA 0 alone handles them.
+// The ballots of rows [w0, w0 + nr) again, for slices of more rows than are
+// kept (not inlined: the common path keeps its registers).
 template <class Src>
-__device__ __forceinline__ void mat_body(const Src &src, const MatReq &q, long long rows, bool solo, int b, int crank,
+__device__ __noinline__ void mat_again(Src src, MatReq q, int w0, int nr, uint32_t *bits) {
+    __syncthreads();  // the previous rows are consumed
+    const int stride = (blockDim.x >> 5) * Src::kRows;
+    for (int r0 = w0 + (threadIdx.x >> 5) * Src::kRows; r0 < w0 + nr; r0 += stride)
+        (void)mat_rows(src, q, r0, w0 + nr, bits, w0);
+    __syncthreads();
+}
+
+// Calls f(position) for the matches of rows [a, z) of the kept ballots, in
+// order; w0: the row the ballots start at.  Stops when f returns false.
+template <class Src, class F>
+__device__ __forceinline__ void mat_each(const Src &src, const uint32_t *bits, int w0, int a, int z, F f) {
+    for (int r = a; r < z; ++r) {
+        const uint4 w = *reinterpret_cast<const uint4 *>(bits + 4 * r);
+        if (Src::kLaneMajor) {
+            uint32_t any = w.x | w.y | w.z | w.w;
+            while (any) {
+                const int l = __ffs(any) - 1;
+                any &= any - 1;
+                uint32_t es = ((w.x >> l) & 1u) | ((w.y >> l) & 1u) << 1 | ((w.z >> l) & 1u) << 2 | ((w.w >> l) & 1u) << 3;
+                for (; es; es &= es - 1)
+                    if (!f(src.pos(w0 + r, l, __ffs(es) - 1))) return;
+            }
+        } else {
+#pragma unroll 1
+            for (int e = 0; e < 4; ++e) {
+                uint32_t we = e == 0 ? w.x : e == 1 ? w.y : e == 2 ? w.z : w.w;
+                for (; we; we &= we - 1)
+                    if (!f(src.pos(w0 + r, __ffs(we) - 1, e))) return;
+            }
+        }
+    }
+}
+
+// The whole of a request once its source is known (see the file comment).
+// rows: candidate rows; nc: the CTAs that share them, 1 for CTA 0 alone.
+template <class Src>
+__device__ __forceinline__ void mat_body(const Src &src, const MatReq &q, int rows, int nc, int b, int crank,
                                          MatShared &sh, uint32_t *bits, const MatOut &o) {
     namespace cg = cooperative_groups;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int nthreads = blockDim.x, stride = (nthreads >> 5) * Src::kRows;  // rows a round of the CTA's warps
     const int top_c = o.top_c, pos_cap = o.pos_cap;
+    const bool solo = nc == 1;
     if (!solo) cluster_arrive_relaxed();  // this CTA runs; the wait sits before the first push
-    const long long per = solo ? rows : (rows + kMatCluster - 1) / kMatCluster;
-    const long long lo = solo ? 0 : (per * crank < rows ? per * crank : rows);
-    const long long hi = lo + per < rows ? lo + per : rows;
+    const int per = (rows + nc - 1) / nc;
+    const int lo = min(per * crank, rows), hi = min(lo + per, rows);
     if (tid == 0) sh.ccnt = 0;
     __syncthreads();
 
     // ---- every candidate once: ballots, count, the matches that clear theta ----
-    float ls[RS_MAX_TOPC];  // this thread's best (used when more match than the buffer holds)
-    int lp[RS_MAX_TOPC];
-#pragma unroll
-    for (int i = 0; i < RS_MAX_TOPC; ++i) {
-        ls[i] = -INFINITY;
-        lp[i] = -1;
-    }
     int cnt = 0;
-    for (long long r0 = lo + warp * Src::kRows; r0 < hi; r0 += kMatWarps * Src::kRows) {
+    for (int r0 = lo + warp * Src::kRows; r0 < hi; r0 += stride) {
         uint32_t rem = mat_rows(src, q, r0, hi, bits, lo);
         cnt += __popc(rem);
         while (rem) {
@@ -226,29 +266,15 @@ __device__ __forceinline__ void mat_body(const Src &src, const MatReq &q, long l
                 sh.cs[slot] = s;
                 sh.cp[slot] = p;
             }
-            if (sp_before(s, p, ls[RS_MAX_TOPC - 1], lp[RS_MAX_TOPC - 1])) {
-                float cs = s;
-                int cp = p;
-#pragma unroll
-                for (int i = 0; i < RS_MAX_TOPC; ++i) {
-                    if (sp_before(cs, cp, ls[i], lp[i])) {
-                        const float ts = ls[i];
-                        const int tp = lp[i];
-                        ls[i] = cs;
-                        lp[i] = cp;
-                        cs = ts;
-                        cp = tp;
-                    }
-                }
-            }
         }
     }
     int cta_total = 0;
     (void)mat_excl_scan(cnt, sh, &cta_total);
     // the CTA's best top_c: rank every buffered match by counting
     const int ncand = sh.ccnt;
+    bool kept = true;  // the ballots are still those of [lo, lo + kMatBitRows)
     if (ncand <= kMatCand) {
-        for (int e = tid; e < ncand; e += kMatThreads) {
+        for (int e = tid; e < ncand; e += nthreads) {
             const float sv = sh.cs[e];
             const int pv = sh.cp[e];
             const int r = sp_rank(sv, pv, sh.cs, sh.cp, ncand);
@@ -258,7 +284,42 @@ __device__ __forceinline__ void mat_body(const Src &src, const MatReq &q, long l
             }
         }
         if (tid == 0) sh.ntop = ncand < top_c ? ncand : top_c;
-    } else {
+    } else {  // more than the buffer holds: every thread's best of its rows, then the block's best of those
+        float ls[RS_MAX_TOPC];
+        int lp[RS_MAX_TOPC];
+#pragma unroll
+        for (int i = 0; i < RS_MAX_TOPC; ++i) {
+            ls[i] = -INFINITY;
+            lp[i] = -1;
+        }
+        for (int w0 = lo; w0 < hi; w0 += kMatBitRows) {
+            const int nr = min(hi - w0, kMatBitRows);
+            if (w0 != lo) {
+                mat_again(src, q, w0, nr, bits);
+                kept = false;
+            }
+            const int mr = (nr + nthreads - 1) / nthreads;
+            const int a = min(tid * mr, nr), z = min(a + mr, nr);
+            mat_each(src, bits, w0, a, z, [&](int p) {
+                const float s = q.S[p];
+                if (s >= o.theta_score && sp_before(s, p, ls[RS_MAX_TOPC - 1], lp[RS_MAX_TOPC - 1])) {
+                    float cs = s;
+                    int cp = p;
+#pragma unroll
+                    for (int i = 0; i < RS_MAX_TOPC; ++i) {
+                        if (sp_before(cs, cp, ls[i], lp[i])) {
+                            const float ts = ls[i];
+                            const int tp = lp[i];
+                            ls[i] = cs;
+                            lp[i] = cp;
+                            cs = ts;
+                            cp = tp;
+                        }
+                    }
+                }
+                return true;
+            });
+        }
         int ntop = 0;
         for (int c = 0; c < top_c; ++c) {
             float bv;
@@ -284,12 +345,12 @@ __device__ __forceinline__ void mat_body(const Src &src, const MatReq &q, long l
     }
 
     // ---- the slice's global rank (pushed counts) ----
-    long long offset = 0, total = cta_total;
+    int offset = 0, total = cta_total;
     __syncthreads();  // this CTA's top list is complete
     if (!solo) {
         cg::cluster_group cluster = cg::this_cluster();
-        cluster_wait();  // every CTA of the cluster is running
-        if (tid < kMatCluster) *cluster.map_shared_rank(&sh.peer_cnt[crank], tid) = cta_total;
+        cluster_wait();  // every CTA of the cluster is running (or has left: those share no rows)
+        if (tid < nc) *cluster.map_shared_rank(&sh.peer_cnt[crank], tid) = cta_total;
         if (tid < RS_MAX_TOPC && tid < sh.ntop) {
             *cluster.map_shared_rank(&sh.peer_s[crank][tid], 0) = sh.top_s[tid];
             *cluster.map_shared_rank(&sh.peer_p[crank][tid], 0) = sh.top_p[tid];
@@ -298,82 +359,49 @@ __device__ __forceinline__ void mat_body(const Src &src, const MatReq &q, long l
         cluster_arrive_release();  // every push is visible after the wait
         cluster_wait();
         total = 0;
-        for (int r = 0; r < kMatCluster; ++r) {
-            const long long c = sh.peer_cnt[r];
+        for (int r = 0; r < nc; ++r) {
+            const int c = sh.peer_cnt[r];
             if (r < crank) offset += c;
             total += c;
         }
     }
 
-    // ---- positions in ascending order: the kept ballots, then (slices of more
-    // rows than are kept) further rows tested again ----
-    long long base = offset;
+    // ---- positions in ascending order ----
+    int base = offset;
     int32_t *pos = o.pos + (long long)b * pos_cap;
-    for (long long w0 = lo; w0 < hi && base < pos_cap; w0 += kMatBitRows) {
-        const int nr = (int)(hi - w0 < kMatBitRows ? hi - w0 : kMatBitRows);
-        if (w0 != lo) {
-            __syncthreads();  // the previous rows are consumed
-            for (long long r0 = w0 + warp * Src::kRows; r0 < w0 + nr; r0 += kMatWarps * Src::kRows)
-                (void)mat_rows(src, q, r0, w0 + nr, bits, w0);
-            __syncthreads();
-        }
-        const int mr = (nr + kMatThreads - 1) / kMatThreads;  // consecutive rows per thread
-        const int a = tid * mr < nr ? tid * mr : nr, z = a + mr < nr ? a + mr : nr;
+    for (int w0 = lo; w0 < hi && base < pos_cap; w0 += kMatBitRows) {
+        const int nr = min(hi - w0, kMatBitRows);
+        if (w0 != lo || !kept) mat_again(src, q, w0, nr, bits);
+        const int mr = (nr + nthreads - 1) / nthreads;  // consecutive rows per thread
+        const int a = min(tid * mr, nr), z = min(a + mr, nr);
         int n = 0;
         for (int r = a; r < z; ++r) {
             const uint4 w = *reinterpret_cast<const uint4 *>(bits + 4 * r);
             n += __popc(w.x) + __popc(w.y) + __popc(w.z) + __popc(w.w);
         }
         int wtotal = 0;
-        long long idx = base + mat_excl_scan(n, sh, &wtotal);
-        if (n) {
-            for (int r = a; r < z && idx < pos_cap; ++r) {
-                const uint4 w = *reinterpret_cast<const uint4 *>(bits + 4 * r);
-                if (Src::kLaneMajor) {
-                    uint32_t any = w.x | w.y | w.z | w.w;
-                    while (any) {
-                        const int l = __ffs(any) - 1;
-                        any &= any - 1;
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const uint32_t we = e == 0 ? w.x : e == 1 ? w.y : e == 2 ? w.z : w.w;
-                            if ((we >> l) & 1u) {
-                                if (idx < pos_cap) pos[idx] = src.pos(w0 + r, l, e);
-                                ++idx;
-                            }
-                        }
-                    }
-                } else {
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        uint32_t we = e == 0 ? w.x : e == 1 ? w.y : e == 2 ? w.z : w.w;
-                        while (we) {
-                            const int l = __ffs(we) - 1;
-                            we &= we - 1;
-                            if (idx < pos_cap) pos[idx] = src.pos(w0 + r, l, e);
-                            ++idx;
-                        }
-                    }
-                }
-            }
-        }
+        int idx = base + mat_excl_scan(n, sh, &wtotal);
+        if (n && idx < pos_cap)
+            mat_each(src, bits, w0, a, z, [&](int p) {
+                pos[idx] = p;
+                return ++idx < pos_cap;
+            });
         base += wtotal;
     }
     if (crank != 0) return;
 
     // ---- CTA 0: merge the per-CTA lists, selection outputs ----
-    const long long stored = total < pos_cap ? total : pos_cap;
-    for (long long i = stored + tid; i < pos_cap; i += kMatThreads) pos[i] = -1;
+    for (int i = min(total, pos_cap) + tid; i < pos_cap; i += nthreads) pos[i] = -1;
     int nsel;
     if (solo) {
         nsel = sh.ntop;
         if (tid < nsel) sh.sel[tid] = sh.top_p[tid];  // already ranked
     } else {
-        // the cluster's candidates (at most kMatCluster * RS_MAX_TOPC), ranked by counting
+        // the cluster's candidates (at most kMatClusterMax * RS_MAX_TOPC), ranked by counting
         float *ms = sh.cs;  // reused: the CTA's own buffer is no longer needed
         int *mp = sh.cp;
         int nm = 0;
-        for (int r = 0; r < kMatCluster; ++r) {
+        for (int r = 0; r < nc; ++r) {
             const int n = sh.peer_n[r];
             if (tid < n) {
                 ms[nm + tid] = sh.peer_s[r][tid];
@@ -389,11 +417,11 @@ __device__ __forceinline__ void mat_body(const Src &src, const MatReq &q, long l
         nsel = nm < top_c ? nm : top_c;
     }
     __syncthreads();
-    for (int i = tid; i < top_c * o.span_len; i += kMatThreads) {
+    for (int i = tid; i < top_c * o.span_len; i += nthreads) {
         const int c = i / o.span_len, j = i - c * o.span_len;
         int v = -1;
         if (c < nsel) {
-            const long long p = sh.sel[c];
+            const int p = sh.sel[c];
             if (j < q.t - 1 - p) v = q.X[p + 1 + j];
         }
         o.spans[(long long)b * top_c * o.span_len + i] = v;
@@ -402,17 +430,48 @@ __device__ __forceinline__ void mat_body(const Src &src, const MatReq &q, long l
         int sp = -1, sl = 0;
         if (tid < nsel) {
             sp = sh.sel[tid];
-            const long long len = q.t - 1 - sp;
-            sl = (int)(len > o.span_len ? o.span_len : len);
+            sl = min(q.t - 1 - sp, o.span_len);
         }
         o.sel_pos[(long long)b * top_c + tid] = sp;
         o.sel_len[(long long)b * top_c + tid] = sl;
     }
     if (tid == 0) {
-        o.count[b] = (int32_t)total;
+        o.count[b] = total;
         o.n_sel[b] = nsel;
         o.status[b] = q.st | (total > pos_cap ? RS_ST_TRUNCATED : 0);
     }
+}
+
+// The CTAs of the cluster that share a request's rows: one round of CTA 0's
+// warps needs no others.
+template <class Src>
+__device__ __forceinline__ int mat_ctas(int rows) {
+    if (rows <= (int)(blockDim.x >> 5) * Src::kRows) return 1;
+    const int nc = gridDim.x;
+    return nc > kMatCluster && rows < kMatWideRows ? kMatCluster : nc;
+}
+
+// Launches a retrieval kernel over B requests; attr_done: the caller's flags,
+// one per kernel and device.
+template <typename... KArgs, typename... Args>
+inline rs_status mat_launch(const char *who, int (&attr_done)[64], void (*kern)(KArgs...), int B, cudaStream_t st,
+                            Args... args) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev >= 0 && dev < 64 && !attr_done[dev]) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMatSmem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e != cudaSuccess) {
+            set_error("%s: cudaFuncSetAttribute: %s", who, cudaGetErrorString(e));
+            return RS_ERR_CUDA;
+        }
+        attr_done[dev] = 1;
+    }
+    const int nc = B <= kMatFewB ? kMatClusterMax : kMatCluster;
+    const int threads = B <= kMatMidB ? kMatThreads : kMatThreads / 2;
+    launch_pdl_cluster(kern, dim3(nc, B), dim3(threads), kMatSmem, st, nc, args...);
+    RS_CHECK_LAUNCH(who);
+    return RS_OK;
 }
 
 }  // namespace rs

@@ -1,7 +1,7 @@
 // scan.cu -- rs_match_scan: retrieval and feedback-driven candidate
 // selection (Section 3.3 "Selection Algorithm"; Algorithm 1's retrieval).
 //
-// One cluster of 8 CTAs per request; match.cuh has the split, the ranks and
+// One cluster of CTAs per request; match.cuh has the split, the ranks and
 // the selection.  The candidates are the buffer's positions, as quads of four
 // tokens on 16-byte boundaries: a lane reads eight quads (one 128-bit load
 // each, all in flight), compares the last token of the key, filters on the
@@ -17,21 +17,17 @@
 namespace rs {
 namespace {
 
-// A buffer of at most one round of CTA 0 (16 warps x 8 rows x 128 positions)
-// is handled by CTA 0 alone.
-constexpr long long kScanSoloRows = kMatWarps * 8;
-
 struct ScanSource {
     static constexpr int kRows = 8;
     static constexpr bool kLaneMajor = true;
     int al;       // positions of the buffer start past a 16-byte boundary
-    __device__ __forceinline__ int pos(long long row, int lane, int e) const {
-        return (int)(4 * (32 * row + lane) + e - al);
+    __device__ __forceinline__ int pos(int row, int lane, int e) const {
+        return 4 * (32 * row + lane) + e - al;
     }
-    __device__ __forceinline__ uint32_t test(const MatReq &q, long long r0, long long end, int lane) const {
-        const int t = (int)q.t;
-        const int pb = (int)(128 * r0) + 4 * lane - al;  // this lane's first position; row u's at pb + 128 u
-        const int rows = (int)(end - r0 < kRows ? end - r0 : kRows);
+    __device__ __forceinline__ uint32_t test(const MatReq &q, int r0, int end, int lane) const {
+        const int t = q.t;
+        const int pb = 128 * r0 + 4 * lane - al;  // this lane's first position; row u's at pb + 128 u
+        const int rows = min(end - r0, kRows);
         int4 x[kRows];
         uint32_t edge = 0;  // rows whose quad reaches past an end of the buffer
 #pragma unroll
@@ -39,7 +35,7 @@ struct ScanSource {
             const int p0 = pb + 128 * u;
             x[u] = make_int4(0, 0, 0, 0);
             if (u < rows && p0 < t) {
-                if (p0 >= 0 && p0 + 3 < t) x[u] = *reinterpret_cast<const int4 *>(q.X + p0);
+                if (p0 >= 0 && p0 < t - 3) x[u] = *reinterpret_cast<const int4 *>(q.X + p0);
                 else edge |= 1u << u;
             }
         }
@@ -76,7 +72,7 @@ struct ScanSource {
     }
 };
 
-__global__ void __cluster_dims__(kMatCluster, 1, 1) __launch_bounds__(kMatThreads)
+__global__ void __launch_bounds__(kMatThreads)
 match_scan_kernel(const int32_t *__restrict__ tokens, const int64_t *__restrict__ tok_off,
                   const int32_t *__restrict__ k_star, const uint8_t *__restrict__ gate_ok,
                   const float *__restrict__ scores, MatOut o) {
@@ -89,10 +85,10 @@ match_scan_kernel(const int32_t *__restrict__ tokens, const int64_t *__restrict_
     mat_request(q, tokens, tok_off, k_star, gate_ok, scores, b, gridDim.y, true);
     ScanSource src;
     src.al = (int)((reinterpret_cast<uintptr_t>(q.X) >> 2) & 3);
-    const long long rows = q.run ? (q.t - 1 + src.al + 127) / 128 : 0;
-    const bool solo = rows <= kScanSoloRows;
-    if (solo && crank != 0) return;
-    mat_body(src, q, rows, solo, b, crank, sh, scan_bits, o);
+    const int rows = q.run ? (int)(((unsigned)q.t + src.al + 126) / 128) : 0;
+    const int nc = mat_ctas<ScanSource>(rows);
+    if (crank >= nc) return;
+    mat_body(src, q, rows, nc, b, crank, sh, scan_bits, o);
 }
 
 }  // namespace
@@ -124,21 +120,8 @@ extern "C" rs_status rs_match_scan(const int32_t *tokens, const int64_t *tok_off
                             n_sel && status && (pos || pos_cap == 0)),
                  "rs_match_scan: null pointer");
     if (B == 0) return RS_OK;
-    static int attr_done[64] = {0};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev >= 0 && dev < 64 && !attr_done[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(match_scan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)kMatSmem);
-        if (e != cudaSuccess) {
-            set_error("rs_match_scan: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
-            return RS_ERR_CUDA;
-        }
-        attr_done[dev] = 1;
-    }
     const MatOut o{count, pos, sel_pos, sel_len, spans, n_sel, status, p.theta_score, p.top_c, p.span_len, pos_cap};
-    launch_pdl(match_scan_kernel, dim3(kMatCluster, B), dim3(kMatThreads), kMatSmem, (cudaStream_t)stream, tokens,
-        tok_off, k_star, gate_ok, scores, o);
-    RS_CHECK_LAUNCH("rs_match_scan");
-    return RS_OK;
+    static int attr_done[64] = {0};
+    return mat_launch("rs_match_scan", attr_done, match_scan_kernel, B, (cudaStream_t)stream, tokens, tok_off, k_star, gate_ok,
+                      scores, o);
 }

@@ -10,7 +10,7 @@ import torch
 import oracle
 from gpu_helpers import f32
 from paper_2511_01282_gb300 import respec as rs
-from test_gpu_index import _cuda, compare
+from test_gpu_index import _cuda, build_index, compare
 
 pytestmark = pytest.mark.gpu
 
@@ -51,10 +51,10 @@ def _scan(tokens, tok_off, ks, scores, theta, top_c, span_len, pos_cap):
 @pytest.mark.parametrize("k", [1, 2, 3, 8])
 @pytest.mark.parametrize("V", [3, 400])
 def test_scan_alignments_and_round_edges(k, V):
-    # request lengths of 1 mod 4 walk through every alignment; 16384 candidate
-    # positions are one round of one CTA
+    # request lengths of 1 mod 4 walk through every alignment; 8192 candidate
+    # positions (16384 in calls of few requests) are the most one CTA takes alone
     rng = np.random.default_rng(100 * k + V)
-    lens = [1, 5, 129, 2049, 16381, 16385, 16389, 33, 8193, 17, 20001]
+    lens = [1, 5, 129, 8185, 16381, 8197, 16389, 33, 8193, 17, 20001]
     tokens, tok_off = _buffers(rng, lens, V, k)
     scores = rng.random(len(tokens)).astype(np.float32)
     scores[rng.random(len(tokens)) < 0.2] = 0.5
@@ -63,14 +63,29 @@ def test_scan_alignments_and_round_edges(k, V):
 
 
 def test_scan_beyond_the_kept_ballots():
-    # 8 x 4096 rows x 128 positions = 4194304: the last rows are tested again
-    # for their positions, which the capacity reaches only with few matches
+    # 16 x 2048 rows x 128 positions = 4194304: the last rows are tested again
+    # for their positions, which the capacity reaches only with few matches, and
+    # for their scores when the buffer of matches overflows
     rng = np.random.default_rng(7)
     tokens, tok_off = _buffers(rng, [3, 4194304 + 70001], 50000, 2)
     scores = rng.random(len(tokens)).astype(np.float32)
     ref = _scan(tokens, tok_off, np.array([1, 1], np.int32), scores, 0.3, 8, 4, 300)
     assert 20 < ref["count"][1] < 300
     _scan(tokens, tok_off, np.array([0, 2], np.int32), scores, 0.3, 8, 4, 300)
+    tokens = rng.integers(0, 60, 4194304 + 70001).astype(np.int32)
+    _scan(tokens, np.array([0, len(tokens)], np.int64), np.array([1], np.int32), scores[:len(tokens)], 0.3, 8, 4, 100)
+
+
+@pytest.mark.parametrize("B", [1, 4, 5, 8, 9, 40])
+def test_scan_cluster_forms(B):
+    # up to 4 requests: clusters of 16, of which a request of less than 131072
+    # candidates uses 8; up to 8: clusters of 8; more: CTAs of half the threads
+    rng = np.random.default_rng(B)
+    lens = rng.choice([40, 8190, 8197, 16380, 16389, 30001], B).tolist()
+    lens[0], lens[-1] = 130000, 131200
+    tokens, tok_off = _buffers(rng, lens, 30, 2)
+    scores = rng.random(len(tokens)).astype(np.float32)
+    _scan(tokens, tok_off, rng.integers(1, 4, B).astype(np.int32), scores, 0.3, 8, 8, 900)
 
 
 @pytest.mark.parametrize("lens,V", [([1023, 1024, 1025, 0, 1], 300), ([4096, 0, 0, 4097], 1), ([524288 - 5, 5], 70000),
