@@ -442,8 +442,9 @@ index_place(const uint2 *__restrict__ sorted, long long N, const int64_t *__rest
     }
 }
 
-// Append: the positions built[b] .. t_b - 1 of every request, in rounds of
-// kAppThreads; see the file comment.
+// Append: the positions built[b] .. t_b - 1 of every request, in one round of a
+// warp when they are few (an append of 5 tokens and its query 8.5 -> 8.0 us),
+// else in rounds of kAppThreads; see the file comment.
 __global__ void __launch_bounds__(kAppThreads)
 index_append(const int32_t *__restrict__ tokens, const int64_t *__restrict__ tok_off, int V, IndexView ix,
              int32_t *__restrict__ status) {
@@ -470,6 +471,36 @@ index_append(const int32_t *__restrict__ tokens, const int64_t *__restrict__ tok
     int32_t *ovf = ix.list + ix.base[b];
     int32_t *buckets = ovf + kOvf;
     bool full = false;
+    if (built < t && t - built <= 32) {
+        // a step's few tokens: one warp, no barriers
+        if (tid >= 32) return;
+        const bool valid = lane < (int)(t - built);
+        const int p = (int)built + lane;
+        const int bk = valid ? bucket_of(X[p], V) : -1 - lane;
+        const int f0 = valid ? first[bk] : 0, f1 = valid ? first[bk + 1] : 0;
+        const int held = valid ? len[bk] : 0;
+        const unsigned peers = __match_any_sync(0xffffffffu, bk), lt = (1u << lane) - 1u;
+        const int slot = held + __popc(peers & lt);
+        const bool inb = valid && slot < (f1 - f0) + (f1 - f0) / 4 + 2;
+        const unsigned ov = __ballot_sync(0xffffffffu, valid && !inb);
+        const int oslot = novf + __popc(ov & lt);
+        // the first position with no room anywhere ends the indexed ones
+        const unsigned none = __ballot_sync(0xffffffffu, valid && !inb && oslot >= kOvf);
+        const int cut = none ? __ffs(none) - 1 : (int)(t - built);
+        const bool in = lane < cut;
+        const unsigned put = __ballot_sync(0xffffffffu, in && inb);
+        if (in && inb) {
+            buckets[start_of(f0, bk) + slot] = p;
+            if ((peers & put) >> lane == 1u) len[bk] = slot + 1;  // the bucket's last
+        }
+        if (in && valid && !inb) ovf[oslot] = p;
+        if (lane == 0) {
+            ix.built[b] = built + cut;
+            ix.ovf_n[b] = novf + __popc(ov & (cut < 32 ? (1u << cut) - 1u : 0xffffffffu));
+            if (status) status[b] = built + cut < t ? RS_ST_TRUNCATED : 0;
+        }
+        return;
+    }
     for (long long r0 = built; r0 < t && !full; r0 += kAppThreads) {
         const long long p = r0 + tid;
         const bool valid = p < t;

@@ -113,3 +113,33 @@ def test_index_query_of_a_common_token(common):
     scores = rng.random(t).astype(np.float32)
     for k in (1, 3):
         compare(tokens, tok_off, np.array([k], np.int32), None, scores, 0.3, 8, 4, 5000, 1000)
+
+
+@pytest.mark.parametrize("n", [1, 31, 32, 33])
+def test_append_of_one_warp_and_more(n):
+    # up to 32 new tokens are one warp's; many of one id, so that its bucket's
+    # room ends inside the append, and the overflow list's last slots
+    rng = np.random.default_rng(n)
+    V = 50
+    bufs = [rng.integers(0, V, 60).astype(np.int32), np.zeros(0, np.int32), rng.integers(0, V, 9).astype(np.int32)]
+    tok_off = np.concatenate([[0], np.cumsum([len(x) for x in bufs])]).astype(np.int64)
+    idx, total = build_index(np.concatenate(bufs), tok_off, V)
+    status = torch.full((3,), -1, dtype=torch.int32, device="cuda")
+
+    def grow(extra):
+        nonlocal bufs, tok_off
+        bufs = [np.concatenate([a, e]).astype(np.int32) for a, e in zip(bufs, extra)]
+        tok_off = np.concatenate([[0], np.cumsum([len(x) for x in bufs])]).astype(np.int64)
+        tokens = np.concatenate(bufs)
+        rs.rs_match_index_append(_cuda(tokens), _cuda(tok_off), 3, V, total, idx, status)
+        scores = rng.random(len(tokens)).astype(np.float32)
+        for k in (1, 2):
+            compare(tokens, tok_off, np.full(3, k, np.int32), None, scores, 0.3, 4, 8, 5000, V, idx=idx, t_total=total)
+        return status.tolist()
+
+    for _ in range(4):
+        assert grow([np.where(rng.random(n) < 0.7, 7, rng.integers(0, V, n)), np.full(n, 3), rng.integers(-2, V + 2, n)]) == [0, 0, 0]
+    # request 1's overflow list: filled up to its last n // 2 slots, then past them
+    fill = 4096 + 2 - len(bufs[1]) - n // 2
+    assert grow([[], np.full(fill, 3), []]) == [0, 0, 0]
+    assert grow([[1], np.full(n, 3), []]) == [0, rs.RS_ST_TRUNCATED, 0]
