@@ -34,18 +34,18 @@
 //
 // Build: the (request, bucket) keys of all tokens are sorted, with their
 // positions, by a stable LSD radix sort over all requests at once (digits of
-// at most 9 bits, so 18-bit keys -- 128K ids, one request -- take two
-// passes).  A pass is three kernels: the digit counts of every tile of keys,
-// their offsets, and the stable scatter, which ranks a tile's keys by warp
-// match and per-warp counters, orders the tile in shared memory and writes
-// whole runs of equal digits.  first[] is then a binary search per bucket in
-// the sorted keys (no atomics: counting buckets with them made a text's most
-// common tokens the bottleneck, 270 of 700 us for 4 x 1M tokens), and the
-// last kernel moves each sorted position to its bucket's slots.  A pass over
-// 4M tokens reads 32 MB and writes 32 MB in L2 and takes ~46 us cold (counts
-// 10, offsets 7.5, scatter 27-31, bound by the ballots and the 64-byte runs).
-// Build, four appends and four queries on 4 x 1M tokens: 1018 -> 150 us in a
-// graph; build, eight appends and eight queries on 4 x 32K: 242 -> 97 us.
+// at most 9 bits).  A pass is three kernels: the digit counts of every tile of
+// keys, their offsets, and the stable scatter, which ranks a tile's keys by
+// ballots and per-warp counters, orders the tile in shared memory and writes
+// whole runs of equal digits.  No atomics: counting buckets with them made a
+// text's most common tokens the bottleneck (270 of 700 us for 4 x 1M tokens).
+// Keys of 10 to 18 bits (32K ids and 8 requests, 128K ids and two) take two
+// passes, and the tiles of the second are cut where the first digit changes:
+// the offsets at the first tile of a digit's keys are then where each bucket
+// begins, so the second scatter writes the positions straight into the buckets
+// and the bucket starts need no search.  Other key lengths (and short buffers,
+// whose few tiles this cut would multiply) sort in plain passes, find first[]
+// by a binary search per bucket and move the sorted positions in one more pass.
 // Append: one CTA per request takes the new positions in rounds of 256; each
 // position's rank among the round's positions of its bucket gives its slot
 // after the bucket's entries; full buckets spill to the overflow list in
@@ -80,6 +80,26 @@ inline long long n_tiles(long long t_total) {
     return (t_total + tile - 1) / tile;
 }
 
+// bits of a sort key (request, bucket): buckets 0 .. V, requests 0 .. B - 1
+inline int bits_for(long long n) {  // smallest b with n < 2^b
+    int b = 0;
+    while (b < 63 && (1ll << b) <= n) ++b;
+    return b;
+}
+inline int key_bits(int B, int V) { return bits_for(V) + bits_for(B > 0 ? B - 1 : 0); }
+// Whether the second pass's tiles are cut at the first digit (see above): 4 x 1M
+// tokens build in 86.6 us so, 96.8 in plain passes; 4 x 32K in 26.9 and 28.5, but
+// with the appends and queries behind it in 88.3 and 87.7.
+constexpr long long kCutMin = 1 << 18;
+inline bool cut_build(int B, int V, long long t_total) {
+    const int bits = key_bits(B, V);
+    return t_total >= kCutMin && bits > kMaxDigitBits && bits <= 2 * kMaxDigitBits;
+}
+// tiles of a pass, at most: with cuts, one more per digit and one past the end
+inline long long hist_tiles(int B, int V, long long t_total) {
+    return n_tiles(t_total) + (cut_build(B, V, t_total) ? kMaxBins + 1 : 0);
+}
+
 struct IndexView {
     int32_t *valid;         // 1 when the build's offsets were consistent (else the index holds nothing)
     int64_t *built, *base;  // per request: positions indexed, first list slot
@@ -89,8 +109,8 @@ struct IndexView {
     int32_t *list;
     // build scratch
     uint2 *pair[2];         // (key, position) of every token
-    int32_t *hist;          // [ntiles][bins]
-    int32_t *dtot;          // [kMaxBins]
+    int32_t *hist;          // [tiles][bins]
+    int32_t *dtot;          // [2][kMaxBins]
 };
 
 inline long long list_slots(int B, int V, long long t_total) {
@@ -109,22 +129,18 @@ inline size_t carve_index(void *base, int B, int V, long long t_total, IndexView
     v->list = cv.take<int32_t>((size_t)list_slots(B, V, t_total));
     v->pair[0] = cv.take<uint2>((size_t)t_total);
     v->pair[1] = cv.take<uint2>((size_t)t_total);
-    v->hist = cv.take<int32_t>((size_t)kMaxBins * n_tiles(t_total));
-    v->dtot = cv.take<int32_t>((size_t)kMaxBins);
+    v->hist = cv.take<int32_t>((size_t)kMaxBins * hist_tiles(B, V, t_total));
+    v->dtot = cv.take<int32_t>((size_t)2 * kMaxBins);
     return cv.used();
 }
 inline size_t index_bytes(int B, int V, long long t_total) {
     IndexView v;
     return carve_index(nullptr, B, V, t_total, &v);
 }
-// bits of a sort key (request, bucket): buckets 0 .. V, requests 0 .. B - 1
-inline int bits_for(long long n) {  // smallest b with n < 2^b
-    int b = 0;
-    while (b < 63 && (1ll << b) <= n) ++b;
-    return b;
-}
-
 __device__ __forceinline__ int bucket_of(int tok, int V) { return (tok >= 0 && tok < V) ? tok : V; }
+__device__ __forceinline__ long long base_of(long long t0, int b, int V) {
+    return t0 + t0 / 4 + (long long)b * (2ll * (V + 1) + kOvf);
+}
 __device__ __forceinline__ long long start_of(int first, int v) { return (long long)first + first / 4 + 2ll * v; }
 
 // (0) the build's offsets: tok_off[0] = 0, ascending, tok_off[B] = t_total;
@@ -227,8 +243,8 @@ __device__ __forceinline__ int radix_excl_scan(int v, int *s_w, int *total) {
 
 // (tile, digit) offsets: each digit's exclusive prefix over the tiles, and
 // its total.  A block takes eight digits (one 32-byte sector of a tile's
-// counts); thread (group g, digit d) takes eight consecutive tiles a round.
-constexpr int kOffDigits = 8, kOffTiles = 8;
+// counts); thread (group g, digit d) takes sixteen consecutive tiles a round.
+constexpr int kOffDigits = 8, kOffTiles = 16;
 __global__ void __launch_bounds__(kRadixThreads)
 radix_offsets(int32_t *__restrict__ hist, long long ntiles, int bins, int32_t *__restrict__ dtot,
               const int32_t *__restrict__ valid) {
@@ -266,55 +282,35 @@ radix_offsets(int32_t *__restrict__ hist, long long ntiles, int bins, int32_t *_
     if (live && g == 0) dtot[blockIdx.x * kOffDigits + d] = carry;
 }
 
-// The stable scatter.  Warp w takes keys w 32 kR .. of the tile, 32 at a time;
-// a key's rank is the count of equal digits before it in the tile (earlier
-// warps, earlier rounds of its warp, lower lanes of its round).  The tile is
-// put in digit order in shared memory and leaves from there, so that equal
-// digits -- consecutive addresses -- are written by neighbouring threads.
-template <class Keys, int kR>
-__global__ void __launch_bounds__(kRadixThreads, 3)
-radix_scatter(Keys src, uint2 *__restrict__ out, long long N, int shift, int bins,
-              const int32_t *__restrict__ hist, const int32_t *__restrict__ dtot, const int32_t *__restrict__ valid) {
-    pdl_enter();
-    if (!*valid) return;
-    constexpr int kTile = kR * kRadixThreads;
-    __shared__ uint2 s_pair[kTile];
-    __shared__ uint16_t s_cnt[kRadixWarps][kMaxBins];
-    __shared__ int s_dst[kMaxBins];  // global index of the digit's first key, less its place in the tile
-    __shared__ int s_w[kRadixWarps];
+// A tile of keys put in digit order in shared memory, stably.  Warp w takes the
+// keys w 32 rounds .. of the tile, 32 at a time; a key's rank is the count of
+// equal digits before it in the tile (earlier warps, earlier rounds of its
+// warp, lower lanes of its round).
+template <int kR>
+struct TileShared {
+    uint2 pair[kR * kRadixThreads];
+    uint16_t cnt[kRadixWarps][kMaxBins];
+    int w[kRadixWarps];
+};
+__device__ __forceinline__ int tile_rounds_of(int n) { return (n + kRadixThreads - 1) / kRadixThreads; }
+__device__ __forceinline__ int tile_elem(int rounds, int q) {
+    return ((int)(threadIdx.x >> 5) * rounds + q) * 32 + (int)(threadIdx.x & 31);
+}
+// k[q]: this thread's keys (tile_elem(rounds, q) below n); starts(x, y): called
+// by every thread with the places of its digits 2 tid and 2 tid + 1 in the
+// ordered tile.  Ends with a barrier.
+template <int kR, class Starts>
+__device__ __forceinline__ void order_tile(TileShared<kR> &sh, const uint2 (&k)[kR], int n, int rounds, int shift, int bins,
+                                           Starts starts) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const long long tile = blockIdx.x, i0 = tile * kTile;
-    const int n = (int)(N - i0 < kTile ? N - i0 : kTile);
-    decltype(src.load(0)) x[kR];
-#pragma unroll
-    for (int q = 0; q < kR; ++q) {
-        const int e = warp * (32 * kR) + q * 32 + lane;
-        x[q] = src.load(i0 + (e < n ? e : 0));
-    }
-    src.tile(i0);
-    // this thread's digits 2 tid and 2 tid + 1 (bins is even): where the tile's
-    // keys of each begin, within the digit and over all digits
-    int2 g = make_int2(0, 0), tot = make_int2(0, 0);
-    if (2 * tid < bins) {
-        g = *reinterpret_cast<const int2 *>(hist + tile * bins + 2 * tid);
-        tot = *reinterpret_cast<const int2 *>(dtot + 2 * tid);
-    }
-    for (int x = tid; x < kRadixWarps * kMaxBins / 2; x += kRadixThreads) reinterpret_cast<uint32_t *>(&s_cnt[0][0])[x] = 0;
-    uint2 k[kR];
-#pragma unroll
-    for (int q = 0; q < kR; ++q) {
-        const int e = warp * (32 * kR) + q * 32 + lane;
-        k[q] = e < n ? src.pair(x[q], i0 + e) : make_uint2(0u, 0u);
-    }
-    int all;
-    const int below = radix_excl_scan(tot.x + tot.y, s_w, &all);  // ends with a barrier
-    g.x += below;
-    g.y += below + tot.x;
+    for (int x = tid; x < kRadixWarps * kMaxBins / 2; x += kRadixThreads) reinterpret_cast<uint32_t *>(&sh.cnt[0][0])[x] = 0;
+    __syncthreads();
     const unsigned lt = (1u << lane) - 1u;
     int rk[kR];
 #pragma unroll
     for (int q = 0; q < kR; ++q) {
-        const bool ok = warp * (32 * kR) + q * 32 + lane < n;
+        if (q >= rounds) break;
+        const bool ok = tile_elem(rounds, q) < n;
         const int dg = (int)((k[q].x >> shift) & (bins - 1));
         // the lanes of this round with the same digit, one ballot per bit
         // (match.any is slow where a round holds many distinct digits: first
@@ -327,9 +323,9 @@ radix_scatter(Keys src, uint2 *__restrict__ out, long long N, int shift, int bin
             const unsigned bal = __ballot_sync(0xffffffffu, one);
             peers &= one ? bal : ~bal;
         }
-        const int before = ok ? s_cnt[warp][dg] : 0;
+        const int before = ok ? sh.cnt[warp][dg] : 0;
         __syncwarp();
-        if (ok && (peers & lt) == 0) s_cnt[warp][dg] = (uint16_t)(before + __popc(peers));
+        if (ok && (peers & lt) == 0) sh.cnt[warp][dg] = (uint16_t)(before + __popc(peers));
         __syncwarp();
         rk[q] = before + __popc(peers & lt);
     }
@@ -338,20 +334,19 @@ radix_scatter(Keys src, uint2 *__restrict__ out, long long N, int shift, int bin
         int run[2] = {0, 0};
 #pragma unroll
         for (int w = 0; w < kRadixWarps; ++w) {
-            uint32_t *p = reinterpret_cast<uint32_t *>(&s_cnt[w][2 * tid]);
+            uint32_t *p = reinterpret_cast<uint32_t *>(&sh.cnt[w][2 * tid]);
             const uint32_t c = *p;
             *p = (uint32_t)run[0] | ((uint32_t)run[1] << 16);
             run[0] += (int)(c & 0xffffu);
             run[1] += (int)(c >> 16);
         }
         int total;
-        const int x = radix_excl_scan(run[0] + run[1], s_w, &total);
-        s_dst[2 * tid] = g.x - x;
-        s_dst[2 * tid + 1] = g.y - (x + run[0]);
+        const int x = radix_excl_scan(run[0] + run[1], sh.w, &total);
+        starts(x, x + run[0]);
         // the counters become places in the ordered tile
 #pragma unroll
         for (int w = 0; w < kRadixWarps; ++w) {
-            uint32_t *p = reinterpret_cast<uint32_t *>(&s_cnt[w][2 * tid]);
+            uint32_t *p = reinterpret_cast<uint32_t *>(&sh.cnt[w][2 * tid]);
             const uint32_t c = *p;
             *p = ((c & 0xffffu) + (uint32_t)x) | (((c >> 16) + (uint32_t)(x + run[0])) << 16);
         }
@@ -359,24 +354,213 @@ radix_scatter(Keys src, uint2 *__restrict__ out, long long N, int shift, int bin
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < kR; ++q) {
-        if (warp * (32 * kR) + q * 32 + lane < n) {
+        if (q < rounds && tile_elem(rounds, q) < n) {
             const int dg = (int)((k[q].x >> shift) & (bins - 1));
-            s_pair[s_cnt[warp][dg] + rk[q]] = k[q];
+            sh.pair[sh.cnt[warp][dg] + rk[q]] = k[q];
         }
     }
     __syncthreads();
+}
+
+// This thread's digits 2 tid and 2 tid + 1 of a row of bins counts (bins is even).
+__device__ __forceinline__ int2 two_digits(const int32_t *row, int bins) {
+    return 2 * (int)threadIdx.x < bins ? *reinterpret_cast<const int2 *>(row + 2 * threadIdx.x) : make_int2(0, 0);
+}
+
+// The stable scatter: equal digits -- consecutive addresses -- are written by
+// neighbouring threads.
+template <class Keys, int kR>
+__global__ void __launch_bounds__(kRadixThreads, 3)
+radix_scatter(Keys src, uint2 *__restrict__ out, long long N, int shift, int bins,
+              const int32_t *__restrict__ hist, const int32_t *__restrict__ dtot, const int32_t *__restrict__ valid) {
+    pdl_enter();
+    if (!*valid) return;
+    constexpr int kTile = kR * kRadixThreads;
+    __shared__ TileShared<kR> sh;
+    __shared__ int s_dst[kMaxBins];  // global index of the digit's first key, less its place in the tile
+    const long long tile = blockIdx.x, i0 = tile * kTile;
+    const int n = (int)(N - i0 < kTile ? N - i0 : kTile), rounds = tile_rounds_of(n);
+    decltype(src.load(0)) x[kR];
+#pragma unroll
+    for (int q = 0; q < kR; ++q) {
+        const int e = tile_elem(rounds, q);
+        x[q] = src.load(i0 + (q < rounds && e < n ? e : 0));
+    }
+    src.tile(i0);
+    // where the tile's keys of each digit begin, within the digit and over all digits
+    int2 g = two_digits(hist + tile * bins, bins);
+    const int2 tot = two_digits(dtot, bins);
+    uint2 k[kR];
+#pragma unroll
+    for (int q = 0; q < kR; ++q) {
+        const int e = tile_elem(rounds, q);
+        k[q] = q < rounds && e < n ? src.pair(x[q], i0 + e) : make_uint2(0u, 0u);
+    }
+    int all;
+    const int below = radix_excl_scan(tot.x + tot.y, sh.w, &all);
+    g.x += below;
+    g.y += below + tot.x;
+    order_tile(sh, k, n, rounds, shift, bins, [&](int x0, int x1) {
+        s_dst[2 * threadIdx.x] = g.x - x0;
+        s_dst[2 * threadIdx.x + 1] = g.y - x1;
+    });
+#pragma unroll
+    for (int q = 0; q < kR; ++q) {
+        const int e = q * kRadixThreads + threadIdx.x;
+        if (e < n) {
+            const uint2 v = sh.pair[e];
+            out[(long long)s_dst[(v.x >> shift) & (bins - 1)] + e] = v;
+        }
+    }
+}
+
+// ---- the second of two passes, with tiles cut at the first digit ----
+// Tile `tile`: its keys [i0, i0 + n) share the first digit `digit`, whose keys
+// begin with tile `first`; n = 0 past the last tile.  dtot: the first digit's
+// totals.
+struct CutTile {
+    int digit, first, n;
+    long long i0;
+};
+__device__ __forceinline__ CutTile cut_tile(const int32_t *dtot, int bins, int tile_keys, int tile, int *s_w, CutTile *s_out) {
+    const int2 c = two_digits(dtot, bins);
+    if (threadIdx.x == 0) s_out->n = 0;
+    const int a = (c.x + tile_keys - 1) / tile_keys, b = (c.y + tile_keys - 1) / tile_keys;
+    int all;
+    const int tx = radix_excl_scan(a + b, s_w, &all);
+    const int kx = radix_excl_scan(c.x + c.y, s_w, &all);
+    if (tile >= tx && tile < tx + a + b) {
+        const bool second = tile >= tx + a;
+        const int first = second ? tx + a : tx, at = (tile - first) * tile_keys, cnt = second ? c.y : c.x;
+        *s_out = CutTile{2 * (int)threadIdx.x + second, first, min(tile_keys, cnt - at), (long long)kx + (second ? c.x : 0) + at};
+    }
+    __syncthreads();
+    return *s_out;
+}
+
+template <int kR>
+__global__ void __launch_bounds__(kRadixThreads)
+cut_hist(const uint2 *__restrict__ in, int bins0, int shift, int bins, const int32_t *__restrict__ dtot,
+         int32_t *__restrict__ hist, const int32_t *__restrict__ valid) {
+    pdl_enter();
+    if (!*valid) return;
+    __shared__ int cnt[kMaxBins];
+    __shared__ int s_w[kRadixWarps];
+    __shared__ CutTile s_tile;
+    for (int d = threadIdx.x; d < bins; d += kRadixThreads) cnt[d] = 0;
+    const CutTile t = cut_tile(dtot, bins0, kR * kRadixThreads, blockIdx.x, s_w, &s_tile);
+    uint32_t x[kR];
+#pragma unroll
+    for (int q = 0; q < kR; ++q) {
+        const int e = q * kRadixThreads + threadIdx.x;
+        x[q] = e < t.n ? in[t.i0 + e].x : 0u;
+    }
+#pragma unroll
+    for (int q = 0; q < kR; ++q)
+        if (q * kRadixThreads + (int)threadIdx.x < t.n) atomicAdd(&cnt[x[q] >> shift], 1);
+    __syncthreads();
+    for (int d = threadIdx.x; d < bins; d += kRadixThreads) hist[(long long)blockIdx.x * bins + d] = cnt[d];  // 0 past the last tile
+}
+
+// Blocks [0, tiles): a tile's positions into their buckets.  With O[tile][h] the
+// keys of second digit h in earlier tiles and base(h) those of smaller second
+// digits, bucket (h, l) begins at sorted index base(h) + O[first tile of l][h].
+// Blocks past them: first[] and len[] of 1024 buckets, from the same sums.
+constexpr int kCutFirst = 1024;
+template <int kR>
+__global__ void __launch_bounds__(kRadixThreads, 3)
+cut_scatter(const uint2 *__restrict__ in, int tiles, int bins0, int lo_bits, int bins, const int32_t *__restrict__ dtot,
+            const int32_t *__restrict__ hist, const int64_t *__restrict__ tok_off, int B, int V, int vbits, IndexView ix) {
+    pdl_enter();
+    if (!*ix.valid) return;
+    constexpr int kTile = kR * kRadixThreads;
+    __shared__ TileShared<kR> sh;
+    __shared__ CutTile s_tile;
+    __shared__ long long s_list[kMaxBins];  // list slot of the digit's first key in the tile, less its place there
+    __shared__ int s_t0[kMaxBins];
+    const int tid = threadIdx.x;
+    const uint32_t vmask = (1u << vbits) - 1u;  // vbits <= 18 here
+    const int2 tot = two_digits(dtot + kMaxBins, bins);
+    int all;
+    const int below = radix_excl_scan(tot.x + tot.y, sh.w, &all);
+    const int base[2] = {below, below + tot.x};
+    if ((int)blockIdx.x >= tiles) {
+        int *s_base = s_t0, *s_first = reinterpret_cast<int *>(s_list);
+        const int2 c = two_digits(dtot, bins0);
+        const int a = (c.x + kTile - 1) / kTile, b = (c.y + kTile - 1) / kTile;
+        const int tx = radix_excl_scan(a + b, sh.w, &all);
+        s_base[2 * tid] = base[0];
+        s_base[2 * tid + 1] = base[1];
+        s_first[2 * tid] = tx;
+        s_first[2 * tid + 1] = tx + a;
+        __syncthreads();
+        const long long end = (long long)B * (V + 2);
+        for (int q = 0; q < kCutFirst / kRadixThreads; ++q) {
+            const long long i = (long long)((int)blockIdx.x - tiles) * kCutFirst + q * kRadixThreads + tid;
+            if (i >= end) break;
+            const int rb = (int)(i / (V + 2)), v = (int)(i - (long long)rb * (V + 2));
+            const long long t0 = tok_off[rb];
+            const int t = (int)(tok_off[rb + 1] - t0);
+            auto first_of = [&](int w) -> int {
+                if (w > V) return t;
+                const uint32_t key = ((uint32_t)rb << vbits) | (uint32_t)w;
+                const int lo = (int)(key & ((1u << lo_bits) - 1u)), hi = (int)(key >> lo_bits);
+                return (int)(s_base[hi] + hist[(long long)s_first[lo] * bins + hi] - t0);
+            };
+            const int f = first_of(v);
+            ix.first[i] = f;
+            if (v <= V) ix.len[(long long)rb * (V + 1) + v] = first_of(v + 1) - f;
+            if (v == 0) {
+                ix.built[rb] = t;
+                ix.base[rb] = base_of(t0, rb, V);
+                ix.ovf_n[rb] = 0;
+            }
+        }
+        return;
+    }
+    const CutTile t = cut_tile(dtot, bins0, kTile, blockIdx.x, sh.w, &s_tile);
+    if (t.n == 0) return;
+    const int rounds = tile_rounds_of(t.n);
+    uint2 k[kR];
+#pragma unroll
+    for (int q = 0; q < kR; ++q) {
+        const int e = tile_elem(rounds, q);
+        k[q] = q < rounds && e < t.n ? in[t.i0 + e] : make_uint2(0u, 0u);
+    }
+    const int2 own = two_digits(hist + (long long)blockIdx.x * bins, bins);
+    const int2 run = two_digits(hist + (long long)t.first * bins, bins);
+    long long list[2] = {0, 0};
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int d = 2 * tid + h;
+        const uint32_t key = ((uint32_t)d << lo_bits) | (uint32_t)t.digit;
+        const int b = (int)(key >> vbits), v = (int)(key & vmask);
+        if (d < bins && b < B && v <= V) {
+            const long long t0 = tok_off[b];
+            const int o = h ? own.y : own.x, r = h ? run.y : run.x;
+            const int f = (int)(base[h] + r - t0);
+            list[h] = base_of(t0, b, V) + kOvf + start_of(f, v) + (o - r);
+            s_t0[d] = (int)t0;
+        }
+    }
+    order_tile(sh, k, t.n, rounds, lo_bits, bins, [&](int x0, int x1) {
+        s_list[2 * tid] = list[0] - x0;
+        s_list[2 * tid + 1] = list[1] - x1;
+    });
 #pragma unroll
     for (int q = 0; q < kR; ++q) {
         const int e = q * kRadixThreads + tid;
-        if (e < n) {
-            const uint2 v = s_pair[e];
-            out[(long long)s_dst[(v.x >> shift) & (bins - 1)] + e] = v;
+        if (e < t.n) {
+            const uint2 v = sh.pair[e];
+            const int d = (int)(v.x >> lo_bits);
+            ix.list[s_list[d] + e] = (int32_t)(v.y - (uint32_t)s_t0[d]);
         }
     }
 }
 static_assert(kMaxBins == 2 * kRadixThreads, "two digits per thread");
 static_assert(kTileRounds * kRadixThreads <= 65535, "16-bit tile counters");
 
+// ---- after plain passes ----
 // first[b][v]: where the keys of (b, v) begin in the sorted order, by binary
 // search; the lengths are the differences.  Blocks of 256 threads cover 255
 // buckets (the last thread only serves its neighbour).
@@ -408,7 +592,7 @@ index_first(const uint2 *__restrict__ sorted, const int64_t *__restrict__ tok_of
     }
     if (blockIdx.x == 0 && tid == 0) {
         ix.built[b] = t1 - t0;
-        ix.base[b] = t0 + t0 / 4 + (long long)b * (2ll * (V + 1) + kOvf);
+        ix.base[b] = base_of(t0, b, V);
         ix.ovf_n[b] = 0;
     }
 }
@@ -573,6 +757,7 @@ index_append(const int32_t *__restrict__ tokens, const int64_t *__restrict__ tok
 // is candidate 128 r + 32 e + l.
 struct ListSource {
     static constexpr int kRows = 2;
+    static constexpr int kWideRows = 128;  // 16384 candidates, each a read of its own
     static constexpr bool kLaneMajor = false;
     const int32_t *blist, *olist;
     int nb, no, ncand, tail0;
@@ -656,7 +841,7 @@ static rs_status check_index(const char *who, int B, int V, int64_t t_total, con
     RS_CHECK_ARG(B >= 0 && B <= 65535, "%s: B=%d outside [0, 65535]", who, B);
     RS_CHECK_ARG(V >= 1 && V < (1 << 30), "%s: V=%d outside [1, 2^30)", who, V);
     RS_CHECK_ARG(t_total >= 0 && t_total < (1ll << 31), "%s: t_total outside [0, 2^31)", who);
-    if (bits_for(V) + bits_for(B > 0 ? B - 1 : 0) > 32) {
+    if (key_bits(B, V) > 32) {
         set_error("%s: B=%d requests with V=%d need more than 32 key bits", who, B, V);
         return RS_ERR_UNSUPPORTED;
     }
@@ -668,12 +853,12 @@ static rs_status check_index(const char *who, int B, int V, int64_t t_total, con
     return RS_OK;
 }
 
-// One pass of the sort: digit `pass` of the keys, from the tokens or from the
-// pairs the last pass left.
+// The sort of a build.  One pass over digit `pass` (of `bits` bits) of the keys,
+// from the tokens or from the pairs the last pass left.
 template <int kR>
-static rs_status radix_pass(const int32_t *tokens, const int64_t *tok_off, int B, int V, int vbits, int keybits,
-                            int passes, int pass, long long N, const IndexView &ix, cudaStream_t st) {
-    const int bits = (keybits + passes - 1) / passes, shift = pass * bits, bins = 1 << bits;
+static rs_status radix_pass(const int32_t *tokens, const int64_t *tok_off, int B, int V, int vbits, int bits, int pass,
+                            long long N, const IndexView &ix, cudaStream_t st) {
+    const int shift = pass * bits, bins = 1 << bits;
     const long long nt = n_tiles(N);
     const TokenKeys tk{tokens, tok_off, B, V, vbits, 0, 0};
     const PairKeys pk{ix.pair[(pass & 1) ^ 1]};
@@ -693,6 +878,49 @@ static rs_status radix_pass(const int32_t *tokens, const int64_t *tok_off, int B
     return RS_OK;
 }
 
+// Plain passes, then the bucket starts and the placement.
+template <int kR>
+static rs_status build_plain(const int32_t *tokens, const int64_t *tok_off, int B, int V, long long N, const IndexView &ix,
+                             cudaStream_t st) {
+    const int vbits = bits_for(V), keybits = key_bits(B, V);
+    const int passes = N > 0 ? (keybits + kMaxDigitBits - 1) / kMaxDigitBits : 0;
+    for (int pass = 0; pass < passes; ++pass) {
+        const rs_status s = radix_pass<kR>(tokens, tok_off, B, V, vbits, (keybits + passes - 1) / passes, pass, N, ix, st);
+        if (s != RS_OK) return s;
+    }
+    const uint2 *sorted = ix.pair[(passes - 1) & 1];
+    launch_pdl(index_first, dim3((unsigned)((V + 2ll + kFirstPer - 1) / kFirstPer), B), dim3(kFirstPer + 1), 0, st, sorted,
+        tok_off, V, vbits, ix);
+    RS_CHECK_LAUNCH("rs_match_index_build/first");
+    if (N == 0) return RS_OK;
+    launch_pdl(index_place, dim3((unsigned)((N + 256 * kPlacePer - 1) / (256 * kPlacePer))), dim3(256), 0, st, sorted, N,
+        tok_off, V, vbits, ix);
+    RS_CHECK_LAUNCH("rs_match_index_build/place");
+    return RS_OK;
+}
+
+// Two passes, the second over tiles cut at the first digit.
+template <int kR>
+static rs_status build_cut(const int32_t *tokens, const int64_t *tok_off, int B, int V, long long N, const IndexView &ix,
+                           cudaStream_t st) {
+    const int vbits = bits_for(V), keybits = key_bits(B, V);
+    const int lo_bits = (keybits + 1) / 2, bins0 = 1 << lo_bits, bins = 1 << (keybits - lo_bits);
+    const rs_status s = radix_pass<kR>(tokens, tok_off, B, V, vbits, lo_bits, 0, N, ix, st);
+    if (s != RS_OK) return s;
+    const int tiles = (int)n_tiles(N) + bins0 + 1;  // the last one is never used: O past every key
+    const dim3 block(kRadixThreads);
+    launch_pdl(cut_hist<kR>, dim3((unsigned)tiles), block, 0, st, ix.pair[0], bins0, lo_bits, bins, ix.dtot, ix.hist, ix.valid);
+    RS_CHECK_LAUNCH("rs_match_index_build/cut_hist");
+    launch_pdl(radix_offsets, dim3((unsigned)(bins + kOffDigits - 1) / kOffDigits), block, 0, st, ix.hist, (long long)tiles,
+        bins, ix.dtot + kMaxBins, ix.valid);
+    RS_CHECK_LAUNCH("rs_match_index_build/cut_offsets");
+    const unsigned firsts = (unsigned)(((long long)B * (V + 2) + kCutFirst - 1) / kCutFirst);
+    launch_pdl(cut_scatter<kR>, dim3((unsigned)tiles + firsts), block, 0, st, ix.pair[0], tiles, bins0, lo_bits, bins, ix.dtot,
+        ix.hist, tok_off, B, V, vbits, ix);
+    RS_CHECK_LAUNCH("rs_match_index_build/cut_scatter");
+    return RS_OK;
+}
+
 extern "C" rs_status rs_match_index_build(const int32_t *tokens, const int64_t *tok_off, int B, int V,
                                           int64_t t_total, void *index, size_t index_bytes_avail, void *stream) {
     clear_error();
@@ -703,26 +931,14 @@ extern "C" rs_status rs_match_index_build(const int32_t *tokens, const int64_t *
     cudaStream_t st = (cudaStream_t)stream;
     IndexView ix;
     carve_index(index, B, V, t_total, &ix);
-    const int vbits = bits_for(V);
-    const int keybits = vbits + bits_for(B - 1);
     launch_pdl(index_check, dim3(1), dim3(1024), 0, st, tok_off, B, (long long)t_total, ix);
     RS_CHECK_LAUNCH("rs_match_index_build/check");
-    const int passes = t_total > 0 ? (keybits + kMaxDigitBits - 1) / kMaxDigitBits : 0;
     const bool small = tile_rounds(t_total) == kTileRoundsSmall;
-    for (int pass = 0; pass < passes; ++pass) {
-        const rs_status s = small ? radix_pass<kTileRoundsSmall>(tokens, tok_off, B, V, vbits, keybits, passes, pass, t_total, ix, st)
-                                  : radix_pass<kTileRounds>(tokens, tok_off, B, V, vbits, keybits, passes, pass, t_total, ix, st);
-        if (s != RS_OK) return s;
-    }
-    const uint2 *sorted = ix.pair[(passes - 1) & 1];
-    launch_pdl(index_first, dim3((unsigned)((V + 2ll + kFirstPer - 1) / kFirstPer), B), dim3(kFirstPer + 1), 0, st, sorted,
-        tok_off, V, vbits, ix);
-    RS_CHECK_LAUNCH("rs_match_index_build/first");
-    if (t_total == 0) return RS_OK;
-    launch_pdl(index_place, dim3((unsigned)((t_total + 256 * kPlacePer - 1) / (256 * kPlacePer))), dim3(256), 0, st, sorted,
-        (long long)t_total, tok_off, V, vbits, ix);
-    RS_CHECK_LAUNCH("rs_match_index_build/place");
-    return RS_OK;
+    if (cut_build(B, V, t_total))
+        return small ? build_cut<kTileRoundsSmall>(tokens, tok_off, B, V, t_total, ix, st)
+                     : build_cut<kTileRounds>(tokens, tok_off, B, V, t_total, ix, st);
+    return small ? build_plain<kTileRoundsSmall>(tokens, tok_off, B, V, t_total, ix, st)
+                 : build_plain<kTileRounds>(tokens, tok_off, B, V, t_total, ix, st);
 }
 
 extern "C" rs_status rs_match_index_append(const int32_t *tokens, const int64_t *tok_off, int B, int V,

@@ -20,7 +20,7 @@
 // holds.  So calls of up to kMatFewB requests take clusters of 16 CTAs of 512
 // threads (4 x 1M tokens: 23.6 us with 8, 15.3 with 16; more of these clusters
 // than GPCs run in turn: 8 requests 23.5 and 27.4), of which a request of
-// less than kMatWideRows rows uses 8; calls of up to kMatMidB requests clusters
+// fewer rows than its source's kWideRows uses 8; calls of up to kMatMidB requests clusters
 // of 8; larger calls clusters of 8 CTAs of 256 threads.
 #pragma once
 
@@ -34,7 +34,6 @@ namespace rs {
 constexpr int kMatCluster = 8;
 constexpr int kMatClusterMax = 16;
 constexpr int kMatFewB = 4, kMatMidB = 8;
-constexpr int kMatWideRows = 1024;  // 131072 candidates
 constexpr int kMatThreads = 512;          // or half of it
 constexpr int kMatWarps = kMatThreads / 32;
 constexpr int kMatCand = 512;             // matches ranked from the shared buffer
@@ -448,7 +447,7 @@ template <class Src>
 __device__ __forceinline__ int mat_ctas(int rows) {
     if (rows <= (int)(blockDim.x >> 5) * Src::kRows) return 1;
     const int nc = gridDim.x;
-    return nc > kMatCluster && rows < kMatWideRows ? kMatCluster : nc;
+    return nc > kMatCluster && rows < Src::kWideRows ? kMatCluster : nc;
 }
 
 // Launches a retrieval kernel over B requests; attr_done: the caller's flags,

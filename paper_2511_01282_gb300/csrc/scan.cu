@@ -19,6 +19,7 @@ namespace {
 
 struct ScanSource {
     static constexpr int kRows = 8;
+    static constexpr int kWideRows = 1024;  // 131072 positions: below, 8 CTAs are as fast as 16
     static constexpr bool kLaneMajor = true;
     int al;       // positions of the buffer start past a 16-byte boundary
     __device__ __forceinline__ int pos(int row, int lane, int e) const {
