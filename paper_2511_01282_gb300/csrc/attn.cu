@@ -37,7 +37,8 @@ __global__ void __launch_bounds__(256)
 attn_prep(const int32_t *__restrict__ node_off, const int32_t *__restrict__ ctx_len,
           const int64_t *__restrict__ kv_off, const int32_t *__restrict__ parents, int R, long long kv_rows,
           int Hq, int Hkv, int D, int seg_rows, ReqInfo *__restrict__ info, uint32_t *__restrict__ anc,
-          float *__restrict__ out, float *__restrict__ lse, int32_t *__restrict__ status) {
+          float *__restrict__ out, float *__restrict__ lse, int32_t *__restrict__ status,
+          int *__restrict__ n_items) {
     // the attention kernel takes whole SMs, so it launches only once this
     // kernel's own wait is over: earlier work has left them by then
     pdl_wait_prev();
@@ -84,65 +85,39 @@ attn_prep(const int32_t *__restrict__ node_off, const int32_t *__restrict__ ctx_
         }
     }
     if (tid == 0) status[b] = st;
+    if (b == 0 && tid == 0) *n_items = 0;
 }
 static_assert(kAncWords == 8, "an ancestor set is two 16-byte words");
 
-// attn_combine: every block first reads all job records (one per attention
-// CTA; a record names the split segment that CTA started) and cuts each job
-// into items of rows by a block scan, then takes items blockIdx.x,
-// blockIdx.x + gridDim.x, ...  A lane merges one column quad of rpw
-// consecutive rows, rpw = 4, 2 or 1 for segments of <= 2, <= 4 or more
-// pieces, so that it issues the loads of up to kCombPairs (row, piece)
-// partials (o, m, l) at once: an item costs one memory round trip for
+// attn_combine: blocks take the items the attention CTAs wrote (blockIdx.x,
+// blockIdx.x + gridDim.x, ...).  A lane merges one column quad of rpw
+// consecutive rows, so that it issues the loads of up to kCombPairs (row,
+// piece) partials (o, m, l) at once: an item costs one memory round trip for
 // segments of up to eight pieces whatever their number.  The pieces of a
 // row are folded in piece order with a running maximum (deterministic):
 // M = max_p m_p, L = sum_p e^(m_p - M) l_p, O = sum_p e^(m_p - M) O_p / L.
-// The pieces of a segment are the partial of CTA c (slot first_slot) and
-// slot 0 of every later CTA up to c1 with a non-empty unit range (the CTAs'
-// ranges are read from the records the attention kernel leaves beside the
-// jobs, so the combine does not depend on how the work was split).
-constexpr int kCombThreads = 256;
 constexpr int kCombPairs = 8;  // (row, piece) loads in flight per lane
 
-// Exclusive prefix of one int per thread of the block, in thread order.
-__device__ __forceinline__ int block_excl_scan(int v, int *s_w, int *total) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) s_w[warp] = x;
-    __syncthreads();
-    int before = 0, sum = 0;
-#pragma unroll
-    for (int w = 0; w < kCombThreads / 32; ++w) {
-        before += w < warp ? s_w[w] : 0;
-        sum += s_w[w];
-    }
-    __syncthreads();
-    *total = sum;
-    return before + x - v;
-}
-
 template <int D>
-__device__ __forceinline__ void combine_item(const AttnArgs &a, const CombJob &job, int np, const int *nonempty,
-                                             int row0, int rpw) {
+__device__ __forceinline__ void combine_item(const AttnArgs &a, const CombItem &it) {
     constexpr int kLpr = D / 4;        // lanes per row, one column quad each
     constexpr int kSub = 32 / kLpr;    // row groups per warp
     const int lane = threadIdx.x & 31;
     const int q = lane % kLpr;
     const int grp = (int)(threadIdx.x >> 5) * kSub + lane / kLpr;
     const int G = a.Hq / a.Hkv;
-    const int rows = min(a.seg_rows, job.N * G - job.mtile * a.seg_rows);
-    const int rbase = row0 + grp * rpw;                 // this lane's first row in the segment
-    const int npairs = max(0, min(rpw, rows - rbase)) * np;
-    // piece p > 0: slot 0 of the p-th CTA with a non-empty range after CTA c
-    auto slot_of = [&](int p) -> long long { return p == 0 ? job.first_slot : 2ll * nonempty[p]; };
+    const int np = it.np;
+    const int rbase = it.row0 + grp * it.rpw;           // this lane's first row in the segment
+    const int npairs = max(0, min(it.rpw, it.rows - rbase)) * np;
+    // (a choice per load between the list and the usual consecutive CTAs took 1 us
+    // longer, and so did two forms of this function: the kernel runs from a cold
+    // instruction cache)
+    const int *slots = a.slots + it.slots;              // of pieces 1 ..
+    auto slot_of = [&](int p) -> int { return p == 0 ? it.first_slot : slots[p]; };
     float M = -INFINITY, L = 0.f;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     int k = 0, p = 0;  // row and piece the fold is at
+    int i = (it.mrow + rbase) / G, hg = it.mrow + rbase - i * G;  // its node and head in the group
     for (int x0 = 0; x0 < npairs; x0 += kCombPairs) {
         float m[kCombPairs], l[kCombPairs];
         float4 o[kCombPairs];
@@ -154,10 +129,10 @@ __device__ __forceinline__ void combine_item(const AttnArgs &a, const CombJob &j
                 l[s] = 0.f;
                 o[s] = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (x0 + s < npairs) {
-                    const long long prow = slot_of(pp) * a.seg_rows + rbase + kk;
+                    const int prow = slot_of(pp) * a.seg_rows + rbase + kk;
                     m[s] = a.part_m[prow];
                     l[s] = a.part_l[prow];
-                    o[s] = *reinterpret_cast<const float4 *>(a.part_o + prow * D + q * 4);
+                    o[s] = *reinterpret_cast<const float4 *>(a.part_o + (long long)prow * D + q * 4);
                     if (++pp == np) {
                         pp = 0;
                         ++kk;
@@ -184,9 +159,7 @@ __device__ __forceinline__ void combine_item(const AttnArgs &a, const CombJob &j
                 }
             }
             if (++p == np) {  // row rbase + k complete
-                const int rr = job.mtile * a.seg_rows + rbase + k;
-                const int i = rr / G, h = job.kvh * G + (rr - i * G);
-                const long long orow = (long long)(job.n0 + i) * a.Hq + h;
+                const long long orow = (long long)(it.n0 + i) * a.Hq + it.kvh * G + hg;
                 const float f = L > 0.f ? 1.f / L : 0.f;
                 *reinterpret_cast<float4 *>(a.out + orow * D + q * 4) =
                     make_float4(acc.x * f, acc.y * f, acc.z * f, acc.w * f);
@@ -196,6 +169,10 @@ __device__ __forceinline__ void combine_item(const AttnArgs &a, const CombJob &j
                 acc = make_float4(0.f, 0.f, 0.f, 0.f);
                 p = 0;
                 ++k;
+                if (++hg == G) {
+                    hg = 0;
+                    ++i;
+                }
             }
         }
     }
@@ -203,68 +180,15 @@ __device__ __forceinline__ void combine_item(const AttnArgs &a, const CombJob &j
 
 template <int D>
 __global__ void __launch_bounds__(kCombThreads, 3)
-attn_combine(AttnArgs a, int Gc) {
+attn_combine(AttnArgs a) {
     pdl_enter();
-    __shared__ CombJob s_job[kAttnMaxGrid];
-    __shared__ int s_np[kAttnMaxGrid], s_rpw[kAttnMaxGrid], s_rank[kAttnMaxGrid];
-    __shared__ int s_ne[kAttnMaxGrid];  // the CTAs with a non-empty range, in order
-    __shared__ int s_pre[kAttnMaxGrid + 1];
-    __shared__ int s_w[kCombThreads / 32];
-    const int t = threadIdx.x;
-    const int G = a.Hq / a.Hkv;
-    constexpr int rows_per_group = kCombThreads / (D / 4);  // rows of an item with rpw = 1
-    // CTA t's job and whether its range is empty
-    CombJob j;
-    j.b = -1;
-    int ne = 0;
-    if (t < Gc) {
-        j = a.jobs[t];
-        s_job[t] = j;
-        const int2 rg = a.ranges[t];
-        ne = rg.y > rg.x;
-    }
-    int rank;
-    if (!__syncthreads_or(t < Gc && !ne)) {  // every range non-empty (the usual case): no scan
-        rank = t;
-        if (t < Gc) {
-            s_rank[t] = t;
-            s_ne[t] = t;
-        }
-    } else {
-        int n_ne;
-        rank = block_excl_scan(ne, s_w, &n_ne);
-        if (t < Gc) {
-            s_rank[t] = rank;
-            if (ne) s_ne[rank] = t;
-        }
-    }
-    __syncthreads();
-    // items of the job of CTA t
-    int items = 0;
-    if (t < Gc && j.b >= 0) {
-        const int np = s_rank[j.c1] - rank + 1;  // CTAs t and c1 both hold a piece
-        const int rpw = np <= 2 ? 4 : (np <= 4 ? 2 : 1);
-        const int rows = min(a.seg_rows, j.N * G - j.mtile * a.seg_rows);
-        const int per = rows_per_group * rpw;
-        s_np[t] = np;
-        s_rpw[t] = rpw;
-        items = (rows + per - 1) / per;
-    }
-    int total;
-    const int pre = block_excl_scan(items, s_w, &total);
-    if (t < Gc) s_pre[t] = pre;
-    if (t == 0) s_pre[Gc] = total;
-    __syncthreads();
-    for (int it = blockIdx.x; it < total; it += gridDim.x) {
-        int lo = 0, hi = Gc - 1;  // last CTA c with s_pre[c] <= it
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (s_pre[mid] <= it) lo = mid;
-            else hi = mid - 1;
-        }
-        const int c = lo;
-        const int row0 = (it - s_pre[c]) * rows_per_group * s_rpw[c];
-        combine_item<D>(a, s_job[c], s_np[c], s_ne + s_rank[c], row0, s_rpw[c]);
+    const int total = *a.n_items;
+    CombItem next = a.items[blockIdx.x];  // read with the count (the array holds more items than there are blocks)
+    for (int x = blockIdx.x; x < total;) {
+        const CombItem it = next;
+        x += gridDim.x;
+        if (x < total) next = a.items[x];
+        combine_item<D>(a, it);
     }
 }
 
@@ -365,8 +289,9 @@ extern "C" size_t rs_tree_verify_attn_workspace_size(int B, int R, int Hq, int H
     cv.take<float>(2 * Gc * rows * (size_t)D);
     cv.take<float>(2 * Gc * rows);
     cv.take<float>(2 * Gc * rows);
-    cv.take<CombJob>(Gc);
-    cv.take<int2>(Gc);
+    cv.take<CombItem>(kCombMaxItems * Gc);
+    cv.take<int>(1);
+    cv.take<int>(Gc * Gc);
     return cv.used();
 }
 
@@ -423,8 +348,9 @@ extern "C" rs_status rs_tree_verify_attn(const uint16_t *q, const uint16_t *k, c
     a.seg_rows = seg_rows;
     a.q_tma = 0;
     a.stage = 0;
-    a.jobs = cv.take<CombJob>((size_t)Gc);
-    a.ranges = cv.take<int2>((size_t)Gc);
+    a.items = cv.take<CombItem>((size_t)kCombMaxItems * Gc);
+    a.n_items = cv.take<int>(1);
+    a.slots = cv.take<int>((size_t)Gc * Gc);
     a.B = B;
     a.Hq = Hq;
     a.Hkv = Hkv;
@@ -489,7 +415,7 @@ extern "C" rs_status rs_tree_verify_attn(const uint16_t *q, const uint16_t *k, c
     }
     launch_pdl(attn_prep, dim3(B), dim3(256), 0, st, node_off, ctx_len, kv_off, parents, R, (long long)kv_rows, Hq,
         Hkv, D, seg_rows, info, anc, out, lse,
-        status);
+        status, a.n_items);
     RS_CHECK_LAUNCH("rs_tree_verify_attn/prep");
 
     int(&attr_done)[64][2] = pair ? g_pair_attr_done : g_attr_done;
@@ -531,8 +457,8 @@ extern "C" rs_status rs_tree_verify_attn(const uint16_t *q, const uint16_t *k, c
     // a full launch: combine blocks parked early beside the attention CTAs
     // (programmatic launch) measured slower (GQA-16K 56.4 -> 58.0 us, batched
     // 89.9 -> 90.1, 7B-shape step 44.3 -> 46.0)
-    if (D == 128) launch_full(attn_combine<128>, dim3(3 * Gc), dim3(kCombThreads), 0, st, a, Gc);
-    else launch_full(attn_combine<64>, dim3(3 * Gc), dim3(kCombThreads), 0, st, a, Gc);
+    if (D == 128) launch_full(attn_combine<128>, dim3(3 * Gc), dim3(kCombThreads), 0, st, a);
+    else launch_full(attn_combine<64>, dim3(3 * Gc), dim3(kCombThreads), 0, st, a);
     RS_CHECK_LAUNCH("rs_tree_verify_attn/combine");
     return RS_OK;
 }

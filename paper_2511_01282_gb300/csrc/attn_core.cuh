@@ -87,14 +87,30 @@ struct ReqInfo {
     int rows;   // (node, q-head-in-group) rows per KV head: N * Hq / Hkv
 };
 
-// The split segment a CTA starts, for attn_combine: the segment that begins
-// in the CTA's range and continues past it (at most one per CTA).
+// The split segment a CTA starts: the segment that begins in the CTA's range and
+// continues past it (at most one per CTA).
 struct CombJob {
     int b;           // request (-1: the CTA starts no split segment)
     int kvh, mtile;  // the segment's KV head and row tile
-    int n0, N;       // the request's first node and node count
     int first_slot;  // partial slot of the segment's first piece
     int c1;          // last CTA holding a piece of the segment
+};
+// Work of attn_combine: some rows of a split segment.  The CTA that starts the
+// segment writes its items, so that a combine block reads one record and can
+// load partials at once (it used to read every CTA's job, scan their items and
+// search for its own: GQA-16K call 57.2 -> 55.9 us, batched 90.4 -> 89.4, tiny
+// step 27.4 -> 26.4).
+constexpr int kCombThreads = 256;
+constexpr int kCombMaxItems = 32;  // of one segment: 256 rows, at least 8 an item
+struct __align__(16) CombItem {
+    int np, rpw;     // pieces; consecutive rows a lane merges
+    int rows;        // rows of the segment
+    int row0;        // the item's first row in the segment
+    int first_slot;  // partial slot of the first piece
+    int slots;       // the slots of the others: entries slots + 1 .. of AttnArgs::slots
+    int kvh, n0;     // KV head, the request's first node
+    int mrow;        // the segment's first (node, q-head-in-group) row in the request
+    int pad[3];
 };
 
 struct AttnArgs {
@@ -103,8 +119,9 @@ struct AttnArgs {
     const int32_t *ctx_len, *node_off;
     const uint32_t *anc;
     float *part_o, *part_m, *part_l;
-    CombJob *jobs;  // [gridDim.x]
-    int2 *ranges;   // [gridDim.x]: each CTA's unit range [x, y)
+    CombItem *items;  // [kCombMaxItems gridDim.x], the first *n_items used (in no particular order)
+    int *n_items;     // zeroed by attn_prep
+    int *slots;       // [gridDim.x][gridDim.x]: row c: the pieces' slots of the split segment CTA c starts
     int kv_stream;  // the launch's K/V is large next to L2: stream tiles read once
     int seg_rows;   // rows per segment and per partial slot: 128, or 256 in the two-tile form
     int stage;      // one-tile form: O rows leave through shared memory (attn_smem_bytes_staged)
@@ -288,20 +305,65 @@ __device__ __forceinline__ Piece piece_at(const ReqInfo *info, const int *s_pref
 template <class S>
 __device__ __forceinline__ CombJob comb_job(const AttnArgs &a, const ReqInfo *info, const int *s_pref, const S &split,
                                             long long u0, long long u1, int c) {
-    CombJob job{-1, 0, 0, 0, 0, 0, 0};
+    CombJob job{-1, 0, 0, 0, 0};
     if (u0 < u1) {
         const Piece pl = piece_at(info, s_pref, a.B, u1 - 1, u0, u1, c);
         if (pl.seg_start >= u0 && pl.seg_end > u1) {
             job.b = pl.b;
             job.kvh = pl.kvh;
             job.mtile = pl.mtile;
-            job.n0 = a.node_off[pl.b];
-            job.N = a.node_off[pl.b + 1] - job.n0;
             job.first_slot = (int)(2 * c + (pl.seg_start > u0 ? 1 : 0));
             job.c1 = (int)split.owner_of_seg_end(pl.b, pl.seg_start, pl.seg_end);
         }
     }
     return job;
+}
+
+// The items of that segment, by one warp.  Its pieces are slot first_slot and
+// slot 0 of every later CTA up to c1 with a non-empty unit range.  rpw = 4, 2 or
+// 1 rows a lane for <= 2, <= 4 or more pieces.
+template <int D, class S>
+__device__ __forceinline__ void write_items(const AttnArgs &a, const ReqInfo *info, const int *s_pref, const S &split,
+                                            long long u0, long long u1, int c) {
+    const int lane = threadIdx.x & 31;
+    const CombJob job = comb_job(a, info, s_pref, split, u0, u1, c);
+    if (job.b < 0) return;
+    int *slots = a.slots + (long long)c * gridDim.x;
+    int np = 1;
+    for (int x0 = c + 1; x0 <= job.c1; x0 += 32) {
+        const int x = x0 + lane;
+        const bool ne = x <= job.c1 && split.range_lo(x) < split.range_lo(x + 1);
+        const unsigned m = __ballot_sync(0xffffffffu, ne);
+        if (ne) slots[np + __popc(m & ((1u << lane) - 1u))] = 2 * x;
+        np += __popc(m);
+    }
+    const ReqInfo ri = info[job.b];
+    CombItem it;
+    it.np = np;
+    it.rpw = np <= 2 ? 4 : (np <= 4 ? 2 : 1);
+    it.mrow = job.mtile * a.seg_rows;
+    it.rows = min(a.seg_rows, ri.rows - it.mrow);
+    it.first_slot = job.first_slot;
+    it.slots = c * (int)gridDim.x;
+    it.kvh = job.kvh;
+    it.n0 = a.node_off[job.b];
+    const int per = kCombThreads / (D / 4) * it.rpw, items = (it.rows + per - 1) / per;
+    int base = 0;
+    if (lane == 0) base = atomicAdd(a.n_items, items);
+    base = __shfl_sync(0xffffffffu, base, 0);
+    for (int i = lane; i < items; i += 32) {
+        it.row0 = i * per;
+        a.items[base + i] = it;
+    }
+}
+
+// The same as a call, for the one-tile kernel, whose softmax code it would cost
+// registers (76 instead of 32 bytes of spills).  Not for the two-tile kernel's
+// TMA warp, which has given registers up: a called function does not know.
+template <int D, class S>
+__device__ __noinline__ void write_items_call(const AttnArgs &a, const ReqInfo *info, const int *s_pref, const S &split,
+                                              long long u0, long long u1, int c) {
+    write_items<D>(a, info, s_pref, split, u0, u1, c);
 }
 
 // 32 mask bits for tree indices [base, base + 32): negative indices are prefix
@@ -457,10 +519,7 @@ attn_tc_kernel(AttnArgs a, const ReqInfo *info, const __grid_constant__ CUtensor
             }
         }
         __syncwarp();
-        if (lane == 1) {  // after the producer loop: off the critical path
-            a.jobs[c] = comb_job(a, info, s_pref, split, u0, u1, (int)c);
-            a.ranges[c] = make_int2((int)u0, (int)u1);
-        }
+        write_items_call<D>(a, info, s_pref, split, u0, u1, (int)c);  // after the producer loop: off the critical path
     } else if (warp == kMmaWarp) {
         // ---------------------------------------------------------- MMA issuer
         if (lane == 0) {

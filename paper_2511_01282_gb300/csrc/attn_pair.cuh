@@ -18,7 +18,7 @@
 //
 // Warps: 0-3 softmax of tile A (thread = row, all 128 keys of a tile),
 // 4-7 softmax of tile B (idle in half mode), 8 TMA producer, 9 MMA issuer,
-// 10-11 idle.  A softmax thread holds a whole 128-key row of S, so the
+// 10 writes the combine items, 11 idle.  A softmax thread holds a whole 128-key row of S, so the
 // producer warpgroup (8-11) gives registers up to the softmax warpgroups
 // (setmaxnreg: 128 x 72 + 256 x 216 = 384 x 168, the launch's budget).
 // Tensor memory (512 columns): O_A [0, 128), O_B [128, 256), S/P buffer 0
@@ -370,11 +370,8 @@ attn_pair_kernel(AttnArgs a, const ReqInfo *info, const __grid_constant__ CUtens
                     }
             }
         }
-        __syncwarp();
-        if (lane == 1) {  // the split segment this CTA starts, for attn_combine
-            a.jobs[c] = comb_job(a, info, s_pref, split, u0, u1, (int)c);
-            a.ranges[c] = make_int2((int)u0, (int)u1);
-        }
+    } else if (warp == kMmaWarp + 1) {
+        write_items<D>(a, info, s_pref, split, u0, u1, (int)c);  // a warp with nothing else to do
     } else if (warp == kMmaWarp) {
         // ---------------------------------------------------------- MMA issuer
         if (lane == 0) {
