@@ -38,6 +38,7 @@ constexpr int kAccVpt = 32;
 constexpr int kAccChunk = kAccThreads * kAccVpt;
 constexpr int kNoId = 0x7fffffff;  // "no candidate": after every real (v, id)
 constexpr int kCandCap = 64;        // per-warp candidate buffer (logits at or above the threshold)
+constexpr int kListBeta = 8;        // list merges hold this many candidates of a chunk in registers
 constexpr int kFuseMax = 8;         // rows of at most this many chunks merge inside their cluster
 
 struct VI {
@@ -66,17 +67,30 @@ struct MS {
     float m, s, w;
 };
 
+// The triple of the union of one triple per lane, over aligned groups of G lanes
+// (each lane of a group gets it): the maximum first, then one exponential a
+// lane and plain sums.  A triple without mass (s = 0) counts for nothing.
+template <int G>
+__device__ __forceinline__ MS ms_union(MS t) {
+    float M = t.m;
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+    const bool some = t.s != 0.f;
+    const float d = t.m - M, c = some ? __expf(d) : 0.f;
+    float s = some ? t.s * c : 0.f, w = some ? c * (t.w + t.s * d) : 0.f;
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) {
+        s += __shfl_xor_sync(0xffffffffu, s, o);
+        w += __shfl_xor_sync(0xffffffffu, w, o);
+    }
+    return MS{M, s, w};
+}
 __device__ __forceinline__ MS ms_merge(MS a, MS b) {
     if (a.s == 0.f) return b;
     if (b.s == 0.f) return a;
     const float M = fmaxf(a.m, b.m);
     const float ca = __expf(a.m - M), cb = __expf(b.m - M);
     return MS{M, a.s * ca + b.s * cb, ca * (a.w + a.s * (a.m - M)) + cb * (b.w + b.s * (b.m - M))};
-}
-
-__device__ __forceinline__ MS ms_shfl(MS a, int o) {
-    return MS{__shfl_xor_sync(0xffffffffu, a.m, o), __shfl_xor_sync(0xffffffffu, a.s, o),
-              __shfl_xor_sync(0xffffffffu, a.w, o)};
 }
 
 // Bitonic sort of one float per lane within aligned groups of G lanes (a
@@ -116,17 +130,53 @@ struct RowOut {
     float *lse, *entropy, *rowmax;  // entropy may be null
 };
 
-// One warp merges row r's chunk results: the chunk (m, s, w) triples into
-// the log-sum-exp (and the entropy), the chunk candidate lists (ncand <=
-// 32 kPer pairs, loaded once into registers) into argmax and top-beta by
-// beta rounds of a warp-wide "best after the previous winner" reduction.
+// One warp merges row r's chunk results: the chunk (m, s, w) triples into the
+// log-sum-exp (and the entropy), the chunk candidate lists into argmax and
+// top-beta.  Lane c < G holds chunk c's list (nchunks <= G, beta <= kBeta); the
+// best of the lists' heads wins a round and its lane moves on.  (Rounds over all
+// candidates with a warp-wide "best after the previous winner" each made the
+// whole merge of 16 chunks and beta = 5 4.3 us behind the row pass, this 2.1.)
+template <int G, int kBeta>
+__device__ __forceinline__ void merge_lists(const VI *cand, const MS *part, int nchunks, int beta, long long r,
+                                            const RowOut &o, int lane) {
+    VI cv[kBeta];
+#pragma unroll
+    for (int k = 0; k < kBeta; ++k)
+        cv[k] = lane < nchunks && k < beta ? cand[lane * beta + k] : VI{-INFINITY, kNoId};
+    const MS ms = ms_union<G>(lane < nchunks ? part[lane] : MS{-INFINITY, 0.f, 0.f});
+    for (int k = 0; k < beta; ++k) {
+        VI best = cv[0];
+#pragma unroll
+        for (int off = G / 2; off > 0; off >>= 1) best = vi_best(best, vi_shfl(best, off));
+        if (cv[0].i == best.i) {
+#pragma unroll
+            for (int q = 0; q + 1 < kBeta; ++q) cv[q] = cv[q + 1];
+            cv[kBeta - 1] = VI{-INFINITY, kNoId};
+        }
+        if (lane == 0) {
+            const int id = best.i == kNoId ? -1 : best.i;
+            o.topk[r * beta + k] = id;
+            if (k == 0) {
+                o.argmax[r] = id;
+                o.rowmax[r] = best.v;
+            }
+        }
+    }
+    if (lane == 0) {
+        o.lse[r] = ms.s > 0.f ? ms.m + __logf(ms.s) : -INFINITY;
+        if (o.entropy) o.entropy[r] = ms.s > 0.f ? (__logf(ms.s) - ms.w / ms.s) : 0.f;
+    }
+}
+
+// The same for more chunks than lanes or longer lists (ncand <= 32 kPer pairs,
+// loaded once into registers): beta rounds of a warp-wide "best after the
+// previous winner" reduction over all candidates.
 template <int kPer>
 __device__ __forceinline__ void merge_row(const VI *cand, int ncand, const MS *part, int nchunks, int beta,
                                           long long r, const RowOut &o, int lane) {
     MS ms{-INFINITY, 0.f, 0.f};
     for (int c = lane; c < nchunks; c += 32) ms = ms_merge(ms, part[c]);
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) ms = ms_merge(ms, ms_shfl(ms, off));
+    ms = ms_union<32>(ms);
     VI cv[kPer];
 #pragma unroll
     for (int q = 0; q < kPer; ++q) {
@@ -343,10 +393,8 @@ accept_rows(const float *__restrict__ logits, int V, int nchunks, int beta, VI *
             }
         }
     }
-    if (warp == 0) {  // the eight warp triples, merged as a 3-level tree
-        MS a = lane < kAccThreads / 32 ? sh.sms[lane] : MS{-INFINITY, 0.f, 0.f};
-#pragma unroll
-        for (int off = 4; off > 0; off >>= 1) a = ms_merge(a, ms_shfl(a, off));
+    if (warp == 0) {  // the eight warp triples
+        const MS a = ms_union<kAccThreads / 32>(sh.sms[lane % (kAccThreads / 32)]);
         if (lane == 0) *dms = a;
     }
     if (kFuse) {
@@ -356,8 +404,10 @@ accept_rows(const float *__restrict__ logits, int V, int nchunks, int beta, VI *
         } else {
             __syncthreads();
         }
-        if (chunk == 0 && warp == 0)
-            merge_row<kFuseMax * RS_MAX_BETA / 32>(sh.rx_cand, nchunks * beta, sh.rx_ms, nchunks, beta, r, o, lane);
+        if (chunk == 0 && warp == 0) {
+            if (beta <= kListBeta) merge_lists<kFuseMax, kListBeta>(sh.rx_cand, sh.rx_ms, nchunks, beta, r, o, lane);
+            else merge_row<kFuseMax * RS_MAX_BETA / 32>(sh.rx_cand, nchunks * beta, sh.rx_ms, nchunks, beta, r, o, lane);
+        }
     }
 }
 
@@ -373,7 +423,9 @@ accept_merge(const VI *__restrict__ cand, const MS *__restrict__ part, int nchun
     const long long r = (long long)blockIdx.x * (kMergeThreads / 32) + (threadIdx.x >> 5);
     if (r >= R) return;
     const int ncand = nchunks * beta;
-    merge_row<kCandPerLane>(cand + r * ncand, ncand, part + r * nchunks, nchunks, beta, r, o, lane);
+    if (nchunks <= 32 && beta <= kListBeta)
+        merge_lists<32, kListBeta>(cand + r * ncand, part + r * nchunks, nchunks, beta, r, o, lane);
+    else merge_row<kCandPerLane>(cand + r * ncand, ncand, part + r * nchunks, nchunks, beta, r, o, lane);
 }
 
 // One thread per node (warps 0-7) and a warp for the chains and selections.
