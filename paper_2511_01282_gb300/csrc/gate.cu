@@ -41,12 +41,23 @@ __device__ __forceinline__ Ent3 ent_merge(Ent3 a, Ent3 b) {
     return r;
 }
 
-__device__ __forceinline__ Ent3 ent_shfl(Ent3 a, int o) {
-    Ent3 b;
-    b.m = __shfl_xor_sync(0xffffffffu, a.m, o);
-    b.s = __shfl_xor_sync(0xffffffffu, a.s, o);
-    b.w = __shfl_xor_sync(0xffffffffu, a.w, o);
-    return b;
+// The triple of the union of one triple per lane, over aligned groups of G lanes
+// (each lane of a group gets it): the maximum first, then one exponential a
+// lane and plain sums.  A triple without mass (s = 0) counts for nothing.
+template <int G>
+__device__ __forceinline__ Ent3 ent_union(Ent3 t) {
+    float M = t.m;
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+    const bool some = t.s != 0.f;
+    const float d = t.m - M, c = some ? __expf(d) : 0.f;
+    float s = some ? t.s * c : 0.f, w = some ? c * (t.w + t.s * d) : 0.f;
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) {
+        s += __shfl_xor_sync(0xffffffffu, s, o);
+        w += __shfl_xor_sync(0xffffffffu, w, o);
+    }
+    return Ent3{M, s, w};
 }
 
 // Row entropy in nats of the whole row's triple.
@@ -145,12 +156,12 @@ entropy_partial(const float *__restrict__ logits, int V, int nchunks, Ent3 *__re
     __shared__ Ent3 sw[kGateThreads / 32];
     if ((tid & 31) == 0) sw[tid >> 5] = t;
     __syncthreads();
-    if (tid == 0) {
-        Ent3 a = sw[0];
-#pragma unroll
-        for (int w = 1; w < kGateThreads / 32; ++w) a = ent_merge(a, sw[w]);
-        if (nchunks == 1) entropy[r] = ent_of(a);  // the chunk is the row: nothing to merge
-        else part[blk] = a;
+    if (tid < 32) {
+        const Ent3 a = ent_union<kGateThreads / 32>(sw[tid % (kGateThreads / 32)]);
+        if (tid == 0) {
+            if (nchunks == 1) entropy[r] = ent_of(a);  // the chunk is the row: nothing to merge
+            else part[blk] = a;
+        }
     }
 }
 
@@ -164,8 +175,7 @@ entropy_merge(const Ent3 *__restrict__ part, int nchunks, int R, float *__restri
     if (r >= R) return;
     Ent3 t{-INFINITY, 0.f, 0.f};
     for (int c = lane; c < nchunks; c += 32) t = ent_merge(t, part[r * nchunks + c]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t = ent_merge(t, ent_shfl(t, o));
+    t = ent_union<32>(t);
     if (lane == 0) entropy[r] = ent_of(t);
 }
 
