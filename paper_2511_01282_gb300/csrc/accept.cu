@@ -8,8 +8,8 @@
 // (logit desc, id asc); the top-beta is exact and sort-free apart from one
 // 16-lane sort that sets the candidate threshold.  No dynamic register
 // indexing.
-// Row merge: one warp per row merges the chunk results into argmax,
-// top-beta, log-sum-exp, the row's largest logit (workspace, for kernel 3)
+// Row merge: two warps per row merge the chunk results into argmax, top-beta,
+// log-sum-exp, the row's largest logit (workspace, for kernel 3)
 // and (optionally) the row entropy.  When a row has at most 8 chunks the
 // row's chunk CTAs form one cluster: each pushes its results into CTA 0's
 // shared memory and CTA 0 merges them after the cluster barrier, so the row
@@ -130,20 +130,30 @@ struct RowOut {
     float *lse, *entropy, *rowmax;  // entropy may be null
 };
 
-// One warp merges row r's chunk results: the chunk (m, s, w) triples into the
-// log-sum-exp (and the entropy), the chunk candidate lists into argmax and
-// top-beta.  Lane c < G holds chunk c's list (nchunks <= G, beta <= kBeta); the
+// Row r's log-sum-exp (and entropy) from its chunk triples, by one warp.
+template <int G>
+__device__ __forceinline__ void merge_triples(const MS *part, int nchunks, long long r, const RowOut &o, int lane) {
+    MS ms{-INFINITY, 0.f, 0.f};
+    for (int c = lane; c < nchunks; c += 32) ms = ms_merge(ms, part[c]);
+    ms = ms_union<G>(ms);
+    if (lane == 0) {
+        o.lse[r] = ms.s > 0.f ? ms.m + __logf(ms.s) : -INFINITY;
+        if (o.entropy) o.entropy[r] = ms.s > 0.f ? (__logf(ms.s) - ms.w / ms.s) : 0.f;
+    }
+}
+
+// Another merges the chunk candidate lists into argmax and top-beta.  Lane c < G
+// holds chunk c's list (nchunks <= G, beta <= kBeta); the
 // best of the lists' heads wins a round and its lane moves on.  (Rounds over all
 // candidates with a warp-wide "best after the previous winner" each made the
 // whole merge of 16 chunks and beta = 5 4.3 us behind the row pass, this 2.1.)
 template <int G, int kBeta>
-__device__ __forceinline__ void merge_lists(const VI *cand, const MS *part, int nchunks, int beta, long long r,
-                                            const RowOut &o, int lane) {
+__device__ __forceinline__ void merge_lists(const VI *cand, int nchunks, int beta, long long r, const RowOut &o,
+                                            int lane) {
     VI cv[kBeta];
 #pragma unroll
     for (int k = 0; k < kBeta; ++k)
         cv[k] = lane < nchunks && k < beta ? cand[lane * beta + k] : VI{-INFINITY, kNoId};
-    const MS ms = ms_union<G>(lane < nchunks ? part[lane] : MS{-INFINITY, 0.f, 0.f});
     for (int k = 0; k < beta; ++k) {
         VI best = cv[0];
 #pragma unroll
@@ -162,21 +172,13 @@ __device__ __forceinline__ void merge_lists(const VI *cand, const MS *part, int 
             }
         }
     }
-    if (lane == 0) {
-        o.lse[r] = ms.s > 0.f ? ms.m + __logf(ms.s) : -INFINITY;
-        if (o.entropy) o.entropy[r] = ms.s > 0.f ? (__logf(ms.s) - ms.w / ms.s) : 0.f;
-    }
 }
 
 // The same for more chunks than lanes or longer lists (ncand <= 32 kPer pairs,
 // loaded once into registers): beta rounds of a warp-wide "best after the
 // previous winner" reduction over all candidates.
 template <int kPer>
-__device__ __forceinline__ void merge_row(const VI *cand, int ncand, const MS *part, int nchunks, int beta,
-                                          long long r, const RowOut &o, int lane) {
-    MS ms{-INFINITY, 0.f, 0.f};
-    for (int c = lane; c < nchunks; c += 32) ms = ms_merge(ms, part[c]);
-    ms = ms_union<32>(ms);
+__device__ __forceinline__ void merge_row(const VI *cand, int ncand, int beta, long long r, const RowOut &o, int lane) {
     VI cv[kPer];
 #pragma unroll
     for (int q = 0; q < kPer; ++q) {
@@ -202,10 +204,6 @@ __device__ __forceinline__ void merge_row(const VI *cand, int ncand, const MS *p
                 o.rowmax[r] = best.v;
             }
         }
-    }
-    if (lane == 0) {
-        o.lse[r] = ms.s > 0.f ? ms.m + __logf(ms.s) : -INFINITY;
-        if (o.entropy) o.entropy[r] = ms.s > 0.f ? (__logf(ms.s) - ms.w / ms.s) : 0.f;
     }
 }
 
@@ -393,7 +391,7 @@ accept_rows(const float *__restrict__ logits, int V, int nchunks, int beta, VI *
             }
         }
     }
-    if (warp == 0) {  // the eight warp triples
+    if (warp == 1) {  // the eight warp triples
         const MS a = ms_union<kAccThreads / 32>(sh.sms[lane % (kAccThreads / 32)]);
         if (lane == 0) *dms = a;
     }
@@ -405,27 +403,29 @@ accept_rows(const float *__restrict__ logits, int V, int nchunks, int beta, VI *
             __syncthreads();
         }
         if (chunk == 0 && warp == 0) {
-            if (beta <= kListBeta) merge_lists<kFuseMax, kListBeta>(sh.rx_cand, sh.rx_ms, nchunks, beta, r, o, lane);
-            else merge_row<kFuseMax * RS_MAX_BETA / 32>(sh.rx_cand, nchunks * beta, sh.rx_ms, nchunks, beta, r, o, lane);
+            if (beta <= kListBeta) merge_lists<kFuseMax, kListBeta>(sh.rx_cand, nchunks, beta, r, o, lane);
+            else merge_row<kFuseMax * RS_MAX_BETA / 32>(sh.rx_cand, nchunks * beta, beta, r, o, lane);
         }
+        if (chunk == 0 && warp == 1) merge_triples<kFuseMax>(sh.rx_ms, nchunks, r, o, lane);
     }
 }
 
-// Row statistics of rows longer than kFuseMax chunks: one warp per row
-// merges the chunk results from the workspace.
-constexpr int kMergeThreads = 256;
+// Row statistics of rows longer than kFuseMax chunks: two warps per row merge
+// the chunk results from the workspace, the lists and the triples.
+constexpr int kMergeThreads = 128;
+constexpr int kMergeRows = kMergeThreads / 64;  // rows per block
 constexpr int kCandPerLane = 8;
 
 __global__ void __launch_bounds__(kMergeThreads)
 accept_merge(const VI *__restrict__ cand, const MS *__restrict__ part, int nchunks, int beta, int R, RowOut o) {
     pdl_enter();
-    const int lane = threadIdx.x & 31;
-    const long long r = (long long)blockIdx.x * (kMergeThreads / 32) + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const long long r = (long long)blockIdx.x * kMergeRows + (warp >> 1);
     if (r >= R) return;
     const int ncand = nchunks * beta;
-    if (nchunks <= 32 && beta <= kListBeta)
-        merge_lists<32, kListBeta>(cand + r * ncand, part + r * nchunks, nchunks, beta, r, o, lane);
-    else merge_row<kCandPerLane>(cand + r * ncand, ncand, part + r * nchunks, nchunks, beta, r, o, lane);
+    if (warp & 1) merge_triples<32>(part + r * nchunks, nchunks, r, o, lane);
+    else if (nchunks <= 32 && beta <= kListBeta) merge_lists<32, kListBeta>(cand + r * ncand, nchunks, beta, r, o, lane);
+    else merge_row<kCandPerLane>(cand + r * ncand, ncand, beta, r, o, lane);
 }
 
 // One thread per node (warps 0-7) and a warp for the chains and selections.
@@ -802,7 +802,7 @@ extern "C" rs_status rs_accept(const float *logits, int R, int V, const int32_t 
             launch_pdl(fn, grid, dim3(kAccThreads), 0, st, logits, V, nchunks, p.beta, cand, part, ro);
         RS_CHECK_LAUNCH("rs_accept/accept_rows");
         if (!fuse) {
-            launch_pdl(accept_merge, dim3((R + kMergeThreads / 32 - 1) / (kMergeThreads / 32)), dim3(kMergeThreads),
+            launch_pdl(accept_merge, dim3((R + kMergeRows - 1) / kMergeRows), dim3(kMergeThreads),
                 0, st, cand, part, nchunks, p.beta, R, ro);
             RS_CHECK_LAUNCH("rs_accept/accept_merge");
         }
