@@ -35,17 +35,18 @@
 // Build: the (request, bucket) keys of all tokens are sorted, with their
 // positions, by a stable LSD radix sort over all requests at once (digits of
 // at most 9 bits).  A pass is three kernels: the digit counts of every tile of
-// keys, their offsets, and the stable scatter, which ranks a tile's keys by
-// ballots and per-warp counters, orders the tile in shared memory and writes
-// whole runs of equal digits.  No atomics: counting buckets with them made a
+// keys, their offsets, and the stable scatter, which ranks a tile's keys with
+// per-warp counters, orders the tile in shared memory and writes whole runs of
+// equal digits.  No atomics on global memory: counting buckets with them made a
 // text's most common tokens the bottleneck (270 of 700 us for 4 x 1M tokens).
 // Keys of 10 to 18 bits (32K ids and 8 requests, 128K ids and two) take two
 // passes, and the tiles of the second are cut where the first digit changes:
 // the offsets at the first tile of a digit's keys are then where each bucket
 // begins, so the second scatter writes the positions straight into the buckets
-// and the bucket starts need no search.  Other key lengths (and short buffers,
-// whose few tiles this cut would multiply) sort in plain passes, find first[]
-// by a binary search per bucket and move the sorted positions in one more pass.
+// and the bucket starts need no search.  Between its passes a key is 32 bits,
+// its second digit over its position.  Other key lengths (and the shortest and
+// longest buffers) sort in plain passes, find first[] by a binary search per
+// bucket and move the sorted positions in one more pass.
 // Append: one CTA per request takes the new positions in rounds of 256; each
 // position's rank among the round's positions of its bucket gives its slot
 // after the bucket's entries; full buckets spill to the overflow list in
@@ -87,13 +88,18 @@ inline int bits_for(long long n) {  // smallest b with n < 2^b
     return b;
 }
 inline int key_bits(int B, int V) { return bits_for(V) + bits_for(B > 0 ? B - 1 : 0); }
-// Whether the second pass's tiles are cut at the first digit (see above): 4 x 1M
-// tokens build in 86.6 us so, 96.8 in plain passes; 4 x 32K in 26.9 and 28.5, but
-// with the appends and queries behind it in 88.3 and 87.7.
-constexpr long long kCutMin = 1 << 18;
+// Whether the second pass's tiles are cut at the first digit (see above), with
+// 32-bit keys between the passes.  Builds of a text so and in plain passes: 4 x 1M
+// tokens 62.8 and 88.0 us, 4 x 200K 38.1 and 47.3, 8 x 60K 34.8 and 37.7, 4 x 32K
+// 27.1 and 29.2.  Shorter ones are a few us of kernels between launches either
+// way, and the counts of the cut tiles are a MB more of index.
+constexpr long long kCutMin = 1 << 16;
+inline int cut_lo_bits(int B, int V) { return (key_bits(B, V) + 1) / 2; }
+inline int cut_pos_bits(long long t_total) { return bits_for(t_total - 1); }
 inline bool cut_build(int B, int V, long long t_total) {
     const int bits = key_bits(B, V);
-    return t_total >= kCutMin && bits > kMaxDigitBits && bits <= 2 * kMaxDigitBits;
+    return t_total >= kCutMin && bits > kMaxDigitBits && bits <= 2 * kMaxDigitBits &&
+           bits - cut_lo_bits(B, V) + cut_pos_bits(t_total) <= 32;
 }
 // tiles of a pass, at most: with cuts, one more per digit and one past the end
 inline long long hist_tiles(int B, int V, long long t_total) {
@@ -154,14 +160,16 @@ index_check(const int64_t *__restrict__ tok_off, int B, long long t_total, Index
     if (threadIdx.x == 0) *ix.valid = bad ? 0 : 1;
 }
 
-// The keys of a pass: pass 0 makes them from the tokens (the request of token
-// i is the last b with tok_off[b] <= i), later passes read the pairs.
+// The keys of a pass, by tile: pass 0 makes them from the tokens (the request
+// of token i is the last b with tok_off[b] <= i), later passes read the pairs.
 struct TokenKeys {
     const int32_t *tokens;
     const int64_t *tok_off;
     int B, V, vbits;
-    int b0;        // the request of the tile's first token
-    long long b1;  // where that request ends
+    uint32_t i0;         // the tile's first token
+    const int32_t *tile;
+    uint32_t high;       // the request bits of that token's key
+    int own;             // the tile's tokens of the same request
     __device__ __forceinline__ int request(long long i) const {
         int lo = 0, hi = B - 1;
         while (lo < hi) {
@@ -171,24 +179,31 @@ struct TokenKeys {
         }
         return lo;
     }
-    __device__ __forceinline__ void tile(long long i0) {
-        b0 = request(i0);
-        b1 = tok_off[b0 + 1];
+    __device__ __forceinline__ uint32_t request_bits(int b) const { return vbits >= 32 ? 0u : (uint32_t)b << vbits; }
+    __device__ __forceinline__ void begin(long long first) {
+        i0 = (uint32_t)first;
+        tile = tokens + first;
     }
     // the load, apart from what is made of it, so that a thread's loads are all
     // in flight before any is used
-    __device__ __forceinline__ int load(long long i) const { return tokens[i]; }
-    __device__ __forceinline__ uint2 pair(int tok, long long i) const {
-        const int b = i < b1 ? b0 : request(i);
-        const uint32_t k = (uint32_t)bucket_of(tok, V) | (vbits >= 32 ? 0u : ((uint32_t)b << vbits));
-        return make_uint2(k, (uint32_t)i);
+    __device__ __forceinline__ int load(int e) const { return tile[e]; }
+    __device__ __forceinline__ void after_loads() {
+        const int b = request(i0);
+        const long long left = tok_off[b + 1] - (long long)i0;
+        high = request_bits(b);
+        own = (int)(left < 0x7fffffff ? left : 0x7fffffff);
+    }
+    __device__ __forceinline__ uint2 pair(int tok, int e) const {
+        const uint32_t i = i0 + (uint32_t)e;
+        return make_uint2((uint32_t)bucket_of(tok, V) | (e < own ? high : request_bits(request(i))), i);
     }
 };
 struct PairKeys {
     const uint2 *in;
-    __device__ __forceinline__ void tile(long long) {}
-    __device__ __forceinline__ uint2 load(long long i) const { return in[i]; }
-    __device__ __forceinline__ uint2 pair(uint2 x, long long) const { return x; }
+    __device__ __forceinline__ void begin(long long first) { in += first; }
+    __device__ __forceinline__ uint2 load(int e) const { return in[e]; }
+    __device__ __forceinline__ void after_loads() {}
+    __device__ __forceinline__ uint2 pair(uint2 x, int) const { return x; }
 };
 
 // Each radix kernel handles one tile of kR * 256 keys; a thread's keys are all
@@ -201,18 +216,20 @@ radix_hist(Keys src, long long N, int shift, int bins, int32_t *__restrict__ his
     __shared__ int cnt[kMaxBins];
     const long long tile = blockIdx.x, i0 = tile * (kR * kRadixThreads);
     for (int d = threadIdx.x; d < bins; d += kRadixThreads) cnt[d] = 0;
+    const int n = (int)(N - i0 < kR * kRadixThreads ? N - i0 : kR * kRadixThreads);
+    src.begin(i0);
     decltype(src.load(0)) x[kR];
 #pragma unroll
     for (int q = 0; q < kR; ++q) {
-        const long long i = i0 + q * kRadixThreads + threadIdx.x;
-        x[q] = src.load(i < N ? i : i0);
+        const int e = q * kRadixThreads + (int)threadIdx.x;
+        x[q] = src.load(e < n ? e : 0);
     }
-    src.tile(i0);
+    src.after_loads();
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < kR; ++q) {
-        const long long i = i0 + q * kRadixThreads + threadIdx.x;
-        if (i < N) atomicAdd(&cnt[(src.pair(x[q], i).x >> shift) & (bins - 1)], 1);
+        const int e = q * kRadixThreads + (int)threadIdx.x;
+        if (e < n) atomicAdd(&cnt[(src.pair(x[q], e).x >> shift) & (bins - 1)], 1);
     }
     __syncthreads();
     for (int d = threadIdx.x; d < bins; d += kRadixThreads) hist[tile * bins + d] = cnt[d];
@@ -243,38 +260,51 @@ __device__ __forceinline__ int radix_excl_scan(int v, int *s_w, int *total) {
 
 // (tile, digit) offsets: each digit's exclusive prefix over the tiles, and
 // its total.  A block takes eight digits (one 32-byte sector of a tile's
-// counts); thread (group g, digit d) takes sixteen consecutive tiles a round.
-constexpr int kOffDigits = 8, kOffTiles = 16;
-__global__ void __launch_bounds__(kRadixThreads)
+// counts); thread (group g, digit d) takes kT consecutive tiles a round, four
+// groups to a warp.
+// Threads: one round for 1024 tiles of 4096 keys (4 x 1M tokens: 65.7 us for the
+// whole build, 68.8 with 1024 threads) or 128 of 1024 (4 x 32K tokens: 28.4,
+// 29.9 with 1024; 4096 tokens: 19.0 and 21.4).
+constexpr int kOffDigits = 8;
+constexpr int off_threads(int rounds) { return rounds == kTileRounds ? 512 : 256; }
+template <int kT>
+__global__ void __launch_bounds__(off_threads(kT))
 radix_offsets(int32_t *__restrict__ hist, long long ntiles, int bins, int32_t *__restrict__ dtot,
               const int32_t *__restrict__ valid) {
     pdl_enter();
     if (!*valid) return;
-    constexpr int kGroups = kRadixThreads / kOffDigits;
-    __shared__ int s_sum[kGroups][kOffDigits + 1];
-    const int d = threadIdx.x % kOffDigits, g = threadIdx.x / kOffDigits;
+    constexpr int kWarps = off_threads(kT) / 32, kGroups = off_threads(kT) / kOffDigits;
+    __shared__ int s_sum[kWarps][kOffDigits];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int d = lane % kOffDigits, g = threadIdx.x / kOffDigits;
     int32_t *col = hist + blockIdx.x * kOffDigits + d;
     const bool live = (int)blockIdx.x * kOffDigits + d < bins;
     int carry = 0;
-    for (long long base = 0; base < ntiles; base += kGroups * kOffTiles) {
-        const long long t = base + g * kOffTiles;
-        int c[kOffTiles], sum = 0;
+    for (long long base = 0; base < ntiles; base += kGroups * kT) {
+        const long long t = base + g * kT;
+        int c[kT], sum = 0;
 #pragma unroll
-        for (int q = 0; q < kOffTiles; ++q) c[q] = live && t + q < ntiles ? col[(t + q) * bins] : 0;
+        for (int q = 0; q < kT; ++q) c[q] = live && t + q < ntiles ? col[(t + q) * bins] : 0;
 #pragma unroll
-        for (int q = 0; q < kOffTiles; ++q) sum += c[q];
-        s_sum[g][d] = sum;
+        for (int q = 0; q < kT; ++q) sum += c[q];
+        int x = sum;
+#pragma unroll
+        for (int o = kOffDigits; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane >= 32 - kOffDigits) s_sum[warp][d] = x;
         __syncthreads();
-        int x = carry;
+        x += carry - sum;
 #pragma unroll
-        for (int h = 0; h < kGroups; ++h) {
-            const int y = s_sum[h][d];
-            x += h < g ? y : 0;
+        for (int w = 0; w < kWarps; ++w) {
+            const int y = s_sum[w][d];
+            x += w < warp ? y : 0;
             carry += y;
         }
         __syncthreads();
 #pragma unroll
-        for (int q = 0; q < kOffTiles; ++q) {
+        for (int q = 0; q < kT; ++q) {
             if (live && t + q < ntiles) col[(t + q) * bins] = x;
             x += c[q];
         }
@@ -286,9 +316,12 @@ radix_offsets(int32_t *__restrict__ hist, long long ntiles, int bins, int32_t *_
 // keys w 32 rounds .. of the tile, 32 at a time; a key's rank is the count of
 // equal digits before it in the tile (earlier warps, earlier rounds of its
 // warp, lower lanes of its round).
-template <int kR>
+template <class W, int kR>
 struct TileShared {
-    uint2 pair[kR * kRadixThreads];
+    union {
+        W word[kR * kRadixThreads];
+        uint32_t peers[kRadixWarps][kMaxBins];  // while ranking: the lanes of the warp's round with that digit
+    };
     uint16_t cnt[kRadixWarps][kMaxBins];
     int w[kRadixWarps];
 };
@@ -296,36 +329,45 @@ __device__ __forceinline__ int tile_rounds_of(int n) { return (n + kRadixThreads
 __device__ __forceinline__ int tile_elem(int rounds, int q) {
     return ((int)(threadIdx.x >> 5) * rounds + q) * 32 + (int)(threadIdx.x & 31);
 }
-// k[q]: this thread's keys (tile_elem(rounds, q) below n); starts(x, y): called
-// by every thread with the places of its digits 2 tid and 2 tid + 1 in the
-// ordered tile.  Ends with a barrier.
-template <int kR, class Starts>
-__device__ __forceinline__ void order_tile(TileShared<kR> &sh, const uint2 (&k)[kR], int n, int rounds, int shift, int bins,
+// k[q]: this thread's keys, those past the tile's last with the largest digit
+// (they come after the others wherever they are counted); digit(k): a key's
+// digit; starts(x, y): called by every thread with the places of its digits 2
+// tid and 2 tid + 1 in the ordered tile.  Ends with a barrier.
+//
+// Bound by shared memory (a key's bit, count, place, and the key itself written
+// and read, most at two to three lanes a bank).  The lanes of a round that
+// share a digit: those of the first lane's by one ballot, the others set their
+// bits in a word per digit.  The ballot takes the digit that many lanes have,
+// as in text and in the later passes, where setting bits would run one lane
+// after the other.  A build of 4 x 1M tokens with this against a ballot per digit
+// bit: a text 63.0 and 85.7 us, uniform tokens 63.1 and 86.6, one token 53.5 and
+// 81.2 (bits alone: text 71, match.any in the second pass: text 60.5, uniform
+// 78.4).
+template <class W, int kR, class Digit, class Starts>
+__device__ __forceinline__ void order_tile(TileShared<W, kR> &sh, const W (&k)[kR], int rounds, Digit digit,
                                            Starts starts) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int x = tid; x < kRadixWarps * kMaxBins / 2; x += kRadixThreads) reinterpret_cast<uint32_t *>(&sh.cnt[0][0])[x] = 0;
+    for (int x = tid; x < kRadixWarps * kMaxBins / 8; x += kRadixThreads) reinterpret_cast<uint4 *>(&sh.cnt[0][0])[x] = uint4{};
+    for (int x = tid; x < kRadixWarps * kMaxBins / 4; x += kRadixThreads)
+        reinterpret_cast<uint4 *>(&sh.peers[0][0])[x] = uint4{};
     __syncthreads();
     const unsigned lt = (1u << lane) - 1u;
     int rk[kR];
 #pragma unroll
     for (int q = 0; q < kR; ++q) {
         if (q >= rounds) break;
-        const bool ok = tile_elem(rounds, q) < n;
-        const int dg = (int)((k[q].x >> shift) & (bins - 1));
-        // the lanes of this round with the same digit, one ballot per bit
-        // (match.any is slow where a round holds many distinct digits: first
-        // pass over 4 x 1M tokens 47.2 us with it, 31.2 so; second pass, few
-        // distinct digits, 25.7 against 27.4)
-        unsigned peers = __ballot_sync(0xffffffffu, ok);
-#pragma unroll
-        for (int bit = 0; bit < kMaxDigitBits; ++bit) {
-            const bool one = (dg >> bit) & 1;
-            const unsigned bal = __ballot_sync(0xffffffffu, one);
-            peers &= one ? bal : ~bal;
-        }
-        const int before = ok ? sh.cnt[warp][dg] : 0;
+        const int dg = digit(k[q]);
+        const bool as_first = dg == __shfl_sync(0xffffffffu, dg, 0);
+        const unsigned firsts = __ballot_sync(0xffffffffu, as_first);
+        if (!as_first) atomicOr(&sh.peers[warp][dg], 1u << lane);
         __syncwarp();
-        if (ok && (peers & lt) == 0) sh.cnt[warp][dg] = (uint16_t)(before + __popc(peers));
+        const unsigned peers = as_first ? firsts : sh.peers[warp][dg];
+        const int before = sh.cnt[warp][dg];
+        __syncwarp();
+        if ((peers & lt) == 0) {
+            sh.cnt[warp][dg] = (uint16_t)(before + __popc(peers));
+            if (!as_first) sh.peers[warp][dg] = 0;
+        }
         __syncwarp();
         rk[q] = before + __popc(peers & lt);
     }
@@ -353,12 +395,8 @@ __device__ __forceinline__ void order_tile(TileShared<kR> &sh, const uint2 (&k)[
     }
     __syncthreads();
 #pragma unroll
-    for (int q = 0; q < kR; ++q) {
-        if (q < rounds && tile_elem(rounds, q) < n) {
-            const int dg = (int)((k[q].x >> shift) & (bins - 1));
-            sh.pair[sh.cnt[warp][dg] + rk[q]] = k[q];
-        }
-    }
+    for (int q = 0; q < kR; ++q)
+        if (q < rounds) sh.word[sh.cnt[warp][digit(k[q])] + rk[q]] = k[q];
     __syncthreads();
 }
 
@@ -367,49 +405,81 @@ __device__ __forceinline__ int2 two_digits(const int32_t *row, int bins) {
     return 2 * (int)threadIdx.x < bins ? *reinterpret_cast<const int2 *>(row + 2 * threadIdx.x) : make_int2(0, 0);
 }
 
+// What a scatter keeps of a key in its tile and writes: the pair itself, or
+// (first pass of a cut build, digit: the low bits of the key) the key over its
+// place in the tile, written as its other bits over its position.
+template <int kR>
+struct WholePair {
+    using W = uint2;
+    static constexpr int kBlocks = 3;
+    int shift, bins;
+    __device__ __forceinline__ W make(uint2 p, int) const { return p; }
+    __device__ __forceinline__ W last() const { return make_uint2(0xffffffffu, 0u); }
+    __device__ __forceinline__ int digit(W w) const { return (int)((w.x >> shift) & (bins - 1)); }
+    __device__ __forceinline__ W out(W w, long long) const { return w; }
+};
+template <int kR>
+struct Packed {
+    using W = uint32_t;
+    static constexpr int kBlocks = 4;
+    static constexpr int kPlace = kR == kTileRounds ? 12 : 10;
+    static_assert(kR * kRadixThreads == 1 << kPlace && 2 * kMaxDigitBits + kPlace <= 32, "a key and a place in 32 bits");
+    int lo_bits, pos_bits;
+    __device__ __forceinline__ W make(uint2 p, int e) const { return p.x << kPlace | (uint32_t)e; }
+    __device__ __forceinline__ W last() const { return 0xffffffffu; }
+    __device__ __forceinline__ int digit(W w) const { return (int)((w >> kPlace) & ((1u << lo_bits) - 1u)); }
+    __device__ __forceinline__ W out(W w, long long i0) const {
+        return ((w >> kPlace) >> lo_bits) << pos_bits | ((uint32_t)i0 + (w & ((1u << kPlace) - 1u)));
+    }
+};
+
 // The stable scatter: equal digits -- consecutive addresses -- are written by
 // neighbouring threads.
-template <class Keys, int kR>
-__global__ void __launch_bounds__(kRadixThreads, 3)
-radix_scatter(Keys src, uint2 *__restrict__ out, long long N, int shift, int bins,
+template <class Keys, int kR, class Words>
+__global__ void __launch_bounds__(kRadixThreads, Words::kBlocks)
+radix_scatter(Keys src, Words words, typename Words::W *__restrict__ out, long long N, int bins,
               const int32_t *__restrict__ hist, const int32_t *__restrict__ dtot, const int32_t *__restrict__ valid) {
     pdl_enter();
     if (!*valid) return;
+    using W = typename Words::W;
     constexpr int kTile = kR * kRadixThreads;
-    __shared__ TileShared<kR> sh;
+    __shared__ TileShared<W, kR> sh;
     __shared__ int s_dst[kMaxBins];  // global index of the digit's first key, less its place in the tile
     const long long tile = blockIdx.x, i0 = tile * kTile;
     const int n = (int)(N - i0 < kTile ? N - i0 : kTile), rounds = tile_rounds_of(n);
+    src.begin(i0);
     decltype(src.load(0)) x[kR];
 #pragma unroll
     for (int q = 0; q < kR; ++q) {
         const int e = tile_elem(rounds, q);
-        x[q] = src.load(i0 + (q < rounds && e < n ? e : 0));
+        x[q] = src.load(q < rounds && e < n ? e : 0);
     }
-    src.tile(i0);
+    src.after_loads();
     // where the tile's keys of each digit begin, within the digit and over all digits
     int2 g = two_digits(hist + tile * bins, bins);
     const int2 tot = two_digits(dtot, bins);
-    uint2 k[kR];
+    W k[kR];
 #pragma unroll
     for (int q = 0; q < kR; ++q) {
         const int e = tile_elem(rounds, q);
-        k[q] = q < rounds && e < n ? src.pair(x[q], i0 + e) : make_uint2(0u, 0u);
+        k[q] = q < rounds && e < n ? words.make(src.pair(x[q], e), e) : words.last();
     }
     int all;
     const int below = radix_excl_scan(tot.x + tot.y, sh.w, &all);
     g.x += below;
     g.y += below + tot.x;
-    order_tile(sh, k, n, rounds, shift, bins, [&](int x0, int x1) {
-        s_dst[2 * threadIdx.x] = g.x - x0;
-        s_dst[2 * threadIdx.x + 1] = g.y - x1;
-    });
+    order_tile(
+        sh, k, rounds, [&](W w) { return words.digit(w); },
+        [&](int x0, int x1) {
+            s_dst[2 * threadIdx.x] = g.x - x0;
+            s_dst[2 * threadIdx.x + 1] = g.y - x1;
+        });
 #pragma unroll
     for (int q = 0; q < kR; ++q) {
         const int e = q * kRadixThreads + threadIdx.x;
         if (e < n) {
-            const uint2 v = sh.pair[e];
-            out[(long long)s_dst[(v.x >> shift) & (bins - 1)] + e] = v;
+            const W v = sh.word[e];
+            out[(long long)s_dst[words.digit(v)] + e] = words.out(v, i0);
         }
     }
 }
@@ -418,9 +488,8 @@ radix_scatter(Keys src, uint2 *__restrict__ out, long long N, int shift, int bin
 // Tile `tile`: its keys [i0, i0 + n) share the first digit `digit`, whose keys
 // begin with tile `first`; n = 0 past the last tile.  dtot: the first digit's
 // totals.
-struct CutTile {
-    int digit, first, n;
-    long long i0;
+struct __align__(16) CutTile {
+    int digit, first, n, i0;
 };
 __device__ __forceinline__ CutTile cut_tile(const int32_t *dtot, int bins, int tile_keys, int tile, int *s_w, CutTile *s_out) {
     const int2 c = two_digits(dtot, bins);
@@ -432,7 +501,7 @@ __device__ __forceinline__ CutTile cut_tile(const int32_t *dtot, int bins, int t
     if (tile >= tx && tile < tx + a + b) {
         const bool second = tile >= tx + a;
         const int first = second ? tx + a : tx, at = (tile - first) * tile_keys, cnt = second ? c.y : c.x;
-        *s_out = CutTile{2 * (int)threadIdx.x + second, first, min(tile_keys, cnt - at), (long long)kx + (second ? c.x : 0) + at};
+        *s_out = CutTile{2 * (int)threadIdx.x + second, first, min(tile_keys, cnt - at), kx + (second ? c.x : 0) + at};
     }
     __syncthreads();
     return *s_out;
@@ -440,8 +509,8 @@ __device__ __forceinline__ CutTile cut_tile(const int32_t *dtot, int bins, int t
 
 template <int kR>
 __global__ void __launch_bounds__(kRadixThreads)
-cut_hist(const uint2 *__restrict__ in, int bins0, int shift, int bins, const int32_t *__restrict__ dtot,
-         int32_t *__restrict__ hist, const int32_t *__restrict__ valid) {
+cut_hist(const uint32_t *__restrict__ in, int bins0, int pos_bits, int bins, const int32_t *__restrict__ dtot,
+         int32_t *__restrict__ hist, CutTile *__restrict__ tiles, const int32_t *__restrict__ valid) {
     pdl_enter();
     if (!*valid) return;
     __shared__ int cnt[kMaxBins];
@@ -449,15 +518,16 @@ cut_hist(const uint2 *__restrict__ in, int bins0, int shift, int bins, const int
     __shared__ CutTile s_tile;
     for (int d = threadIdx.x; d < bins; d += kRadixThreads) cnt[d] = 0;
     const CutTile t = cut_tile(dtot, bins0, kR * kRadixThreads, blockIdx.x, s_w, &s_tile);
+    if (threadIdx.x == 0) tiles[blockIdx.x] = t;
     uint32_t x[kR];
 #pragma unroll
     for (int q = 0; q < kR; ++q) {
         const int e = q * kRadixThreads + threadIdx.x;
-        x[q] = e < t.n ? in[t.i0 + e].x : 0u;
+        x[q] = e < t.n ? in[t.i0 + e] : 0u;
     }
 #pragma unroll
     for (int q = 0; q < kR; ++q)
-        if (q * kRadixThreads + (int)threadIdx.x < t.n) atomicAdd(&cnt[x[q] >> shift], 1);
+        if (q * kRadixThreads + (int)threadIdx.x < t.n) atomicAdd(&cnt[x[q] >> pos_bits], 1);
     __syncthreads();
     for (int d = threadIdx.x; d < bins; d += kRadixThreads) hist[(long long)blockIdx.x * bins + d] = cnt[d];  // 0 past the last tile
 }
@@ -468,29 +538,28 @@ cut_hist(const uint2 *__restrict__ in, int bins0, int shift, int bins, const int
 // Blocks past them: first[] and len[] of 1024 buckets, from the same sums.
 constexpr int kCutFirst = 1024;
 template <int kR>
-__global__ void __launch_bounds__(kRadixThreads, 3)
-cut_scatter(const uint2 *__restrict__ in, int tiles, int bins0, int lo_bits, int bins, const int32_t *__restrict__ dtot,
+__global__ void __launch_bounds__(kRadixThreads, 4)
+cut_scatter(const uint32_t *__restrict__ in, const CutTile *__restrict__ cuts, int tiles, int bins0, int lo_bits, int pos_bits, int bins, const int32_t *__restrict__ dtot,
             const int32_t *__restrict__ hist, const int64_t *__restrict__ tok_off, int B, int V, int vbits, IndexView ix) {
     pdl_enter();
     if (!*ix.valid) return;
     constexpr int kTile = kR * kRadixThreads;
-    __shared__ TileShared<kR> sh;
-    __shared__ CutTile s_tile;
+    __shared__ TileShared<uint32_t, kR> sh;
     __shared__ long long s_list[kMaxBins];  // list slot of the digit's first key in the tile, less its place there
     __shared__ int s_t0[kMaxBins];
     const int tid = threadIdx.x;
     const uint32_t vmask = (1u << vbits) - 1u;  // vbits <= 18 here
     const int2 tot = two_digits(dtot + kMaxBins, bins);
+    const CutTile t = (int)blockIdx.x < tiles ? cuts[blockIdx.x] : CutTile{};
     int all;
-    const int below = radix_excl_scan(tot.x + tot.y, sh.w, &all);
-    const int base[2] = {below, below + tot.x};
     if ((int)blockIdx.x >= tiles) {
+        const int below = radix_excl_scan(tot.x + tot.y, sh.w, &all);
         int *s_base = s_t0, *s_first = reinterpret_cast<int *>(s_list);
         const int2 c = two_digits(dtot, bins0);
         const int a = (c.x + kTile - 1) / kTile, b = (c.y + kTile - 1) / kTile;
         const int tx = radix_excl_scan(a + b, sh.w, &all);
-        s_base[2 * tid] = base[0];
-        s_base[2 * tid + 1] = base[1];
+        s_base[2 * tid] = below;
+        s_base[2 * tid + 1] = below + tot.x;
         s_first[2 * tid] = tx;
         s_first[2 * tid + 1] = tx + a;
         __syncthreads();
@@ -518,17 +587,19 @@ cut_scatter(const uint2 *__restrict__ in, int tiles, int bins0, int lo_bits, int
         }
         return;
     }
-    const CutTile t = cut_tile(dtot, bins0, kTile, blockIdx.x, sh.w, &s_tile);
     if (t.n == 0) return;
     const int rounds = tile_rounds_of(t.n);
-    uint2 k[kR];
+    const uint32_t last = (uint32_t)(bins - 1) << pos_bits;
+    uint32_t k[kR];
 #pragma unroll
     for (int q = 0; q < kR; ++q) {
         const int e = tile_elem(rounds, q);
-        k[q] = q < rounds && e < t.n ? in[t.i0 + e] : make_uint2(0u, 0u);
+        k[q] = q < rounds && e < t.n ? in[t.i0 + e] : last;
     }
     const int2 own = two_digits(hist + (long long)blockIdx.x * bins, bins);
     const int2 run = two_digits(hist + (long long)t.first * bins, bins);
+    const int below = radix_excl_scan(tot.x + tot.y, sh.w, &all);
+    const int base[2] = {below, below + tot.x};
     long long list[2] = {0, 0};
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
@@ -543,17 +614,19 @@ cut_scatter(const uint2 *__restrict__ in, int tiles, int bins0, int lo_bits, int
             s_t0[d] = (int)t0;
         }
     }
-    order_tile(sh, k, t.n, rounds, lo_bits, bins, [&](int x0, int x1) {
-        s_list[2 * tid] = list[0] - x0;
-        s_list[2 * tid + 1] = list[1] - x1;
-    });
+    order_tile(
+        sh, k, rounds, [&](uint32_t w) { return (int)(w >> pos_bits); },
+        [&](int x0, int x1) {
+            s_list[2 * tid] = list[0] - x0;
+            s_list[2 * tid + 1] = list[1] - x1;
+        });
 #pragma unroll
     for (int q = 0; q < kR; ++q) {
         const int e = q * kRadixThreads + tid;
         if (e < t.n) {
-            const uint2 v = sh.pair[e];
-            const int d = (int)(v.x >> lo_bits);
-            ix.list[s_list[d] + e] = (int32_t)(v.y - (uint32_t)s_t0[d]);
+            const uint32_t v = sh.word[e];
+            const int d = (int)(v >> pos_bits);
+            ix.list[s_list[d] + e] = (int32_t)((v & ((1u << pos_bits) - 1u)) - (uint32_t)s_t0[d]);
         }
     }
 }
@@ -853,27 +926,18 @@ static rs_status check_index(const char *who, int B, int V, int64_t t_total, con
     return RS_OK;
 }
 
-// The sort of a build.  One pass over digit `pass` (of `bits` bits) of the keys,
-// from the tokens or from the pairs the last pass left.
-template <int kR>
-static rs_status radix_pass(const int32_t *tokens, const int64_t *tok_off, int B, int V, int vbits, int bits, int pass,
-                            long long N, const IndexView &ix, cudaStream_t st) {
-    const int shift = pass * bits, bins = 1 << bits;
+// The digit counts of a pass over the keys `src` and their offsets, then the scatter.
+template <int kR, class Keys, class Words>
+static rs_status radix_pass(const Keys &src, const Words &words, typename Words::W *out, int shift, int bins, long long N,
+                            const IndexView &ix, cudaStream_t st) {
     const long long nt = n_tiles(N);
-    const TokenKeys tk{tokens, tok_off, B, V, vbits, 0, 0};
-    const PairKeys pk{ix.pair[(pass & 1) ^ 1]};
     const dim3 grid((unsigned)nt), block(kRadixThreads);
-    if (pass == 0) launch_pdl(radix_hist<TokenKeys, kR>, grid, block, 0, st, tk, N, shift, bins, ix.hist, ix.valid);
-    else launch_pdl(radix_hist<PairKeys, kR>, grid, block, 0, st, pk, N, shift, bins, ix.hist, ix.valid);
+    launch_pdl(radix_hist<Keys, kR>, grid, block, 0, st, src, N, shift, bins, ix.hist, ix.valid);
     RS_CHECK_LAUNCH("rs_match_index_build/radix_hist");
-    launch_pdl(radix_offsets, dim3((unsigned)(bins + kOffDigits - 1) / kOffDigits), block, 0, st, ix.hist, nt, bins, ix.dtot,
+    launch_pdl(radix_offsets<kR>, dim3((unsigned)(bins + kOffDigits - 1) / kOffDigits), dim3(off_threads(kR)), 0, st, ix.hist, nt, bins, ix.dtot,
                ix.valid);
     RS_CHECK_LAUNCH("rs_match_index_build/radix_offsets");
-    if (pass == 0)
-        launch_pdl(radix_scatter<TokenKeys, kR>, grid, block, 0, st, tk, ix.pair[0], N, shift, bins, ix.hist, ix.dtot, ix.valid);
-    else
-        launch_pdl(radix_scatter<PairKeys, kR>, grid, block, 0, st, pk, ix.pair[pass & 1], N, shift, bins, ix.hist, ix.dtot,
-                   ix.valid);
+    launch_pdl(radix_scatter<Keys, kR, Words>, grid, block, 0, st, src, words, out, N, bins, ix.hist, ix.dtot, ix.valid);
     RS_CHECK_LAUNCH("rs_match_index_build/radix_scatter");
     return RS_OK;
 }
@@ -885,7 +949,12 @@ static rs_status build_plain(const int32_t *tokens, const int64_t *tok_off, int 
     const int vbits = bits_for(V), keybits = key_bits(B, V);
     const int passes = N > 0 ? (keybits + kMaxDigitBits - 1) / kMaxDigitBits : 0;
     for (int pass = 0; pass < passes; ++pass) {
-        const rs_status s = radix_pass<kR>(tokens, tok_off, B, V, vbits, (keybits + passes - 1) / passes, pass, N, ix, st);
+        const int bits = (keybits + passes - 1) / passes, shift = pass * bits, bins = 1 << bits;
+        const WholePair<kR> words{shift, bins};
+        uint2 *out = ix.pair[pass & 1];
+        const rs_status s =
+            pass == 0 ? radix_pass<kR>(TokenKeys{tokens, tok_off, B, V, vbits, 0, nullptr, 0, 0}, words, out, shift, bins, N, ix, st)
+                      : radix_pass<kR>(PairKeys{ix.pair[(pass & 1) ^ 1]}, words, out, shift, bins, N, ix, st);
         if (s != RS_OK) return s;
     }
     const uint2 *sorted = ix.pair[(passes - 1) & 1];
@@ -904,18 +973,21 @@ template <int kR>
 static rs_status build_cut(const int32_t *tokens, const int64_t *tok_off, int B, int V, long long N, const IndexView &ix,
                            cudaStream_t st) {
     const int vbits = bits_for(V), keybits = key_bits(B, V);
-    const int lo_bits = (keybits + 1) / 2, bins0 = 1 << lo_bits, bins = 1 << (keybits - lo_bits);
-    const rs_status s = radix_pass<kR>(tokens, tok_off, B, V, vbits, lo_bits, 0, N, ix, st);
+    const int lo_bits = cut_lo_bits(B, V), pos_bits = cut_pos_bits(N), bins0 = 1 << lo_bits, bins = 1 << (keybits - lo_bits);
+    uint32_t *words = reinterpret_cast<uint32_t *>(ix.pair[0]);
+    CutTile *cuts = reinterpret_cast<CutTile *>(ix.pair[1]);  // at most N / 1024 + 514 records of 16 bytes, N >= kCutMin
+    const rs_status s = radix_pass<kR>(TokenKeys{tokens, tok_off, B, V, vbits, 0, nullptr, 0, 0}, Packed<kR>{lo_bits, pos_bits}, words, 0,
+                                       bins0, N, ix, st);
     if (s != RS_OK) return s;
     const int tiles = (int)n_tiles(N) + bins0 + 1;  // the last one is never used: O past every key
     const dim3 block(kRadixThreads);
-    launch_pdl(cut_hist<kR>, dim3((unsigned)tiles), block, 0, st, ix.pair[0], bins0, lo_bits, bins, ix.dtot, ix.hist, ix.valid);
+    launch_pdl(cut_hist<kR>, dim3((unsigned)tiles), block, 0, st, words, bins0, pos_bits, bins, ix.dtot, ix.hist, cuts, ix.valid);
     RS_CHECK_LAUNCH("rs_match_index_build/cut_hist");
-    launch_pdl(radix_offsets, dim3((unsigned)(bins + kOffDigits - 1) / kOffDigits), block, 0, st, ix.hist, (long long)tiles,
+    launch_pdl(radix_offsets<kR>, dim3((unsigned)(bins + kOffDigits - 1) / kOffDigits), dim3(off_threads(kR)), 0, st, ix.hist, (long long)tiles,
         bins, ix.dtot + kMaxBins, ix.valid);
     RS_CHECK_LAUNCH("rs_match_index_build/cut_offsets");
     const unsigned firsts = (unsigned)(((long long)B * (V + 2) + kCutFirst - 1) / kCutFirst);
-    launch_pdl(cut_scatter<kR>, dim3((unsigned)tiles + firsts), block, 0, st, ix.pair[0], tiles, bins0, lo_bits, bins, ix.dtot,
+    launch_pdl(cut_scatter<kR>, dim3((unsigned)tiles + firsts), block, 0, st, words, cuts, tiles, bins0, lo_bits, pos_bits, bins, ix.dtot,
         ix.hist, tok_off, B, V, vbits, ix);
     RS_CHECK_LAUNCH("rs_match_index_build/cut_scatter");
     return RS_OK;

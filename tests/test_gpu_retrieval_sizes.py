@@ -90,11 +90,13 @@ def test_scan_cluster_forms(B):
 
 @pytest.mark.parametrize("lens,V", [([1023, 1024, 1025, 0, 1], 300), ([4096, 0, 0, 4097], 1), ([524288 - 5, 5], 70000),
                                     ([524289], 511), ([70001] * 3, 512), ([3] * 700, 1 << 18), ([262143], 40000),
-                                    ([0, 262144, 0], 40000), ([300001, 0, 280000, 3], 20000), ([9000] * 4, 1 << 17)])
+                                    ([0, 262144, 0], 40000), ([65535], 40000), ([0, 65536, 0], 40000),
+                                    ([8388608], 1 << 17), ([8388609], 1 << 17), ([300001, 0, 280000, 3], 20000), ([9000] * 4, 1 << 17)])
 def test_index_sort_edges(lens, V):
     # tiles of 1024 and 4096 keys (524288 tokens is the last total with small
-    # tiles), one to four passes, with two of them from 262144 tokens on tiles cut
-    # at the first digit, empty requests, ids that nothing holds
+    # tiles), one to four passes, with two of them from 65536 tokens on tiles cut
+    # at the first digit (as long as a key's second digit and its position, 9 and
+    # 23 bits of 8388608 tokens, fit one word), empty requests, ids that nothing holds
     rng = np.random.default_rng(len(lens) + V)
     tokens, tok_off = _buffers(rng, lens, max(V, 2), 1)  # V = 1: ids 0 and (foreign) 1
     scores = rng.random(len(tokens)).astype(np.float32)
