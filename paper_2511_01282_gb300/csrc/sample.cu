@@ -176,71 +176,57 @@ __device__ __forceinline__ float ex2f(float x) {
     return y;
 }
 
-// This thread's 32 logits of chunk c0 (ids >= V read as -inf).
-template <int kW>
-__device__ __forceinline__ void load32(const float *__restrict__ row, int V, int c0, float (&z)[kSmpVpt]) {
-    const int base = c0 + threadIdx.x * kSmpVpt;
-    if (kW >= 4 && base + kSmpVpt <= V) {
-        const float4 *p = reinterpret_cast<const float4 *>(row + base);
-#pragma unroll
-        for (int q = 0; q < kSmpVpt / 4; ++q) {
-            const float4 x = __ldg(p + q);
-            z[4 * q] = x.x;
-            z[4 * q + 1] = x.y;
-            z[4 * q + 2] = x.z;
-            z[4 * q + 3] = x.w;
-        }
-    } else {
-#pragma unroll
-        for (int j = 0; j < kSmpVpt; ++j) z[j] = base + j < V ? __ldg(row + base + j) : -INFINITY;
-    }
-}
-
-// The same 32 logits, read through shared memory: the CTA streams the chunk
-// with coalesced 128-bit loads into a buffer padded by four floats after
-// every 32 (so that neither the stores nor the per-thread 128-bit reads of 32
-// consecutive ids meet bank conflicts), then each thread takes its own ids.
-// Chunks that end past V fall back to load32.  The values are the same either
-// way, so the per-thread sums do not depend on the path.
+// This thread's 32 consecutive logits of chunk c0 (ids >= V read as -inf), through
+// shared memory: the CTA streams the chunk with coalesced loads into a buffer
+// padded by four floats after every 32 (so that neither the stores nor the
+// per-thread 128-bit reads of 32 consecutive ids meet bank conflicts), then
+// each thread takes its own ids.  A row's last chunk goes the same way, and so
+// do rows of any alignment, by single logits: with these read straight from
+// global memory, 128 bytes apart from lane to lane, a call on 145 rows of 128257
+// logits took 100 us and of 32000 (a quarter of them in last chunks) 21.0;
+// so 33.9 and 18.8.
 constexpr int kSmpPadded = kSmpChunk + kSmpChunk / 8;  // 36 floats per thread
 
 // kW: logits per streaming load (8: V % 8 == 0 and 32-byte aligned logits;
-// 4: V % 4 == 0 and 16-byte alignment; 1: no staging).
+// 4: V % 4 == 0 and 16-byte alignment; 1: any).
+// Loads past the row read the chunk's first logits again (s_buf holds those
+// there), so that one piece of code serves every chunk (145 rows of 128256
+// logits: 32.1 us, with another for the last chunks 33.9).
 template <int kW>
 __device__ __forceinline__ void load32_staged(const float *__restrict__ row, int V, int c0, float *s_buf,
                                               float (&z)[kSmpVpt]) {
-    if (kW >= 4 && c0 + kSmpChunk <= V) {  // uniform over the CTA
-        const int tid = threadIdx.x;
-        if (kW == 8) {
+    const int tid = threadIdx.x, left = V - c0;  // a multiple of kW
+    const float *chunk = row + c0;
 #pragma unroll
-            for (int j = 0; j < kSmpVpt / 8; ++j) {
-                const int e = 8 * (j * kSmpThreads + tid);  // 8 ids in one padded 32-group
-                float x[8];
-                ldg_stream8(row + c0 + e, x);
-                float4 *d = reinterpret_cast<float4 *>(s_buf + e + 4 * (e >> 5));
-                d[0] = make_float4(x[0], x[1], x[2], x[3]);
-                d[1] = make_float4(x[4], x[5], x[6], x[7]);
-            }
+    for (int j = 0; j < kSmpVpt / kW; ++j) {
+        const int e = kW * (j * kSmpThreads + tid);  // kW ids of one padded 32-group
+        const float *p = chunk + (e < left ? e : 0);
+        float *d = s_buf + e + 4 * (e >> 5);
+        if constexpr (kW == 8) {
+            float x[8];
+            ldg_stream8(p, x);
+            reinterpret_cast<float4 *>(d)[0] = make_float4(x[0], x[1], x[2], x[3]);
+            reinterpret_cast<float4 *>(d)[1] = make_float4(x[4], x[5], x[6], x[7]);
+        } else if constexpr (kW == 4) {
+            *reinterpret_cast<float4 *>(d) = ldg_stream4(reinterpret_cast<const float4 *>(p));
         } else {
-#pragma unroll
-            for (int j = 0; j < kSmpVpt / 4; ++j) {
-                const int e = 4 * (j * kSmpThreads + tid);
-                const float4 x = ldg_stream4(reinterpret_cast<const float4 *>(row + c0 + e));
-                *reinterpret_cast<float4 *>(s_buf + e + 4 * (e >> 5)) = x;
-            }
+            *d = ldg_stream(p);
         }
-        __syncthreads();
-        const float4 *p = reinterpret_cast<const float4 *>(s_buf + tid * (kSmpVpt + 4));
+    }
+    __syncthreads();
+    const float4 *p = reinterpret_cast<const float4 *>(s_buf + tid * (kSmpVpt + 4));
 #pragma unroll
-        for (int q = 0; q < kSmpVpt / 4; ++q) {
-            const float4 x = p[q];
-            z[4 * q] = x.x;
-            z[4 * q + 1] = x.y;
-            z[4 * q + 2] = x.z;
-            z[4 * q + 3] = x.w;
-        }
-    } else {
-        load32<kW>(row, V, c0, z);
+    for (int q = 0; q < kSmpVpt / 4; ++q) {
+        const float4 x = p[q];
+        z[4 * q] = x.x;
+        z[4 * q + 1] = x.y;
+        z[4 * q + 2] = x.z;
+        z[4 * q + 3] = x.w;
+    }
+    if (left < kSmpChunk) {  // uniform over the CTA
+#pragma unroll
+        for (int j = 0; j < kSmpVpt; ++j)
+            if (tid * kSmpVpt + j >= left) z[j] = -INFINITY;
     }
 }
 
@@ -262,19 +248,22 @@ __device__ __forceinline__ float block_max(float v, float *s_w) {
 __device__ __forceinline__ float term(float z, float m, float scale) { return ex2f((z - m) * scale); }
 
 __device__ __forceinline__ void thread_terms(const float (&z)[kSmpVpt], float m, float scale, float &s, float &q) {
-    float e[kSmpVpt];
-    q = 0.f;
+    // two ids an instruction (145 rows of 128256 logits: 32.3 -> 31.6 us)
+    float2 e[kSmpVpt / 2], nq{0.f, 0.f};
+    const float2 nm{-m, -m}, sc{scale, scale};
 #pragma unroll
-    for (int j = 0; j < kSmpVpt; ++j) {
-        const float x = (z[j] - m) * scale;
-        e[j] = ex2f(x);
-        q = fmaf(e[j], fminf(-x, 3.0e38f), q);  // x <= 0; z = -inf gives e = 0 (and a finite factor)
+    for (int j = 0; j < kSmpVpt / 2; ++j) {
+        const float2 x = mul2(add2(float2{z[2 * j], z[2 * j + 1]}, nm), sc);
+        e[j] = float2{ex2f(x.x), ex2f(x.y)};
+        // x <= 0; z = -inf gives e = 0 (and a finite factor)
+        nq = fma2(e[j], float2{fmaxf(x.x, -3.0e38f), fmaxf(x.y, -3.0e38f)}, nq);
     }
+    q = -(nq.x + nq.y);
 #pragma unroll
-    for (int w = 1; w < kSmpVpt; w <<= 1)
+    for (int w = 1; w < kSmpVpt / 2; w <<= 1)
 #pragma unroll
-        for (int j = 0; j < kSmpVpt; j += 2 * w) e[j] += e[j + w];
-    s = e[0];
+        for (int j = 0; j < kSmpVpt / 2; j += 2 * w) e[j] = add2(e[j], e[j + w]);
+    s = e[0].x + e[0].y;
 }
 
 __device__ __forceinline__ double warp_incl_scan_d(double v) {
@@ -505,7 +494,6 @@ sample_pick(const float *__restrict__ logits, int V, int nchunks, float scale, f
         return;
     }
     const int c = d.chunk;
-    const bool staged = kW >= 4 && c * kSmpChunk + kSmpChunk <= V;
     float z[kSmpVpt];
     load32_staged<kW>(row, V, c * kSmpChunk, s_buf, z);
     const float m = d.mc;
@@ -542,13 +530,12 @@ sample_pick(const float *__restrict__ logits, int V, int nchunks, float scale, f
     const DF ex = df_add_f(s_wo[warp], xe);
     const int h = block_first(s > 0.f && df_gt(df_add_f(ex, s), d.tl), &s_i);
     if (h != INT_MAX && warp == (h >> 5)) {
-        // the holder's 32 ids, one per lane (from the staged chunk, or the
-        // row), scanned in fp32 (depth 5); the draw's two margins in
-        // double-float
+        // the holder's 32 ids, one per lane (from the staged chunk), scanned
+        // in fp32 (depth 5); the draw's two margins in double-float
         const DF ntl = df_neg(d.tl);
         const DF exh = shfl_df(ex, h & 31);
         const int base = c * kSmpChunk + h * kSmpVpt;
-        const float zl = staged ? s_buf[h * (kSmpVpt + 4) + lane] : base + lane < V ? row[base + lane] : -INFINITY;
+        const float zl = base + lane < V ? s_buf[h * (kSmpVpt + 4) + lane] : -INFINITY;
         float loc = term(zl, m, scale);
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
