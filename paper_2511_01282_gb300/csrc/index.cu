@@ -56,7 +56,7 @@
 // Query: the candidates (the key's last token's bucket, the overflow list,
 // then the tail) are tested by one cluster per request as match.cuh
 // describes (70K candidates for a text's most common token: 79-120 us with one
-// CTA, 10.8 so; a handful: 10.4 -> 8.8, the chain of reads).
+// CTA, 9.2 so; a handful 5.7, the chain of reads).
 #include "match.cuh"
 
 #include <algorithm>
@@ -832,6 +832,7 @@ struct ListSource {
     static constexpr int kRows = 2;
     static constexpr int kWideRows = 128;  // 16384 candidates, each a read of its own
     static constexpr bool kLaneMajor = false;
+    static constexpr bool kBound = false;  // (its code, 16 registers more, costs every query 0.4 us)
     const int32_t *blist, *olist;
     int nb, no, ncand, tail0;
     __device__ __forceinline__ int cand(int c) const {

@@ -37,6 +37,7 @@ constexpr int kMatFewB = 4, kMatMidB = 8;
 constexpr int kMatThreads = 512;          // or half of it
 constexpr int kMatWarps = kMatThreads / 32;
 constexpr int kMatCand = 512;             // matches ranked from the shared buffer
+constexpr int kMatRankAll = 64;           // of which so many at once
 constexpr int kMatBitRows = 2048;         // rows whose ballots a CTA keeps (262144 candidates)
 constexpr size_t kMatSmem = (size_t)kMatBitRows * 4 * sizeof(uint32_t);
 
@@ -56,6 +57,8 @@ __device__ __forceinline__ int sp_rank(float s, int p, const float *cs, const in
 struct MatShared {
     float cs[kMatCand];  // matches with S >= theta_score (first kMatCand)
     int cp[kMatCand];
+    float gs[kMatCand / 32 * RS_MAX_TOPC];  // the best of every 32 of them
+    int gp[kMatCand / 32 * RS_MAX_TOPC];
     int ccnt;
     int warp_sums[kMatWarps];
     float wv[kMatWarps];
@@ -180,7 +183,7 @@ __device__ __forceinline__ void mat_block_best(float hv, int hp, MatShared &sh, 
 
 // The tests of a source's rows [r0, r0 + kRows) by one warp: this lane's hits,
 // bit 4 u + e for element e of row r0 + u; rows at or past `end` give none.
-// The warp's ballots go to bits[4 (r0 - base) ..] (rows below cap only).
+// The warp's ballots go to bits[4 (r0 - base) ..] (rows below `end` and the kept ones only).
 template <class Src>
 __device__ __forceinline__ uint32_t mat_rows(const Src &src, const MatReq &q, int r0, int end, uint32_t *bits,
                                              int base) {
@@ -192,7 +195,7 @@ __device__ __forceinline__ uint32_t mat_rows(const Src &src, const MatReq &q, in
         const uint32_t bal = __ballot_sync(0xffffffffu, (hits >> j) & 1u);
         mine = lane == j ? bal : mine;
     }
-    if (lane < 4 * Src::kRows && r0 - base + (lane >> 2) < kMatBitRows) bits[4 * (r0 - base) + lane] = mine;
+    if (lane < 4 * Src::kRows && r0 + (lane >> 2) < end && r0 - base + (lane >> 2) < kMatBitRows) bits[4 * (r0 - base) + lane] = mine;
     return hits;
 }
 
@@ -207,29 +210,74 @@ __device__ __noinline__ void mat_again(Src src, MatReq q, int w0, int nr, uint32
     __syncthreads();
 }
 
-// Calls f(position) for the matches of rows [a, z) of the kept ballots, in
-// order; w0: the row the ballots start at.  Stops when f returns false.
-template <class Src, class F>
-__device__ __forceinline__ void mat_each(const Src &src, const uint32_t *bits, int w0, int a, int z, F f) {
-    for (int r = a; r < z; ++r) {
-        const uint4 w = *reinterpret_cast<const uint4 *>(bits + 4 * r);
-        if (Src::kLaneMajor) {
-            uint32_t any = w.x | w.y | w.z | w.w;
-            while (any) {
-                const int l = __ffs(any) - 1;
-                any &= any - 1;
-                uint32_t es = ((w.x >> l) & 1u) | ((w.y >> l) & 1u) << 1 | ((w.z >> l) & 1u) << 2 | ((w.w >> l) & 1u) << 3;
-                for (; es; es &= es - 1)
-                    if (!f(src.pos(w0 + r, l, __ffs(es) - 1))) return;
-            }
-        } else {
-#pragma unroll 1
-            for (int e = 0; e < 4; ++e) {
-                uint32_t we = e == 0 ? w.x : e == 1 ? w.y : e == 2 ? w.z : w.w;
-                for (; we; we &= we - 1)
-                    if (!f(src.pos(w0 + r, __ffs(we) - 1, e))) return;
-            }
+// Calls use(idx, position, load(position)) for the matches of rows [a, z) of the
+// kept ballots (by one warp), idx counting them in order from `base`, below `cap`;
+// w0: the row the ballots start at.  32 rows at a time, either a lane per row (few matches in
+// each: every row's first at once) or row by row with all lanes (many: a
+// row's matches at once), whichever takes fewer steps, as each may wait for a
+// read: 999 positions of one token in a list took 57 us a lane per row, 12 so.
+template <class Src, class L, class U>
+__device__ __forceinline__ void mat_each(const Src &src, const uint32_t *bits, int w0, int a, int z, int base, int cap,
+                                         L load, U use) {
+    auto f = [&](int idx, int p) { use(idx, p, load(p)); };
+    const int lane = threadIdx.x & 31;
+    const uint32_t lt = (1u << lane) - 1u;
+    for (int c0 = a; c0 < z && base < cap; c0 += 32) {
+        const int own = c0 + lane;
+        uint4 w = make_uint4(0u, 0u, 0u, 0u);
+        if (own < z) w = *reinterpret_cast<const uint4 *>(bits + 4 * own);
+        const int n = __popc(w.x) + __popc(w.y) + __popc(w.z) + __popc(w.w);
+        int incl = n;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
         }
+        int idx = base + incl - n;
+        base += __shfl_sync(0xffffffffu, incl, 31);
+        uint32_t rows = __ballot_sync(0xffffffffu, n > 0 && idx < cap);
+        if (__reduce_max_sync(0xffffffffu, (unsigned)n) <= (unsigned)__popc(rows)) {
+            if (Src::kLaneMajor) {
+                uint32_t any = w.x | w.y | w.z | w.w;
+                for (; any && idx < cap; any &= any - 1) {
+                    const int l = __ffs(any) - 1;
+                    uint32_t es =
+                        ((w.x >> l) & 1u) | ((w.y >> l) & 1u) << 1 | ((w.z >> l) & 1u) << 2 | ((w.w >> l) & 1u) << 3;
+                    for (; es && idx < cap; es &= es - 1) f(idx++, src.pos(w0 + own, l, __ffs(es) - 1));
+                }
+            } else {
+#pragma unroll 1
+                for (int e = 0; e < 4; ++e) {
+                    uint32_t we = e == 0 ? w.x : e == 1 ? w.y : e == 2 ? w.z : w.w;
+                    for (; we && idx < cap; we &= we - 1) f(idx++, src.pos(w0 + own, __ffs(we) - 1, e));
+                }
+            }
+            __syncwarp();
+            continue;
+        }
+        for (; rows; rows &= rows - 1) {
+            const int q = __ffs(rows) - 1, r = c0 + q;
+            const uint4 v = *reinterpret_cast<const uint4 *>(bits + 4 * r);
+            const uint32_t we[4] = {v.x, v.y, v.z, v.w};
+            int at = __shfl_sync(0xffffffffu, idx, q);
+            if (Src::kLaneMajor) at += __popc(v.x & lt) + __popc(v.y & lt) + __popc(v.z & lt) + __popc(v.w & lt);
+            int p[4], k[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const bool hit = (we[e] >> lane) & 1u;
+                k[e] = Src::kLaneMajor ? at : at + __popc(we[e] & lt);
+                at += Src::kLaneMajor ? (int)hit : __popc(we[e]);
+                if (!hit) k[e] = cap;
+                p[e] = hit ? src.pos(w0 + r, lane, e) : 0;
+            }
+            float s[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) s[e] = k[e] < cap ? load(p[e]) : 0.f;
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (k[e] < cap) use(k[e], p[e], s[e]);
+        }
+        __syncwarp();
     }
 }
 
@@ -240,7 +288,7 @@ __device__ __forceinline__ void mat_body(const Src &src, const MatReq &q, int ro
                                          MatShared &sh, uint32_t *bits, const MatOut &o) {
     namespace cg = cooperative_groups;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int nthreads = blockDim.x, stride = (nthreads >> 5) * Src::kRows;  // rows a round of the CTA's warps
+    const int nthreads = blockDim.x;
     const int top_c = o.top_c, pos_cap = o.pos_cap;
     const bool solo = nc == 1;
     if (!solo) cluster_arrive_relaxed();  // this CTA runs; the wait sits before the first push
@@ -250,40 +298,109 @@ __device__ __forceinline__ void mat_body(const Src &src, const MatReq &q, int ro
     __syncthreads();
 
     // ---- every candidate once: ballots, count, the matches that clear theta ----
+    // (consecutive rows per warp, as the positions are written)
+    const int mr = (hi - lo + (nthreads >> 5) - 1) / (nthreads >> 5);
+    const int wa = min(lo + warp * mr, hi), wz = min(wa + mr, hi);
     int cnt = 0;
-    for (int r0 = lo + warp * Src::kRows; r0 < hi; r0 += stride) {
-        uint32_t rem = mat_rows(src, q, r0, hi, bits, lo);
-        cnt += __popc(rem);
-        while (rem) {
-            const int j = __ffs(rem) - 1;
-            rem &= rem - 1;
-            const int p = src.pos(r0 + (j >> 2), lane, j & 3);
-            const float s = q.S[p];
-            if (!(s >= o.theta_score)) continue;
-            const int slot = atomicAdd(&sh.ccnt, 1);
-            if (slot < kMatCand) {
-                sh.cs[slot] = s;
-                sh.cp[slot] = p;
+    for (int r0 = wa; r0 < wz; r0 += Src::kRows) {
+        const uint32_t hits = mat_rows(src, q, r0, wz, bits, lo);
+        cnt += __popc(hits);
+        // their scores, four of each lane at once; one slot count per warp and
+        // round.  Once the buffer has run over, its contents count no more
+        for (uint32_t rem = hits;;) {
+            const bool over = *(volatile int *)&sh.ccnt > kMatCand;
+            if (!__any_sync(0xffffffffu, rem != 0 && !over)) break;
+            int p[4], at[4], n = 0;
+            float s[4];
+            bool pass[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int j = __ffs(rem) - 1;
+                p[e] = rem ? src.pos(r0 + (j >> 2), lane, j & 3) : -1;
+                s[e] = rem ? q.S[p[e]] : 0.f;
+                rem &= rem - 1;
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                pass[e] = p[e] >= 0 && s[e] >= o.theta_score;
+                const uint32_t bal = __ballot_sync(0xffffffffu, pass[e]);
+                at[e] = n + __popc(bal & ((1u << lane) - 1u));
+                n += __popc(bal);
+            }
+            if (n == 0) continue;
+            int slot = 0;
+            if (lane == 0) slot = atomicAdd(&sh.ccnt, n);
+            slot = __shfl_sync(0xffffffffu, slot, 0);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                if (pass[e] && slot + at[e] < kMatCand) {
+                    sh.cs[slot + at[e]] = s[e];
+                    sh.cp[slot + at[e]] = p[e];
+                }
             }
         }
     }
-    int cta_total = 0;
-    (void)mat_excl_scan(cnt, sh, &cta_total);
+    cnt = (int)__reduce_add_sync(0xffffffffu, (unsigned)cnt);
+    if (lane == 0) sh.warp_sums[warp] = cnt;
+    __syncthreads();
+    int cta_total = 0, before = 0;  // before: the matches of the earlier warps
+#pragma unroll
+    for (int w = 0; w < kMatWarps; ++w) {
+        const int y = w < (nthreads >> 5) ? sh.warp_sums[w] : 0;
+        before += w < warp ? y : 0;
+        cta_total += y;
+    }
     // the CTA's best top_c: rank every buffered match by counting
     const int ncand = sh.ccnt;
+    const bool over = ncand > kMatCand;
     bool kept = true;  // the ballots are still those of [lo, lo + kMatBitRows)
-    if (ncand <= kMatCand) {
-        for (int e = tid; e < ncand; e += nthreads) {
-            const float sv = sh.cs[e];
-            const int pv = sh.cp[e];
-            const int r = sp_rank(sv, pv, sh.cs, sh.cp, ncand);
+    if (!over || Src::kBound) {
+        const float *cs = sh.cs;
+        const int *cp = sh.cp;
+        int n = Src::kBound ? min(ncand, kMatCand) : ncand;
+        if (n > kMatRankAll) {
+            // the best top_c of every 32 first (300 matches of a list: 12.5 us with
+            // all ranked against each other, 9.3 so)
+            for (int g = warp; g * 32 < n; g += nthreads >> 5) {
+                const int e = g * 32 + lane;
+                const float sv = e < n ? cs[e] : -INFINITY;
+                const int pv = e < n ? cp[e] : -1 - lane;  // after every match
+                int r = 0;
+#pragma unroll 8
+                for (int i = 0; i < 32; ++i)
+                    r += sp_before(__shfl_sync(0xffffffffu, sv, i), __shfl_sync(0xffffffffu, pv, i), sv, pv);
+                if (r < top_c) {
+                    sh.gs[g * top_c + r] = sv;
+                    sh.gp[g * top_c + r] = pv;
+                }
+            }
+            __syncthreads();
+            n = (n + 31) / 32 * top_c;
+            cs = sh.gs;
+            cp = sh.gp;
+        }
+        for (int e = tid; e < n; e += nthreads) {
+            const float sv = cs[e];
+            const int pv = cp[e];
+            const int r = sp_rank(sv, pv, cs, cp, n);
             if (r < top_c) {
                 sh.top_s[r] = sv;
                 sh.top_p[r] = pv;
             }
         }
         if (tid == 0) sh.ntop = ncand < top_c ? ncand : top_c;
-    } else {  // more than the buffer holds: every thread's best of its rows, then the block's best of those
+    }
+    if (over) {  // more than the buffer holds: every thread's best of its rows, then the block's best of those
+        // kBound: only those not behind the best top_c of the buffer (read
+        // before the first of these is replaced, behind a barrier): 16 x 300000
+        // positions, half of them matches, 98.5 -> 58.7 us
+        float ts = -INFINITY;
+        int tp = -1;
+        if (Src::kBound) {
+            __syncthreads();
+            ts = sh.top_s[top_c - 1];
+            tp = sh.top_p[top_c - 1];
+        }
         float ls[RS_MAX_TOPC];
         int lp[RS_MAX_TOPC];
 #pragma unroll
@@ -297,11 +414,11 @@ __device__ __forceinline__ void mat_body(const Src &src, const MatReq &q, int ro
                 mat_again(src, q, w0, nr, bits);
                 kept = false;
             }
-            const int mr = (nr + nthreads - 1) / nthreads;
-            const int a = min(tid * mr, nr), z = min(a + mr, nr);
-            mat_each(src, bits, w0, a, z, [&](int p) {
-                const float s = q.S[p];
-                if (s >= o.theta_score && sp_before(s, p, ls[RS_MAX_TOPC - 1], lp[RS_MAX_TOPC - 1])) {
+            const int per_warp = (nr + (nthreads >> 5) - 1) / (nthreads >> 5);
+            const int a = min(warp * per_warp, nr), z = min(a + per_warp, nr);
+            mat_each(src, bits, w0, a, z, 0, 0x7fffffff, [&](int p) { return q.S[p]; },
+                     [&](int, int p, float s) {
+                if (s >= o.theta_score && !(Src::kBound && sp_before(ts, tp, s, p)) && sp_before(s, p, ls[RS_MAX_TOPC - 1], lp[RS_MAX_TOPC - 1])) {
                     float cs = s;
                     int cp = p;
 #pragma unroll
@@ -316,7 +433,6 @@ __device__ __forceinline__ void mat_body(const Src &src, const MatReq &q, int ro
                         }
                     }
                 }
-                return true;
             });
         }
         int ntop = 0;
@@ -366,26 +482,28 @@ __device__ __forceinline__ void mat_body(const Src &src, const MatReq &q, int ro
     }
 
     // ---- positions in ascending order ----
-    int base = offset;
     int32_t *pos = o.pos + (long long)b * pos_cap;
-    for (int w0 = lo; w0 < hi && base < pos_cap; w0 += kMatBitRows) {
-        const int nr = min(hi - w0, kMatBitRows);
-        if (w0 != lo || !kept) mat_again(src, q, w0, nr, bits);
-        const int mr = (nr + nthreads - 1) / nthreads;  // consecutive rows per thread
-        const int a = min(tid * mr, nr), z = min(a + mr, nr);
-        int n = 0;
-        for (int r = a; r < z; ++r) {
-            const uint4 w = *reinterpret_cast<const uint4 *>(bits + 4 * r);
-            n += __popc(w.x) + __popc(w.y) + __popc(w.z) + __popc(w.w);
+    auto none = [](int) { return 0.f; };
+    auto put = [&](int i, int p, float) { pos[i] = p; };
+    if (kept && hi - lo <= kMatBitRows) {
+        mat_each(src, bits, lo, wa - lo, wz - lo, offset + before, pos_cap, none, put);
+    } else {
+        int base = offset;
+        for (int w0 = lo; w0 < hi && base < pos_cap; w0 += kMatBitRows) {
+            const int nr = min(hi - w0, kMatBitRows);
+            if (w0 != lo || !kept) mat_again(src, q, w0, nr, bits);
+            const int per_warp = (nr + (nthreads >> 5) - 1) / (nthreads >> 5);
+            const int a = min(warp * per_warp, nr), z = min(a + per_warp, nr);
+            int n = 0;
+            for (int r = a + lane; r < z; r += 32) {
+                const uint4 w = *reinterpret_cast<const uint4 *>(bits + 4 * r);
+                n += __popc(w.x) + __popc(w.y) + __popc(w.z) + __popc(w.w);
+            }
+            int wtotal = 0;
+            const int idx = __shfl_sync(0xffffffffu, base + mat_excl_scan(n, sh, &wtotal), 0);
+            mat_each(src, bits, w0, a, z, idx, pos_cap, none, put);
+            base += wtotal;
         }
-        int wtotal = 0;
-        int idx = base + mat_excl_scan(n, sh, &wtotal);
-        if (n && idx < pos_cap)
-            mat_each(src, bits, w0, a, z, [&](int p) {
-                pos[idx] = p;
-                return ++idx < pos_cap;
-            });
-        base += wtotal;
     }
     if (crank != 0) return;
 

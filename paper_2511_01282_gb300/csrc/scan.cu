@@ -3,24 +3,28 @@
 //
 // One cluster of CTAs per request; match.cuh has the split, the ranks and
 // the selection.  The candidates are the buffer's positions, as quads of four
-// tokens on 16-byte boundaries: a lane reads eight quads (one 128-bit load
+// tokens on 16-byte boundaries: a lane reads four quads (one 128-bit load
 // each, all in flight), compares the last token of the key, filters on the
 // one before it from its neighbour's register, and only what is left reads
 // the other key tokens and, if it matches, its score.  Nothing is staged in
 // shared memory and nothing is read twice.  Staging 8192-position windows of
 // tokens and scores (4-byte asynchronous copies, a second staging for the
 // positions) took 51 us on 4 x 262144 tokens of text, a key of two; this takes
-// 10.2 (graph), the reads of 32 SMs at 4 MB and the dependent rounds around
-// them.  2048 tokens take as long as they did (7 us cold, all latency).
+// 8.4 (graph), the reads of 32 SMs at 4 MB and the dependent rounds around
+// them.  The shortest calls of one to four requests pay for the larger cluster:
+// 2000 tokens 5.7 us, 4.6 before; of 16 requests 4.0, 4.7 before.
 #include "match.cuh"
 
 namespace rs {
 namespace {
 
 struct ScanSource {
-    static constexpr int kRows = 8;
+    // (eight rows: 2 x 1.3M tokens 17.6 us instead of 18.8, but every call of a
+    // round or two 1.2 us longer)
+    static constexpr int kRows = 4;
     static constexpr int kWideRows = 1024;  // 131072 positions: below, 8 CTAs are as fast as 16
     static constexpr bool kLaneMajor = true;
+    static constexpr bool kBound = true;
     int al;       // positions of the buffer start past a 16-byte boundary
     __device__ __forceinline__ int pos(int row, int lane, int e) const {
         return 4 * (32 * row + lane) + e - al;
@@ -30,44 +34,42 @@ struct ScanSource {
         const int pb = 128 * r0 + 4 * lane - al;  // this lane's first position; row u's at pb + 128 u
         const int rows = min(end - r0, kRows);
         int4 x[kRows];
-        uint32_t edge = 0;  // rows whose quad reaches past an end of the buffer
 #pragma unroll
         for (int u = 0; u < kRows; ++u) {
             const int p0 = pb + 128 * u;
             x[u] = make_int4(0, 0, 0, 0);
             if (u < rows && p0 < t) {
-                if (p0 >= 0 && p0 < t - 3) x[u] = *reinterpret_cast<const int4 *>(q.X + p0);
-                else edge |= 1u << u;
+                if (p0 >= 0 && p0 < t - 3) {
+                    x[u] = *reinterpret_cast<const int4 *>(q.X + p0);
+                } else {  // the quad reaches past an end of the buffer
+                    if (p0 >= 0) x[u].x = q.X[p0];
+                    if (p0 + 1 >= 0 && p0 + 1 < t) x[u].y = q.X[p0 + 1];
+                    if (p0 + 2 >= 0 && p0 + 2 < t) x[u].z = q.X[p0 + 2];
+                    if (p0 + 3 < t) x[u].w = q.X[p0 + 3];
+                }
             }
         }
         const int kl = q.k1, k2 = q.k2;
         const bool one = q.k < 2;
-        // the token before the quad is a neighbour's, unless this is lane 0 or
-        // the neighbour's quad was not loaded (it starts before the buffer)
-        const bool alone = lane == 0 || pb < 4;
         uint32_t hits = 0;
 #pragma unroll
         for (int u = 0; u < kRows; ++u) {
             const int before = __shfl_up_sync(0xffffffffu, x[u].w, 1);
-            const bool m0 = x[u].x == kl && (one || alone || before == k2);
+            const bool m0 = x[u].x == kl && (one || lane == 0 || before == k2);  // lane 0: not in a register
             const bool m1 = x[u].y == kl && (one || x[u].x == k2);
             const bool m2 = x[u].z == kl && (one || x[u].y == k2);
             const bool m3 = x[u].w == kl && (one || x[u].z == k2);
             hits |= ((m0 ? 1u : 0u) | (m1 ? 2u : 0u) | (m2 ? 4u : 0u) | (m3 ? 8u : 0u)) << (4 * u);
         }
-        // what is left is checked one by one: quads that were not loaded (all
-        // four positions), the range of matches (k - 1 .. t - 2), the key
-        // tokens the registers did not show
-        uint32_t rem = 0;
-        for (uint32_t m = edge; m; m &= m - 1) rem |= 0xfu << (4 * (__ffs(m) - 1));
-        hits &= ~rem;
-        for (rem |= hits; rem; rem &= rem - 1) {
+        // what is left is checked one by one: the range of matches (k - 1 ..
+        // t - 2), which the positions not loaded miss, and the key tokens the
+        // registers did not show
+        for (uint32_t rem = hits; rem; rem &= rem - 1) {
             const int j = __ffs(rem) - 1;
             const int p = pb + 128 * (j >> 2) + (j & 3);
             bool ok = (j >> 2) < rows && p >= q.k - 1 && p <= t - 2;
-            if (ok && ((edge >> (j >> 2)) & 1u)) ok = q.X[p] == kl && (one || mat_prefix(q, p));
-            else if (ok && !(one || (q.k == 2 && !(alone && (j & 3) == 0)))) ok = mat_prefix(q, p);
-            hits = ok ? hits | (1u << j) : hits & ~(1u << j);
+            if (ok && !(one || (q.k == 2 && (lane != 0 || (j & 3) != 0)))) ok = mat_prefix(q, p);
+            if (!ok) hits &= ~(1u << j);
         }
         return hits;
     }

@@ -51,10 +51,10 @@ def _scan(tokens, tok_off, ks, scores, theta, top_c, span_len, pos_cap):
 @pytest.mark.parametrize("k", [1, 2, 3, 8])
 @pytest.mark.parametrize("V", [3, 400])
 def test_scan_alignments_and_round_edges(k, V):
-    # request lengths of 1 mod 4 walk through every alignment; 8192 candidate
-    # positions (16384 in calls of few requests) are the most one CTA takes alone
+    # request lengths of 1 mod 4 walk through every alignment; 4096 candidate
+    # positions (8192 in calls of few requests) are the most one CTA takes alone
     rng = np.random.default_rng(100 * k + V)
-    lens = [1, 5, 129, 8185, 16381, 8197, 16389, 33, 8193, 17, 20001]
+    lens = [1, 5, 129, 8185, 16381, 8197, 16389, 33, 8193, 17, 20001, 4089, 4097, 4101]
     tokens, tok_off = _buffers(rng, lens, V, k)
     scores = rng.random(len(tokens)).astype(np.float32)
     scores[rng.random(len(tokens)) < 0.2] = 0.5
@@ -147,3 +147,26 @@ def test_append_of_one_warp_and_more(n):
     fill = 4096 + 2 - len(bufs[1]) - n // 2
     assert grow([[], np.full(fill, 3), []]) == [0, 0, 0]
     assert grow([[1], np.full(n, 3), []]) == [0, rs.RS_ST_TRUNCATED, 0]
+
+
+@pytest.mark.parametrize("form", ["scan", "index"])
+@pytest.mark.parametrize("B", [2, 9])
+@pytest.mark.parametrize("share", [0.02, 0.12, 0.7])
+def test_many_matches(form, B, share):
+    # rows of 128 candidates with few and with many matches (a lane per row, then
+    # row by row), more matches than are ranked at once (64), than a CTA's
+    # buffer holds (512), equal scores among them, and a capacity inside a row
+    rng = np.random.default_rng(int(100 * share) + B)
+    lens = rng.choice([300, 3000, 9000, 40001], B).tolist()
+    lens[0] = 40001
+    tokens, tok_off = _buffers(rng, lens, 500, 1)
+    tokens[rng.random(len(tokens)) < share] = 7
+    tokens[tok_off[1:] - 1] = 7
+    scores = rng.random(len(tokens)).astype(np.float32)
+    scores[tok_off[1]:] = np.where(rng.random(len(tokens) - tok_off[1]) < 0.5, 0.75, scores[tok_off[1]:])
+    ks = np.ones(B, np.int32)
+    for pos_cap, theta in ((130, 0.3), (5000, 0.9)):
+        if form == "scan":
+            _scan(tokens, tok_off, ks, scores, theta, 5, 8, pos_cap)
+        else:
+            compare(tokens, tok_off, ks, None, scores, theta, 5, 8, pos_cap, 500)
