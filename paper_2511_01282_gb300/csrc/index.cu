@@ -262,11 +262,14 @@ __device__ __forceinline__ int radix_excl_scan(int v, int *s_w, int *total) {
 // its total.  A block takes eight digits (one 32-byte sector of a tile's
 // counts); thread (group g, digit d) takes kT consecutive tiles a round, four
 // groups to a warp.
-// Threads: one round for 1024 tiles of 4096 keys (4 x 1M tokens: 65.7 us for the
-// whole build, 68.8 with 1024 threads) or 128 of 1024 (4 x 32K tokens: 28.4,
-// 29.9 with 1024; 4096 tokens: 19.0 and 21.4).
+// Two sizes: up to kOffFew tiles in one round of 256 threads (4096 tokens: 19.0 us
+// for the whole build, 21.4 with 1024 threads), more in rounds of 1024 tiles by
+// 512 threads (4 x 1M tokens: 65.7 us, 68.8 with 1024 threads; 8 x 60K tokens 31.7,
+// 34.6 in rounds of 128).
 constexpr int kOffDigits = 8;
-constexpr int off_threads(int rounds) { return rounds == kTileRounds ? 512 : 256; }
+constexpr int kOffManyT = 16, kOffFewT = 4, kOffFew = 128;
+constexpr int off_threads(int per_thread) { return per_thread == kOffManyT ? 512 : 256; }
+static_assert(kOffFew == off_threads(kOffFewT) / kOffDigits * kOffFewT, "one round");
 template <int kT>
 __global__ void __launch_bounds__(off_threads(kT))
 radix_offsets(int32_t *__restrict__ hist, long long ntiles, int bins, int32_t *__restrict__ dtot,
@@ -927,6 +930,15 @@ static rs_status check_index(const char *who, int B, int V, int64_t t_total, con
     return RS_OK;
 }
 
+static void radix_offsets_launch(int32_t *hist, long long ntiles, int bins, int32_t *dtot, const int32_t *valid,
+                                 cudaStream_t st) {
+    const dim3 grid((unsigned)(bins + kOffDigits - 1) / kOffDigits);
+    if (ntiles <= kOffFew)
+        launch_pdl(radix_offsets<kOffFewT>, grid, dim3(off_threads(kOffFewT)), 0, st, hist, ntiles, bins, dtot, valid);
+    else
+        launch_pdl(radix_offsets<kOffManyT>, grid, dim3(off_threads(kOffManyT)), 0, st, hist, ntiles, bins, dtot, valid);
+}
+
 // The digit counts of a pass over the keys `src` and their offsets, then the scatter.
 template <int kR, class Keys, class Words>
 static rs_status radix_pass(const Keys &src, const Words &words, typename Words::W *out, int shift, int bins, long long N,
@@ -935,8 +947,7 @@ static rs_status radix_pass(const Keys &src, const Words &words, typename Words:
     const dim3 grid((unsigned)nt), block(kRadixThreads);
     launch_pdl(radix_hist<Keys, kR>, grid, block, 0, st, src, N, shift, bins, ix.hist, ix.valid);
     RS_CHECK_LAUNCH("rs_match_index_build/radix_hist");
-    launch_pdl(radix_offsets<kR>, dim3((unsigned)(bins + kOffDigits - 1) / kOffDigits), dim3(off_threads(kR)), 0, st, ix.hist, nt, bins, ix.dtot,
-               ix.valid);
+    radix_offsets_launch(ix.hist, nt, bins, ix.dtot, ix.valid, st);
     RS_CHECK_LAUNCH("rs_match_index_build/radix_offsets");
     launch_pdl(radix_scatter<Keys, kR, Words>, grid, block, 0, st, src, words, out, N, bins, ix.hist, ix.dtot, ix.valid);
     RS_CHECK_LAUNCH("rs_match_index_build/radix_scatter");
@@ -984,8 +995,7 @@ static rs_status build_cut(const int32_t *tokens, const int64_t *tok_off, int B,
     const dim3 block(kRadixThreads);
     launch_pdl(cut_hist<kR>, dim3((unsigned)tiles), block, 0, st, words, bins0, pos_bits, bins, ix.dtot, ix.hist, cuts, ix.valid);
     RS_CHECK_LAUNCH("rs_match_index_build/cut_hist");
-    launch_pdl(radix_offsets<kR>, dim3((unsigned)(bins + kOffDigits - 1) / kOffDigits), dim3(off_threads(kR)), 0, st, ix.hist, (long long)tiles,
-        bins, ix.dtot + kMaxBins, ix.valid);
+    radix_offsets_launch(ix.hist, (long long)tiles, bins, ix.dtot + kMaxBins, ix.valid, st);
     RS_CHECK_LAUNCH("rs_match_index_build/cut_offsets");
     const unsigned firsts = (unsigned)(((long long)B * (V + 2) + kCutFirst - 1) / kCutFirst);
     launch_pdl(cut_scatter<kR>, dim3((unsigned)tiles + firsts), block, 0, st, words, cuts, tiles, bins0, lo_bits, pos_bits, bins, ix.dtot,
