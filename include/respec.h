@@ -350,7 +350,7 @@ rs_status rs_accept(const float *logits, int R, int V, const int32_t *node_off, 
  * rs_match_scan_indexed: rs_match_scan's inputs, outputs and meaning, plus
  *   V, t_total (as given to the build) and the index.  Positions the index
  *   does not hold (appended without rs_match_index_append, or left out as
- *   above) are tested one by one.  One CTA per request.
+ *   above) are tested one by one.  One cluster of CTAs per request.
  */
 size_t rs_match_index_bytes(int B, int V, int64_t t_total);
 rs_status rs_match_index_build(const int32_t *tokens, const int64_t *tok_off, int B, int V, int64_t t_total,

@@ -16,7 +16,8 @@
 //   attn_prep validates each tree and builds a 256-bit ancestor set per
 //   node; the tree part of the mask is a bit test on it.
 // Launches: attn_prep (B CTAs) -> attn_tc_kernel (one CTA per SM; see
-// attn_core.cuh) -> attn_combine (three CTAs per SM over the split segments' rows).
+// attn_core.cuh) or attn_pair_kernel (attn_pair.cuh) -> attn_combine (three
+// CTAs per SM over the work items that the attention CTAs wrote).
 #include <cudaTypedefs.h>
 #include <math.h>
 

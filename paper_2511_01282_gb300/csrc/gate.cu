@@ -8,10 +8,11 @@
 // chunk's.  Row entropy is then H = ln s - w / s for the merged triple (the
 // log-sum-exp form of -sum p ln p).
 // Kernel 2 (entropy_merge): one warp per row merges its chunk triples into
-// the row entropy (rows of one chunk need no merge: kernel 1 writes theirs).  Kernel 3 (gate_push): one CTA per request pushes the
-// committed rows' entropies into the history and evaluates H_k, C_k, k* and
-// the trigger in fp64.  rs_entropy_gate_rows runs kernel 3 alone on row
-// entropies that rs_accept already produced from the same logits.
+// the row entropy (rows of one chunk need no merge: kernel 1 writes theirs).
+// Kernel 3 (gate_push): one CTA per request pushes the committed rows'
+// entropies into the history and evaluates H_k, C_k, k* and the trigger in
+// fp64.  rs_entropy_gate_rows runs kernel 3 alone on row entropies that
+// rs_accept already produced from the same logits.
 #include <math.h>
 
 #include <mutex>

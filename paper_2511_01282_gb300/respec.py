@@ -1,4 +1,4 @@
-"""Thin ctypes binding of ``librespec.so`` (declared in ``include/respec.h``).
+"""Thin binding of ``librespec.so`` (declared in ``include/respec.h``).
 
 Argument marshalling only: every function here has the name and argument
 order of its C entry point, turns torch tensors into device pointers, calls
