@@ -56,7 +56,7 @@
 // Query: the candidates (the key's last token's bucket, the overflow list,
 // then the tail) are tested by one cluster per request as match.cuh
 // describes (70K candidates for a text's most common token: 79-120 us with one
-// CTA, 9.2 so; a handful 5.7, the chain of reads).
+// CTA, 9.2 so; a handful 4.6, the chain of reads).
 #include "match.cuh"
 
 #include <algorithm>
@@ -872,7 +872,7 @@ struct ListSource {
     }
 };
 
-__global__ void __launch_bounds__(kMatThreads)
+__global__ void __launch_bounds__(kMatHalf)
 index_query(const int32_t *__restrict__ tokens, const int64_t *__restrict__ tok_off, int V,
             const int32_t *__restrict__ k_star, const uint8_t *__restrict__ gate_ok,
             const float *__restrict__ scores, IndexView ix, MatOut o) {
@@ -898,7 +898,8 @@ index_query(const int32_t *__restrict__ tokens, const int64_t *__restrict__ tok_
         src.ncand = src.nb + src.no + (nt > 0 ? nt : 0);
     }
     const int rows = (src.ncand + 127) / 128;
-    const int nc = mat_ctas<ListSource>(rows);
+    q.threads = kMatHalf;
+    const int nc = mat_ctas<ListSource>(rows, q.threads);
     if (crank >= nc) return;
     mat_body(src, q, rows, nc, b, crank, sh, qry_bits, o);
 }
@@ -1061,6 +1062,6 @@ extern "C" rs_status rs_match_scan_indexed(const int32_t *tokens, const int64_t 
     carve_index(const_cast<void *>(index), B, V, t_total, &ix);
     const MatOut o{count, pos, sel_pos, sel_len, spans, n_sel, status, p.theta_score, p.top_c, p.span_len, pos_cap};
     static int attr_done[64] = {0};
-    return mat_launch("rs_match_scan_indexed", attr_done, index_query, B, (cudaStream_t)stream, tokens, tok_off, V, k_star,
+    return mat_launch("rs_match_scan_indexed", kMatHalf, attr_done, index_query, B, (cudaStream_t)stream, tokens, tok_off, V, k_star,
                       gate_ok, scores, ix, o);
 }

@@ -15,13 +15,17 @@
 // barrier nobody touches another CTA's shared memory.
 //
 // What bounds it: a chain of dependent reads (offsets, key, candidates,
-// scores, spans) of about 0.5 us each, then for long buffers the reads of one
-// request's SMs (~100 GB/s per SM), then, with many requests, the CTAs an SM
-// holds.  So calls of up to kMatFewB requests take clusters of 16 CTAs of 512
-// threads (4 x 1M tokens: 23.6 us with 8, 15.3 with 16; more of these clusters
-// than GPCs run in turn: 8 requests 23.5 and 27.4), of which a request of
-// fewer rows than its source's kWideRows uses 8; calls of up to kMatMidB requests clusters
-// of 8; larger calls clusters of 8 CTAs of 256 threads.
+// scores, spans) of about 0.5 us each and the barriers between them, then for
+// long buffers the reads of one request's SMs (~100 GB/s per SM), then, with
+// many requests, the CTAs an SM holds.  So calls of up to kMatFewB requests take
+// clusters of 16 CTAs (scans of 4 x 1M tokens: 25 us with 8, 17 with 16; more of
+// these clusters than GPCs run in turn: 8 requests 23.5 and 27.4 in an earlier form), of
+// which a request of fewer rows than its source's kWideRows uses 8; others
+// clusters of 8.  CTAs have 512 threads in the scans of up to kMatMidB requests,
+// whose reads in flight bound them (4 x 1M tokens: 17 us, 25 with 256), but
+// only 256 stay for a request of one round of these, and 256 are launched for
+// everything else: twice the warps at each barrier cost a query of 4 x 32K
+// tokens 0.7 of 5.2 us, a scan of 30000 positions 1.0 of 6.8.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -34,7 +38,7 @@ namespace rs {
 constexpr int kMatCluster = 8;
 constexpr int kMatClusterMax = 16;
 constexpr int kMatFewB = 4, kMatMidB = 8;
-constexpr int kMatThreads = 512;          // or half of it
+constexpr int kMatThreads = 512, kMatHalf = kMatThreads / 2;
 constexpr int kMatWarps = kMatThreads / 32;
 constexpr int kMatCand = 512;             // matches ranked from the shared buffer
 constexpr int kMatRankAll = 64;           // of which so many at once
@@ -88,6 +92,7 @@ struct MatReq {
     bool run;
     int key[RS_MAX_L];  // key[i] = X[t - k + i]
     int k1, k2;         // its last token, and the one before (-1: none)
+    int threads;        // of the CTA at work on it
 };
 
 // ok: the caller's own condition for reading the request (its index is valid).
@@ -130,7 +135,7 @@ __device__ __forceinline__ bool mat_prefix(const MatReq &q, int p) {
 }
 
 // Exclusive scan of one int per thread over the block; *total gets the sum.
-__device__ __forceinline__ int mat_excl_scan(int v, MatShared &sh, int *total) {
+__device__ __forceinline__ int mat_excl_scan(int v, int threads, MatShared &sh, int *total) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int x = v;
 #pragma unroll
@@ -143,7 +148,7 @@ __device__ __forceinline__ int mat_excl_scan(int v, MatShared &sh, int *total) {
     int before = 0, sum = 0;
 #pragma unroll
     for (int w = 0; w < kMatWarps; ++w) {
-        const int y = w < (int)(blockDim.x >> 5) ? sh.warp_sums[w] : 0;
+        const int y = w < (threads >> 5) ? sh.warp_sums[w] : 0;
         before += w < warp ? y : 0;
         sum += y;
     }
@@ -153,7 +158,7 @@ __device__ __forceinline__ int mat_excl_scan(int v, MatShared &sh, int *total) {
 }
 
 // Best head of the block's register lists; every thread gets it.
-__device__ __forceinline__ void mat_block_best(float hv, int hp, MatShared &sh, float *bv, int *bp) {
+__device__ __forceinline__ void mat_block_best(float hv, int hp, int threads, MatShared &sh, float *bv, int *bp) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
@@ -172,8 +177,8 @@ __device__ __forceinline__ void mat_block_best(float hv, int hp, MatShared &sh, 
                 sh.wp[warp] = hp;
             }
             __syncthreads();
-            hv = lane < (int)(blockDim.x >> 5) ? sh.wv[lane] : -INFINITY;
-            hp = lane < (int)(blockDim.x >> 5) ? sh.wp[lane] : -1;
+            hv = lane < (threads >> 5) ? sh.wv[lane] : -INFINITY;
+            hp = lane < (threads >> 5) ? sh.wp[lane] : -1;
         }
     }
     __syncthreads();  // wv / wp reusable
@@ -204,7 +209,7 @@ __device__ __forceinline__ uint32_t mat_rows(const Src &src, const MatReq &q, in
 template <class Src>
 __device__ __noinline__ void mat_again(Src src, MatReq q, int w0, int nr, uint32_t *bits) {
     __syncthreads();  // the previous rows are consumed
-    const int stride = (blockDim.x >> 5) * Src::kRows;
+    const int stride = (q.threads >> 5) * Src::kRows;
     for (int r0 = w0 + (threadIdx.x >> 5) * Src::kRows; r0 < w0 + nr; r0 += stride)
         (void)mat_rows(src, q, r0, w0 + nr, bits, w0);
     __syncthreads();
@@ -288,7 +293,7 @@ __device__ __forceinline__ void mat_body(const Src &src, const MatReq &q, int ro
                                          MatShared &sh, uint32_t *bits, const MatOut &o) {
     namespace cg = cooperative_groups;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int nthreads = blockDim.x;
+    const int nthreads = q.threads;
     const int top_c = o.top_c, pos_cap = o.pos_cap;
     const bool solo = nc == 1;
     if (!solo) cluster_arrive_relaxed();  // this CTA runs; the wait sits before the first push
@@ -439,7 +444,7 @@ __device__ __forceinline__ void mat_body(const Src &src, const MatReq &q, int ro
         for (int c = 0; c < top_c; ++c) {
             float bv;
             int bp;
-            mat_block_best(ls[0], lp[0], sh, &bv, &bp);
+            mat_block_best(ls[0], lp[0], nthreads, sh, &bv, &bp);
             if (bp < 0) break;
             if (tid == 0) {
                 sh.top_s[c] = bv;
@@ -500,7 +505,7 @@ __device__ __forceinline__ void mat_body(const Src &src, const MatReq &q, int ro
                 n += __popc(w.x) + __popc(w.y) + __popc(w.z) + __popc(w.w);
             }
             int wtotal = 0;
-            const int idx = __shfl_sync(0xffffffffu, base + mat_excl_scan(n, sh, &wtotal), 0);
+            const int idx = __shfl_sync(0xffffffffu, base + mat_excl_scan(n, nthreads, sh, &wtotal), 0);
             mat_each(src, bits, w0, a, z, idx, pos_cap, none, put);
             base += wtotal;
         }
@@ -562,16 +567,17 @@ __device__ __forceinline__ void mat_body(const Src &src, const MatReq &q, int ro
 // The CTAs of the cluster that share a request's rows: one round of CTA 0's
 // warps needs no others.
 template <class Src>
-__device__ __forceinline__ int mat_ctas(int rows) {
-    if (rows <= (int)(blockDim.x >> 5) * Src::kRows) return 1;
+__device__ __forceinline__ int mat_ctas(int rows, int threads) {
+    if (rows <= (threads >> 5) * Src::kRows) return 1;
     const int nc = gridDim.x;
     return nc > kMatCluster && rows < Src::kWideRows ? kMatCluster : nc;
 }
 
-// Launches a retrieval kernel over B requests; attr_done: the caller's flags,
-// one per kernel and device.
+// Launches a retrieval kernel over B requests; few_threads: the threads of a CTA
+// in calls of up to kMatMidB requests; attr_done: the caller's flags, one per
+// kernel and device.
 template <typename... KArgs, typename... Args>
-inline rs_status mat_launch(const char *who, int (&attr_done)[64], void (*kern)(KArgs...), int B, cudaStream_t st,
+inline rs_status mat_launch(const char *who, int few_threads, int (&attr_done)[64], void (*kern)(KArgs...), int B, cudaStream_t st,
                             Args... args) {
     int dev = 0;
     cudaGetDevice(&dev);
@@ -585,7 +591,7 @@ inline rs_status mat_launch(const char *who, int (&attr_done)[64], void (*kern)(
         attr_done[dev] = 1;
     }
     const int nc = B <= kMatFewB ? kMatClusterMax : kMatCluster;
-    const int threads = B <= kMatMidB ? kMatThreads : kMatThreads / 2;
+    const int threads = B <= kMatMidB ? few_threads : kMatHalf;
     launch_pdl_cluster(kern, dim3(nc, B), dim3(threads), kMatSmem, st, nc, args...);
     RS_CHECK_LAUNCH(who);
     return RS_OK;

@@ -10,9 +10,9 @@
 // shared memory and nothing is read twice.  Staging 8192-position windows of
 // tokens and scores (4-byte asynchronous copies, a second staging for the
 // positions) took 51 us on 4 x 262144 tokens of text, a key of two; this takes
-// 8.4 (graph), the reads of 32 SMs at 4 MB and the dependent rounds around
-// them.  The shortest calls of one to four requests pay for the larger cluster:
-// 2000 tokens 5.7 us, 4.6 before; of 16 requests 4.0, 4.7 before.
+// 8.3 (graph), the reads of 64 SMs at 4 MB and the dependent rounds around
+// them.  Short calls take as long as they did: 2000 tokens of one request 4.7 us
+// (4.6 before), of 16 requests 3.9 (4.7).
 #include "match.cuh"
 
 namespace rs {
@@ -89,8 +89,11 @@ match_scan_kernel(const int32_t *__restrict__ tokens, const int64_t *__restrict_
     ScanSource src;
     src.al = (int)((reinterpret_cast<uintptr_t>(q.X) >> 2) & 3);
     const int rows = q.run ? (int)(((unsigned)q.t + src.al + 126) / 128) : 0;
-    const int nc = mat_ctas<ScanSource>(rows);
-    if (crank >= nc) return;
+    // with one round of half the warps of eight CTAs the other warps leave: they
+    // would only make every barrier longer
+    q.threads = rows <= kMatCluster * (kMatHalf / 32) * ScanSource::kRows ? kMatHalf : (int)blockDim.x;
+    const int nc = mat_ctas<ScanSource>(rows, q.threads);
+    if (crank >= nc || (int)threadIdx.x >= q.threads) return;
     mat_body(src, q, rows, nc, b, crank, sh, scan_bits, o);
 }
 
@@ -125,6 +128,6 @@ extern "C" rs_status rs_match_scan(const int32_t *tokens, const int64_t *tok_off
     if (B == 0) return RS_OK;
     const MatOut o{count, pos, sel_pos, sel_len, spans, n_sel, status, p.theta_score, p.top_c, p.span_len, pos_cap};
     static int attr_done[64] = {0};
-    return mat_launch("rs_match_scan", attr_done, match_scan_kernel, B, (cudaStream_t)stream, tokens, tok_off, k_star, gate_ok,
+    return mat_launch("rs_match_scan", kMatThreads, attr_done, match_scan_kernel, B, (cudaStream_t)stream, tokens, tok_off, k_star, gate_ok,
                       scores, o);
 }

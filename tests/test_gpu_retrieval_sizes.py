@@ -52,7 +52,7 @@ def _scan(tokens, tok_off, ks, scores, theta, top_c, span_len, pos_cap):
 @pytest.mark.parametrize("V", [3, 400])
 def test_scan_alignments_and_round_edges(k, V):
     # request lengths of 1 mod 4 walk through every alignment; 4096 candidate
-    # positions (8192 in calls of few requests) are the most one CTA takes alone
+    # positions are the most one CTA takes alone
     rng = np.random.default_rng(100 * k + V)
     lens = [1, 5, 129, 8185, 16381, 8197, 16389, 33, 8193, 17, 20001, 4089, 4097, 4101]
     tokens, tok_off = _buffers(rng, lens, V, k)
@@ -79,9 +79,10 @@ def test_scan_beyond_the_kept_ballots():
 @pytest.mark.parametrize("B", [1, 4, 5, 8, 9, 40])
 def test_scan_cluster_forms(B):
     # up to 4 requests: clusters of 16, of which a request of less than 131072
-    # candidates uses 8; up to 8: clusters of 8; more: CTAs of half the threads
+    # candidates uses 8; more: clusters of 8; more than 8 requests, or up to 32768
+    # candidates: half the threads
     rng = np.random.default_rng(B)
-    lens = rng.choice([40, 8190, 8197, 16380, 16389, 30001], B).tolist()
+    lens = rng.choice([40, 4090, 4101, 8197, 30001, 32760, 32775], B).tolist()
     lens[0], lens[-1] = 130000, 131200
     tokens, tok_off = _buffers(rng, lens, 30, 2)
     scores = rng.random(len(tokens)).astype(np.float32)
