@@ -468,12 +468,10 @@ __device__ __forceinline__ int ones_from(const uint32_t *w, int pos, int L) {
 // where the first half overlaps the row kernels, 18.2 -> 14.3 and 29.0 -> 23.7.
 template <bool kEarly>
 __global__ void __launch_bounds__(kDecThreads)
-accept_decide(const float *__restrict__ logits, int R, int V, const int32_t *__restrict__ node_off,
-              const int32_t *__restrict__ tokens, const int32_t *__restrict__ parents,
-              const uint8_t *__restrict__ source, const int8_t *__restrict__ chain,
-              const int32_t *__restrict__ sel_pos, const int64_t *__restrict__ tok_off, rs_params p,
-              int acc_cap, const int32_t *argmax, const int32_t *topk, const float *lse, const float *rowmax,
-              float *__restrict__ p_tok, int32_t *__restrict__ acc_len, int32_t *__restrict__ acc_nodes,
+accept_decide(const float *logits, int R, int V, const int32_t *node_off, const int32_t *tokens,
+              const int32_t *parents, const uint8_t *source, const int8_t *chain, const int32_t *sel_pos,
+              const int64_t *tok_off, rs_params p, int acc_cap, const int32_t *argmax, const int32_t *topk,
+              const float *lse, const float *rowmax, float *__restrict__ p_tok, int32_t *__restrict__ acc_len, int32_t *__restrict__ acc_nodes,
               int32_t *__restrict__ bonus, int32_t *__restrict__ winner, uint8_t *__restrict__ commit, float *scores,
               int32_t *__restrict__ status) {
     pdl_launch_next();

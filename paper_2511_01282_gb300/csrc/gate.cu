@@ -221,7 +221,7 @@ __device__ __forceinline__ int push_scan(int v, int *s_w, int *total) {
 // 5.3 us (kEarly) and 6.5 -> 6.1 us.
 template <bool kEarly>
 __global__ void __launch_bounds__(kPushThreads)
-gate_push(const float *entropy, const int32_t *__restrict__ row_off, const uint8_t *__restrict__ row_commit, int R,
+gate_push(const float *entropy, const int32_t *row_off, const uint8_t *row_commit, int R,
           rs_params p, float *hist, int32_t *hist_n, int32_t *__restrict__ k_star, float *__restrict__ h_best,
           uint8_t *__restrict__ entropy_ok) {
     pdl_launch_next();

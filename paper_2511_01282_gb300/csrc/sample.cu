@@ -466,8 +466,8 @@ sample_partial(const float *__restrict__ logits, int V, int nchunks, float scale
 // flagged list (row, maximum) for the exact pass.
 template <int kW>
 __global__ void __launch_bounds__(kSmpThreads)
-sample_pick(const float *__restrict__ logits, int V, int nchunks, float scale, float lam_h, float lam_l,
-            const Exp2Tab tab, const ChunkMass *part, const float *__restrict__ uniforms, int force,
+sample_pick(const float *logits, int V, int nchunks, float scale, float lam_h, float lam_l,
+            const Exp2Tab tab, const ChunkMass *part, const float *uniforms, int force,
             int *__restrict__ n_flag, FlagRow *__restrict__ flags, int *__restrict__ done,
             int32_t *__restrict__ draw) {
     pdl_launch_next();
@@ -664,8 +664,8 @@ __device__ int last_with_mass(const float *row, long long end, float M, double i
 // sums and scans in double-float on the fp32 pipe; fp64 only on the rare
 // paths (u Z below 2^-40 Z, the last id with mass).
 __global__ void __launch_bounds__(kSmpThreads)
-sample_exact(const float *__restrict__ logits, int V, int nslices, float lam_h, float lam_l, double inv_t, double T,
-             const Exp2Tab tab, const float *__restrict__ uniforms, const int *n_flag,
+sample_exact(const float *logits, int V, int nslices, float lam_h, float lam_l, double inv_t, double T,
+             const Exp2Tab tab, const float *uniforms, const int *n_flag,
              const FlagRow *flags, int *__restrict__ done, float2 *__restrict__ slice_sum,
              int32_t *__restrict__ draw) {
     pdl_launch_next();
@@ -817,9 +817,8 @@ sample_exact(const float *__restrict__ logits, int V, int nslices, float lam_h, 
 // before the wait for them; only the draws are read after it.
 template <bool kEarly>
 __global__ void __launch_bounds__(32)
-sample_walk(const int32_t *__restrict__ node_off, int R, const int32_t *__restrict__ tokens,
-            const int32_t *__restrict__ parents, const uint8_t *__restrict__ source,
-            const int32_t *draw, int acc_cap, int32_t *__restrict__ acc_len,
+sample_walk(const int32_t *node_off, int R, const int32_t *tokens, const int32_t *parents,
+            const uint8_t *source, const int32_t *draw, int acc_cap, int32_t *__restrict__ acc_len,
             int32_t *__restrict__ acc_nodes, int32_t *__restrict__ bonus, int32_t *__restrict__ status) {
     pdl_launch_next();
     if (!kEarly) pdl_wait_prev();
