@@ -231,8 +231,7 @@ __device__ __forceinline__ void merge_row(const VI *cand, int ncand, int beta, l
 //     cluster barrier; otherwise they go to the workspace for accept_merge.
 template <bool kVec, bool kEnt, bool kFuse>
 __global__ void __launch_bounds__(kAccThreads, 4)
-accept_rows(const float *__restrict__ logits, int V, int nchunks, int beta, VI *__restrict__ cand,
-            MS *__restrict__ part, RowOut o) {
+accept_rows(const float *logits, int V, int nchunks, int beta, VI *cand, MS *part, RowOut o) {
     // the kernels behind this one read the caller's arrays before they wait for
     // it (accept_decide), so they may launch only once its own wait is over
     pdl_wait_prev();
@@ -421,7 +420,7 @@ constexpr int kMergeRows = kMergeThreads / 64;  // rows per block
 constexpr int kCandPerLane = 8;
 
 __global__ void __launch_bounds__(kMergeThreads)
-accept_merge(const VI *__restrict__ cand, const MS *__restrict__ part, int nchunks, int beta, int R, RowOut o) {
+accept_merge(const VI *cand, const MS *part, int nchunks, int beta, int R, RowOut o) {
     pdl_enter();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long r = (long long)blockIdx.x * kMergeRows + (warp >> 1);
@@ -471,9 +470,8 @@ __global__ void __launch_bounds__(kDecThreads)
 accept_decide(const float *logits, int R, int V, const int32_t *node_off, const int32_t *tokens,
               const int32_t *parents, const uint8_t *source, const int8_t *chain, const int32_t *sel_pos,
               const int64_t *tok_off, rs_params p, int acc_cap, const int32_t *argmax, const int32_t *topk,
-              const float *lse, const float *rowmax, float *__restrict__ p_tok, int32_t *__restrict__ acc_len, int32_t *__restrict__ acc_nodes,
-              int32_t *__restrict__ bonus, int32_t *__restrict__ winner, uint8_t *__restrict__ commit, float *scores,
-              int32_t *__restrict__ status) {
+              const float *lse, const float *rowmax, float *p_tok, int32_t *acc_len, int32_t *acc_nodes,
+              int32_t *bonus, int32_t *winner, uint8_t *commit, float *scores, int32_t *status) {
     pdl_launch_next();
     if (!kEarly) pdl_wait_prev();
     const int b = blockIdx.x;

@@ -35,11 +35,9 @@ namespace rs {
 namespace {
 
 __global__ void __launch_bounds__(256)
-attn_prep(const int32_t *__restrict__ node_off, const int32_t *__restrict__ ctx_len,
-          const int64_t *__restrict__ kv_off, const int32_t *__restrict__ parents, int R, long long kv_rows,
-          int Hq, int Hkv, int D, int seg_rows, ReqInfo *__restrict__ info, uint32_t *__restrict__ anc,
-          float *__restrict__ out, float *__restrict__ lse, int32_t *__restrict__ status,
-          int *__restrict__ n_items) {
+attn_prep(const int32_t *node_off, const int32_t *ctx_len, const int64_t *kv_off, const int32_t *parents, int R,
+          long long kv_rows, int Hq, int Hkv, int D, int seg_rows, ReqInfo *info, uint32_t *anc, float *out, float *lse,
+          int32_t *status, int *n_items) {
     // the attention kernel takes whole SMs, so it launches only once this
     // kernel's own wait is over: earlier work has left them by then
     pdl_wait_prev();

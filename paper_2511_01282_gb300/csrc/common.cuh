@@ -113,10 +113,11 @@ long long l2_bytes();  // L2 size of the current device (cached per device)
 // Let the next kernel start launching, then wait for the previous kernel.
 __device__ __forceinline__ void pdl_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait_prev() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-// A kernel with work before pdl_wait_prev takes its inputs through pointers that
-// are not `const __restrict__`: loads through those may become ld.global.nc,
-// which the compiler is free to move above the wait.  (That also holds where the
-// wait comes first in one instance of a template and later in another.)
+// No pointer here is __restrict__: with it the compiler may take it that nothing
+// else writes what a kernel reads, turn the loads into ld.global.nc and move them
+// above the wait (sample_exact met that), where what the predecessor writes --
+// scores, commit flags, a key length, this call's own intermediate results -- is
+// read too early.  The streaming loads below are volatile and stay behind it.
 __device__ __forceinline__ void pdl_enter() {
     pdl_launch_next();
     pdl_wait_prev();

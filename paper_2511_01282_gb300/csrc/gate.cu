@@ -74,8 +74,7 @@ __device__ __forceinline__ float ex2f_approx(float x) {
 // 0 and 16-byte alignment; else 1).
 template <int kW>
 __global__ void __launch_bounds__(kGateThreads)
-entropy_partial(const float *__restrict__ logits, int V, int nchunks, Ent3 *__restrict__ part,
-                float *__restrict__ entropy) {
+entropy_partial(const float *logits, int V, int nchunks, Ent3 *part, float *entropy) {
     // gate_push reads the caller's arrays before it waits for this call's row
     // kernels, so it may launch only once this kernel's own wait is over
     pdl_wait_prev();
@@ -169,7 +168,7 @@ entropy_partial(const float *__restrict__ logits, int V, int nchunks, Ent3 *__re
 constexpr int kMergeThreads = 256;
 
 __global__ void __launch_bounds__(kMergeThreads)
-entropy_merge(const Ent3 *__restrict__ part, int nchunks, int R, float *__restrict__ entropy) {
+entropy_merge(const Ent3 *part, int nchunks, int R, float *entropy) {
     pdl_enter();
     const int lane = threadIdx.x & 31;
     const long long r = (long long)blockIdx.x * (kMergeThreads / 32) + (threadIdx.x >> 5);
@@ -222,8 +221,8 @@ __device__ __forceinline__ int push_scan(int v, int *s_w, int *total) {
 template <bool kEarly>
 __global__ void __launch_bounds__(kPushThreads)
 gate_push(const float *entropy, const int32_t *row_off, const uint8_t *row_commit, int R,
-          rs_params p, float *hist, int32_t *hist_n, int32_t *__restrict__ k_star, float *__restrict__ h_best,
-          uint8_t *__restrict__ entropy_ok) {
+          rs_params p, float *hist, int32_t *hist_n, int32_t *k_star, float *h_best,
+          uint8_t *entropy_ok) {
     pdl_launch_next();
     const int b = blockIdx.x, tid = threadIdx.x;
     const int l = p.l;

@@ -152,7 +152,7 @@ __device__ __forceinline__ long long start_of(int first, int v) { return (long l
 // (0) the build's offsets: tok_off[0] = 0, ascending, tok_off[B] = t_total;
 // every later build kernel does nothing unless they are
 __global__ void __launch_bounds__(1024)
-index_check(const int64_t *__restrict__ tok_off, int B, long long t_total, IndexView ix) {
+index_check(const int64_t *tok_off, int B, long long t_total, IndexView ix) {
     pdl_enter();
     int bad = threadIdx.x == 0 && (tok_off[0] != 0 || tok_off[B] != t_total);
     for (int b = threadIdx.x; b < B; b += blockDim.x) bad |= tok_off[b + 1] < tok_off[b];
@@ -210,7 +210,7 @@ struct PairKeys {
 // loaded before any is used.
 template <class Keys, int kR>
 __global__ void __launch_bounds__(kRadixThreads)
-radix_hist(Keys src, long long N, int shift, int bins, int32_t *__restrict__ hist, const int32_t *__restrict__ valid) {
+radix_hist(Keys src, long long N, int shift, int bins, int32_t *hist, const int32_t *valid) {
     pdl_enter();
     if (!*valid) return;
     __shared__ int cnt[kMaxBins];
@@ -272,8 +272,8 @@ constexpr int off_threads(int per_thread) { return per_thread == kOffManyT ? 512
 static_assert(kOffFew == off_threads(kOffFewT) / kOffDigits * kOffFewT, "one round");
 template <int kT>
 __global__ void __launch_bounds__(off_threads(kT))
-radix_offsets(int32_t *__restrict__ hist, long long ntiles, int bins, int32_t *__restrict__ dtot,
-              const int32_t *__restrict__ valid) {
+radix_offsets(int32_t *hist, long long ntiles, int bins, int32_t *dtot,
+              const int32_t *valid) {
     pdl_enter();
     if (!*valid) return;
     constexpr int kWarps = off_threads(kT) / 32, kGroups = off_threads(kT) / kOffDigits;
@@ -440,8 +440,8 @@ struct Packed {
 // neighbouring threads.
 template <class Keys, int kR, class Words>
 __global__ void __launch_bounds__(kRadixThreads, Words::kBlocks)
-radix_scatter(Keys src, Words words, typename Words::W *__restrict__ out, long long N, int bins,
-              const int32_t *__restrict__ hist, const int32_t *__restrict__ dtot, const int32_t *__restrict__ valid) {
+radix_scatter(Keys src, Words words, typename Words::W *out, long long N, int bins,
+              const int32_t *hist, const int32_t *dtot, const int32_t *valid) {
     pdl_enter();
     if (!*valid) return;
     using W = typename Words::W;
@@ -512,8 +512,8 @@ __device__ __forceinline__ CutTile cut_tile(const int32_t *dtot, int bins, int t
 
 template <int kR>
 __global__ void __launch_bounds__(kRadixThreads)
-cut_hist(const uint32_t *__restrict__ in, int bins0, int pos_bits, int bins, const int32_t *__restrict__ dtot,
-         int32_t *__restrict__ hist, CutTile *__restrict__ tiles, const int32_t *__restrict__ valid) {
+cut_hist(const uint32_t *in, int bins0, int pos_bits, int bins, const int32_t *dtot,
+         int32_t *hist, CutTile *tiles, const int32_t *valid) {
     pdl_enter();
     if (!*valid) return;
     __shared__ int cnt[kMaxBins];
@@ -542,8 +542,8 @@ cut_hist(const uint32_t *__restrict__ in, int bins0, int pos_bits, int bins, con
 constexpr int kCutFirst = 1024;
 template <int kR>
 __global__ void __launch_bounds__(kRadixThreads, 4)
-cut_scatter(const uint32_t *__restrict__ in, const CutTile *__restrict__ cuts, int tiles, int bins0, int lo_bits, int pos_bits, int bins, const int32_t *__restrict__ dtot,
-            const int32_t *__restrict__ hist, const int64_t *__restrict__ tok_off, int B, int V, int vbits, IndexView ix) {
+cut_scatter(const uint32_t *in, const CutTile *cuts, int tiles, int bins0, int lo_bits, int pos_bits, int bins,
+            const int32_t *dtot, const int32_t *hist, const int64_t *tok_off, int B, int V, int vbits, IndexView ix) {
     pdl_enter();
     if (!*ix.valid) return;
     constexpr int kTile = kR * kRadixThreads;
@@ -642,7 +642,7 @@ static_assert(kTileRounds * kRadixThreads <= 65535, "16-bit tile counters");
 // buckets (the last thread only serves its neighbour).
 constexpr int kFirstPer = 255;
 __global__ void __launch_bounds__(kFirstPer + 1)
-index_first(const uint2 *__restrict__ sorted, const int64_t *__restrict__ tok_off, int V, int vbits, IndexView ix) {
+index_first(const uint2 *sorted, const int64_t *tok_off, int V, int vbits, IndexView ix) {
     pdl_enter();
     if (!*ix.valid) return;
     __shared__ int s_first[kFirstPer + 1];
@@ -677,7 +677,7 @@ index_first(const uint2 *__restrict__ sorted, const int64_t *__restrict__ tok_of
 // positions of that bucket is its sorted index minus the bucket's first.
 constexpr int kPlacePer = 4;
 __global__ void __launch_bounds__(256)
-index_place(const uint2 *__restrict__ sorted, long long N, const int64_t *__restrict__ tok_off, int V, int vbits,
+index_place(const uint2 *sorted, long long N, const int64_t *tok_off, int V, int vbits,
             IndexView ix) {
     pdl_enter();
     if (!*ix.valid) return;
@@ -706,8 +706,8 @@ index_place(const uint2 *__restrict__ sorted, long long N, const int64_t *__rest
 // warp when they are few (an append of 5 tokens and its query 8.5 -> 8.0 us),
 // else in rounds of kAppThreads; see the file comment.
 __global__ void __launch_bounds__(kAppThreads)
-index_append(const int32_t *__restrict__ tokens, const int64_t *__restrict__ tok_off, int V, IndexView ix,
-             int32_t *__restrict__ status) {
+index_append(const int32_t *tokens, const int64_t *tok_off, int V, IndexView ix,
+             int32_t *status) {
     pdl_enter();
     constexpr int kW = kAppThreads / 32;
     __shared__ int s_bk[kAppThreads];
@@ -873,11 +873,10 @@ struct ListSource {
 };
 
 __global__ void __launch_bounds__(kMatHalf)
-index_query(const int32_t *__restrict__ tokens, const int64_t *__restrict__ tok_off, int V,
-            const int32_t *__restrict__ k_star, const uint8_t *__restrict__ gate_ok,
-            const float *__restrict__ scores, IndexView ix, MatOut o) {
-    pdl_enter();
+index_query(const int32_t *tokens, const int64_t *tok_off, int V, const int32_t *k_star, const uint8_t *gate_ok,
+            const float *scores, IndexView ix, MatOut o) {
     __shared__ MatShared sh;
+    mat_enter(sh);
     extern __shared__ __align__(16) uint32_t qry_bits[];
     const int crank = (int)cooperative_groups::this_cluster().block_rank();
     const int b = blockIdx.y;

@@ -95,10 +95,19 @@ struct MatReq {
     int threads;        // of the CTA at work on it
 };
 
+// A retrieval kernel's first act.  The one barrier that no read depends on comes
+// before the wait for the predecessor, and no thread stops at it between the
+// request's records and its candidates.
+__device__ __forceinline__ void mat_enter(MatShared &sh) {
+    pdl_launch_next();
+    if (threadIdx.x == 0) sh.ccnt = 0;
+    __syncthreads();
+    pdl_wait_prev();
+}
+
 // ok: the caller's own condition for reading the request (its index is valid).
-__device__ __forceinline__ void mat_request(MatReq &q, const int32_t *__restrict__ tokens,
-                                            const int64_t *__restrict__ tok_off, const int32_t *__restrict__ k_star,
-                                            const uint8_t *__restrict__ gate_ok, const float *__restrict__ scores, int b,
+__device__ __forceinline__ void mat_request(MatReq &q, const int32_t *tokens, const int64_t *tok_off,
+                                            const int32_t *k_star, const uint8_t *gate_ok, const float *scores, int b,
                                             int B, bool ok) {
     const long long t0 = tok_off[b], t1 = tok_off[b + 1], tend = tok_off[B];
     q.k = k_star[b];
@@ -299,8 +308,6 @@ __device__ __forceinline__ void mat_body(const Src &src, const MatReq &q, int ro
     if (!solo) cluster_arrive_relaxed();  // this CTA runs; the wait sits before the first push
     const int per = (rows + nc - 1) / nc;
     const int lo = min(per * crank, rows), hi = min(lo + per, rows);
-    if (tid == 0) sh.ccnt = 0;
-    __syncthreads();
 
     // ---- every candidate once: ballots, count, the matches that clear theta ----
     // (consecutive rows per warp, as the positions are written)

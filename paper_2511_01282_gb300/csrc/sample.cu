@@ -196,7 +196,7 @@ constexpr int kSmpPadded = kSmpChunk + kSmpChunk / 8;  // 36 floats per thread
 // logits: 16.4 us, 19.1 with all thirty-two at once; eight at a time 15.2, but
 // 145 rows of 128257 36.5 instead of 32.8).
 template <int kW>
-__device__ __forceinline__ void load32_staged(const float *__restrict__ row, int V, int c0, float *s_buf,
+__device__ __forceinline__ void load32_staged(const float *row, int V, int c0, float *s_buf,
                                               float (&z)[kSmpVpt]) {
     const int tid = threadIdx.x, left = V - c0;  // a multiple of kW
     const float *chunk = row + c0;
@@ -423,8 +423,7 @@ __device__ __forceinline__ RowDecision decide_row(const ChunkMass *pr, int nchun
 // mass s_c and q_c (staged loads, terms, butterfly then tree sums).
 template <int kW>
 __global__ void __launch_bounds__(kSmpThreads)
-sample_partial(const float *__restrict__ logits, int V, int nchunks, float scale, ChunkMass *__restrict__ part,
-               int *__restrict__ n_flag) {
+sample_partial(const float *logits, int V, int nchunks, float scale, ChunkMass *part, int *n_flag) {
     // the later kernels read the caller's arrays before they wait for this
     // call's (uniforms, the chosen logits' tree), so they may launch only once
     // this kernel's own wait is over
@@ -468,8 +467,8 @@ template <int kW>
 __global__ void __launch_bounds__(kSmpThreads)
 sample_pick(const float *logits, int V, int nchunks, float scale, float lam_h, float lam_l,
             const Exp2Tab tab, const ChunkMass *part, const float *uniforms, int force,
-            int *__restrict__ n_flag, FlagRow *__restrict__ flags, int *__restrict__ done,
-            int32_t *__restrict__ draw) {
+            int *n_flag, FlagRow *flags, int *done,
+            int32_t *draw) {
     pdl_launch_next();
     __shared__ float2 s_tab[64];
     __shared__ RowDecision s_dec;
@@ -666,8 +665,8 @@ __device__ int last_with_mass(const float *row, long long end, float M, double i
 __global__ void __launch_bounds__(kSmpThreads)
 sample_exact(const float *logits, int V, int nslices, float lam_h, float lam_l, double inv_t, double T,
              const Exp2Tab tab, const float *uniforms, const int *n_flag,
-             const FlagRow *flags, int *__restrict__ done, float2 *__restrict__ slice_sum,
-             int32_t *__restrict__ draw) {
+             const FlagRow *flags, int *done, float2 *slice_sum,
+             int32_t *draw) {
     pdl_launch_next();
     __shared__ float2 s_tab[64];
     __shared__ DF s_w[kSmpWarps + 1];
@@ -818,8 +817,8 @@ sample_exact(const float *logits, int V, int nslices, float lam_h, float lam_l, 
 template <bool kEarly>
 __global__ void __launch_bounds__(32)
 sample_walk(const int32_t *node_off, int R, const int32_t *tokens, const int32_t *parents,
-            const uint8_t *source, const int32_t *draw, int acc_cap, int32_t *__restrict__ acc_len,
-            int32_t *__restrict__ acc_nodes, int32_t *__restrict__ bonus, int32_t *__restrict__ status) {
+            const uint8_t *source, const int32_t *draw, int acc_cap, int32_t *acc_len,
+            int32_t *acc_nodes, int32_t *bonus, int32_t *status) {
     pdl_launch_next();
     if (!kEarly) pdl_wait_prev();
     constexpr int kPer = RS_MAX_NODES / 32;

@@ -76,11 +76,10 @@ struct ScanSource {
 };
 
 __global__ void __launch_bounds__(kMatThreads)
-match_scan_kernel(const int32_t *__restrict__ tokens, const int64_t *__restrict__ tok_off,
-                  const int32_t *__restrict__ k_star, const uint8_t *__restrict__ gate_ok,
-                  const float *__restrict__ scores, MatOut o) {
-    pdl_enter();
+match_scan_kernel(const int32_t *tokens, const int64_t *tok_off, const int32_t *k_star, const uint8_t *gate_ok,
+                  const float *scores, MatOut o) {
     __shared__ MatShared sh;
+    mat_enter(sh);
     extern __shared__ __align__(16) uint32_t scan_bits[];
     const int crank = (int)cooperative_groups::this_cluster().block_rank();
     const int b = blockIdx.y;

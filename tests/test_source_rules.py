@@ -44,22 +44,21 @@ def _kernels():
     return out
 
 
-def _read_only(args):
-    return re.findall(r"const\s+[^,()]*\*\s*__restrict__\s+(\w+)", args)
-
-
 def test_every_kernel_is_found():
     names = {k for _, k, _, _ in _kernels()}
     assert {"gate_push", "accept_decide", "sample_walk", "attn_prep", "attn_tc_kernel", "index_query", "cut_scatter"} <= names
     assert len(names) >= 20
 
 
-@pytest.mark.parametrize("kernel", [k for k in _kernels()], ids=lambda k: k[1])
-def test_kernels_that_work_before_their_wait_have_plain_inputs(kernel):
-    # a load through `const __restrict__` may be moved above the wait; with code
-    # there the compiler has a place to move it to
-    f, name, args, body = kernel
-    before = re.split(r"pdl_enter\(\)|pdl_wait_prev\(\)", body)[0]
-    early = re.sub(r"pdl_launch_next\(\)|[;\s]", "", before)
-    assert "pdl_" in body, "%s neither waits for its predecessor nor says why" % name
-    assert not early or not _read_only(args), "%s (%s): %s" % (name, f, _read_only(args))
+@pytest.mark.parametrize("kernel", _kernels(), ids=lambda k: k[1])
+def test_kernels_wait_for_their_predecessor(kernel):
+    _, name, _, body = kernel
+    assert re.search(r"\bpdl_(enter|wait_prev)\(\)|\bmat_enter\(", body), name
+
+
+@pytest.mark.parametrize("name", SOURCES)
+def test_loads_stay_behind_the_wait(name):
+    # a load through a __restrict__ pointer (or __ldg) may be moved above the wait
+    # for the kernel before, which may still be writing what is read; inlined, the
+    # parameters of device functions are as good as the kernel's
+    assert not re.findall(r"__restrict__|__ldg\b", _text(name))
