@@ -63,7 +63,9 @@ typedef enum {
                                layout broken, or a node count out of range     */
 #define RS_ST_TRUNCATED  2  /* an output list was longer than its capacity     */
 #define RS_ST_BAD_POS    4  /* a selected position lies outside the buffer     */
-#define RS_ST_TOO_LARGE  8  /* more than RS_MAX_NODES tree nodes               */
+#define RS_ST_TOO_LARGE  8  /* more than RS_MAX_NODES tree nodes, a key of more
+                               than RS_MAX_L or a buffer of more than 2^31 - 1
+                               tokens                                          */
 #define RS_ST_TIMEOUT   16  /* a pipeline wait inside a kernel gave up (bounded
                                wait, ~2 s; the environment variable
                                RS_DEBUG_WAIT_LIMIT, in clock cycles, shortens it
@@ -192,7 +194,8 @@ rs_status rs_entropy_gate_noalloc(const float *logits, int R, int V, const int32
  *   tokens   [sum t_b] int32: per request the committed token buffer
  *            (prompt + generated, ending with the root token), request b at
  *            tokens[tok_off[b] .. tok_off[b+1]).
- *   tok_off  [B+1] int64.
+ *   tok_off  [B+1] int64; a request of more than 2^31 - 1 tokens is skipped with
+ *            RS_ST_TOO_LARGE (positions are int32).
  *   k_star   [B] int32 key lengths (rs_entropy_gate's output); k <= 0 skips
  *            the request, k > RS_MAX_L skips it with RS_ST_TOO_LARGE.
  *   gate_ok  [B] uint8 or NULL: when given, requests with gate_ok[b] == 0

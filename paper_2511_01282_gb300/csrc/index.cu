@@ -837,19 +837,20 @@ struct ListSource {
     static constexpr bool kLaneMajor = false;
     static constexpr bool kBound = false;  // (its code, 16 registers more, costs every query 0.4 us)
     const int32_t *blist, *olist;
-    int nb, no, ncand, tail0;
+    int nb, no, tail0;
+    ListPos at{0};  // at most 2^31 - 1 in all: no position is in two lists
     __device__ __forceinline__ int cand(int c) const {
         if (c < nb) return blist[c];
-        if (c < nb + no) return olist[c - nb];
-        return tail0 + (c - nb - no);
+        c -= nb;
+        return c < no ? olist[c] : tail0 + (c - no);
     }
-    __device__ __forceinline__ int pos(int row, int lane, int e) const { return cand(128 * row + 32 * e + lane); }
+    __device__ __forceinline__ int pos(int row, int lane, int e) const { return cand(at.number(row, 32 * e + lane)); }
     __device__ __forceinline__ uint32_t test(const MatReq &q, int r0, int end, int lane) const {
         int p[4 * kRows], x0[4 * kRows], x1[4 * kRows];
 #pragma unroll
         for (int j = 0; j < 4 * kRows; ++j) {
-            const int c = 128 * (r0 + (j >> 2)) + 32 * (j & 3) + lane;
-            p[j] = r0 + (j >> 2) < end && c < ncand ? cand(c) : -1;
+            const int o = 32 * j + lane;  // rows follow one another
+            p[j] = r0 + (j >> 2) < end && at.in(r0, o) ? cand(at.number(r0, o)) : -1;
         }
 #pragma unroll
         for (int j = 0; j < 4 * kRows; ++j) {
@@ -885,7 +886,7 @@ index_query(const int32_t *tokens, const int64_t *tok_off, int V, const int32_t 
     const int novf = ix.ovf_n[b];
     MatReq q;
     mat_request(q, tokens, tok_off, k_star, gate_ok, scores, b, gridDim.y, *ix.valid != 0);
-    ListSource src{nullptr, nullptr, 0, 0, 0, q.t};
+    ListSource src{nullptr, nullptr, 0, 0, 0, ListPos{0}};
     if (q.run) {
         const int bk = bucket_of(q.k1, V);
         src.olist = ix.list + base;
@@ -894,9 +895,9 @@ index_query(const int32_t *tokens, const int64_t *tok_off, int V, const int32_t 
         src.no = novf;
         src.tail0 = (int)(built < q.t ? built : q.t);
         const int nt = q.t - 1 - src.tail0;  // tail: positions tail0 .. t - 2
-        src.ncand = src.nb + src.no + (nt > 0 ? nt : 0);
+        src.at.n = src.nb + src.no + (nt > 0 ? nt : 0);
     }
-    const int rows = (src.ncand + 127) / 128;
+    const int rows = src.at.rows();
     q.threads = kMatHalf;
     const int nc = mat_ctas<ListSource>(rows, q.threads);
     if (crank >= nc) return;

@@ -32,6 +32,7 @@
 #include <math.h>
 
 #include "common.cuh"
+#include "match_pos.h"
 
 namespace rs {
 
@@ -87,7 +88,7 @@ struct MatOut {
 struct MatReq {
     const int32_t *X;
     const float *S;
-    int t;      // tokens (positions are int32: longer buffers are cut at 2^31 - 1)
+    int t;      // tokens (0 for a request that is not read)
     int k, st;  // key length; status bits
     bool run;
     int key[RS_MAX_L];  // key[i] = X[t - k + i]
@@ -113,13 +114,18 @@ __device__ __forceinline__ void mat_request(MatReq &q, const int32_t *tokens, co
     q.k = k_star[b];
     const bool gate = gate_ok == nullptr || gate_ok[b] != 0;
     const long long t = t1 - t0;
-    // the buffers hold tok_off[B] tokens: a range outside them is not read
-    const bool off_ok = ok && t0 >= 0 && t >= 0 && t0 + t <= tend;
+    // the buffers hold tok_off[B] tokens: a range outside them is not read, and
+    // neither is one of more tokens than positions can name
+    const bool off_ok = ok && t0 >= 0 && (unsigned long long)t <= kMatMaxTokens && t1 <= tend;
     q.X = tokens + (off_ok ? t0 : 0);
     q.S = scores + (off_ok ? t0 : 0);
-    q.t = off_ok ? (int)(t < 0x7fffffff ? t : 0x7fffffff) : 0;
-    q.st = off_ok ? 0 : RS_ST_BAD_OFFSET;
+    q.t = off_ok ? (int)t : 0;
+    q.st = 0;
     q.run = off_ok && q.k > 0 && gate;
+    if (!off_ok) {
+        if (!ok || t0 < 0 || t1 < t0 || t1 > tend) q.st = RS_ST_BAD_OFFSET;
+        else if (q.k > 0 && gate) q.st = RS_ST_TOO_LARGE;
+    }
     if (q.run && q.k > RS_MAX_L) {
         q.st = RS_ST_TOO_LARGE;
         q.run = false;

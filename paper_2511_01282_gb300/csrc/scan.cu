@@ -25,27 +25,24 @@ struct ScanSource {
     static constexpr int kWideRows = 1024;  // 131072 positions: below, 8 CTAs are as fast as 16
     static constexpr bool kLaneMajor = true;
     static constexpr bool kBound = true;
-    int al;       // positions of the buffer start past a 16-byte boundary
-    __device__ __forceinline__ int pos(int row, int lane, int e) const {
-        return 4 * (32 * row + lane) + e - al;
-    }
+    ScanPos at;
+    __device__ __forceinline__ int pos(int row, int lane, int e) const { return (int)(at.quad(row, lane) + (uint32_t)e); }
     __device__ __forceinline__ uint32_t test(const MatReq &q, int r0, int end, int lane) const {
-        const int t = q.t;
-        const int pb = 128 * r0 + 4 * lane - al;  // this lane's first position; row u's at pb + 128 u
+        const uint32_t pb = at.quad(r0, lane);  // this lane's first position; row u's at pb + 128 u
         const int rows = min(end - r0, kRows);
         int4 x[kRows];
 #pragma unroll
         for (int u = 0; u < kRows; ++u) {
-            const int p0 = pb + 128 * u;
+            const uint32_t p0 = pb + 128u * u;
             x[u] = make_int4(0, 0, 0, 0);
-            if (u < rows && p0 < t) {
-                if (p0 >= 0 && p0 < t - 3) {
+            if (u < rows) {
+                if (at.whole(p0)) {
                     x[u] = *reinterpret_cast<const int4 *>(q.X + p0);
                 } else {  // the quad reaches past an end of the buffer
-                    if (p0 >= 0) x[u].x = q.X[p0];
-                    if (p0 + 1 >= 0 && p0 + 1 < t) x[u].y = q.X[p0 + 1];
-                    if (p0 + 2 >= 0 && p0 + 2 < t) x[u].z = q.X[p0 + 2];
-                    if (p0 + 3 < t) x[u].w = q.X[p0 + 3];
+                    if (at.in(p0)) x[u].x = q.X[p0];
+                    if (at.in(p0 + 1u)) x[u].y = q.X[p0 + 1u];
+                    if (at.in(p0 + 2u)) x[u].z = q.X[p0 + 2u];
+                    if (at.in(p0 + 3u)) x[u].w = q.X[p0 + 3u];
                 }
             }
         }
@@ -66,9 +63,9 @@ struct ScanSource {
         // registers did not show
         for (uint32_t rem = hits; rem; rem &= rem - 1) {
             const int j = __ffs(rem) - 1;
-            const int p = pb + 128 * (j >> 2) + (j & 3);
-            bool ok = (j >> 2) < rows && p >= q.k - 1 && p <= t - 2;
-            if (ok && !(one || (q.k == 2 && (lane != 0 || (j & 3) != 0)))) ok = mat_prefix(q, p);
+            const uint32_t p = pb + 128u * (uint32_t)(j >> 2) + (uint32_t)(j & 3);
+            bool ok = (j >> 2) < rows && at.end(p, q.k);
+            if (ok && !(one || (q.k == 2 && (lane != 0 || (j & 3) != 0)))) ok = mat_prefix(q, (int)p);
             if (!ok) hits &= ~(1u << j);
         }
         return hits;
@@ -85,9 +82,8 @@ match_scan_kernel(const int32_t *tokens, const int64_t *tok_off, const int32_t *
     const int b = blockIdx.y;
     MatReq q;
     mat_request(q, tokens, tok_off, k_star, gate_ok, scores, b, gridDim.y, true);
-    ScanSource src;
-    src.al = (int)((reinterpret_cast<uintptr_t>(q.X) >> 2) & 3);
-    const int rows = q.run ? (int)(((unsigned)q.t + src.al + 126) / 128) : 0;
+    ScanSource src{ScanPos{(uint32_t)q.t, (uint32_t)(reinterpret_cast<uintptr_t>(q.X) >> 2) & 3u}};
+    const int rows = q.run ? (int)src.at.rows() : 0;
     // with one round of half the warps of eight CTAs the other warps leave: they
     // would only make every barrier longer
     q.threads = rows <= kMatCluster * (kMatHalf / 32) * ScanSource::kRows ? kMatHalf : (int)blockDim.x;
