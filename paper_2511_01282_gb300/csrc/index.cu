@@ -57,9 +57,11 @@
 // then the tail) are tested by one cluster per request as match.cuh
 // describes (70K candidates for a text's most common token: 79-120 us with one
 // CTA, 9.2 so; a handful 4.6, the chain of reads).
-#include "match.cuh"
+#include <stddef.h>
 
 #include <algorithm>
+
+#include "match.cuh"
 
 namespace rs {
 namespace {
@@ -320,7 +322,7 @@ radix_offsets(int32_t *hist, long long ntiles, int bins, int32_t *dtot,
 // equal digits before it in the tile (earlier warps, earlier rounds of its
 // warp, lower lanes of its round).
 template <class W, int kR>
-struct TileShared {
+struct alignas(16) TileShared {
     union {
         W word[kR * kRadixThreads];
         uint32_t peers[kRadixWarps][kMaxBins];  // while ranking: the lanes of the warp's round with that digit
@@ -349,6 +351,8 @@ __device__ __forceinline__ int tile_elem(int rounds, int q) {
 template <class W, int kR, class Digit, class Starts>
 __device__ __forceinline__ void order_tile(TileShared<W, kR> &sh, const W (&k)[kR], int rounds, Digit digit,
                                            Starts starts) {
+    using Tile = TileShared<W, kR>;
+    static_assert(offsetof(Tile, peers) % 16 == 0 && offsetof(Tile, cnt) % 16 == 0, "cleared by 16-byte words");
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     for (int x = tid; x < kRadixWarps * kMaxBins / 8; x += kRadixThreads) reinterpret_cast<uint4 *>(&sh.cnt[0][0])[x] = uint4{};
     for (int x = tid; x < kRadixWarps * kMaxBins / 4; x += kRadixThreads)

@@ -62,3 +62,17 @@ def test_loads_stay_behind_the_wait(name):
     # for the kernel before, which may still be writing what is read; inlined, the
     # parameters of device functions are as good as the kernel's
     assert not re.findall(r"__restrict__|__ldg\b", _text(name))
+
+
+def test_shared_structs_read_as_16_byte_words_are_aligned():
+    # &sh.member as uint4: the struct's own alignment has to carry it, not what
+    # else the kernel happens to keep in shared memory
+    seen = 0
+    for f in SOURCES:
+        s = _text(f)
+        for var, member in re.findall(r"reinterpret_cast<(?:const )?(?:u?int4|float4) \*>\(&(\w+)\.(\w+)", s):
+            for struct in set(re.findall(r"(\w+)<[^<>]*>\s*&%s\b" % var, s)):
+                assert re.search(r"struct\s+alignas\(16\)\s+%s\b" % struct, s), (f, struct)
+                assert re.search(r"offsetof\(\w+, %s\) %% 16 == 0" % member, s), (f, struct, member)
+                seen += 1
+    assert seen >= 2
