@@ -47,10 +47,10 @@ __device__ __forceinline__ Ent3 ent_merge(Ent3 a, Ent3 b) {
 // lane and plain sums.  A triple without mass (s = 0) counts for nothing.
 template <int G>
 __device__ __forceinline__ Ent3 ent_union(Ent3 t) {
-    float M = t.m;
+    const bool some = t.s != 0.f;
+    float M = some ? t.m : -INFINITY;  // of a triple without mass m may be +inf
 #pragma unroll
     for (int o = G / 2; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
-    const bool some = t.s != 0.f;
     const float d = t.m - M, c = some ? __expf(d) : 0.f;
     float s = some ? t.s * c : 0.f, w = some ? c * (t.w + t.s * d) : 0.f;
 #pragma unroll
