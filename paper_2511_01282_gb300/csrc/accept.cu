@@ -39,6 +39,7 @@ constexpr int kAccChunk = kAccThreads * kAccVpt;
 constexpr int kNoId = 0x7fffffff;  // "no candidate": after every real (v, id)
 constexpr int kCandCap = 64;        // per-warp candidate buffer (logits at or above the threshold)
 constexpr int kListBeta = 8;        // list merges hold this many candidates of a chunk in registers
+constexpr float kFarLogit = 5e8f;   // from here on logits lie 32 or more apart
 constexpr int kFuseMax = 8;         // rows of at most this many chunks merge inside their cluster
 
 struct VI {
@@ -67,6 +68,11 @@ struct MS {
     float m, s, w;
 };
 
+// How far a triple's maximum lies below the union's.  Bounded, so that its product
+// with s stays finite: a slice of masked logits (-FLT_MAX, say) has s = the number
+// of them, and 0 times infinity is no 0.
+__device__ __forceinline__ float ms_below(float m, float M) { return fmaxf(m - M, -1e30f); }
+
 // The triple of the union of one triple per lane, over aligned groups of G lanes
 // (each lane of a group gets it): the maximum first, then one exponential a
 // lane and plain sums.  A triple without mass (s = 0) counts for nothing.
@@ -76,7 +82,7 @@ __device__ __forceinline__ MS ms_union(MS t) {
     float M = some ? t.m : -INFINITY;  // of a triple without mass m may be +inf
 #pragma unroll
     for (int o = G / 2; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
-    const float d = t.m - M, c = some ? __expf(d) : 0.f;
+    const float d = ms_below(t.m, M), c = some ? __expf(d) : 0.f;
     float s = some ? t.s * c : 0.f, w = some ? c * (t.w + t.s * d) : 0.f;
 #pragma unroll
     for (int o = G / 2; o > 0; o >>= 1) {
@@ -88,9 +94,9 @@ __device__ __forceinline__ MS ms_union(MS t) {
 __device__ __forceinline__ MS ms_merge(MS a, MS b) {
     if (a.s == 0.f) return b;
     if (b.s == 0.f) return a;
-    const float M = fmaxf(a.m, b.m);
-    const float ca = __expf(a.m - M), cb = __expf(b.m - M);
-    return MS{M, a.s * ca + b.s * cb, ca * (a.w + a.s * (a.m - M)) + cb * (b.w + b.s * (b.m - M))};
+    const float M = fmaxf(a.m, b.m), da = ms_below(a.m, M), db = ms_below(b.m, M);
+    const float ca = __expf(da), cb = __expf(db);
+    return MS{M, a.s * ca + b.s * cb, ca * (a.w + a.s * da) + cb * (b.w + b.s * db)};
 }
 
 // Bitonic sort of one float per lane within aligned groups of G lanes (a
@@ -216,7 +222,11 @@ __device__ __forceinline__ void merge_row(const VI *cand, int ncand, int beta, l
 //     calls on rows of 128257 logits took 1.6 times those on 128256).
 //   * Every lane exponentiates against its warp's maximum, so a warp's
 //     triple is a plain shuffle sum; two logits an instruction where the unit
-//     has the form (145 rows of 128256 logits: 20.9 -> 20.7 us).
+//     has the form (145 rows of 128256 logits: 20.9 -> 20.7 us).  Scaling and
+//     subtracting in one fma leaves the rounding of max log2(e) in the exponent:
+//     nothing beside the logits' own spacing, but a factor of 2^860 for a warp
+//     whose logits are all masked with -1e10.  Where the spacing is 32 or more
+//     only logits equal to the maximum count, and they are counted.
 //   * Top-beta: the sixteen half-warp maxima are logits of sixteen disjoint
 //     parts of the chunk, so the beta-th largest of them (one 16-lane sort)
 //     is a lower bound T on the chunk's beta-th largest logit.  Only logits
@@ -316,6 +326,11 @@ accept_rows(const float *logits, int V, int nchunks, int beta, VI *cand, MS *par
         }
         float ss = (s2[0].x + s2[0].y) + (s2[1].x + s2[1].y);
         float ww = (w2[0].x + w2[0].y) + (w2[1].x + w2[1].y);
+        if (fabsf(wmax) >= kFarLogit) {  // (a logit of +inf leaves no finite sum: no mass)
+            ss = ww = 0.f;
+#pragma unroll
+            for (int j = 0; j < kAccVpt; ++j) ss += v[j] == wmax && wmax < INFINITY ? 1.f : 0.f;
+        }
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) {
             ss += __shfl_xor_sync(0xffffffffu, ss, off);

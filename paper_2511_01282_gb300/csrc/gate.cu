@@ -30,16 +30,17 @@ struct Ent3 {
     float m, s, w;
 };
 
+// How far a triple's maximum lies below the union's.  Bounded, so that its product
+// with s stays finite: a slice of masked logits (-FLT_MAX, say) has s = the number
+// of them, and 0 times infinity is no 0.
+__device__ __forceinline__ float ent_below(float m, float M) { return fmaxf(m - M, -1e30f); }
+
 __device__ __forceinline__ Ent3 ent_merge(Ent3 a, Ent3 b) {
     if (a.s == 0.f) return b;
     if (b.s == 0.f) return a;
-    float M = fmaxf(a.m, b.m);
-    float ca = __expf(a.m - M), cb = __expf(b.m - M);
-    Ent3 r;
-    r.m = M;
-    r.s = a.s * ca + b.s * cb;
-    r.w = ca * (a.w + a.s * (a.m - M)) + cb * (b.w + b.s * (b.m - M));
-    return r;
+    const float M = fmaxf(a.m, b.m), da = ent_below(a.m, M), db = ent_below(b.m, M);
+    const float ca = __expf(da), cb = __expf(db);
+    return Ent3{M, a.s * ca + b.s * cb, ca * (a.w + a.s * da) + cb * (b.w + b.s * db)};
 }
 
 // The triple of the union of one triple per lane, over aligned groups of G lanes
@@ -51,7 +52,7 @@ __device__ __forceinline__ Ent3 ent_union(Ent3 t) {
     float M = some ? t.m : -INFINITY;  // of a triple without mass m may be +inf
 #pragma unroll
     for (int o = G / 2; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
-    const float d = t.m - M, c = some ? __expf(d) : 0.f;
+    const float d = ent_below(t.m, M), c = some ? __expf(d) : 0.f;
     float s = some ? t.s * c : 0.f, w = some ? c * (t.w + t.s * d) : 0.f;
 #pragma unroll
     for (int o = G / 2; o > 0; o >>= 1) {

@@ -66,3 +66,35 @@ def test_a_slice_without_mass_counts_for_nothing(V):
             at = int(np.argmax(z[r]))
             rest[r, (ids // 8192 == at // 8192) & (ids % 8192 // lanes % 8 == at % 8192 // lanes % 8)] = -np.inf
         assert np.abs(got - oracle.entropy_rows(rest.astype(np.float32))).max() < 1e-3
+
+
+@pytest.mark.parametrize("V", SIZES)
+@pytest.mark.parametrize("mask", [-np.finfo(np.float32).max, -2.5e38, -1e30, -1e10, -1e9, -4e8, -65504])
+def test_masks_of_the_lowest_value(V, mask):
+    # masked ids in whole chunks, in whole slices of a warp, alone, and everywhere
+    # but at one id: they carry no mass, whatever the finite value
+    rng = np.random.default_rng(V)
+    z = (3 * rng.standard_normal((7, V))).astype(np.float32)
+    ids = np.arange(V)
+    z[0, max(1, V // 3):] = mask
+    z[1, :V - 5] = mask
+    z[2, ids // 128 % 8 != 3] = mask
+    z[3, ids % 3 != 1] = mask
+    z[4, ids != V // 2] = mask
+    z[5, :] = mask                       # nothing is left: a uniform row
+    z[6, ids % 2 == 0] = -np.inf
+    H = oracle.entropy_rows(z)
+    assert np.abs(gate_entropy(z) - H).max() < 1e-3
+    zd = z.astype(np.float64)
+    m = zd.max(1)
+    lse = m + np.log(np.exp(zd - m[:, None]).sum(1))
+    for with_entropy in (True, False):
+        o = accept_rows(z, with_entropy)
+        if with_entropy:
+            assert np.abs(o["entropy"].astype(np.float64) - H).max() < 1e-3
+        assert np.allclose(o["lse"].astype(np.float64), lse, rtol=1e-5, atol=1e-6)
+        p = np.exp(m[:-1] - lse[:-1])    # every node's token is its parent's best
+        got = o["p_tok"][1:].astype(np.float64)
+        assert np.allclose(np.delete(got, 5), np.delete(p, 5), rtol=1e-4, atol=1e-7)
+        assert 0 <= got[5] <= 1          # both logit and lse are the mask: ln V may be below its rounding
+        assert (o["argmax"] == z.argmax(1)).all()
