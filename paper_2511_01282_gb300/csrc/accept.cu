@@ -326,11 +326,6 @@ accept_rows(const float *logits, int V, int nchunks, int beta, VI *cand, MS *par
         }
         float ss = (s2[0].x + s2[0].y) + (s2[1].x + s2[1].y);
         float ww = (w2[0].x + w2[0].y) + (w2[1].x + w2[1].y);
-        if (fabsf(wmax) >= kFarLogit) {  // (a logit of +inf leaves no finite sum: no mass)
-            ss = ww = 0.f;
-#pragma unroll
-            for (int j = 0; j < kAccVpt; ++j) ss += v[j] == wmax && wmax < INFINITY ? 1.f : 0.f;
-        }
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) {
             ss += __shfl_xor_sync(0xffffffffu, ss, off);
@@ -338,6 +333,13 @@ accept_rows(const float *logits, int V, int nchunks, int beta, VI *cand, MS *par
         }
         t.s = ss;
         t.w = ww * 0.6931471805599453f;
+        if (fabsf(wmax) >= kFarLogit) {  // (a logit of +inf leaves no finite sum: no mass)
+            int n = 0;
+#pragma unroll
+            for (int j = 0; j < kAccVpt; ++j) n += __popc(__ballot_sync(0xffffffffu, v[j] == wmax));
+            t.s = wmax < INFINITY ? (float)n : 0.f;
+            t.w = 0.f;
+        }
     }
     if (lane == 0) sh.sms[warp] = t;
     __syncthreads();
