@@ -35,6 +35,30 @@ int num_sms() {
     return cache[dev];
 }
 
+unsigned long long context_id() {
+    typedef int (*ctx_get_current_t)(void **);
+    typedef int (*ctx_get_id_t)(void *, unsigned long long *);
+    static std::once_flag once;
+    static ctx_get_current_t get_current = nullptr;
+    static ctx_get_id_t get_id = nullptr;
+    std::call_once(once, [] {
+        void *a = nullptr, *b = nullptr;
+        cudaDriverEntryPointQueryResult qa, qb;
+        if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &a, 12000, cudaEnableDefault, &qa) ==
+                cudaSuccess && qa == cudaDriverEntryPointSuccess &&
+            cudaGetDriverEntryPointByVersion("cuCtxGetId", &b, 12000, cudaEnableDefault, &qb) == cudaSuccess &&
+            qb == cudaDriverEntryPointSuccess) {
+            get_current = reinterpret_cast<ctx_get_current_t>(a);
+            get_id = reinterpret_cast<ctx_get_id_t>(b);
+        }
+    });
+    if (!get_current || !get_id) return 0;
+    void *ctx = nullptr;
+    unsigned long long id = 0;
+    if (get_current(&ctx) != 0 || !ctx || get_id(ctx, &id) != 0) return 0;
+    return id;
+}
+
 long long l2_bytes() {
     static std::mutex mu;
     static long long cache[64] = {0};

@@ -108,6 +108,10 @@ struct Carve {
 
 int num_sms();  // SM count of the current device (cached per device)
 long long l2_bytes();  // L2 size of the current device (cached per device)
+// Unique id of the calling thread's current CUDA context (0 when it cannot be
+// read).  Context ids are never reused within a process, so a device reset or
+// another context on the same device gives a new id.
+unsigned long long context_id();
 
 // ---------------------------------------------------------------- device side
 // Let the next kernel start launching, then wait for the previous kernel.

@@ -837,6 +837,7 @@ index_append(const int32_t *tokens, const int64_t *tok_off, int V, IndexView ix,
 // is candidate 128 r + 32 e + l.
 struct ListSource {
     static constexpr int kRows = 2;
+    static constexpr int kThreads = kMatHalf, kFewB = 4;
     static constexpr int kWideRows = 128;  // 16384 candidates, each a read of its own
     static constexpr bool kLaneMajor = false;
     static constexpr bool kBound = false;  // (its code, 16 registers more, costs every query 0.4 us)
@@ -1065,7 +1066,7 @@ extern "C" rs_status rs_match_scan_indexed(const int32_t *tokens, const int64_t 
     IndexView ix;
     carve_index(const_cast<void *>(index), B, V, t_total, &ix);
     const MatOut o{count, pos, sel_pos, sel_len, spans, n_sel, status, p.theta_score, p.top_c, p.span_len, pos_cap};
-    static int attr_done[64] = {0};
-    return mat_launch("rs_match_scan_indexed", kMatHalf, attr_done, index_query, B, (cudaStream_t)stream, tokens, tok_off, V, k_star,
-                      gate_ok, scores, ix, o);
+    static MatWide wide;
+    return mat_launch<ListSource>("rs_match_scan_indexed", wide, index_query, B, (cudaStream_t)stream, tokens, tok_off, V, k_star,
+                                  gate_ok, scores, ix, o);
 }

@@ -17,28 +17,32 @@
 // What bounds it: a chain of dependent reads (offsets, key, candidates,
 // scores, spans) of about 0.5 us each and the barriers between them, then for
 // long buffers the reads of one request's SMs (~100 GB/s per SM), then, with
-// many requests, the CTAs an SM holds.  So calls of up to kMatFewB requests take
-// clusters of 16 CTAs (scans of 4 x 1M tokens: 25 us with 8, 17 with 16; more of
-// these clusters than GPCs run in turn: 8 requests 23.5 and 27.4 in an earlier form), of
-// which a request of fewer rows than its source's kWideRows uses 8; others
-// clusters of 8.  CTAs have 512 threads in the scans of up to kMatMidB requests,
-// whose reads in flight bound them (4 x 1M tokens: 17 us, 25 with 256), but
-// only 256 stay for a request of one round of these, and 256 are launched for
-// everything else: twice the warps at each barrier cost a query of 4 x 32K
-// tokens 0.7 of 5.2 us, a scan of 30000 positions 1.0 of 6.8.
+// many requests, the CTAs an SM holds.  So calls of few requests take clusters of
+// 16 CTAs (match_cluster), of which a request of fewer rows than its source's
+// kWideRows uses 8; others clusters of 8.  Scans do so while the GPU runs all of
+// them at once, which with 512 threads is 7 (5 and 7 requests of 200000 tokens
+// 9.5 and 12.5 us with 8 CTAs, 8.0 and 9.7 with 16; of 1M tokens 33 and 20; but 8
+// of 20000 tokens 5.6 and 9.3: the eighth waits), queries up to 4 requests (5 to 14
+// would gain 1 us of 7.6 for a text's common token, but short ones lose 0.1 of 4.8,
+// and 8 to 14 with many matches 0.4 of 13).  CTAs have 512 threads in the scans of
+// up to kMatMidB requests, whose reads in flight bound them (4 x 1M tokens: 17 us,
+// 25 with 256), but only 256 stay for a request of one round of these, and 256 are
+// launched for everything else: twice the warps at each barrier cost a query of
+// 4 x 32K tokens 0.7 of 5.2 us, a scan of 30000 positions 1.0 of 6.8.
 #pragma once
 
 #include <cooperative_groups.h>
 #include <math.h>
+#include <stdlib.h>
+
+#include <mutex>
 
 #include "common.cuh"
 #include "match_pos.h"
 
 namespace rs {
 
-constexpr int kMatCluster = 8;
-constexpr int kMatClusterMax = 16;
-constexpr int kMatFewB = 4, kMatMidB = 8;
+constexpr int kMatMidB = 8;
 constexpr int kMatThreads = 512, kMatHalf = kMatThreads / 2;
 constexpr int kMatWarps = kMatThreads / 32;
 constexpr int kMatCand = 512;             // matches ranked from the shared buffer
@@ -586,25 +590,53 @@ __device__ __forceinline__ int mat_ctas(int rows, int threads) {
     return nc > kMatCluster && rows < Src::kWideRows ? kMatCluster : nc;
 }
 
-// Launches a retrieval kernel over B requests; few_threads: the threads of a CTA
-// in calls of up to kMatMidB requests; attr_done: the caller's flags, one per
-// kernel and device.
-template <typename... KArgs, typename... Args>
-inline rs_status mat_launch(const char *who, int few_threads, int (&attr_done)[64], void (*kern)(KArgs...), int B, cudaStream_t st,
-                            Args... args) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev >= 0 && dev < 64 && !attr_done[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMatSmem);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        if (e != cudaSuccess) {
-            set_error("%s: cudaFuncSetAttribute: %s", who, cudaGetErrorString(e));
-            return RS_ERR_CUDA;
+static_assert(sizeof(MatShared) + kMatSmem <= 48 * 1024, "within what a kernel may use without asking");
+
+// How many clusters of kMatClusterMax CTAs the current context can run at once: 0
+// where it has no GPC of so many SMs (a part of a GPU).  Remembered with the
+// context's id, as the attribute that allows them goes with the context.
+// RS_DEBUG_MATCH_CLUSTER=8 (a test hook, read where this is asked) answers 0.
+class MatWide {
+    std::mutex mu_;
+    unsigned long long ctx_[64] = {};
+    int n_[64] = {};
+
+public:
+    int ask(const void *kern, int threads) {
+        int dev = -1;
+        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+        const unsigned long long id = context_id();
+        std::lock_guard<std::mutex> lk(mu_);
+        if (id != 0 && ctx_[dev] == id) return n_[dev];
+        int n = 0;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(kMatClusterMax);
+        cfg.blockDim = dim3(threads);
+        cfg.dynamicSmemBytes = kMatSmem;
+        cudaLaunchAttribute at;
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = kMatClusterMax;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
+            n = 0;
+            (void)cudaGetLastError();  // smaller clusters do as well
         }
-        attr_done[dev] = 1;
+        if (const char *e = getenv("RS_DEBUG_MATCH_CLUSTER"))
+            if (atoi(e) == kMatCluster) n = 0;
+        n_[dev] = n;
+        ctx_[dev] = context_id();  // the questions made the context current if it was not
+        return n;
     }
-    const int nc = B <= kMatFewB ? kMatClusterMax : kMatCluster;
-    const int threads = B <= kMatMidB ? few_threads : kMatHalf;
+};
+
+// Launches the retrieval kernel of a source over B requests; wide: the kernel's own.
+template <class Src, typename... KArgs, typename... Args>
+inline rs_status mat_launch(const char *who, MatWide &wide, void (*kern)(KArgs...), int B, cudaStream_t st, Args... args) {
+    const int nc = match_cluster(B, Src::kFewB, B <= Src::kFewB ? wide.ask(reinterpret_cast<const void *>(kern), Src::kThreads) : 0);
+    const int threads = B <= kMatMidB ? Src::kThreads : kMatHalf;
     launch_pdl_cluster(kern, dim3(nc, B), dim3(threads), kMatSmem, st, nc, args...);
     RS_CHECK_LAUNCH(who);
     return RS_OK;

@@ -16,6 +16,14 @@ namespace rs {
 
 constexpr long long kMatMaxTokens = 0x7fffffff;
 
+constexpr int kMatCluster = 8;        // the portable cluster size
+constexpr int kMatClusterMax = 16;
+
+// CTAs of a request's cluster in a call over B requests; few: the kernel's own
+// limit for clusters of 16; wide: how many of these the context can run at once
+// (more would run in turn).
+RS_HD int match_cluster(int B, int few, int wide) { return B <= few && B <= wide ? kMatClusterMax : kMatCluster; }
+
 // A scan's candidates: the buffer's positions, as quads of four on 16-byte
 // boundaries.  t: tokens, al: positions that the buffer begins past a boundary.
 // Unsigned: a position in front of the buffer wraps to a number past every buffer,

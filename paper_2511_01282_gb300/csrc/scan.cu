@@ -22,6 +22,7 @@ struct ScanSource {
     // (eight rows: 2 x 1.3M tokens 17.6 us instead of 18.8, but every call of a
     // round or two 1.2 us longer)
     static constexpr int kRows = 4;
+    static constexpr int kThreads = kMatThreads, kFewB = kMatMidB;
     static constexpr int kWideRows = 1024;  // 131072 positions: below, 8 CTAs are as fast as 16
     static constexpr bool kLaneMajor = true;
     static constexpr bool kBound = true;
@@ -122,7 +123,7 @@ extern "C" rs_status rs_match_scan(const int32_t *tokens, const int64_t *tok_off
                  "rs_match_scan: null pointer");
     if (B == 0) return RS_OK;
     const MatOut o{count, pos, sel_pos, sel_len, spans, n_sel, status, p.theta_score, p.top_c, p.span_len, pos_cap};
-    static int attr_done[64] = {0};
-    return mat_launch("rs_match_scan", kMatThreads, attr_done, match_scan_kernel, B, (cudaStream_t)stream, tokens, tok_off, k_star, gate_ok,
-                      scores, o);
+    static MatWide wide;
+    return mat_launch<ScanSource>("rs_match_scan", wide, match_scan_kernel, B, (cudaStream_t)stream, tokens, tok_off, k_star, gate_ok,
+                                  scores, o);
 }

@@ -50,6 +50,12 @@ int main() {
                 if (l.in((int)row, o)) CHECK(l.number((int)row, o) == c);
             }
     }
+    {  // clusters of 16 where the context can run all of the call's at once
+        long long t = 0, al = 0, row = 0; int lane = 0, k = 0;
+        CHECK(match_cluster(1, 4, 7) == 16 && match_cluster(4, 4, 7) == 16 && match_cluster(5, 4, 7) == 8);
+        CHECK(match_cluster(7, 8, 7) == 16 && match_cluster(8, 8, 7) == 8 && match_cluster(4, 8, 3) == 8);
+        CHECK(match_cluster(1, 4, 0) == 8 && match_cluster(1, 8, 0) == 8);
+    }
     printf("bad %d\n", bad);
     return bad != 0;
 }
