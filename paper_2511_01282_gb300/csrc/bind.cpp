@@ -8,8 +8,9 @@
 // GB300 (0.23 us a tensor for three attribute calls, 2.9 us to build a stream
 // object, 1.8 us of conversions), more than some of the kernels behind it.
 //
-// Integers and floats are converted as ctypes converts them (an int wraps to
-// the C type; anything else is refused).
+// Arguments are converted as ctypes converts them: an int wraps to the C type, an
+// instance of the C type or an object whose _as_parameter_ is one will do, and
+// anything else is refused.  A tensor subclass answers for itself.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 #include <c10/cuda/CUDAStream.h>
@@ -24,8 +25,20 @@
 namespace {
 
 PyObject *g_params_type = nullptr, *g_argument_error = nullptr;
+PyObject *g_c_int = nullptr, *g_c_int64 = nullptr, *g_c_float = nullptr, *g_c_void_p = nullptr;  // ctypes' types
 
 struct PyFail {};  // a Python exception is set
+
+// A reference of our own.
+struct Ref {
+    PyObject *o;
+    explicit Ref(PyObject *x) : o(x) {
+        if (!o) throw PyFail{};
+    }
+    ~Ref() { Py_DECREF(o); }
+    Ref(const Ref &) = delete;
+    Ref &operator=(const Ref &) = delete;
+};
 
 // The arguments of one call, taken in order.
 struct Args {
@@ -42,10 +55,44 @@ struct Args {
         PyErr_Format(g_argument_error, "argument %zd: TypeError: %s instead of %s instance", i, what, Py_TYPE(o)->tp_name);
         throw PyFail{};
     }
+    // What stands for o where plain(o) does not hold: the first of o,
+    // o._as_parameter_ ... that is an instance of the ctypes type or plain.
+    // use(x, is_instance) makes the result of it.
+    template <class Plain, class Use>
+    auto stand_in(PyObject *o, PyObject *type, const char *what, Plain plain, Use use) {
+        PyObject *x = Py_NewRef(o);
+        for (int depth = 0;; ++depth) {
+            const Ref own(x);
+            const int is = PyObject_IsInstance(x, type);
+            if (is < 0) throw PyFail{};
+            if (is || plain(x)) return use(x, is != 0);
+            x = depth < 64 ? PyObject_GetAttrString(x, "_as_parameter_") : nullptr;
+            if (!x) {
+                PyErr_Clear();
+                refuse(what, o);
+            }
+        }
+    }
+    // The same for numbers: use(x) with x or an instance's value.
+    template <class Plain, class Use>
+    auto number_for(PyObject *o, PyObject *type, const char *what, Plain plain, Use use) {
+        return stand_in(o, type, what, plain, [use](PyObject *x, bool instance) {
+            if (!instance) return use(x);
+            const Ref v(PyObject_GetAttrString(x, "value"));
+            return use(v.o);
+        });
+    }
+    // A handle: None, an int, a c_void_p or what stands for one.
+    void *handle(PyObject *h, const char *what) {
+        auto plain = [](PyObject *x) { return x == Py_None || PyLong_Check(x); };
+        auto use = [this](PyObject *x) { return x == Py_None ? nullptr : reinterpret_cast<void *>(masked(x)); };
+        if (plain(h)) return use(h);
+        return number_for(h, g_c_void_p, what, plain, use);
+    }
     // The address of a tensor, or of an object with a tensor's attributes; its
     // bytes too where asked for.
     void *address(PyObject *o, size_t *bytes) {
-        if (THPVariable_Check(o)) {
+        if (THPVariable_CheckExact(o)) {
             const at::Tensor &t = THPVariable_Unpack(o);
             check(t.is_cuda(), t.is_contiguous(), o);
             if (bytes) *bytes = (size_t)t.numel() * (size_t)t.element_size();
@@ -56,7 +103,8 @@ struct Args {
         if (bytes)
             *bytes = (size_t)(number(PyObject_CallMethod(o, "numel", nullptr)) *
                               number(PyObject_CallMethod(o, "element_size", nullptr)));
-        return reinterpret_cast<void *>(number(PyObject_CallMethod(o, "data_ptr", nullptr)));
+        const Ref p(PyObject_CallMethod(o, "data_ptr", nullptr));
+        return handle(p.o, "address expected");
     }
     void check(bool cuda, bool contiguous, PyObject *o) {
         if (!cuda) {
@@ -71,10 +119,11 @@ struct Args {
         }
     }
     unsigned long long number(PyObject *x) {  // takes the reference
-        if (!x) throw PyFail{};
-        const unsigned long long r = PyLong_Check(x) ? PyLong_AsUnsignedLongLongMask(x) : (unsigned long long)PyObject_IsTrue(x);
-        Py_DECREF(x);
-        return r;
+        const Ref own(x);
+        if (PyLong_Check(x)) return masked(x);
+        const int yes = PyObject_IsTrue(x);
+        if (yes < 0) throw PyFail{};
+        return (unsigned long long)yes;
     }
     template <class T>
     T *ptr() {
@@ -88,28 +137,43 @@ struct Args {
         if (x == (unsigned long long)-1 && PyErr_Occurred()) throw PyFail{};
         return x;
     }
-    long long i64() {
+    long long i64() { return integer(g_c_int64); }
+    int i32() { return (int)integer(g_c_int); }
+    long long integer(PyObject *type) {
         PyObject *o = next();
-        if (!PyLong_Check(o)) refuse("int expected", o);
-        return (long long)masked(o);
+        if (PyLong_Check(o)) return (long long)masked(o);
+        return number_for(o, type, "int expected", [](PyObject *x) { return PyLong_Check(x) != 0; },
+                          [this](PyObject *x) { return (long long)masked(x); });
     }
-    int i32() { return (int)i64(); }
+    // whether x converts to a double, without an exception
+    static bool real(PyObject *x, double *d) {
+        *d = PyFloat_AsDouble(x);
+        if (*d != -1.0 || !PyErr_Occurred()) return true;
+        PyErr_Clear();
+        return false;
+    }
     float f32() {
         PyObject *o = next();
-        const double x = PyFloat_AsDouble(o);
-        if (x == -1.0 && PyErr_Occurred()) {
-            PyErr_Clear();
-            refuse("float expected", o);
-        }
-        return (float)x;
+        double d;
+        if (real(o, &d)) return (float)d;
+        return number_for(o, g_c_float, "float expected",
+                          [](PyObject *x) {
+                              double y;
+                              return real(x, &y);
+                          },
+                          [](PyObject *x) {
+                              double y;
+                              real(x, &y);
+                              return (float)y;
+                          });
     }
     rs_params params() {
-        PyObject *o = next();
-        const int is = PyObject_IsInstance(o, g_params_type);
-        if (is < 0) throw PyFail{};
-        if (!is) refuse("expected rs_params", o);
+        return stand_in(next(), g_params_type, "expected rs_params", [](PyObject *) { return false; },
+                        [](PyObject *x, bool) { return params_of(x); });
+    }
+    static rs_params params_of(PyObject *x) {
         Py_buffer b;
-        if (PyObject_GetBuffer(o, &b, PyBUF_SIMPLE) != 0) throw PyFail{};
+        if (PyObject_GetBuffer(x, &b, PyBUF_SIMPLE) != 0) throw PyFail{};
         rs_params p;
         const bool fits = b.len == (Py_ssize_t)sizeof p;
         if (fits) memcpy(&p, b.buf, sizeof p);
@@ -131,14 +195,8 @@ struct Args {
         PyObject *o = next();
         if (o == Py_None) return c10::cuda::getCurrentCUDAStream().stream();
         if (PyLong_Check(o)) return reinterpret_cast<void *>(masked(o));
-        PyObject *h = PyObject_GetAttrString(o, "cuda_stream");
-        if (!h) throw PyFail{};
-        unsigned long long x = 0;
-        const bool ok = PyLong_Check(h);
-        if (ok) x = PyLong_AsUnsignedLongLongMask(h);
-        Py_DECREF(h);
-        if (!ok) refuse("stream handle expected", o);
-        return reinterpret_cast<void *>(x);
+        const Ref h(PyObject_GetAttrString(o, "cuda_stream"));
+        return handle(h.o, "stream handle expected");
     }
 };
 
@@ -394,8 +452,12 @@ PyMODINIT_FUNC PyInit__respec_bind() {
     PyObject *ctypes = PyImport_ImportModule("ctypes");
     if (!ctypes) return nullptr;
     g_argument_error = PyObject_GetAttrString(ctypes, "ArgumentError");
+    g_c_int = PyObject_GetAttrString(ctypes, "c_int");
+    g_c_int64 = PyObject_GetAttrString(ctypes, "c_int64");
+    g_c_float = PyObject_GetAttrString(ctypes, "c_float");
+    g_c_void_p = PyObject_GetAttrString(ctypes, "c_void_p");
     Py_DECREF(ctypes);
-    if (!g_argument_error) return nullptr;
+    if (!g_argument_error || !g_c_int || !g_c_int64 || !g_c_float || !g_c_void_p) return nullptr;
     PyObject *m = PyModule_Create(&kModule);
     if (m && PyModule_AddStringConstant(m, "torch_version", TORCH_VERSION) != 0) Py_CLEAR(m);
     return m;
