@@ -90,11 +90,13 @@ def build(force=False, verbose=False, extra_flags=()):
     if jobs:
         with cf.ThreadPoolExecutor(max_workers=min(len(jobs), os.cpu_count() or 4)) as ex:
             list(ex.map(run, jobs))
-    if force or jobs or _stale(LIB, objs):
+    if force or jobs or _stale(LIB, objs + [__file__]):
         tmp = LIB + ".tmp.%d" % os.getpid()
-        run([nvcc] + ARCH + ["-shared", "-o", tmp] + objs)
+        # by its name the binding finds it where respec.py has already loaded it,
+        # whatever else of that file name is on the loader's path
+        run([nvcc] + ARCH + ["-shared", "-Xlinker", "-soname=" + os.path.basename(LIB), "-o", tmp] + objs)
         os.replace(tmp, LIB)
-    if force or _stale(BIND, [bind_obj]):
+    if force or _stale(BIND, [bind_obj, __file__]):
         tmp = BIND + ".tmp.%d" % os.getpid()
         run(["g++", "-shared", "-o", tmp, bind_obj, "-L", HERE, "-l:" + os.path.basename(LIB), "-L", torch_lib,
              "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda", "-Wl,-rpath,$ORIGIN",
