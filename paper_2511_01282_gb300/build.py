@@ -4,7 +4,8 @@ Each CUDA translation unit under ``csrc/`` is compiled in parallel with nvcc,
 then linked into one shared library next to this file.  The CUDA runtime is
 linked statically, so the library needs only the driver at run time.
 ``csrc/bind.cpp`` (the marshalling of ``respec.py``) is compiled beside them
-with g++ against the installed torch and linked to the library.
+with g++ against the installed torch; it gets the library's entry points from
+``respec.py``, which loads the library by its path.
 """
 import concurrent.futures as cf
 import importlib.util
@@ -92,15 +93,12 @@ def build(force=False, verbose=False, extra_flags=()):
             list(ex.map(run, jobs))
     if force or jobs or _stale(LIB, objs + [__file__]):
         tmp = LIB + ".tmp.%d" % os.getpid()
-        # by its name the binding finds it where respec.py has already loaded it,
-        # whatever else of that file name is on the loader's path
-        run([nvcc] + ARCH + ["-shared", "-Xlinker", "-soname=" + os.path.basename(LIB), "-o", tmp] + objs)
+        run([nvcc] + ARCH + ["-shared", "-o", tmp] + objs)
         os.replace(tmp, LIB)
     if force or _stale(BIND, [bind_obj, __file__]):
         tmp = BIND + ".tmp.%d" % os.getpid()
-        run(["g++", "-shared", "-o", tmp, bind_obj, "-L", HERE, "-l:" + os.path.basename(LIB), "-L", torch_lib,
-             "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda", "-Wl,-rpath,$ORIGIN",
-             "-Wl,-rpath," + torch_lib])
+        run(["g++", "-shared", "-o", tmp, bind_obj, "-L", torch_lib, "-ltorch_python", "-ltorch",
+             "-ltorch_cpu", "-lc10", "-lc10_cuda", "-Wl,-rpath," + torch_lib])
         os.replace(tmp, BIND)
     return LIB
 

@@ -22,10 +22,22 @@
 
 #include "respec.h"
 
+#define RS_ENTRIES(X)                                                                                            \
+    X(entropy_gate) X(entropy_gate_noalloc) X(entropy_gate_rows) X(match_scan) X(tree_verify_attn) X(accept)     \
+    X(match_index_build) X(match_index_append) X(match_scan_indexed) X(tree_sample)
+
 namespace {
 
 PyObject *g_params_type = nullptr, *g_argument_error = nullptr;
 PyObject *g_c_int = nullptr, *g_c_int64 = nullptr, *g_c_float = nullptr, *g_c_void_p = nullptr;  // ctypes' types
+
+// The library's entry points, as respec.py has loaded them: linked by file name the
+// loader might find another librespec.so first.
+struct Library {
+#define RS_ENTRY(name) decltype(&rs_##name) name = nullptr;
+    RS_ENTRIES(RS_ENTRY)
+#undef RS_ENTRY
+} lib;
 
 struct PyFail {};  // a Python exception is set
 
@@ -242,7 +254,7 @@ RS_BIND(entropy_gate) {
         size_t wb;
         void *ws = a.sized(&wb, true), *st = a.stream();
         return [=] {
-            return rs_entropy_gate(logits, R, V, row_off, row_commit, B, p, hist, hist_n, entropy, k_star, h_best, ok, ws, wb, st);
+            return lib.entropy_gate(logits, R, V, row_off, row_commit, B, p, hist, hist_n, entropy, k_star, h_best, ok, ws, wb, st);
         };
     });
 }
@@ -263,7 +275,7 @@ RS_BIND(entropy_gate_noalloc) {
         auto *ok = a.ptr<uint8_t>();
         void *st = a.stream();
         return [=] {
-            return rs_entropy_gate_noalloc(logits, R, V, row_off, row_commit, B, p, hist, hist_n, entropy, k_star, h_best, ok, st);
+            return lib.entropy_gate_noalloc(logits, R, V, row_off, row_commit, B, p, hist, hist_n, entropy, k_star, h_best, ok, st);
         };
     });
 }
@@ -281,7 +293,7 @@ RS_BIND(entropy_gate_rows) {
         auto *h_best = a.ptr<float>();
         auto *ok = a.ptr<uint8_t>();
         void *st = a.stream();
-        return [=] { return rs_entropy_gate_rows(entropy, row_off, row_commit, B, p, hist, hist_n, k_star, h_best, ok, st); };
+        return [=] { return lib.entropy_gate_rows(entropy, row_off, row_commit, B, p, hist, hist_n, k_star, h_best, ok, st); };
     });
 }
 
@@ -300,7 +312,7 @@ RS_BIND(match_scan) {
         size_t wb;
         void *ws = a.sized(&wb, true), *st = a.stream();
         return [=] {
-            return rs_match_scan(tokens, tok_off, B, k_star, gate_ok, scores, p, cap, count, pos, sel_pos, sel_len, spans, n_sel,
+            return lib.match_scan(tokens, tok_off, B, k_star, gate_ok, scores, p, cap, count, pos, sel_pos, sel_len, spans, n_sel,
                                  status, ws, wb, st);
         };
     });
@@ -319,7 +331,7 @@ RS_BIND(tree_verify_attn) {
         size_t wb;
         void *ws = a.sized(&wb, true), *st = a.stream();
         return [=] {
-            return rs_tree_verify_attn(q, k, vv, kv_rows, kv_off, ctx_len, node_off, parents, B, R, Hq, Hkv, D, scale, out, lse,
+            return lib.tree_verify_attn(q, k, vv, kv_rows, kv_off, ctx_len, node_off, parents, B, R, Hq, Hkv, D, scale, out, lse,
                                        status, ws, wb, st);
         };
     });
@@ -347,7 +359,7 @@ RS_BIND(accept) {
         size_t wb;
         void *ws = a.sized(&wb, true), *st = a.stream();
         return [=] {
-            return rs_accept(logits, R, V, node_off, B, tokens, parents, source, chain, sel_pos, tok_off, p, cap, argmax, topk, lse,
+            return lib.accept(logits, R, V, node_off, B, tokens, parents, source, chain, sel_pos, tok_off, p, cap, argmax, topk, lse,
                              p_tok, entropy, acc_len, acc_nodes, bonus, winner, commit, scores, status, ws, wb, st);
         };
     });
@@ -361,7 +373,7 @@ RS_BIND(match_index_build) {
         const int64_t total = a.i64();
         size_t ib;
         void *index = a.sized(&ib, false), *st = a.stream();
-        return [=] { return rs_match_index_build(tokens, tok_off, B, V, total, index, ib, st); };
+        return [=] { return lib.match_index_build(tokens, tok_off, B, V, total, index, ib, st); };
     });
 }
 
@@ -375,7 +387,7 @@ RS_BIND(match_index_append) {
         void *index = a.sized(&ib, false);
         auto *status = a.ptr<int32_t>();
         void *st = a.stream();
-        return [=] { return rs_match_index_append(tokens, tok_off, B, V, total, index, ib, status, st); };
+        return [=] { return lib.match_index_append(tokens, tok_off, B, V, total, index, ib, status, st); };
     });
 }
 
@@ -396,7 +408,7 @@ RS_BIND(match_scan_indexed) {
         size_t ib;
         void *index = a.sized(&ib, false), *st = a.stream();
         return [=] {
-            return rs_match_scan_indexed(tokens, tok_off, B, k_star, gate_ok, scores, p, cap, count, pos, sel_pos, sel_len, spans,
+            return lib.match_scan_indexed(tokens, tok_off, B, k_star, gate_ok, scores, p, cap, count, pos, sel_pos, sel_len, spans,
                                          n_sel, status, V, total, index, ib, st);
         };
     });
@@ -418,31 +430,37 @@ RS_BIND(tree_sample) {
         size_t wb;
         void *ws = a.sized(&wb, true), *st = a.stream();
         return [=] {
-            return rs_tree_sample(logits, R, V, node_off, B, tokens, parents, source, T, uniforms, cap, draw, acc_len, acc_nodes,
+            return lib.tree_sample(logits, R, V, node_off, B, tokens, parents, source, T, uniforms, cap, draw, acc_len, acc_nodes,
                                   bonus, status, ws, wb, st);
         };
     });
 }
 
-// setup(rs_params type): the type the params argument must have.
-PyObject *setup(PyObject *, PyObject *type) {
+// setup(rs_params type, {name: address of rs_name}): the type the params argument
+// must have and the library's entry points.
+PyObject *setup(PyObject *, PyObject *args) {
+    PyObject *type, *entries;
+    if (!PyArg_ParseTuple(args, "OO!", &type, &PyDict_Type, &entries)) return nullptr;
+    Library l;
+#define RS_ENTRY(name)                                                                              \
+    if (PyObject *a = PyDict_GetItemString(entries, "rs_" #name))                                   \
+        l.name = reinterpret_cast<decltype(l.name)>(PyLong_AsVoidPtr(a));                           \
+    if (!l.name) {                                                                                  \
+        if (!PyErr_Occurred()) PyErr_SetString(PyExc_KeyError, "rs_" #name);                        \
+        return nullptr;                                                                             \
+    }
+    RS_ENTRIES(RS_ENTRY)
+#undef RS_ENTRY
+    lib = l;
     Py_INCREF(type);
     Py_XSETREF(g_params_type, type);
     Py_RETURN_NONE;
 }
 
 #define RS_METHOD(name) {"rs_" #name, reinterpret_cast<PyCFunction>(reinterpret_cast<void *>(name)), METH_FASTCALL, nullptr}
-PyMethodDef kMethods[] = {RS_METHOD(entropy_gate),
-                          RS_METHOD(entropy_gate_noalloc),
-                          RS_METHOD(entropy_gate_rows),
-                          RS_METHOD(match_scan),
-                          RS_METHOD(tree_verify_attn),
-                          RS_METHOD(accept),
-                          RS_METHOD(match_index_build),
-                          RS_METHOD(match_index_append),
-                          RS_METHOD(match_scan_indexed),
-                          RS_METHOD(tree_sample),
-                          {"setup", setup, METH_O, nullptr},
+#define RS_ENTRY(name) RS_METHOD(name),
+PyMethodDef kMethods[] = {RS_ENTRIES(RS_ENTRY)
+                          {"setup", setup, METH_VARARGS, nullptr},
                           {nullptr, nullptr, 0, nullptr}};
 PyModuleDef kModule = {PyModuleDef_HEAD_INIT, "_respec_bind", nullptr, -1, kMethods, nullptr, nullptr, nullptr, nullptr};
 

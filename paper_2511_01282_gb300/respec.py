@@ -109,7 +109,7 @@ def _native():
     """The C++ marshalling module, built in-tree beside the library."""
     global _bind
     if _bind is None:
-        lib()
+        L = lib()
         if not os.path.exists(BIND_PATH):
             raise RuntimeError("_respec_bind.so is not built: run paper_2511_01282_gb300.build.build() "
                                "(or __graft_entry__.build())")
@@ -119,7 +119,7 @@ def _native():
         if not torch.__version__.startswith(m.torch_version):
             raise RuntimeError("_respec_bind.so was built for torch %s, this is %s: rebuild it"
                                % (m.torch_version, torch.__version__))
-        m.setup(rs_params)
+        m.setup(rs_params, {name: C.cast(getattr(L, name), _P).value for name in _SIGS})
         _bind = m
     return _bind
 
