@@ -56,6 +56,18 @@ def _stale(target, deps):
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def _read(path):
+    if not os.path.exists(path):
+        return None
+    with open(path) as f:
+        return f.read()
+
+
+def _write(path, text):
+    with open(path, "w") as f:
+        f.write(text)
+
+
 def build(force=False, verbose=False, extra_flags=()):
     nvcc = _nvcc()
     os.makedirs(BUILD, exist_ok=True)
@@ -74,7 +86,12 @@ def build(force=False, verbose=False, extra_flags=()):
     torch_lib = os.path.join(torch_dir, "lib")
     cuda_include = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc))), "include")
     bind_obj = os.path.join(BUILD, "bind.o")
-    if force or _stale(bind_obj, [BIND_SRC, os.path.join(torch_dir, "version.py")] + hdrs):
+    # the torch that the binding is for, by path and version (an older one that is
+    # installed later has older files)
+    stamp = os.path.join(BUILD, "bind.torch")
+    torch_is = torch_dir + "\n" + (_read(os.path.join(torch_dir, "version.py")) or "")
+    rebind = force or _read(stamp) != torch_is or _stale(bind_obj, [BIND_SRC] + hdrs)
+    if rebind:
         jobs.append(["g++", "-O2", "-std=c++17", "-fPIC", "-I", INCLUDE, "-I", sysconfig.get_paths()["include"],
                      "-I", os.path.join(torch_dir, "include"),
                      "-I", os.path.join(torch_dir, "include", "torch", "csrc", "api", "include"),
@@ -91,15 +108,16 @@ def build(force=False, verbose=False, extra_flags=()):
     if jobs:
         with cf.ThreadPoolExecutor(max_workers=min(len(jobs), os.cpu_count() or 4)) as ex:
             list(ex.map(run, jobs))
-    if force or jobs or _stale(LIB, objs + [__file__]):
+    if force or any(j[0] == nvcc for j in jobs) or _stale(LIB, objs + [__file__]):
         tmp = LIB + ".tmp.%d" % os.getpid()
         run([nvcc] + ARCH + ["-shared", "-o", tmp] + objs)
         os.replace(tmp, LIB)
-    if force or _stale(BIND, [bind_obj, __file__]):
+    if rebind or _stale(BIND, [bind_obj, __file__]):
         tmp = BIND + ".tmp.%d" % os.getpid()
         run(["g++", "-shared", "-o", tmp, bind_obj, "-L", torch_lib, "-ltorch_python", "-ltorch",
              "-ltorch_cpu", "-lc10", "-lc10_cuda", "-Wl,-rpath," + torch_lib])
         os.replace(tmp, BIND)
+        _write(stamp, torch_is)
     return LIB
 
 

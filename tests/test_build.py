@@ -26,3 +26,23 @@ def test_the_binding_calls_the_library_beside_it(tmp_path):
     path = str(tmp_path) + os.pathsep + os.environ.get("LD_LIBRARY_PATH", "")
     r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, env=dict(os.environ, LD_LIBRARY_PATH=path), capture_output=True, text=True)
     assert r.returncode == 0, r.stderr[-1500:]
+
+
+def test_another_torch_rebuilds_the_binding(monkeypatch, tmp_path):
+    # files of an older torch that is installed later are older than the binding
+    made = []
+    real = subprocess.run
+    monkeypatch.setattr(build.subprocess, "run", lambda cmd, **kw: made.append(cmd) or real(["true"], **kw))
+    monkeypatch.setattr(build.os, "replace", lambda a, b: None)
+    monkeypatch.setattr(build, "_write", lambda path, text: None)
+    build.build()
+    assert not made                                   # nothing to do
+    other = tmp_path / "torch"
+    (other / "include").mkdir(parents=True)
+    (other / "version.py").write_text("__version__ = '2.0.0'\n")
+    os.utime(other / "version.py", (0, 0))
+    monkeypatch.setattr(build, "_torch_dir", lambda: str(other))
+    build.build()
+    assert any(build.BIND_SRC in c for c in made) and any(str(other / "include") in c for c in made)
+    assert any("-shared" in c and any(a.startswith(build.BIND) for a in c) for c in made)
+    assert not any(c[0].endswith("nvcc") for c in made)
