@@ -5,7 +5,8 @@ then linked into one shared library next to this file.  The CUDA runtime is
 linked statically, so the library needs only the driver at run time.
 ``csrc/bind.cpp`` (the marshalling of ``respec.py``) is compiled beside them
 with g++ against the installed torch; it gets the library's entry points from
-``respec.py``, which loads the library by its path.
+``respec.py``, which loads the library by its path.  Without torch only the
+library is built (for callers of the C ABI).
 """
 import concurrent.futures as cf
 import importlib.util
@@ -35,9 +36,7 @@ def _nvcc():
 
 def _torch_dir():
     spec = importlib.util.find_spec("torch")
-    if spec is None:
-        raise RuntimeError("torch not found")
-    return list(spec.submodule_search_locations)[0]
+    return None if spec is None else list(spec.submodule_search_locations)[0]
 
 
 def sources():
@@ -83,14 +82,13 @@ def build(force=False, verbose=False, extra_flags=()):
             jobs.append([nvcc] + flags + ["-c", src, "-o", obj])
 
     torch_dir = _torch_dir()
-    torch_lib = os.path.join(torch_dir, "lib")
     cuda_include = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc))), "include")
     bind_obj = os.path.join(BUILD, "bind.o")
     # the torch that the binding is for, by path and version (an older one that is
     # installed later has older files)
     stamp = os.path.join(BUILD, "bind.torch")
-    torch_is = torch_dir + "\n" + (_read(os.path.join(torch_dir, "version.py")) or "")
-    rebind = force or _read(stamp) != torch_is or _stale(bind_obj, [BIND_SRC] + hdrs)
+    torch_is = torch_dir and torch_dir + "\n" + (_read(os.path.join(torch_dir, "version.py")) or "")
+    rebind = torch_dir and (force or _read(stamp) != torch_is or _stale(bind_obj, [BIND_SRC] + hdrs))
     if rebind:
         jobs.append(["g++", "-O2", "-std=c++17", "-fPIC", "-I", INCLUDE, "-I", sysconfig.get_paths()["include"],
                      "-I", os.path.join(torch_dir, "include"),
@@ -112,8 +110,9 @@ def build(force=False, verbose=False, extra_flags=()):
         tmp = LIB + ".tmp.%d" % os.getpid()
         run([nvcc] + ARCH + ["-shared", "-o", tmp] + objs)
         os.replace(tmp, LIB)
-    if rebind or _stale(BIND, [bind_obj, __file__]):
+    if torch_dir and (rebind or _stale(BIND, [bind_obj, __file__])):
         tmp = BIND + ".tmp.%d" % os.getpid()
+        torch_lib = os.path.join(torch_dir, "lib")
         run(["g++", "-shared", "-o", tmp, bind_obj, "-L", torch_lib, "-ltorch_python", "-ltorch",
              "-ltorch_cpu", "-lc10", "-lc10_cuda", "-Wl,-rpath," + torch_lib])
         os.replace(tmp, BIND)

@@ -46,3 +46,8 @@ def test_another_torch_rebuilds_the_binding(monkeypatch, tmp_path):
     assert any(build.BIND_SRC in c for c in made) and any(str(other / "include") in c for c in made)
     assert any("-shared" in c and any(a.startswith(build.BIND) for a in c) for c in made)
     assert not any(c[0].endswith("nvcc") for c in made)
+
+
+def test_the_library_builds_without_torch(monkeypatch):
+    monkeypatch.setattr(build.importlib.util, "find_spec", lambda name: None)
+    assert build.build() == build.LIB and os.path.exists(build.LIB)
