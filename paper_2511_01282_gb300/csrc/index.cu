@@ -1015,7 +1015,7 @@ extern "C" rs_status rs_match_index_build(const int32_t *tokens, const int64_t *
     clear_error();
     const rs_status e = check_index("rs_match_index_build", B, V, t_total, index, index_bytes_avail);
     if (e != RS_OK) return e;
-    RS_CHECK_ARG(B == 0 || (tokens && tok_off) || t_total == 0, "rs_match_index_build: null pointer");
+    RS_CHECK_ARG(B == 0 || (tok_off && (tokens || t_total == 0)), "rs_match_index_build: null pointer");
     if (B == 0) return RS_OK;
     cudaStream_t st = (cudaStream_t)stream;
     IndexView ix;

@@ -90,3 +90,26 @@ def test_subclasses_answer_for_themselves(rs):  # noqa: F811
     _scan(rs, tokens=torch.zeros(4, dtype=torch.int32).as_subclass(Sub))
     with pytest.raises(ValueError, match="CUDA"):  # a Parameter is a plain tensor
         _scan(rs, tokens=torch.nn.Parameter(torch.zeros(4)))
+
+
+def test_an_index_of_no_tokens_still_needs_its_offsets(rs):  # noqa: F811
+    # the build reads them on the device whatever the total
+    class Index:
+        is_cuda, device = True, "like"
+
+        def is_contiguous(self):
+            return True
+
+        def data_ptr(self):
+            return 4096
+
+        def numel(self):
+            return 1 << 30
+
+        def element_size(self):
+            return 1
+
+    with pytest.raises(rs.RespecError, match="null pointer") as e:
+        rs.rs_match_index_build(None, None, 1, 4, 0, Index(), stream=0)
+    assert e.value.status == rs.RS_ERR_INVALID_ARG
+    rs.rs_match_index_build(None, None, 0, 4, 0, Index(), stream=0)
