@@ -214,10 +214,12 @@ __device__ __forceinline__ uint32_t mat_rows(const Src &src, const MatReq &q, in
     const int lane = threadIdx.x & 31;
     const uint32_t hits = src.test(q, r0, end, lane);
     uint32_t mine = 0;
+    if (!Src::kSparse || __any_sync(0xffffffffu, hits != 0)) {
 #pragma unroll
-    for (int j = 0; j < 4 * Src::kRows; ++j) {
-        const uint32_t bal = __ballot_sync(0xffffffffu, (hits >> j) & 1u);
-        mine = lane == j ? bal : mine;
+        for (int j = 0; j < 4 * Src::kRows; ++j) {
+            const uint32_t bal = __ballot_sync(0xffffffffu, (hits >> j) & 1u);
+            mine = lane == j ? bal : mine;
+        }
     }
     if (lane < 4 * Src::kRows && r0 + (lane >> 2) < end && r0 - base + (lane >> 2) < kMatBitRows) bits[4 * (r0 - base) + lane] = mine;
     return hits;
@@ -329,9 +331,8 @@ __device__ __forceinline__ void mat_body(const Src &src, const MatReq &q, int ro
         cnt += __popc(hits);
         // their scores, four of each lane at once; one slot count per warp and
         // round.  Once the buffer has run over, its contents count no more
-        for (uint32_t rem = hits;;) {
-            const bool over = *(volatile int *)&sh.ccnt > kMatCand;
-            if (!__any_sync(0xffffffffu, rem != 0 && !over)) break;
+        for (uint32_t rem = hits; __any_sync(0xffffffffu, rem != 0);) {
+            if (__any_sync(0xffffffffu, *(volatile int *)&sh.ccnt > kMatCand)) break;
             int p[4], at[4], n = 0;
             float s[4];
             bool pass[4];
@@ -508,7 +509,7 @@ __device__ __forceinline__ void mat_body(const Src &src, const MatReq &q, int ro
     auto none = [](int) { return 0.f; };
     auto put = [&](int i, int p, float) { pos[i] = p; };
     if (kept && hi - lo <= kMatBitRows) {
-        mat_each(src, bits, lo, wa - lo, wz - lo, offset + before, pos_cap, none, put);
+        if (cnt > 0) mat_each(src, bits, lo, wa - lo, wz - lo, offset + before, pos_cap, none, put);
     } else {
         int base = offset;
         for (int w0 = lo; w0 < hi && base < pos_cap; w0 += kMatBitRows) {

@@ -25,6 +25,9 @@ struct ScanSource {
     static constexpr int kThreads = kMatThreads, kFewB = kMatMidB;
     static constexpr int kWideRows = 1024;  // 131072 positions: below, 8 CTAs are as fast as 16
     static constexpr bool kLaneMajor = true;
+    // most rows of a scan hold no match and need no ballots (4 x 262144 tokens of
+    // text 7.8 -> 7.3 us, no match in 2000 tokens 3.6 -> 3.4; 0.03 more where all do)
+    static constexpr bool kSparse = true;
     static constexpr bool kBound = true;
     ScanPos at;
     __device__ __forceinline__ int pos(int row, int lane, int e) const { return (int)(at.quad(row, lane) + (uint32_t)e); }
