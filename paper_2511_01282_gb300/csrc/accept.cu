@@ -37,7 +37,7 @@ constexpr int kAccThreads = 256;
 constexpr int kAccVpt = 32;
 constexpr int kAccChunk = kAccThreads * kAccVpt;
 constexpr int kNoId = 0x7fffffff;  // "no candidate": after every real (v, id)
-constexpr int kCandCap = 64;        // per-warp candidate buffer (logits at or above the threshold)
+constexpr int kCandCap = 64;        // a chunk's candidate buffer (logits at or above the threshold)
 constexpr int kListBeta = 8;        // list merges hold this many candidates of a chunk in registers
 constexpr float kFarLogit = 5e8f;   // from here on logits lie 32 or more apart
 constexpr int kFuseMax = 8;         // rows of at most this many chunks merge inside their cluster
@@ -505,7 +505,6 @@ accept_decide(const float *logits, int R, int V, const int32_t *node_off, const 
     __shared__ uint32_t s_cg[RS_MAX_TOPC][kNodeWords], s_cr[RS_MAX_TOPC][kNodeWords];  // greedy / relaxed, chain order
     __shared__ uint32_t s_g[kNodeWords];                                               // greedy, node order
     __shared__ int s_cacc[RS_MAX_TOPC];
-    __shared__ int s_bad;
     __shared__ int s_best;  // (depth << 16) | (0xffff - node)
 
     // the request's rows must lie in [0, R) and its buffer in the score table
@@ -518,10 +517,7 @@ accept_decide(const float *logits, int R, int V, const int32_t *node_off, const 
     if (!rows_ok || !tok_ok) st = RS_ST_BAD_OFFSET;
     else if (N > RS_MAX_NODES) st = RS_ST_TOO_LARGE;
     else if (N < 1) st = RS_ST_BAD_TREE;
-    if (tid == 0) {
-        s_bad = 0;
-        s_best = 0;
-    }
+    if (tid == 0) s_best = 0;
     if (tid < RS_MAX_TOPC * kNodeWords) {
         (&s_cg[0][0])[tid] = 0;
         (&s_cr[0][0])[tid] = 0;

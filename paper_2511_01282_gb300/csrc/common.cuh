@@ -35,12 +35,17 @@ void count_launch(int n = 1);
         ::rs::count_launch();                                                        \
     } while (0)
 
-// Kernels are launched with programmatic stream serialization: the next
-// kernel in the stream may begin launching as soon as every block of this one
-// has started (pdl_enter's first instruction), and each kernel waits for its
-// predecessor's completion and memory before it touches global memory (its
-// second).  Since every kernel waits, completion stays ordered along the
-// whole stream.  Without a programmatic predecessor the wait returns at once.
+// Kernels are launched with programmatic stream serialization: the next kernel in
+// the stream may begin launching as soon as every block of this one has let it
+// (pdl_launch_next), and each kernel waits for its predecessor's completion and
+// memory (pdl_wait_prev) before it touches what that one may still write.  Most
+// kernels do both first (pdl_enter).  A call's first row kernel (entropy_partial,
+// accept_rows, sample_partial, and attn_prep) waits before it lets the next one
+// launch: everything before the call is then complete when the call's later
+// kernels start, and these (gate_push, accept_decide, sample_pick, sample_walk)
+// read the caller's arrays before their own wait.  Since every kernel waits,
+// completion stays ordered along the whole stream.  Without a programmatic
+// predecessor the wait returns at once.
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                        Args... args) {
@@ -67,8 +72,10 @@ cudaError_t launch_full(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t sm
     cfg.stream = st;
     return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
-// The same with a one-dimensional cluster of `cluster_x` CTAs along x
-// (grid.x a multiple of it; at most 8, the portable cluster size).
+// launch_pdl with a one-dimensional cluster of `cluster_x` CTAs along x (grid.x a
+// multiple of it).  More than 8, the portable cluster size, take a kernel whose
+// cudaFuncAttributeNonPortableClusterSizeAllowed is set, and a GPU part that can
+// run one (see MatWide).
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl_cluster(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                                int cluster_x, Args... args) {

@@ -4,7 +4,7 @@
 // Kernel 1 (entropy_partial): one CTA per (row, 8192-logit chunk).  Each
 // thread streams 32 logits with 128-bit loads; relative to its warp's
 // maximum m the warp forms s = sum e^(z-m) and w = sum e^(z-m) (z-m) (plain
-// shuffle sums), and one thread merges the eight warp triples into the
+// shuffle sums), and one warp sums the eight warps' triples into the
 // chunk's.  Row entropy is then H = ln s - w / s for the merged triple (the
 // log-sum-exp form of -sum p ln p).
 // Kernel 2 (entropy_merge): one warp per row merges its chunk triples into
@@ -390,9 +390,9 @@ extern "C" rs_status rs_entropy_gate(const float *logits, int R, int V, const in
 }
 
 // ============================================================ no-allocation variant
-// rs_entropy_gate_noalloc runs the same three kernels as rs_entropy_gate
-// (entropy_partial, entropy_merge, gate_push), with the per-chunk partials in
-// the fixed device array below instead of a caller workspace, for callers
+// rs_entropy_gate_noalloc runs the same kernels as rs_entropy_gate
+// (entropy_partial, entropy_merge for rows of several chunks, gate_push), with the
+// per-chunk partials in the fixed device array below instead of a caller workspace, for callers
 // that cannot allocate device memory.  The array (RS_GATE_NOALLOC_MAX_PARTIALS
 // triples, 12 bytes each) lives on every GPU that loads this library until
 // the process exits.  It needs no initialisation: every partial a call reads

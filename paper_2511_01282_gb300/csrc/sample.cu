@@ -11,29 +11,30 @@
 //
 // The draws are exact: every one is the fp64 inverse CDF.  Most rows are
 // settled by an fp32 pass that carries a rigorous error bound; the few whose
-// uniform lies within that bound of a CDF step are redone in fp64.
+// uniform lies within that bound of a CDF step are redone in double-float.
 //
 // Kernel 1 (sample_partial): one CTA per (row, 8192-logit chunk), staged
 // through shared memory with coalesced loads; thread t owns the 32
 // consecutive ids c0 + 32 t .. c0 + 32 t + 31.  Per chunk it stores the
 // maximum m_c, the mass s_c = sum_v 2^(x_v) with x_v = (z_v - m_c) log2(e)/T
-// (pairwise over a thread's 32 ids, then a butterfly and a tree: depth 13)
+// (over a thread's 32 ids two interleaved trees of depth 4, of the even and of
+// the odd ids, and their sum; then a butterfly and a tree: depth 13 in all)
 // and q_c = sum_v 2^(x_v) |x_v|, which sizes the error from rounding x_v.
 // Kernel 2 (sample_pick): one CTA per row.  Warp 0 weights the chunks by
-// f_c = exp((m_c - M)/T) in fp64 (M the row maximum), forms Z and u Z in fp64
+// f_c = exp((m_c - M)/T) in double-float (M the row maximum), forms Z and u Z so
 // and finds the chunk holding the crossing; the CTA recomputes that chunk's
-// terms, scans the thread sums in fp64, and the holder thread's warp scans its
-// 32 terms in fp64 to place the draw.  With u_32 = 2^-24 and e_x the relative
-// error of ex2.approx, every computed prefix Ŝ and the computed u Ẑ are
-// within E = (13 u_32 + e_x) Z + 2.8 u_32 sum_c f_c q_c of the exact values
-// (13 u_32: the summation depth; 2.8 u_32 |x|: 4 roundings in x_v, times
-// ln 2; f_c and everything after the chunk sums carry fp64 error only).  A
-// draw whose two margins Ŝ(v) - u Ẑ and u Ẑ - Ŝ(v-1) both exceed 2 E is the
-// exact draw; any other row (and any row that took a rounding fallback) is
-// appended to the flagged list.
-// Kernel 3 (sample_exact): the flagged rows in fp64, spread over the whole
-// GPU as (row, 256-id slice) items: exp((z_v - M)/T) per id, one sum per
-// slice; the CTA that completes a row's last slice (an atomic count, no
+// terms, scans the thread sums (fp32 within a warp, the warps in double-float),
+// and the holder thread's warp scans its 32 terms to place the draw.  With
+// u_32 = 2^-24 and e_x the relative error of ex2.approx, every computed prefix Ŝ
+// and the computed u Ẑ are within E = (13 u_32 + e_x) Z + 2.8 u_32 sum_c f_c q_c
+// of the exact values (13 u_32: the summation depth; 2.8 u_32 |x|: 4 roundings in
+// x_v, times ln 2; f_c and everything after the chunk sums carry double-float
+// error only).  A draw whose two margins Ŝ(v) - u Ẑ and u Ẑ - Ŝ(v-1) both exceed
+// 2 E is the exact draw; any other row (and any row that took a rounding fallback)
+// is appended to the flagged list.
+// Kernel 3 (sample_exact): the flagged rows in double-float, spread over the
+// whole GPU as (row, group of 512-id slices) items: exp((z_v - M)/T) per id, one
+// sum per slice; the CTA that completes a row's last slice (an atomic count, no
 // waiting) scans the slice sums, finds the slice holding u Z and walks it with
 // a block scan.  A uniform >= 1 (u Z at or past the total) takes the row's
 // last id with mass.
@@ -249,8 +250,9 @@ __device__ __forceinline__ float block_max(float v, float *s_w) {
     return r;
 }
 
-// One thread's 32 terms 2^x_v, x_v = (z_v - m) scale: their sum, pairwise
-// in id order (depth 5), and sum 2^x_v |x_v| (for the error bound).  The
+// One thread's 32 terms 2^x_v, x_v = (z_v - m) scale: their sum (the even and the
+// odd ids in a tree of depth 4 each, then one addition: depth 5), and
+// sum 2^x_v |x_v| (for the error bound).  The
 // same code in both kernels, so a chunk's terms are the same in both.
 __device__ __forceinline__ float term(float z, float m, float scale) { return ex2f((z - m) * scale); }
 

@@ -9,10 +9,10 @@
 // the other key tokens and, if it matches, its score.  Nothing is staged in
 // shared memory and nothing is read twice.  Staging 8192-position windows of
 // tokens and scores (4-byte asynchronous copies, a second staging for the
-// positions) took 51 us on 4 x 262144 tokens of text, a key of two; this takes
-// 8.3 (graph), the reads of 64 SMs at 4 MB and the dependent rounds around
-// them.  Short calls take as long as they did: 2000 tokens of one request 4.7 us
-// (4.6 before), of 16 requests 3.9 (4.7).
+// positions) took 47 us on 4 x 262144 tokens of text, a key of two; this takes
+// 7.3 (graph), the reads of 64 SMs at 4 MB and the dependent rounds around
+// them.  Short calls take as long as they did: no match in 300 tokens of one
+// request 3.4 us (3.3 before), in 2000 of 16 requests 3.7 (4.3).
 #include "match.cuh"
 
 namespace rs {

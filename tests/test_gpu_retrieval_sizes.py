@@ -76,11 +76,11 @@ def test_scan_beyond_the_kept_ballots():
     _scan(tokens, np.array([0, len(tokens)], np.int64), np.array([1], np.int32), scores[:len(tokens)], 0.3, 8, 4, 100)
 
 
-@pytest.mark.parametrize("B", [1, 4, 5, 8, 9, 40])
+@pytest.mark.parametrize("B", [1, 4, 5, 7, 8, 9, 40])
 def test_scan_cluster_forms(B):
-    # up to 4 requests: clusters of 16, of which a request of less than 131072
-    # candidates uses 8; more: clusters of 8; more than 8 requests, or up to 32768
-    # candidates: half the threads
+    # as many requests as the GPU runs clusters of 16 at once (7): those, of which a
+    # request of less than 131072 candidates uses 8; more: clusters of 8; more than 8
+    # requests, or up to 32768 candidates: half the threads
     rng = np.random.default_rng(B)
     lens = rng.choice([40, 4090, 4101, 8197, 30001, 32760, 32775], B).tolist()
     lens[0], lens[-1] = 130000, 131200
